@@ -1,0 +1,1152 @@
+// Bit-stream kernels: C^(i) and sum_i D^(i) for every feature count and code width that the Int4 kernels for
+// multiples of 8 do not take -- code widths other than 4 bits (the method "at lower and higher precision", paper
+// Section 4 / Figure 3), and any E, k or row stride (k = E/64 is a multiple of 8 for few widths E).
+//
+// A token's codes are L*B bits long (L = E - k slots of B bits), so rows start at any bit of the code stream and
+// the 8 adjacent slots of a group lie across its words.  Both kernels therefore work on a group of 8 slots per
+// thread, as the Int4 kernels do, and put the bit offset into shared memory, where an unaligned field costs one
+// funnel shift:
+//   quantise    a block quantises 8 rows into per-row bit strings in shared memory, then writes the tile's bytes
+//               (8*L*B bits are a whole number of bytes) as consecutive 32-bit words funnelled out of the strings;
+//   dequantise  a block's panel of code words comes in by 16-byte copies from the aligned place at or below each
+//               row's first bit; a thread funnels its group's bits out of the landed words.
+// Arithmetic as everywhere: u = fl(x * inv_s), clamp, round to nearest even; acc = fma(code, s, acc) over the
+// devices in ascending order.
+#include <cuda_bf16.h>
+
+#include "tpq_internal.h"
+
+namespace {
+
+__device__ __forceinline__ uint32_t lop3_and_or(uint32_t x, uint32_t mask, uint32_t magic)
+{
+    uint32_t d;
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(x), "r"(mask), "r"(magic));
+    return d;
+}
+
+// ----------------------------------------------------------------------------------------------
+// Quantise + pack
+// ----------------------------------------------------------------------------------------------
+constexpr int QS_MAX_BATCH = 16;  // shards of one launch
+constexpr int QS_ROWS = 8;        // rows of a tile: 8*L*B bits are whole bytes for every L and B
+constexpr int QS_THREADS = 320;   // most threads of a block; four blocks share an SM, so that one's barriers hide
+                                  // behind the others' loads
+
+struct QSParams {
+    const uint16_t *y[QS_MAX_BATCH];
+    uint8_t *payload[QS_MAX_BATCH];
+    int64_t T, stride, lp_bytes, n_tiles;
+    int E, k, L, n_holes;
+    int row_words;       // words of a row's bit string in shared memory (even)
+    const float *inv_s;  // [n][E], first shard of the batch
+    const uint32_t *grp;
+    const int32_t *hp_idx, *hole, *filler;
+};
+
+__host__ __device__ inline int qs_row_words(int L, int B) { return ((((L + 7) / 8) * B + 3) / 4 + 2) & ~1; }
+inline size_t qt_smem_bytes(int L, int B) { return (size_t)QS_ROWS * qs_row_words(L, B) * 4; }
+
+// the code of one value in the low bits (two's complement; bits above B are garbage)
+template <int B>
+__device__ __forceinline__ uint32_t qs_code(float x, float inv)
+{
+    constexpr float lo = -(float)(1 << (B - 1)), hi = (float)((1 << (B - 1)) - 1);
+    const float u = fminf(fmaxf(__fmul_rn(x, inv), lo), hi);
+    return __float_as_uint(__fadd_rn(u, 12582912.0f));  // + 1.5 * 2^23: nearest even, the code in the low bits
+}
+
+// 8 values (one uint4 of BF16) -> 4 codes in each of two 32-bit halves, packed from bit 0.  As in the Int4
+// kernels the patterns 0x4B400000 + code are summed with one shift-add each and the constant part is removed at
+// the end: what is left is the sum of the signed codes times their weights, and adding the weights' 2^(B-1)
+// makes the digits non-negative, so that they do not borrow from one another.
+template <int B>
+__device__ __forceinline__ void qs_quant8(const uint4 v, const float2 (&inv)[4], uint32_t (&half)[2])
+{
+    constexpr float lo = -(float)(1 << (B - 1)), hi = (float)((1 << (B - 1)) - 1);
+    constexpr uint32_t ones = 1u + (1u << B) + (1u << (2 * B)) + (1u << (3 * B));
+    constexpr uint32_t sign = ones << (B - 1);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t acc = 0;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t x = w[2 * h + i];
+            float2 u = __fmul2_rn(make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u)), inv[2 * h + i]);
+            u.x = fminf(fmaxf(u.x, lo), hi);
+            u.y = fminf(fmaxf(u.y, lo), hi);
+            const float2 r = __fadd2_rn(u, make_float2(12582912.0f, 12582912.0f));
+            acc += __float_as_uint(r.x) << (2 * i * B);
+            acc += __float_as_uint(r.y) << ((2 * i + 1) * B);
+        }
+        half[h] = (acc - 0x4B400000u * ones + sign) ^ sign;
+    }
+}
+
+// B bytes of codes (the two halves of a group) -> shared memory, B-byte aligned
+template <int B>
+__device__ __forceinline__ void qs_store_group(uint8_t *dst, const uint32_t (&half)[2])
+{
+    const uint64_t bits = (uint64_t)half[0] | ((uint64_t)half[1] << (4 * B));
+    if (B == 8) {
+        *reinterpret_cast<uint2 *>(dst) = make_uint2(half[0], half[1]);
+    } else if (B == 4) {
+        *reinterpret_cast<uint32_t *>(dst) = (uint32_t)bits;
+    } else if (B == 2 || B == 6) {
+#pragma unroll
+        for (int j = 0; j < B / 2; ++j) reinterpret_cast<uint16_t *>(dst)[j] = (uint16_t)(bits >> (16 * j));
+    } else {
+#pragma unroll
+        for (int j = 0; j < B; ++j) dst[j] = (uint8_t)(bits >> (8 * j));
+    }
+}
+
+// A tile's bit strings (rows of LB bits, RW words apart) -> bytes from b0 on of a payload's code section.  Row r's
+// words are those that start in it: from its bit o on, all funnelled by the same shift; the last one takes its upper
+// bits from the next row (rows are at least 32 bits long).  A word shared with a neighbouring tile is written by
+// bytes; the last tile writes the section's zero padding.
+__device__ __forceinline__ void qs_write_tile(uint8_t *pl, const uint32_t *strings, int RW, int LB, int64_t b0, int rows, bool last,
+                                              int64_t lp_bytes, int tid, int NT)
+{
+    const int lead = (int)(b0 & 3);  // bytes of the first word that belong to the tile before
+    uint32_t *out = reinterpret_cast<uint32_t *>(pl) + ((b0 + 3) >> 2);
+    if (lead && tid < 4 - lead) pl[b0 + tid] = (uint8_t)(strings[0] >> (8 * tid));
+    int o = (32 - 8 * lead) & 31;
+    for (int r = 0; r < rows; ++r) {
+        const uint32_t *const s = strings + r * RW;
+        const int n = (LB - o + 31) >> 5;  // words that start in the row
+        for (int j = tid; j < n; j += NT) {
+            const int at = o + 32 * j, left = LB - at;
+            uint32_t v = __funnelshift_r(s[at >> 5], s[(at >> 5) + 1], at & 31);
+            if (left < 32) {
+                v &= (1u << left) - 1u;
+                if (r + 1 < rows) {
+                    v |= s[RW] << left;
+                } else if (!last) {  // the tile's last word is the next tile's first one
+                    for (int c = 0; c < left >> 3; ++c) reinterpret_cast<uint8_t *>(out + j)[c] = (uint8_t)(v >> (8 * c));
+                    continue;
+                }
+            }
+            out[j] = v;
+        }
+        out += n;
+        o += 32 * n - LB;
+    }
+    if (last)
+        for (uint32_t *w = out + tid; w < reinterpret_cast<uint32_t *>(pl + lp_bytes); w += NT) *w = 0u;
+}
+
+// Any E and row stride (and rows too long for the ring of the pipelined kernel below).
+// One tile of QS_ROWS rows of one shard per block (grid = (tiles, shards)); a row's bit string is written to shared
+// memory group by group, the fillers' codes are put into the holes, and the strings leave as words of the stream.
+// VEC: rows are 16-byte aligned and whole groups long (E and stride multiples of 8).
+template <int B, bool VEC>
+__global__ void __launch_bounds__(QS_THREADS, VEC ? 4 : 2) quantize_stream_tile(const QSParams p)
+{
+    extern __shared__ __align__(16) uint32_t qs_smem[];  // QS_ROWS bit strings
+    const int tid = threadIdx.x, NT = blockDim.x;
+    const int E = p.E, k = p.k, L = p.L, G = (L + 7) >> 3, RW = p.row_words, n_holes = p.n_holes;
+    const int LB = L * B;  // bits of a row
+    const int64_t tile = blockIdx.x, t0 = tile * QS_ROWS;
+    const int rows = (int)(p.T - t0 < QS_ROWS ? p.T - t0 : QS_ROWS);
+    const uint16_t *const y = p.y[blockIdx.y] + t0 * p.stride;
+    uint8_t *const pl = p.payload[blockIdx.y];
+    const float *const inv_s = p.inv_s + (size_t)blockIdx.y * E;
+    tpq_grid_dep_launch();
+
+    // this thread's first item of each kind: a hole's filler value, a selected feature's value
+    const int f_r = n_holes ? tid / n_holes : QS_ROWS, f_h = n_holes ? tid - f_r * n_holes : 0;
+    int f_col = 0, f_slot = 0;
+    float f_inv = 0.0f;
+    if (f_r < rows) {
+        f_col = __ldg(p.filler + f_h);
+        f_slot = __ldg(p.hole + f_h);
+        f_inv = __ldg(inv_s + f_col);
+    }
+    const int s_r = k ? tid / k : QS_ROWS;
+    const int s_col = s_r < rows ? __ldg(p.hp_idx + (tid - s_r * k)) : 0;
+
+    tpq_grid_dep_wait();  // the input and the payload buffer may still be in use by the kernel ahead
+    uint32_t f_x = 0;
+    uint16_t s_x = 0;
+    if (f_r < rows) f_x = y[f_r * p.stride + f_col];
+    if (s_r < rows) s_x = y[s_r * p.stride + s_col];
+    for (int g = tid; g < G; g += NT) {
+        float2 inv[4];
+        if (VEC) {
+            const float4 a = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g));
+            const float4 b = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g + 4));
+            inv[0] = make_float2(a.x, a.y); inv[1] = make_float2(a.z, a.w);
+            inv[2] = make_float2(b.x, b.y); inv[3] = make_float2(b.z, b.w);
+        } else {
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+                inv[n] = make_float2(8 * g + 2 * n < E ? __ldg(inv_s + 8 * g + 2 * n) : 0.0f,
+                                     8 * g + 2 * n + 1 < E ? __ldg(inv_s + 8 * g + 2 * n + 1) : 0.0f);
+        }
+        const uint32_t mask = __ldg(p.grp + g) & 0xFFu;
+        const uint16_t *src = y + 8 * g;
+        uint8_t *dst = reinterpret_cast<uint8_t *>(qs_smem) + g * B;
+#pragma unroll
+        for (int r0 = 0; r0 < QS_ROWS; r0 += 4) {
+            if (r0 >= rows) break;
+            uint4 v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {  // all loads first; rows past the end re-read the last row
+                if (VEC) {
+                    v[r] = __ldg(reinterpret_cast<const uint4 *>(src));
+                } else {
+                    uint32_t x[8];
+#pragma unroll
+                    for (int n = 0; n < 8; ++n) x[n] = 8 * g + n < E ? src[n] : 0u;
+                    v[r] = make_uint4(x[0] | x[1] << 16, x[2] | x[3] << 16, x[4] | x[5] << 16, x[6] | x[7] << 16);
+                }
+                if (r0 + r + 1 < rows) src += p.stride;
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                uint32_t half[2];
+                qs_quant8<B>(v[r], inv, half);
+                if (mask) {  // the holes' codes come later
+#pragma unroll
+                    for (int n = 0; n < 8; ++n)
+                        if (mask & (1u << n)) half[n >> 2] &= ~(((1u << B) - 1u) << ((n & 3) * B));
+                }
+                qs_store_group<B>(dst + (r0 + r) * RW * 4, half);
+            }
+        }
+    }
+    __syncthreads();
+    // fillers' codes into the holes (two holes may share a word), selected features to the BF16 block
+    auto fill = [&](int r, int slot, uint32_t x, float inv) {
+        const uint32_t q = qs_code<B>(__uint_as_float(x << 16), inv) & ((1u << B) - 1u);
+        const uint32_t bit = (uint32_t)slot * B, sh = bit & 31;
+        uint32_t *const w = qs_smem + r * RW + (bit >> 5);
+        atomicOr(w, q << sh);
+        if (32 % B != 0 && sh + B > 32) atomicOr(w + 1, q >> (32 - sh));
+    };
+    if (f_r < rows) fill(f_r, f_slot, f_x, f_inv);
+    for (int i = tid + NT; i < rows * n_holes; i += NT) {
+        const int r = i / n_holes, h = i - r * n_holes, f = __ldg(p.filler + h);
+        fill(r, __ldg(p.hole + h), y[r * p.stride + f], __ldg(inv_s + f));
+    }
+    uint16_t *const hp_out = reinterpret_cast<uint16_t *>(pl + p.lp_bytes) + t0 * k;
+    if (s_r < rows) hp_out[tid] = s_x;
+    for (int i = tid + NT; i < rows * k; i += NT) {
+        const int r = i / k;
+        hp_out[i] = y[r * p.stride + __ldg(p.hp_idx + (i - r * k))];
+    }
+    __syncthreads();
+    qs_write_tile(pl, qs_smem, RW, LB, tile * (int64_t)LB, rows, tile == p.n_tiles - 1, p.lp_bytes, tid, NT);
+}
+
+template <int B>
+cudaError_t launch_quantize_tile(const QSParams &p, bool vec, int threads, dim3 grid, cudaStream_t st)
+{
+    const size_t smem = qt_smem_bytes(p.L, B);
+    auto kern = vec ? quantize_stream_tile<B, true> : quantize_stream_tile<B, false>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return tpq_launch_pdl(kern, grid, dim3(threads), smem, st, p);
+}
+
+// The pipelined kernel for rows that bulk copies can fetch (E and stride multiples of 8) and whose ring fits.
+// As the Int4 kernel for multiples of 8 (quantize.cu): one persistent block per SM on a run of adjacent rows, a
+// producer warp that streams stages of QS_STAGE rows into a ring, consumer lanes that own a group of 8 features with
+// its steps in registers, holes patched through warp shuffles.  There is no barrier between the warps:
+//   a consumer warp packs its 32 groups' codes of a row into a bit string of its own in shared memory and writes the
+//   words of the stream that START in its groups; it needs up to 31 bits more for the last one, so its last one or two
+//   groups (qs_ahead) are the next warp's first ones, packed by both;
+//   the edge warp writes the words in which one row ends and the next begins (one code per lane: 16 of a row's last
+//   and 16 of its first, or-ed together), for every row of the block and the row ahead of it.
+// A block may therefore start at any row.  (Built before this and measured at 4 x 2048 x 5120, 51 selected: strings of
+// whole tiles with a barrier of all consumers per 4 rows 43 us; one tile of 8 rows per block, four blocks per SM, 29.5 us;
+// this kernel 26.9 us against 15.9 us for its bytes at 6.65 TB/s; the shape-generic kernel 114 us.
+// 3 bits 41.1 -> 28.4 us, 8 x 1000 x 4608 at 8 bits 39.5 -> 29.7 us.  115 warp instructions per 32 groups: the ALU pipe.)
+constexpr int QS_STAGE = 4;             // rows of a stage
+constexpr int QS_MAX_THREADS = 768;     // 80 registers a thread
+constexpr int QS_MAX_GPT = 2;           // groups of a consumer lane
+constexpr int QS_MAX_STAGES = 6;
+constexpr int QS_PREFETCH_ROWS = 8;     // rows whose bytes a block asks L2 for ahead of the dependency wait
+
+__host__ __device__ constexpr int qs_ahead(int B) { return B < 4 ? 2 : 1; }  // groups whose bits cover 31
+// words of a warp's bit string of one row (even; a funnel may look one word past the last group)
+__host__ __device__ constexpr int qs_warp_words(int B) { return 8 * B + 2; }
+
+struct QPipeParams {
+    QSParams q;
+    int bps;                 // blocks per shard
+    int nstage;
+    int64_t rows_per_block;
+    int *status;
+    // push mode (one shard, n_dst copies of its payload: q.payload[0 .. n_dst))
+    int n_dst;
+    uint32_t epoch;
+    uint32_t *arrived[QS_MAX_BATCH];
+    unsigned int *done;
+};
+
+// consumer warps for rows of G groups, gpt per lane
+inline int qs_warps(int G, int B, int gpt)
+{
+    const int own = (32 - qs_ahead(B)) * gpt;
+    return (G + own - 1) / own;
+}
+inline size_t qs_pipe_bytes(int E, int B, int warps, int gpt, int nstage)
+{
+    return (size_t)nstage * QS_STAGE * E * 2 + (size_t)warps * gpt * QS_STAGE * qs_warp_words(B) * 4 + (size_t)nstage * 16 +
+           256;  // (lanes with no word to write may look up to 64 words past their string's start)
+}
+
+template <int B, int GPT, bool PUSH>
+__global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipeParams pp)
+{
+    constexpr int OWN = 32 - qs_ahead(B), WW = qs_warp_words(B);
+    extern __shared__ __align__(128) uint8_t qs_pipe[];
+    __shared__ int s_failed;  // (push mode) a wait of this block ran out
+    const QSParams &p = pp.q;
+    // warp 0 is the producer, warp 1 the edge warp, then come the NT consumers: where several warps of a scheduler can
+    // issue, the first goes first, and the few instructions of these two must not wait behind the consumers' many
+    // (as last warps 27.3 us at 4 x 2048 x 5120, 51 selected; 27.0 us so)
+    const int NT = blockDim.x - 64, tid = (int)threadIdx.x - 64;
+    if (PUSH && threadIdx.x == 0) s_failed = 0;  // (ordered before any use by the barrier of the prologue)
+    const int E = p.E, k = p.k, L = p.L, G = (L + 7) >> 3, nstage = pp.nstage;
+    const int LB = L * B;  // bits of a row
+    const int sb = blockIdx.x / pp.bps, bx = blockIdx.x - sb * pp.bps;
+    const uint16_t *const y = p.y[sb];
+    const float *const inv_s = p.inv_s + (size_t)sb * E;
+    const uint32_t row_bytes = (uint32_t)E * 2u, stage_bytes = QS_STAGE * row_bytes;
+    uint8_t *const ring = qs_pipe;
+    uint32_t *const strings = reinterpret_cast<uint32_t *>(ring + (size_t)nstage * stage_bytes);
+    uint64_t *const full = reinterpret_cast<uint64_t *>(strings + (size_t)(NT / 32) * GPT * QS_STAGE * WW);
+    uint64_t *const empty = full + nstage;
+    const int64_t t_begin = (int64_t)bx * pp.rows_per_block;
+    const int rows_mine = (int)(p.T - t_begin < pp.rows_per_block ? p.T - t_begin : pp.rows_per_block);
+    const int lane = threadIdx.x & 31;
+
+    tpq_grid_dep_launch();
+    if (threadIdx.x < 32) {
+        // ---------------- producer warp
+        if (lane == 0) {
+            for (int s = 0; s < nstage; ++s) {
+                mbar_init(smem_u32(&full[s]), 1);
+                mbar_init(smem_u32(&empty[s]), NT / 32 + 1);
+            }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");  // the barriers exist
+        if (lane == 0 && p.stride == E) {  // a hint only: L2 is the point of coherence
+            const int rows = rows_mine < QS_PREFETCH_ROWS ? rows_mine : QS_PREFETCH_ROWS;
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(y + t_begin * p.stride), "r"(rows * row_bytes) : "memory");
+        }
+        tpq_grid_dep_wait();  // the input and the payload buffer may still be in use by the kernel ahead
+        int st = 0;
+        uint32_t parity = 1;
+        for (int it = 0, r0 = 0; r0 < rows_mine; ++it, r0 += QS_STAGE) {
+            const int rows = rows_mine - r0 < QS_STAGE ? rows_mine - r0 : QS_STAGE;
+            const uint32_t bar = smem_u32(&full[st]);
+            int ok = 1;
+            if (lane == 0) {
+                if (it >= nstage && !mbar_wait(smem_u32(&empty[st]), parity)) {
+                    atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
+                    ok = 0;
+                } else {
+                    mbar_expect_tx(bar, rows * row_bytes);
+                }
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            if (!ok) break;
+            const uint32_t dst = smem_u32(ring + (size_t)st * stage_bytes);
+            const uint16_t *const src = y + (t_begin + r0) * p.stride;
+            if (p.stride == E) {
+                if (lane == 0) bulk_g2s(dst, src, rows * row_bytes, bar);
+            } else if (lane < rows) {
+                bulk_g2s(dst + lane * row_bytes, src + lane * p.stride, row_bytes, bar);
+            }
+            if (++st == nstage) {
+                st = 0;
+                parity ^= 1u;
+            }
+        }
+        return;
+    }
+
+    int st = 0;
+    uint32_t parity = 0;
+    if (tid < 0) {
+        // ---------------- edge warp: lanes 0..15 hold a row's last 16 codes, lanes 16..31 its first 16
+        const int slot = lane < 16 ? L - 16 + lane : lane - 16;
+        const bool on = slot >= 0 && slot < L;
+        int f = 0;
+        float inv = 0.0f;
+        if (on) {  // the feature in the slot: itself, or the filler of a hole
+            const uint32_t gd = __ldg(p.grp + (slot >> 3));
+            f = slot;
+            if (gd >> (slot & 7) & 1u) f = __ldg(p.filler + (int)(gd >> 8) + __popc(gd & ((1u << (slot & 7)) - 1u)));
+            inv = __ldg(inv_s + f);
+        }
+        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+        auto code = [&](uint32_t x) { return on ? qs_code<B>(__uint_as_float(x << 16), inv) & ((1u << B) - 1u) : 0u; };
+        // the word in which a row ends after `in` bits (its codes `last` in lanes 0..15) and the next begins (`first`)
+        auto edge = [&](int in, int64_t w, uint32_t last, uint32_t first) {
+            const int at = lane < 16 ? in - (16 - lane) * B : in + (lane - 16) * B;  // the code's place in the word
+            const uint32_t q = lane < 16 ? last : first;
+            const uint32_t part = at >= 32 || at <= -B ? 0u : at >= 0 ? q << at : q >> -at;
+            const uint32_t word = __reduce_or_sync(0xffffffffu, part);
+            if (in && lane < (PUSH ? pp.n_dst : 1)) reinterpret_cast<uint32_t *>(p.payload[PUSH ? lane : sb])[w] = word;
+        };
+        uint32_t last = 0;
+        bool dead = false;
+        for (int r0 = 0; r0 < rows_mine; r0 += QS_STAGE) {
+            const int rows = rows_mine - r0 < QS_STAGE ? rows_mine - r0 : QS_STAGE;
+            if (!mbar_wait(smem_u32(&full[st]), parity)) {
+                atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
+                if (PUSH) s_failed = 1;
+                dead = true;
+            }
+            if (__any_sync(0xffffffffu, dead)) {
+                dead = true;
+                break;
+            }
+            // (the copies of this stage were issued behind the dependency wait, so this read is as well)
+            if (r0 == 0 && t_begin > 0) last = code(y[(t_begin - 1) * p.stride + f]);
+            const uint16_t *const stage = reinterpret_cast<const uint16_t *>(ring + (size_t)st * stage_bytes);
+            const int64_t bit0 = (t_begin + r0) * LB, w_stage = bit0 >> 5;
+            const int in0 = (int)(bit0 & 31);
+            uint32_t q[QS_STAGE];
+#pragma unroll
+            for (int r = 0; r < QS_STAGE; ++r) q[r] = stage[r * E + f];  // (rows past the stage's end: old bytes, unused)
+#pragma unroll
+            for (int r = 0; r < QS_STAGE; ++r) {
+                if (r >= rows) break;
+                const uint32_t first = code(q[r]);
+                if (r0 + r > 0 || t_begin > 0) edge((in0 + r * LB) & 31, w_stage + ((in0 + r * LB) >> 5), last, first);
+                last = first;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
+            if (++st == nstage) {
+                st = 0;
+                parity ^= 1u;
+            }
+        }
+        if (t_begin + rows_mine == p.T && !dead) {  // the shard's last word and the section's zero padding
+            edge((int)((p.T * (int64_t)LB) & 31), (p.T * (int64_t)LB) >> 5, last, 0u);
+            const int64_t w0 = (p.T * (int64_t)LB + 31) >> 5;
+            for (int d = 0; d < (PUSH ? pp.n_dst : 1); ++d)
+                if (w0 + lane < p.lp_bytes / 4) reinterpret_cast<uint32_t *>(p.payload[PUSH ? d : sb])[w0 + lane] = 0u;
+        }
+        if (PUSH) asm volatile("bar.sync 2, %0;" ::"r"(NT + 32) : "memory");
+        return;
+    }
+
+    // ---------------- consumers: constants (see quantize_tiled)
+    const int warp = tid >> 5;  // consumer warp
+    float2 inv[GPT][4];
+    uint32_t mask[GPT], w_off[GPT], f_sh[GPT][2], h_in[GPT][2], keep[GPT][2];
+    int hb[GPT], n_wh[GPT], src0[GPT];
+    float w_inv[GPT];
+    bool serial[GPT];
+    const int my_hp = tid < k ? __ldg(p.hp_idx + tid) : 0;
+#pragma unroll
+    for (int a = 0; a < GPT; ++a) {
+        const int g = (warp + a * (NT / 32)) * OWN + lane;
+        mask[a] = 0;
+        hb[a] = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) inv[a][i] = make_float2(0.0f, 0.0f);
+        if (g < G) {
+            const float4 i0 = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g));
+            const float4 i1 = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g + 4));
+            const uint32_t gd = __ldg(p.grp + g);
+            inv[a][0] = make_float2(i0.x, i0.y); inv[a][1] = make_float2(i0.z, i0.w);
+            inv[a][2] = make_float2(i1.x, i1.y); inv[a][3] = make_float2(i1.z, i1.w);
+            mask[a] = gd & 0xFFu;
+            if (8 * g + 8 > L) mask[a] &= (1u << (L - 8 * g)) - 1u;  // (features at or above L have no slot)
+            hb[a] = (int)(gd >> 8);
+        }
+        const int nh = __popc(mask[a]);
+        int incl = nh;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
+        }
+        src0[a] = incl - nh;
+        n_wh[a] = __shfl_sync(0xffffffffu, incl, 31);
+        const int hb_warp = __shfl_sync(0xffffffffu, hb[a], 0);
+        serial[a] = n_wh[a] > 32 || __any_sync(0xffffffffu, nh > 2);
+        w_off[a] = 0;
+        w_inv[a] = 0.0f;
+        if (lane < n_wh[a] && !serial[a]) {
+            const int f = __ldg(p.filler + hb_warp + lane);
+            w_off[a] = (uint32_t)f * 2u;
+            w_inv[a] = __ldg(inv_s + f);
+        }
+        keep[a][0] = keep[a][1] = 0xFFFFFFFFu;
+        f_sh[a][0] = f_sh[a][1] = 0;
+        h_in[a][0] = h_in[a][1] = 0;
+        uint32_t m = mask[a];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (!m) break;
+            const int n = __ffs(m) - 1;
+            const uint32_t sh = (uint32_t)((n & 3) * B), field = ((1u << B) - 1u) << sh;
+            f_sh[a][h] = sh;
+            h_in[a][h] = n < 4 ? 1u : 2u;  // 0: no such hole, 1: in the lower half, 2: in the upper one
+            keep[a][0] &= n < 4 ? ~field : 0xFFFFFFFFu;
+            keep[a][1] &= n < 4 ? 0xFFFFFFFFu : ~field;
+            m &= m - 1;
+        }
+    }
+    asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");  // the producer has set up the barriers
+
+    for (int r0 = 0; r0 < rows_mine; r0 += QS_STAGE) {
+        const int rows = rows_mine - r0 < QS_STAGE ? rows_mine - r0 : QS_STAGE;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), parity))) {
+            atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
+            if (PUSH) s_failed = 1;
+            break;
+        }
+        const uint8_t *const stage8 = ring + (size_t)st * stage_bytes;
+        const int64_t bit0 = (t_begin + r0) * LB, w_stage = bit0 >> 5;  // the stage's first bit, the word it lies in ...
+        const int in0 = (int)(bit0 & 31);                               // ... and its place there
+#pragma unroll
+        for (int a = 0; a < GPT; ++a) {
+            const int wg = warp + a * (NT / 32);  // this warp's place among the row's
+            const int g = wg * OWN + lane;
+            const uint8_t *const src = stage8 + (g < G ? 16 * g : 0);
+            uint32_t *const ws = strings + (size_t)(warp * GPT + a) * (QS_STAGE * WW);
+            // the words that start in this warp's own groups and end in the row, relative to the stage's first word:
+            // string bit `o` is the first word boundary, the same for every lane
+            const int a0 = wg * (OWN * 8 * B);  // the string's first bit in the row
+            const int a1 = a0 + OWN * 8 * B < LB - 31 ? a0 + OWN * 8 * B : LB - 31;
+            auto put = [&](int r, int j, int o, uint32_t word) {
+                if (a0 + o + 32 * (lane + 32 * j) < a1) {
+                    const uint32_t w = ((uint32_t)(in0 + r * LB + a0 + 31) >> 5) + lane + 32 * j;
+                    for (int d = 0; d < (PUSH ? pp.n_dst : 1); ++d)
+                        (reinterpret_cast<uint32_t *>(p.payload[PUSH ? d : sb]) + w_stage)[w] = word;
+                }
+            };
+            auto row_o = [&](int r) { return 31 - ((in0 + r * LB + a0 + 31) & 31); };
+            // a row's codes: at 4 bits a group is a word, so its neighbour's comes by a shuffle; else to the bit string
+            auto emit = [&](int r, const uint32_t (&half)[2], bool store) {
+                if (B == 4) {
+                    const uint32_t own = half[0] | half[1] << 16, next = __shfl_down_sync(0xffffffffu, own, 1);
+                    const int o = row_o(r);
+                    if (store) put(r, 0, o, __funnelshift_r(own, next, o));
+                } else {
+                    qs_store_group<B>(reinterpret_cast<uint8_t *>(ws + r * WW) + lane * B, half);
+                }
+            };
+            if (!serial[a]) {
+                // QS_STAGE independent rows (a short stage's missing ones hold old bytes and are never written)
+                uint4 v[QS_STAGE];
+                uint32_t fx[QS_STAGE];
+#pragma unroll
+                for (int r = 0; r < QS_STAGE; ++r) {
+                    v[r] = *reinterpret_cast<const uint4 *>(src + r * row_bytes);
+                    fx[r] = *reinterpret_cast<const uint16_t *>(stage8 + r * row_bytes + w_off[a]);
+                }
+#pragma unroll
+                for (int r = 0; r < QS_STAGE; ++r) {
+                    uint32_t half[2];
+                    qs_quant8<B>(v[r], inv[a], half);
+                    if (n_wh[a]) {  // uniform over the warp
+                        const uint32_t qv = qs_code<B>(__uint_as_float(fx[r] << 16), w_inv[a]) & ((1u << B) - 1u);
+                        const uint32_t c0 = __shfl_sync(0xffffffffu, qv, src0[a]) << f_sh[a][0];
+                        const uint32_t c1 = __shfl_sync(0xffffffffu, qv, src0[a] + 1) << f_sh[a][1];
+                        half[0] = (half[0] & keep[a][0]) | (h_in[a][0] == 1u ? c0 : 0u) | (h_in[a][1] == 1u ? c1 : 0u);
+                        half[1] = (half[1] & keep[a][1]) | (h_in[a][0] == 2u ? c0 : 0u) | (h_in[a][1] == 2u ? c1 : 0u);
+                    }
+                    emit(r, half, r < rows);
+                }
+            } else {
+                for (int r = 0; r < rows; ++r) {  // a warp on the serial path: every hole patched by its owner
+                    uint32_t half[2];
+                    qs_quant8<B>(*reinterpret_cast<const uint4 *>(src + r * row_bytes), inv[a], half);
+                    uint32_t m = mask[a];
+                    for (int h = 0; m; ++h) {
+                        const int n = __ffs(m) - 1;
+                        m &= m - 1;
+                        const int f = __ldg(p.filler + hb[a] + h);
+                        const uint32_t x = *reinterpret_cast<const uint16_t *>(stage8 + r * row_bytes + 2 * f);
+                        const uint32_t c = qs_code<B>(__uint_as_float(x << 16), __ldg(inv_s + f)) & ((1u << B) - 1u);
+                        const uint32_t sh = (uint32_t)((n & 3) * B);
+                        if (n < 4) half[0] = (half[0] & ~(((1u << B) - 1u) << sh)) | (c << sh);
+                        else half[1] = (half[1] & ~(((1u << B) - 1u) << sh)) | (c << sh);
+                    }
+                    __syncwarp();
+                    emit(r, half, true);
+                }
+            }
+            if (B != 4) {
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < QS_STAGE; ++r) {
+                    if (r >= rows) break;
+                    const int o = row_o(r);
+                    const uint32_t *const s = ws + r * WW + lane;
+#pragma unroll
+                    for (int j = 0; j < (OWN * 8 * B + 1023) / 1024; ++j)
+                        put(r, j, o, __funnelshift_r(s[32 * j], s[32 * j + 1], o));
+                }
+                __syncwarp();
+            }
+        }
+        for (int h = tid; h < k; h += NT) {
+            const uint16_t *const x = reinterpret_cast<const uint16_t *>(stage8) + (h == tid ? my_hp : __ldg(p.hp_idx + h));
+            const int64_t at = (t_begin + r0) * k + h;
+            for (int d = 0; d < (PUSH ? pp.n_dst : 1); ++d) {
+                uint16_t *const o = reinterpret_cast<uint16_t *>(p.payload[PUSH ? d : sb] + p.lp_bytes) + at;
+                for (int r = 0; r < rows; ++r) o[r * k] = x[r * E];
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
+        if (++st == nstage) {
+            st = 0;
+            parity ^= 1u;
+        }
+    }
+    if constexpr (PUSH) {
+        // publication, as quantize_tiled: the block that counts last has observed every block's stores
+        asm volatile("bar.sync 2, %0;" ::"r"(NT + 32) : "memory");
+        if (tid == 0) {
+            __threadfence_system();
+            const unsigned int prev = atomicAdd(pp.done, s_failed ? 0x10001u : 1u);
+            if ((prev & 0xFFFFu) == gridDim.x - 1) {
+                *pp.done = 0u;
+                if ((prev >> 16) == 0 && !s_failed) {
+                    __threadfence_system();
+                    for (int d = 0; d < pp.n_dst; ++d)
+                        asm volatile("st.relaxed.sys.global.u32 [%0], %1;" ::"l"(pp.arrived[d]), "r"(pp.epoch) : "memory");
+                }
+            }
+        }
+    }
+}
+
+// groups per lane and ring depth of the pipelined kernel; false: the shape is the tile kernel's
+bool qs_pipe_plan(const tpq_ctx *c, int64_t stride, int *gpt_out, int *warps_out, int *nstage_out)
+{
+    const int E = c->E, G = (E - c->k + 7) / 8;
+    if (E % 8 || stride % 8) return false;
+    for (int gpt = 1; gpt <= QS_MAX_GPT; ++gpt) {
+        const int warps = qs_warps(G, c->bits, gpt);
+        if (warps * 32 + 64 > QS_MAX_THREADS) continue;
+        for (int n = QS_MAX_STAGES; n > 1; --n)
+            if (qs_pipe_bytes(E, c->bits, warps, gpt, n) <= (size_t)c->smem_optin) {
+                *gpt_out = gpt; *warps_out = warps; *nstage_out = n;
+                return true;
+            }
+    }
+    return false;
+}
+
+template <int B>
+cudaError_t launch_quantize_pipe(const QPipeParams &pp, bool push, int gpt, int threads, unsigned grid, size_t smem, cudaStream_t st)
+{
+    auto kern = gpt == 1 ? (push ? quantize_stream<B, 1, true> : quantize_stream<B, 1, false>)
+                         : (push ? quantize_stream<B, 2, true> : quantize_stream<B, 2, false>);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return tpq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, pp);
+}
+
+// ----------------------------------------------------------------------------------------------
+// Dequantise + reduce
+//
+// The layout of the copy-ring panel kernel (dequant.cu): a block owns a panel of CG groups and walks chunks of RC
+// rows; the panel's steps of all devices sit in shared memory in slot order; the code words of a step (NB devices
+// x RC rows) come by 16-byte asynchronous copies into a ring, one block barrier per step; a hole's lane holds its
+// filler feature's sum, which an item thread moves to its own column after the chunk's stores.  What differs is
+// the alignment: a segment starts at any bit, so the copies start at the 16-byte boundary at or below it and a
+// thread funnels its 8*B bits out of two (three) words; the shift is the same for all devices, so it is worked
+// out once per chunk and row.  Blocks are half the size, two to an SM, so that one's barrier hides behind the other's work.
+// Measured (before: the shape-generic kernel, or one thread per group with byte loads for other widths): 4 x 2048 x 5120
+// with 51 selected 91.7 -> 17.8 us, 3 bits 26.2 -> 16.5 us; 8 x 1000 x 4608 at 8 bits 20.1 -> 16.2 us; one block of 512
+// threads per SM 18.8, 16.9 and 22.1 us.  Bound by instruction issue (22 per 8 codes) and the chunk's barriers.
+// ----------------------------------------------------------------------------------------------
+constexpr int DS_THREADS = 256;  // two blocks share an SM, so that one's barrier hides behind the other's work
+constexpr int DS_CG = 64;        // groups of a panel
+constexpr int DS_R = 4;       // rows per thread
+constexpr int DS_STAGES = 4;  // ring depth (steps)
+
+__host__ __device__ constexpr int ds_nb(int B) { return B <= 4 ? 4 : 2; }  // devices per step
+
+struct DSParams {
+    const uint8_t *pl[TPQ_MAX_SHARDS];
+    int N, E, k, L;
+    int64_t T, lp_bytes, out_stride, n_chunks;
+    const float *s_slot;  // [N][E] steps in slot order
+    const uint32_t *grp;
+    const int32_t *lp_idx, *hp_idx, *filler;
+    int n_holes, panels, gy;
+    bool vec;  // 8 adjacent outputs are 16-byte aligned (E and the output stride multiples of 8)
+    void *out;
+    const float *bias;  // [E] added after the sum, or NULL
+    tpq_arrivals arr;   // arrival words to wait for before the first payload read (words == NULL: none)
+};
+
+__host__ __device__ constexpr int ds_seg_pieces(int B) { return DS_CG * B / 16 + 1; }
+__host__ __device__ constexpr size_t ds_stage_bytes(int B)
+{
+    return (size_t)ds_nb(B) * (DS_THREADS / DS_CG * DS_R) * ds_seg_pieces(B) * 16;
+}
+__host__ __device__ constexpr size_t ds_smem_bytes(int B, int N)
+{
+    return (size_t)N * DS_CG * 32 + DS_STAGES * ds_stage_bytes(B) + 16;  // (a funnel may look one word past the ring)
+}
+
+// bit position, inside the float's mantissa, at which code n of a half is decoded
+__host__ __device__ constexpr int ds_pos(int B, int n) { return (B <= 5 ? (n & 3) : (n & 1)) * B; }
+
+// 4 codes of a half (x: the half's bits from bit 0 on, more above), accumulated: (x & mask) | 0x4B000000 is the
+// float 2^23 + (code + 2^(B-1)) 2^pos once the sign bits are flipped; subtracting 2^23 + 2^(B-1+pos) is exact and the
+// steps are pre-divided by 2^pos, so the FMA rounds exactly like fma(code, s, acc).  A code must end below bit 23:
+// up to 5 bits all four do, wider ones take codes 2 and 3 from the half shifted down.
+template <int B>
+__device__ __forceinline__ void ds_decode4(uint32_t x, const float2 s01, const float2 s23, float2 &a01, float2 &a23)
+{
+    constexpr uint32_t m = (1u << B) - 1u;
+    constexpr uint32_t sign = (1u << (B - 1)) * (1u + (1u << B) + (1u << (2 * B)) + (1u << (3 * B)));
+    constexpr float b0 = -(8388608.0f + (float)(1u << (B - 1)));
+    constexpr float b1 = -(8388608.0f + (float)(1u << (2 * B - 1)));
+    x ^= sign;
+    const uint32_t x2 = B <= 5 ? x : x >> (2 * B);
+    constexpr int p2 = ds_pos(B, 2), p3 = ds_pos(B, 3);
+    constexpr float b2 = -(8388608.0f + (float)(1u << (B - 1 + p2)));
+    constexpr float b3 = -(8388608.0f + (float)(1u << (B - 1 + p3)));
+    const float2 f01 = make_float2(__uint_as_float(lop3_and_or(x, m, 0x4B000000u)),
+                                   __uint_as_float(lop3_and_or(x, m << B, 0x4B000000u)));
+    const float2 f23 = make_float2(__uint_as_float(lop3_and_or(x2, m << p2, 0x4B000000u)),
+                                   __uint_as_float(lop3_and_or(x2, m << p3, 0x4B000000u)));
+    a01 = __ffma2_rn(__fadd2_rn(f01, make_float2(b0, b1)), s01, a01);
+    a23 = __ffma2_rn(__fadd2_rn(f23, make_float2(b2, b3)), s23, a23);
+}
+
+__device__ __forceinline__ void ds_cp16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+template <bool FP32OUT>
+__device__ __forceinline__ void ds_store_one(void *out, int64_t off, float v)
+{
+    if (FP32OUT)
+        static_cast<float *>(out)[off] = v;
+    else
+        static_cast<__nv_bfloat16 *>(out)[off] = __float2bfloat16_rn(v);
+}
+
+template <int B, bool FP32OUT>
+__global__ void __launch_bounds__(DS_THREADS, 2) dequant_stream(const DSParams p)
+{
+    extern __shared__ __align__(128) uint8_t ds_smem[];
+    constexpr int NB = ds_nb(B), CG = DS_CG;
+    constexpr int RS = DS_THREADS / CG, RC = RS * DS_R;
+    constexpr int SEGC = ds_seg_pieces(B), SEGW = SEGC * 4;
+    constexpr int PIECES = NB * RC * SEGC;
+    constexpr int NCP = (PIECES + DS_THREADS - 1) / DS_THREADS;
+    constexpr uint32_t STAGE_BYTES = PIECES * 16;
+
+    if (p.arr.words) {  // (first thing, with no load of its own in flight)
+        tpq_block_wait_arrivals(p.arr);
+        __syncthreads();
+    }
+    const int N = p.N, E = p.E, k = p.k, L = p.L;
+    const uint32_t LB = (uint32_t)L * B;
+    const int tid = threadIdx.x;
+    float4 *const steps = reinterpret_cast<float4 *>(ds_smem);  // [N][2][CG]
+    uint8_t *const ring = ds_smem + (size_t)N * CG * 32;
+    const uint32_t ring_s = smem_u32(ring);
+    const int panel = blockIdx.x % p.panels, by = blockIdx.x / p.panels;
+    const int cg = tid & (CG - 1), rs = tid / CG;
+    const int g = panel * CG + cg;
+    const int lanes = L - 8 * g < 8 ? L - 8 * g : 8;  // slots of the thread's group (the last one may be short)
+    const uint32_t panel_bit = (uint32_t)panel * (CG * 8 * B);
+
+    // copy side: piece c = tid + j * DS_THREADS of a step is piece `within` of segment (device, row) and lands at
+    // byte 16 c of the stage
+    int cp_dev[NCP];
+    uint32_t cp_bit[NCP], cp_in[NCP];  // first bit of the segment relative to the chunk, byte inside the segment
+#pragma unroll
+    for (int j = 0; j < NCP; ++j) {
+        const int c = tid + j * DS_THREADS;
+        const int seg = c / SEGC, within = c - seg * SEGC;
+        const int i = seg / RC, row = seg - i * RC;
+        cp_dev[j] = c < PIECES ? i : -1;
+        cp_bit[j] = (uint32_t)row * LB + panel_bit;
+        cp_in[j] = (uint32_t)within * 16u;
+    }
+    int64_t ich = by;
+    int ib = 0;
+    const int nbatch = (N + NB - 1) / NB;
+    uint32_t idst = ring_s + (uint32_t)tid * 16u;
+    auto issue = [&]() {
+        if (ich < p.n_chunks) {
+            const int64_t bit = ich * RC * (int64_t)LB;
+            const int64_t base = (bit >> 3) & ~(int64_t)15;        // the chunk's 16-byte aligned start ...
+            const uint32_t rem = (uint32_t)(bit - base * 8);       // ... and its first bit behind it
+            const int64_t left = p.lp_bytes - base;
+            const uint32_t lim = (uint32_t)(left < (int64_t)0x7FFFFFF0 ? left : (int64_t)0x7FFFFFF0);
+            const int i0 = ib * NB;
+#pragma unroll
+            for (int j = 0; j < NCP; ++j) {
+                // pieces past the end of the code section (a multiple of 16 bytes) and devices past N are skipped;
+                // what they would have filled is never stored
+                const uint32_t at = ((((rem + cp_bit[j]) >> 3) & ~15u) + cp_in[j]);
+                if (cp_dev[j] >= 0 && i0 + cp_dev[j] < N && at + 16u <= lim)
+                    ds_cp16(idst + (uint32_t)(j * DS_THREADS * 16), p.pl[i0 + cp_dev[j]] + base + at);
+            }
+            if (++ib == nbatch) {
+                ib = 0;
+                ich += p.gy;
+            }
+            idst += STAGE_BYTES;
+            if (idst == ring_s + (uint32_t)tid * 16u + DS_STAGES * STAGE_BYTES) idst = ring_s + (uint32_t)tid * 16u;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");  // (possibly empty: keeps the count in step with the consumer)
+    };
+    for (int a = tid; a < N * CG; a += DS_THREADS) {
+        const int i = a / CG, c = a & (CG - 1), c0 = 8 * (panel * CG + c);
+        float s[8];
+        const float *const src = p.s_slot + (size_t)i * E + c0;
+        if (p.vec && c0 < L) {
+            const float4 u = __ldg(reinterpret_cast<const float4 *>(src)), v = __ldg(reinterpret_cast<const float4 *>(src) + 1);
+            s[0] = u.x; s[1] = u.y; s[2] = u.z; s[3] = u.w; s[4] = v.x; s[5] = v.y; s[6] = v.z; s[7] = v.w;
+        } else {
+#pragma unroll
+            for (int n = 0; n < 8; ++n) s[n] = c0 + n < L ? __ldg(src + n) : 0.0f;
+        }
+#pragma unroll
+        for (int n = 0; n < 8; ++n) s[n] *= 1.0f / (float)(1u << ds_pos(B, n));
+        steps[(2 * i) * CG + c] = make_float4(s[0], s[1], s[2], s[3]);
+        steps[(2 * i + 1) * CG + c] = make_float4(s[4], s[5], s[6], s[7]);
+    }
+    tpq_grid_dep_wait();  // the payloads and the output buffer may still be in use by the kernel ahead
+    tpq_grid_dep_launch();
+#pragma unroll
+    for (int s = 0; s < DS_STAGES - 1; ++s) issue();
+    const float4 *const my_steps = steps + cg;
+    const uint32_t *const ring_w = reinterpret_cast<const uint32_t *>(ring);
+    const uint32_t *sw = ring_w;
+
+    // Items (one per row of the chunk and selected feature): the panel's holes, ranks [hs, he); the last panel also
+    // takes the selected features at or above L, ranks [n_holes, k).
+    const int n_holes = p.n_holes;
+    const int hs = (int)(__ldg(p.grp + panel * CG) >> 8);
+    const int he = (panel == p.panels - 1) ? k : (int)(__ldg(p.grp + (panel + 1) * CG) >> 8);
+    const int n_it = he - hs;
+    const int items = RC * n_it;
+    const int my_r = (tid < items) ? tid / n_it : 0;
+    const int my_h = (tid < items) ? hs + (tid - my_r * n_it) : 0;
+    const int my_col = (tid < items) ? __ldg(p.hp_idx + my_h) : 0;
+    const int my_fcol = (tid < items && my_h < n_holes) ? __ldg(p.filler + my_h) : -1;
+    auto read_out = [&](int64_t at) -> float {  // the bits of an output element
+        if (FP32OUT) return __ldcg(static_cast<const float *>(p.out) + at);
+        return __uint_as_float((uint32_t)__ldcg(static_cast<const uint16_t *>(p.out) + at));
+    };
+    auto write_out = [&](int64_t at, float bits) {
+        if (FP32OUT)
+            static_cast<float *>(p.out)[at] = bits;
+        else
+            static_cast<uint16_t *>(p.out)[at] = (uint16_t)__float_as_uint(bits);
+    };
+    // an item's read of the hole's column is issued a step ahead of its stores (a store right behind the read of
+    // the same address would hold up the memory pipe until the read is done)
+    bool fl_on = false;
+    float fl_f = 0.0f, fl_v = 0.0f;
+    int64_t fl_row = 0;
+    auto flush = [&]() {
+        if (fl_on) {
+            if (my_fcol >= 0) write_out(fl_row + my_fcol, fl_f);
+            ds_store_one<FP32OUT>(p.out, fl_row + my_col, p.bias ? __fadd_rn(fl_v, __ldg(p.bias + my_col)) : fl_v);
+            fl_on = false;
+        }
+    };
+    auto fixup = [&](int64_t tcp, bool on, float v) {
+        if (on) {
+            fl_row = (tcp + my_r) * p.out_stride;
+            if (my_fcol >= 0) fl_f = read_out(fl_row + my_col);
+            fl_v = v;
+            fl_on = true;
+        }
+        for (int a = tid + DS_THREADS; a < items; a += DS_THREADS) {  // panels with more items than threads
+            const int r = a / n_it, h = hs + (a - r * n_it);
+            if (tcp + r >= p.T) break;
+            const int64_t off = p.lp_bytes + ((tcp + r) * k + h) * 2, orow = (tcp + r) * p.out_stride;
+            float u = 0.0f;
+            for (int i = 0; i < N; ++i)
+                u = __fadd_rn(u, __uint_as_float((uint32_t)__ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + off)) << 16));
+            const int col = __ldg(p.hp_idx + h);
+            if (h < n_holes) write_out(orow + __ldg(p.filler + h), read_out(orow + col));
+            ds_store_one<FP32OUT>(p.out, orow + col, p.bias ? __fadd_rn(u, __ldg(p.bias + col)) : u);
+        }
+    };
+    bool pend = false, pend_on = false;
+    float pend_v = 0.0f;
+    int64_t pend_tc = 0;
+
+    for (int64_t ch = by; ch < p.n_chunks; ch += p.gy) {
+        const int64_t tc = ch * RC, t0 = tc + rs * DS_R;
+        const bool it_on = tid < items && tc + my_r < p.T;
+        const int64_t it_off = p.lp_bytes + ((tc + my_r) * k + my_h) * 2;
+        float hv = 0.0f;
+        uint16_t hvv[NB] = {};
+        float2 acc[DS_R][4];
+        int wofs[DS_R];       // this thread's first word of row r inside a device's part of a stage ...
+        uint32_t wsh[DS_R];   // ... and the bit it starts at
+        const uint32_t rem = (uint32_t)((ch * RC * (int64_t)LB) & 127);
+#pragma unroll
+        for (int r = 0; r < DS_R; ++r) {
+            const int rowc = rs * DS_R + r;
+            const uint32_t bit = ((rem + (uint32_t)rowc * LB + panel_bit) & 127u) + (uint32_t)cg * (8 * B);
+            wofs[r] = rowc * SEGW + (int)(bit >> 5);
+            wsh[r] = bit & 31u;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) acc[r][h] = make_float2(0.0f, 0.0f);
+        }
+        const float4 *st4 = my_steps;
+        for (int i0 = 0; i0 < N; i0 += NB, st4 += NB * 2 * CG) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(DS_STAGES - 2) : "memory");
+            __syncthreads();  // the step has landed for everybody; the stage consumed last is free
+            issue();
+            flush();
+            if (pend) {  // (first step of a chunk) the barrier above is also behind the previous chunk's row stores
+                if (n_it > 0) fixup(pend_tc, pend_on, pend_v);
+                pend = false;
+            }
+            if (it_on) {  // add the values loaded a step ago (ascending device order), then load this step's
+                if (i0 > 0) {
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) hv = __fadd_rn(hv, __uint_as_float((uint32_t)hvv[i] << 16));
+                }
+#pragma unroll
+                for (int i = 0; i < NB; ++i)
+                    if (i0 + i < N) hvv[i] = __ldcs(reinterpret_cast<const uint16_t *>(p.pl[i0 + i] + it_off));
+            }
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+                if (i0 + i >= N) break;
+                const float4 a = st4[(2 * i) * CG], b = st4[(2 * i + 1) * CG];
+#pragma unroll
+                for (int r = 0; r < DS_R; ++r) {
+                    const uint32_t *const s = sw + i * RC * SEGW + wofs[r];
+                    const uint32_t lo = __funnelshift_r(s[0], s[1], wsh[r]);
+                    uint32_t hi;  // codes 4..7
+                    if (B <= 4)
+                        hi = lo >> (B < 8 ? 4 * B : 0);
+                    else {
+                        const uint32_t up = __funnelshift_r(s[1], s[2], wsh[r]);
+                        hi = B == 8 ? up : __funnelshift_r(lo, up, 4 * B & 31);
+                    }
+                    ds_decode4<B>(lo, make_float2(a.x, a.y), make_float2(a.z, a.w), acc[r][0], acc[r][1]);
+                    ds_decode4<B>(hi, make_float2(b.x, b.y), make_float2(b.z, b.w), acc[r][2], acc[r][3]);
+                }
+            }
+            sw += STAGE_BYTES / 4;
+            if (sw == ring_w + DS_STAGES * (STAGE_BYTES / 4)) sw = ring_w;
+        }
+        if (it_on) {  // the last step's values (a partial batch has fewer than NB of them)
+            const int nl = N - (N - 1) / NB * NB;
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (i < nl) hv = __fadd_rn(hv, __uint_as_float((uint32_t)hvv[i] << 16));
+        }
+        if (p.bias && lanes > 0) {
+            const uint32_t holes = __ldg(p.grp + g) & 0xFFu;
+            float b[8];  // lane n belongs to feature 8g+n, or, at a hole, to the filler whose codes sit in the slot
+#pragma unroll
+            for (int n = 0; n < 8; ++n)
+                b[n] = n < lanes ? __ldg(p.bias + ((holes & (1u << n)) ? __ldg(p.lp_idx + 8 * g + n) : 8 * g + n)) : 0.0f;
+#pragma unroll
+            for (int r = 0; r < DS_R; ++r)
+#pragma unroll
+                for (int h = 0; h < 4; ++h) acc[r][h] = __fadd2_rn(acc[r][h], make_float2(b[2 * h], b[2 * h + 1]));
+        }
+#pragma unroll
+        for (int r = 0; r < DS_R; ++r) {
+            if (t0 + r >= p.T) break;
+            const int64_t o = (t0 + r) * p.out_stride + 8 * (int64_t)g;
+            if (p.vec && lanes >= 8) {
+                if (FP32OUT) {
+                    float4 *const dst = reinterpret_cast<float4 *>(static_cast<float *>(p.out) + o);
+                    __stcs(dst, make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y));
+                    __stcs(dst + 1, make_float4(acc[r][2].x, acc[r][2].y, acc[r][3].x, acc[r][3].y));
+                } else {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const __nv_bfloat162 v = __floats2bfloat162_rn(acc[r][h].x, acc[r][h].y);
+                        w[h] = *reinterpret_cast<const uint32_t *>(&v);
+                    }
+                    __stcs(reinterpret_cast<uint4 *>(static_cast<uint16_t *>(p.out) + o), make_uint4(w[0], w[1], w[2], w[3]));
+                }
+            } else {
+#pragma unroll
+                for (int n = 0; n < 8; ++n)
+                    if (n < lanes) ds_store_one<FP32OUT>(p.out, o + n, (n & 1) ? acc[r][n >> 1].y : acc[r][n >> 1].x);
+            }
+        }
+        pend = true;
+        pend_on = it_on;
+        pend_v = hv;
+        pend_tc = tc;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    flush();
+    if (pend) {
+        __syncthreads();
+        if (n_it > 0) fixup(pend_tc, pend_on, pend_v);
+        flush();
+    }
+}
+
+template <int B>
+cudaError_t launch_dequant_stream(const DSParams &p, int fp32_out, cudaStream_t st)
+{
+    const size_t smem = ds_smem_bytes(B, p.N);
+    auto kern = fp32_out ? dequant_stream<B, true> : dequant_stream<B, false>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return tpq_launch_pdl(kern, dim3((unsigned)(p.panels * p.gy)), dim3(DS_THREADS), smem, st, p);
+}
+
+}  // namespace
+
+// Rows of at least 32 bits (a word of the stream spans two rows at most), bit strings that fit in shared memory,
+// bit offsets inside a tile or chunk that fit 32 bits.
+bool tpq_stream_ok(const tpq_ctx *c, int64_t T)
+{
+    const int64_t L = c->E - c->k;
+    return T > 0 && T < (int64_t)QS_ROWS * 0x7FFFFFFF && L * c->bits >= 32 && c->E <= (1 << 18) && qt_smem_bytes((int)L, c->bits) <= (size_t)c->smem_optin &&
+           ds_smem_bytes(c->bits, c->N) <= (size_t)c->smem_optin;
+}
+
+static cudaError_t launch_stream(const tpq_ctx *c, int shard0, int n, const void *const *ys, int64_t T, int64_t stride,
+                                 void *const *payloads, int n_dst, uint32_t *const *arrived, uint32_t epoch, cudaStream_t st,
+                                 int64_t *launches)
+{
+    const int E = c->E, k = c->k, L = E - k, G = (L + 7) / 8;
+    int gpt = 0, warps = 0, nstage = 0;
+    const bool pipe = qs_pipe_plan(c, stride, &gpt, &warps, &nstage);
+    QPipeParams pp;
+    QSParams &p = pp.q;
+    p.T = T; p.stride = stride; p.lp_bytes = tpq_lp_bytes_i(T, E, k, c->bits);
+    p.n_tiles = (T + QS_ROWS - 1) / QS_ROWS;
+    p.E = E; p.k = k; p.L = L; p.n_holes = c->n_holes;
+    p.row_words = qs_row_words(L, c->bits);
+    p.grp = c->t.grp; p.hp_idx = c->t.hp_idx; p.hole = c->t.hole; p.filler = c->t.filler;
+    for (int b0 = 0; b0 < n; b0 += QS_MAX_BATCH) {
+        const int nb = n - b0 < QS_MAX_BATCH ? n - b0 : QS_MAX_BATCH;
+        for (int b = 0; b < nb; ++b) {
+            p.y[b] = static_cast<const uint16_t *>(ys[b0 + b]);
+            p.payload[b] = static_cast<uint8_t *>(payloads[b0 + b]);
+        }
+        p.inv_s = c->t.inv_s + (size_t)(shard0 + b0) * E;
+        cudaError_t e;
+        if (pipe) {
+            // the SMs are divided among the shards; no block has more than a row above the mean
+            pp.nstage = nstage; pp.status = c->t.status; pp.done = c->t.push_done;
+            pp.n_dst = n_dst; pp.epoch = epoch;
+            for (int d = 0; d < n_dst; ++d) {
+                p.payload[d] = static_cast<uint8_t *>(payloads[d]);
+                pp.arrived[d] = arrived[d];
+            }
+            int64_t bps = c->sm_count / nb > 0 ? c->sm_count / nb : 1;
+            if (bps > T) bps = T;
+            pp.rows_per_block = (T + bps - 1) / bps;
+            bps = (T + pp.rows_per_block - 1) / pp.rows_per_block;
+            pp.bps = (int)bps;
+            const int threads = warps * 32 + 64;
+            const size_t smem = qs_pipe_bytes(E, c->bits, warps, gpt, nstage);
+            const unsigned grid = (unsigned)(bps * nb);
+            const bool push = n_dst > 0;
+            switch (c->bits) {
+            case 2: e = launch_quantize_pipe<2>(pp, push, gpt, threads, grid, smem, st); break;
+            case 3: e = launch_quantize_pipe<3>(pp, push, gpt, threads, grid, smem, st); break;
+            case 4: e = launch_quantize_pipe<4>(pp, push, gpt, threads, grid, smem, st); break;
+            case 5: e = launch_quantize_pipe<5>(pp, push, gpt, threads, grid, smem, st); break;
+            case 6: e = launch_quantize_pipe<6>(pp, push, gpt, threads, grid, smem, st); break;
+            case 7: e = launch_quantize_pipe<7>(pp, push, gpt, threads, grid, smem, st); break;
+            default: e = launch_quantize_pipe<8>(pp, push, gpt, threads, grid, smem, st); break;
+            }
+        } else {
+            const bool vec = E % 8 == 0 && stride % 8 == 0;
+            const int per = (G + QS_THREADS - 1) / QS_THREADS;  // an even share of the row's groups per thread
+            int threads = ((G + per - 1) / per + 31) / 32 * 32;
+            if (threads < 128) threads = 128;
+            const dim3 grid((unsigned)p.n_tiles, (unsigned)nb);
+            switch (c->bits) {
+            case 2: e = launch_quantize_tile<2>(p, vec, threads, grid, st); break;
+            case 3: e = launch_quantize_tile<3>(p, vec, threads, grid, st); break;
+            case 4: e = launch_quantize_tile<4>(p, vec, threads, grid, st); break;
+            case 5: e = launch_quantize_tile<5>(p, vec, threads, grid, st); break;
+            case 6: e = launch_quantize_tile<6>(p, vec, threads, grid, st); break;
+            case 7: e = launch_quantize_tile<7>(p, vec, threads, grid, st); break;
+            default: e = launch_quantize_tile<8>(p, vec, threads, grid, st); break;
+            }
+        }
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t tpq_launch_quantize_stream(const tpq_ctx *c, int shard0, int n, const void *const *ys, int64_t T, int64_t stride,
+                                       void *const *payloads, cudaStream_t st, int64_t *launches)
+{
+    return launch_stream(c, shard0, n, ys, T, stride, payloads, 0, nullptr, 0u, st, launches);
+}
+
+bool tpq_stream_pipe_ok(const tpq_ctx *c, int64_t T, int64_t stride)
+{
+    int gpt, warps, nstage;
+    return tpq_stream_ok(c, T) && qs_pipe_plan(c, stride, &gpt, &warps, &nstage);
+}
+
+cudaError_t tpq_launch_quantize_stream_push(const tpq_ctx *c, int shard, const void *y, int64_t T, int64_t stride, void *const *dst,
+                                            uint32_t *const *arrived, int n_dst, uint32_t epoch, cudaStream_t st, int64_t *launches)
+{
+    return launch_stream(c, shard, 1, &y, T, stride, dst, n_dst, arrived, epoch, st, launches);
+}
+
+cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *payloads, int64_t T, void *out, int fp32_out,
+                                      int64_t out_stride, cudaStream_t st, int64_t *launches)
+{
+    const int E = c->E, k = c->k, L = E - k, G = (L + 7) / 8;
+    DSParams p;
+    for (int i = 0; i < c->N; ++i) p.pl[i] = static_cast<const uint8_t *>(payloads[i]);
+    p.N = c->N; p.E = E; p.k = k; p.L = L; p.T = T;
+    p.lp_bytes = tpq_lp_bytes_i(T, E, k, c->bits);
+    p.out_stride = out_stride;
+    p.s_slot = c->t.s_slot; p.grp = c->t.grp; p.lp_idx = c->t.lp_idx; p.hp_idx = c->t.hp_idx;
+    p.filler = c->t.filler; p.n_holes = c->n_holes;
+    p.vec = E % 8 == 0 && out_stride % 8 == 0;
+    p.out = out; p.bias = c->call_bias; p.arr = c->call_arr;
+    constexpr int RC = DS_THREADS / DS_CG * DS_R;
+    p.panels = (G + DS_CG - 1) / DS_CG;
+    p.n_chunks = (T + RC - 1) / RC;
+    const int per_sm = 2 * (ds_smem_bytes(c->bits, c->N) + 1024) <= 228 * 1024 ? 2 : 1;
+    int64_t gy = (int64_t)c->sm_count * per_sm / p.panels;
+    if (gy > p.n_chunks) gy = p.n_chunks;
+    if (gy < 1) gy = 1;
+    p.gy = (int)gy;
+    cudaError_t e;
+    switch (c->bits) {
+    case 2: e = launch_dequant_stream<2>(p, fp32_out, st); break;
+    case 3: e = launch_dequant_stream<3>(p, fp32_out, st); break;
+    case 4: e = launch_dequant_stream<4>(p, fp32_out, st); break;
+    case 5: e = launch_dequant_stream<5>(p, fp32_out, st); break;
+    case 6: e = launch_dequant_stream<6>(p, fp32_out, st); break;
+    case 7: e = launch_dequant_stream<7>(p, fp32_out, st); break;
+    default: e = launch_dequant_stream<8>(p, fp32_out, st); break;
+    }
+    if (e == cudaSuccess) ++*launches;
+    return e;
+}

@@ -1,0 +1,70 @@
+"""The bit-stream kernels (code widths other than 4 bits; feature counts, strides and selected counts that are
+multiples of nothing) against the shape-generic kernels, which the parity tests pin to the oracle: payload bytes
+and FP32 / BF16 sums bit for bit.  The shapes sit where the layout can go wrong: rows of 32 bits and a little
+more, a last group of 1 to 7 slots, tiles of 8 rows and one row less or more, a tile that ends inside a word,
+panels of 128 and 32 groups with one group more, rows that a block takes in several rounds, one and two buffers."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+from paper_2411_07942_b200 import binding, synth  # noqa: E402
+
+import gpu_util as gu  # noqa: E402
+
+CASES = [  # N, T, E, k, bits, row padding, bias
+    (1, 1, 33, 1, 2, 0, False), (2, 7, 17, 0, 2, 0, True), (3, 8, 65, 1, 3, 3, True), (2, 9, 130, 2, 4, 0, False),
+    (2, 33, 1033, 8, 4, 0, True), (4, 16, 1024 + 51, 51, 4, 0, False), (4, 67, 5120, 51, 4, 64, True),
+    (8, 40, 2304, 36, 4, 0, False), (8, 129, 4608, 72, 8, 0, True), (5, 31, 5120, 80, 5, 8, False),
+    (3, 65, 1041, 17, 7, 0, True), (3, 24, 1047, 23, 6, 1, False), (16, 50, 832, 13, 5, 0, True),
+    (33, 18, 520, 9, 4, 0, False), (64, 70, 264, 8, 8, 0, True), (2, 20, 8192, 128, 8, 0, False), (2, 11, 16384, 9, 8, 0, False),
+    (1, 300, 5121, 5000, 4, 0, False), (2, 600, 200, 3, 3, 0, False), (1, 2500, 1000, 15, 4, 0, True),
+]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    gu.ensure_lib()
+
+
+@pytest.mark.parametrize("N,T,E,k,bits,pad,with_bias", CASES)
+def test_stream_kernels_equal_generic(N, T, E, k, bits, pad, with_bias):
+    rng = np.random.default_rng(E + T)
+    T += -(-(1 << 18) // (8 * E)) * 8
+    w = synth.Workload("stream", N, T, E, 0.7, max(1, E // 100), 20.0, 200.0, 1, 8, E + 7 * T + bits)
+    scale = synth.column_scales(w)
+    t = binding.Tpq(N, E, bits=bits)
+    gu.calibrate_both(t, [synth.calibration_np(w, i, scale=scale) for i in range(N)])
+    bias = torch.from_numpy(rng.standard_normal(E).astype(np.float32)).cuda() if with_bias else None
+    ys = []
+    for i in range(N):
+        wide = torch.full((T, E + pad), float("nan"), dtype=torch.bfloat16, device="cuda")
+        wide[:, :E] = gu.dev_bf16(synth.activations_np(w, i, T, scale=scale)).view(torch.bfloat16).view(T, E)
+        ys.append(wide)
+    # the selector's set, one run that ends inside a group, and both ends of the feature range
+    start = int(rng.integers(0, E - k + 1))
+    sets = [None, list(range(start, start + k)), sorted(set(range(k // 2)) | set(range(E - (k - k // 2), E)))]
+    for hp in sets if k else [None]:
+        t.select_features(k) if hp is None else t.set_features(hp)
+        P = t.payload_bytes(T)
+        got = {}
+        for path in (binding.PATH_GENERIC, binding.PATH_AUTO):
+            t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+            guarded = [gu.guarded(P) for _ in range(N)]
+            ptrs = [v.data_ptr() for _, v in guarded]
+            t.quantize_pack_batch(0, [y.data_ptr() for y in ys], T, ptrs, P, row_stride=E + pad)
+            outs = []
+            for dt, size in ((binding.TPQ_OUT_FP32, 4), (binding.TPQ_OUT_BF16, 2)):
+                whole, out = gu.guarded(T * (E + pad) * size)
+                t.dequant_reduce(ptrs, T, out.data_ptr(), dt, out_row_stride=E + pad, bias_ptr=bias.data_ptr() if with_bias else None)
+                torch.cuda.synchronize()
+                assert gu.guards_intact(whole, T * (E + pad) * size)
+                outs.append(out.cpu().numpy())
+            assert t.device_status() == 0
+            assert all(gu.guards_intact(whole, P) for whole, _ in guarded)
+            got[path] = ([v.cpu().numpy() for _, v in guarded], outs)
+        for a, b in zip(got[binding.PATH_GENERIC], got[binding.PATH_AUTO]):
+            for x, y in zip(a, b):
+                assert np.array_equal(x, y), (hp, np.nonzero(x != y)[0][:8])
+    t.close()
