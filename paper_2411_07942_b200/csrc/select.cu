@@ -30,94 +30,113 @@ __global__ void __launch_bounds__(256) ranges_kernel(const float *__restrict__ m
 }
 
 // Feature j is selected iff fewer than k features beat it, where a beats j when
-// Rbar_a > Rbar_j, or Rbar_a == Rbar_j and a < j.  O(E^2) comparisons, tiled through shared memory.
-__global__ void __launch_bounds__(256) topk_flags_kernel(const float *__restrict__ Rbar, int E, int k,
-                                                         uint8_t *__restrict__ flag)
+// Rbar_a > Rbar_j, or Rbar_a == Rbar_j and a < j.  O(E^2) comparisons, a warp per feature: its lanes compare side by
+// side, four values per load (Rbar is a few tens of KB, so the loads hit L1).  (One thread per feature, the values
+// through shared memory, left all but 18 SMs idle: 68 us at E = 4608.  With this kernel and the two below
+// the whole selection call takes 61 instead of 135 us at 8 x 4608, 82 instead of 227 us at 16 x 8192.)
+constexpr int TK_WARPS = 8;
+
+__global__ void __launch_bounds__(32 * TK_WARPS) topk_flags_kernel(const float *__restrict__ Rbar, int E, int k,
+                                                                   uint8_t *__restrict__ flag)
 {
-    __shared__ float tile[1024];
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const float mine = (j < E) ? Rbar[j] : 0.0f;
+    const int j = blockIdx.x * TK_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (j >= E) return;
+    const float mine = __ldg(Rbar + j);
     int beats = 0;
-    for (int a0 = 0; a0 < E; a0 += 1024) {
-        __syncthreads();
-        for (int a = threadIdx.x; a < 1024; a += blockDim.x) tile[a] = (a0 + a < E) ? Rbar[a0 + a] : 0.0f;
-        __syncthreads();
-        const int n = (E - a0 < 1024) ? E - a0 : 1024;
-        for (int a = 0; a < n; ++a) {
-            const float v = tile[a];
-            beats += (v > mine) || (v == mine && (a0 + a) < j);
-        }
+    const int E4 = E >> 2;
+#pragma unroll 4
+    for (int q = lane; q < E4; q += 32) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(Rbar) + q);
+        const int a = 4 * q;
+        beats += (v.x > mine || (v.x == mine && a < j)) + (v.y > mine || (v.y == mine && a + 1 < j)) +
+                 (v.z > mine || (v.z == mine && a + 2 < j)) + (v.w > mine || (v.w == mine && a + 3 < j));
     }
-    if (j < E) flag[j] = (beats < k) ? 1 : 0;
+    if (lane < (E & 3)) {
+        const int a = 4 * E4 + lane;
+        const float v = __ldg(Rbar + a);
+        beats += v > mine || (v == mine && a < j);
+    }
+    beats = __reduce_add_sync(0xffffffffu, beats);
+    if (lane == 0) flag[j] = beats < k ? 1 : 0;
 }
 
-// One block: exclusive scan of the flags -> selected list, hole / filler lists, slot order,
-// per-feature slots, the dequantiser's zeroed-step and slot-order step copies and the per-8-feature
-// group descriptors.
-__global__ void __launch_bounds__(1024) tables_kernel(tpq_tables t, int N, int E, int k)
+// One block: exclusive scan of the flags -> selected list, hole / filler lists.  A thread scans an even share of
+// adjacent features, so there is one block-wide scan whatever E is.
+__global__ void __launch_bounds__(1024) scan_kernel(tpq_tables t, int E, int k)
 {
     __shared__ int warp_sums[32];
-    __shared__ int carry;
+    __shared__ int s_below;  // selected features below L
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int L = E - k;
-    if (tid == 0) carry = 0;
+    const int per = (E + 1023) / 1024, j0 = tid * per < E ? tid * per : E, j1 = j0 + per < E ? j0 + per : E;
+    int mine = 0;
+    for (int j = j0; j < j1; ++j) mine += t.flag[j];
+    int incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += o;
+    }
+    if (lane == 31) warp_sums[wid] = incl;
+    if (tid == 0) s_below = k;  // (L == E: every selected feature -- there is none -- is below L)
     __syncthreads();
-    for (int j0 = 0; j0 < E; j0 += 1024) {
-        const int j = j0 + tid;
-        const int f = (j < E) ? t.flag[j] : 0;
-        int incl = f;
+    if (wid == 0) {
+        const int w = warp_sums[lane];
+        int wi = w;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            int o = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += o;
+            const int o = __shfl_up_sync(0xffffffffu, wi, d);
+            if (lane >= d) wi += o;
         }
-        if (lane == 31) warp_sums[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            int w = warp_sums[lane];
-            int wi = w;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                int o = __shfl_up_sync(0xffffffffu, wi, d);
-                if (lane >= d) wi += o;
-            }
-            warp_sums[lane] = wi - w;  // exclusive
-        }
-        __syncthreads();
-        const int before = carry + warp_sums[wid] + incl - f;  // selected features before j
-        if (j < E) {
-            t.hpre[j] = before;
-            if (f) t.hp_idx[before] = j;
-            for (int i = 0; i < N; ++i) t.s_k[(size_t)i * E + j] = f ? 0.0f : t.s[(size_t)i * E + j];
-        }
-        __syncthreads();
-        if (tid == 1023) carry = before + f;
-        __syncthreads();
-    }
-    // holes: selected features below L; fillers: unselected features at or above L (equally many)
-    const int m = (L < E) ? t.hpre[L] : 0;
-    for (int j = tid; j < E; j += 1024) {
-        const int f = t.flag[j];
-        if (f && j < L) t.hole[t.hpre[j]] = j;
-        if (!f && j >= L) t.filler[(j - L) - (t.hpre[j] - m)] = j;
+        warp_sums[lane] = wi - w;  // exclusive
     }
     __syncthreads();
-    for (int j = tid; j < E; j += 1024) {
+    const int start = warp_sums[wid] + incl - mine;  // selected features before j0
+    int before = start;
+    for (int j = j0; j < j1; ++j) {
         const int f = t.flag[j];
-        const int src = (j < L) ? (f ? t.filler[t.hpre[j]] : j) : -1;  // feature held by slot j
-        if (j < L) t.lp_idx[j] = src;
-        for (int i = 0; i < N; ++i) t.s_slot[(size_t)i * E + j] = (src >= 0) ? t.s[(size_t)i * E + src] : 0.0f;
-        if (f)
-            t.pos[j] = -(t.hpre[j] + 1);
-        else
-            t.pos[j] = (j < L) ? j : t.hole[(j - L) - (t.hpre[j] - m)];
+        t.hpre[j] = before;
+        if (j == L) s_below = before;
+        if (f) {
+            t.hp_idx[before] = j;
+            if (j < L) t.hole[before] = j;
+        }
+        before += f;
     }
-    const int n_grp = (E + 7) / 8;
-    for (int g = tid; g < n_grp; g += 1024) {
+    __syncthreads();
+    // holes: selected features below L; fillers: unselected features at or above L (equally many)
+    const int m = s_below;
+    before = start;
+    for (int j = j0; j < j1; ++j) {
+        const int f = t.flag[j];
+        if (!f && j >= L) t.filler[(j - L) - (before - m)] = j;
+        before += f;
+    }
+}
+
+// Per feature, over the whole GPU: slot order, per-feature slots, the dequantiser's zeroed-step and slot-order step
+// copies and the per-8-feature group descriptors.  (As loops of the scan's one block these N*E-long copies took most of
+// its 35 us at 8 x 4608.)
+__global__ void __launch_bounds__(256) tables_kernel(tpq_tables t, int N, int E, int k)
+{
+    const int j = blockIdx.x * 256 + threadIdx.x;
+    if (j >= E) return;
+    const int L = E - k, f = t.flag[j], pre = t.hpre[j];
+    const int m = L < E ? t.hpre[L] : 0;
+    const int src = j < L ? (f ? t.filler[pre] : j) : -1;  // feature held by slot j
+    if (j < L) t.lp_idx[j] = src;
+#pragma unroll 4
+    for (int i = 0; i < N; ++i) {
+        const size_t row = (size_t)i * E;
+        t.s_k[row + j] = f ? 0.0f : t.s[row + j];
+        t.s_slot[row + j] = src >= 0 ? t.s[row + src] : 0.0f;
+    }
+    t.pos[j] = f ? -(pre + 1) : j < L ? j : t.hole[(j - L) - (pre - m)];
+    if ((j & 7) == 0) {
         uint32_t mask = 0;
         for (int n = 0; n < 8; ++n)
-            if (8 * g + n < E && t.flag[8 * g + n]) mask |= 1u << n;
-        t.grp[g] = ((uint32_t)t.hpre[8 * g] << 8) | mask;
+            if (j + n < E && t.flag[j + n]) mask |= 1u << n;
+        t.grp[j >> 3] = ((uint32_t)pre << 8) | mask;
     }
 }
 
@@ -132,14 +151,16 @@ cudaError_t tpq_launch_ranges(const tpq_tables &t, int N, int E, int bits, cudaS
 
 cudaError_t tpq_launch_topk_flags(const tpq_tables &t, int E, int k, cudaStream_t st, int64_t *launches)
 {
-    topk_flags_kernel<<<(E + 255) / 256, 256, 0, st>>>(t.Rbar, E, k, t.flag);
+    topk_flags_kernel<<<(E + TK_WARPS - 1) / TK_WARPS, 32 * TK_WARPS, 0, st>>>(t.Rbar, E, k, t.flag);
     ++*launches;
     return cudaGetLastError();
 }
 
 cudaError_t tpq_launch_tables(const tpq_tables &t, int N, int E, int k, cudaStream_t st, int64_t *launches)
 {
-    tables_kernel<<<1, 1024, 0, st>>>(t, N, E, k);
+    scan_kernel<<<1, 1024, 0, st>>>(t, E, k);
+    ++*launches;
+    tables_kernel<<<(E + 255) / 256, 256, 0, st>>>(t, N, E, k);
     ++*launches;
     return cudaGetLastError();
 }
