@@ -8,7 +8,12 @@
 // logic: a group of 8 columns is either one 32-bit word of codes or 8 BF16 values of the BF16 block.
 //
 // Kernel: tcgen05 (5th-generation tensor cores), persistent: one block per SM walks 128 x BN tiles of the
-// output.  Operands are staged by TMA (128-byte swizzle) in a ring of shared-memory stages that runs on
+// output, or a PAIR of blocks (a cluster of two SMs, tcgen05 cta_group::2) walks 256 x BN tiles.  What bounds a
+// block is its shared memory's bandwidth, which the copies that write the operands and the MMAs that read them share: a
+// 64-wide k-block of a 128 x 256 tile is 48 KB each way, 385 ns, against 260 ns of MMA.  In a pair each block fetches its
+// own 128 rows of x and HALF of the weight tile, and the tensor cores of both read the halves from either's shared
+// memory: 32 KB in and 48 KB out per block and k-block.
+// Operands are staged by TMA (128-byte swizzle) in a ring of shared-memory stages that runs on
 // across tiles; one thread issues tcgen05.mma (M = 128, N = BN, K = 16, BF16 x BF16 -> FP32) into one of TWO
 // accumulators in tensor memory; four epilogue warps read the other one back (tcgen05.ld), round to BF16
 // (the layer's output type), quantise and store, while the tensor cores work on the next tile.
@@ -27,21 +32,25 @@ namespace {
 constexpr int LQ_BM = 128, LQ_BK = 64, LQ_THREADS = 192;
 constexpr int LQ_WAIT_LIMIT = 1 << 24;  // try_wait attempts (each suspends for a hardware time slice) ...
 constexpr unsigned long long LQ_WAIT_NS = 1000000000ull;  // ... and one second, whichever ends first
-constexpr uint32_t LQ_A_BYTES = LQ_BM * LQ_BK * 2;
+constexpr uint32_t LQ_A_BYTES = LQ_BM * LQ_BK * 2;  // the x tile of a 64-wide k-block
+constexpr uint32_t LQ_SMEM_MAX = 227u * 1024u;
 
-__host__ __device__ constexpr uint32_t lq_stage_bytes(int BN) { return LQ_A_BYTES + (uint32_t)BN * LQ_BK * 2; }
-__host__ __device__ constexpr int lq_stages(int BN)
+// CG: blocks that share a tile (1, or 2: a pair, each with half of the weight tile)
+// KB: 64-wide k-blocks of a stage
+__host__ __device__ constexpr uint32_t lq_b_bytes(int BN, int CG) { return (uint32_t)(BN / CG) * LQ_BK * 2; }
+__host__ __device__ constexpr uint32_t lq_stage_bytes(int BN, int CG, int KB) { return KB * (LQ_A_BYTES + lq_b_bytes(BN, CG)); }
+__host__ __device__ constexpr int lq_stages(int BN, int CG, int KB)
 {
-    int n = (int)((200u * 1024u) / lq_stage_bytes(BN));
+    const int n = (int)((LQ_SMEM_MAX - 1024u - 176u - 8u * BN) / lq_stage_bytes(BN, CG, KB));
     return n > 8 ? 8 : n;
 }
 // two accumulators (the epilogue drains one while the tensor cores fill the other), a power of two of columns
 __host__ __device__ constexpr uint32_t lq_tmem_cols(int BN) { return 2 * BN <= 64 ? 64 : 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512; }
-__host__ __device__ constexpr size_t lq_smem_bytes(int BN)
+__host__ __device__ constexpr size_t lq_smem_bytes(int BN, int CG, int KB)
 {
     // 1024 B of slack for the manual alignment; stages; 176 B: barriers (full[8], empty[8], accumulators 2 x 2)
     // and the tensor-memory address; the reciprocal steps of two tiles
-    return 1024 + (size_t)lq_stages(BN) * lq_stage_bytes(BN) + 176 + 2 * (size_t)BN * 4;
+    return 1024 + (size_t)lq_stages(BN, CG, KB) * lq_stage_bytes(BN, CG, KB) + 176 + 2 * (size_t)BN * 4;
 }
 
 struct LQParams {
@@ -51,6 +60,8 @@ struct LQParams {
     const float *inv_s;     // [E] of this device, feature order
     const int32_t *lp_idx;  // [L] slot -> feature
     uint8_t *payload;
+    int x_rows;             // rows of an x box: 128, or where T is below that, T rounded up to 8 (the tile's other rows hold
+                            // whatever was in shared memory; a row of the sum depends on its own row of x only)
     uint16_t *y_slots;      // optional [T][E] BF16 partial sums in slot order (NULL: not written)
     int *status;
 };
@@ -78,31 +89,105 @@ __device__ __forceinline__ bool lq_mbar_wait(uint32_t bar, uint32_t parity)
     return false;
 }
 
-// ---- tcgen05
+// ---- tcgen05; CG = 2: the instruction spans the pair of blocks
+template <int CG>
 __device__ __forceinline__ void tc_alloc(uint32_t smem_dst, uint32_t cols)
 {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (CG == 2) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
 }
+template <int CG>
 __device__ __forceinline__ void tc_dealloc(uint32_t taddr, uint32_t cols)
 {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+    if (CG == 2)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// arrives at the barrier (of a pair: at the barrier at that offset in both blocks) when the MMAs so far are done
+template <int CG>
 __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    if (CG == 2)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+                     "h"((uint16_t)3)
+                     : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 // D[tmem] (+)= A[smem] * B[smem]; BF16 inputs, FP32 accumulation
+template <int CG>
 __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
 {
+    if (CG == 2)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            : "memory");
+}
+// the same place in the shared memory of block `rank` of the cluster
+__device__ __forceinline__ uint32_t lq_peer(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void lq_cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Stage kb of a tile's operand: rows y .. of KB 64-wide k-blocks, one behind the other.  KB = 1: a box of the 2-D map;
+// more: one box of the 3-D map (64 values, rows, k-blocks).  CG = 2: `bar` is a cluster address in the pair's first block.
+template <int CG, int KB>
+__device__ __forceinline__ void lq_load(uint32_t dst, const void *map, int kb, int y, uint32_t bar)
+{
+    if (KB == 1 && CG == 2)
+        asm volatile(
+            "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+                dst),
+            "l"(map), "r"(kb * LQ_BK), "r"(y), "r"(bar)
+            : "memory");
+    else if (KB == 1)
+        tma_load_2d(dst, map, kb * LQ_BK, y, bar);
+    else if (CG == 2)
+        asm volatile(
+            "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+                dst),
+            "l"(map), "r"(0), "r"(y), "r"(kb * KB), "r"(bar)
+            : "memory");
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+            "l"(map), "r"(0), "r"(y), "r"(kb * KB), "r"(bar)
+            : "memory");
+}
+// true in one lane of a converged warp, known to the compiler as a single active thread
+__device__ __forceinline__ bool lq_elect()
+{
+    uint32_t one;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
+        "elect.sync _|p, 0xFFFFFFFF;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(one));
+    return one != 0;
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread <-> its lane's row
 __device__ __forceinline__ void tc_ld_32x32(uint32_t taddr, uint32_t (&r)[32])
@@ -130,10 +215,10 @@ __device__ __forceinline__ uint64_t lq_smem_desc(uint32_t addr)
            | ((uint64_t)1 << 46)                // descriptor version of this architecture
            | ((uint64_t)2 << 61);               // 128-byte swizzle
 }
-// Instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, M = 128, N = BN.
-__host__ __device__ constexpr uint32_t lq_instr_desc(int BN)
+// Instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, M = 128 (of a pair 256), N = BN.
+__host__ __device__ constexpr uint32_t lq_instr_desc(int BN, int CG)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(LQ_BM >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(CG * LQ_BM >> 4) << 24);
 }
 
 // C^(i) of one value (Section 3): two binary32 roundings, clamp, round half to even; the low 4 bits of
@@ -149,23 +234,25 @@ __device__ __forceinline__ uint32_t lq_code(float x, float inv)
 // innermost.  Blocks that run together share a weight tile, and a band's rows of x (LQ_GROUP_M x 128 x K
 // values) stay in L2 while every column tile passes over them, whatever T is.
 constexpr int LQ_GROUP_M = 16;
+template <int CG>  // (a pair's tile is 256 rows: half as many make a band)
 __device__ __forceinline__ void lq_tile_origin(int tile, int mt, int nt, int BN, int &m0, int &n0)
 {
-    const int per_band = LQ_GROUP_M * nt;
+    constexpr int GM = LQ_GROUP_M / CG;
+    const int per_band = GM * nt;
     const int band = tile / per_band, in_band = tile - band * per_band;
-    const int rows = (mt - band * LQ_GROUP_M < LQ_GROUP_M) ? mt - band * LQ_GROUP_M : LQ_GROUP_M;  // the last band may be short
-    const int n = in_band / rows, m = band * LQ_GROUP_M + (in_band - n * rows);
-    m0 = m * LQ_BM;
+    const int rows = (mt - band * GM < GM) ? mt - band * GM : GM;  // the last band may be short
+    const int n = in_band / rows, m = band * GM + (in_band - n * rows);
+    m0 = m * (CG * LQ_BM);
     n0 = n * BN;
 }
 
-template <int BN>
+template <int BN, int CG, int KB>
 __global__ void __launch_bounds__(LQ_THREADS, 1)
 linear_quantize(const LQParams p, const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w)
 {
     extern __shared__ uint8_t lq_raw[];
-    constexpr int NS = lq_stages(BN);
-    constexpr uint32_t STAGE = lq_stage_bytes(BN);
+    constexpr int NS = lq_stages(BN, CG, KB);
+    constexpr uint32_t STAGE = lq_stage_bytes(BN, CG, KB);
     constexpr uint32_t TCOLS = lq_tmem_cols(BN);
     const uint32_t base = (smem_u32(lq_raw) + 1023u) & ~1023u;  // swizzled tiles want 1024-byte alignment
     uint8_t *const gen = lq_raw + (base - smem_u32(lq_raw));
@@ -181,9 +268,13 @@ linear_quantize(const LQParams p, const __grid_constant__ CUtensorMap map_x, con
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int L = p.E - p.k, L8 = L >> 3;
-    const int nkb = (p.K + LQ_BK - 1) / LQ_BK;
-    const int mt = (int)((p.T + LQ_BM - 1) / LQ_BM), nt = (p.E + BN - 1) / BN;
+    const int nkb = (p.K + KB * LQ_BK - 1) / (KB * LQ_BK);  // stages per tile
+    const int mt = (int)((p.T + CG * LQ_BM - 1) / (CG * LQ_BM)), nt = (p.E + BN - 1) / BN;
     const int tiles = mt * nt;
+    // a pair: block `rank` owns rows rank * 128 .. of the tile and fetches half `rank` of the weight tile; the first
+    // block's barriers count both blocks' copies and its MMA warp works for both
+    const uint32_t rank = CG == 2 ? blockIdx.x & 1u : 0u;
+    const int first_tile = blockIdx.x / CG, tile_step = gridDim.x / CG;
 
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
@@ -192,15 +283,16 @@ linear_quantize(const LQParams p, const __grid_constant__ CUtensorMap map_x, con
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(acc_full(b), 1);
-            mbar_init(acc_empty(b), 4);  // one arrival per epilogue warp
+            mbar_init(acc_empty(b), 4 * CG);  // one arrival per epilogue warp
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 1) tc_alloc(smem_u32(tmem_slot), TCOLS);
+    if (warp == 1) tc_alloc<CG>(smem_u32(tmem_slot), TCOLS);
     tc_fence_before();
     tpq_grid_dep_wait();  // the operands and the payload buffer may still be in use by the kernel ahead
     __syncthreads();
+    if (CG == 2) lq_cluster_sync();  // the other block's barriers exist
     tpq_grid_dep_launch();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
@@ -209,64 +301,79 @@ linear_quantize(const LQParams p, const __grid_constant__ CUtensorMap map_x, con
     if (warp == 0) {
         if (lane == 0) {
             int it = 0;  // k-blocks issued so far, over all of this block's tiles
-            for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+            for (int tile = first_tile; tile < tiles && ok; tile += tile_step) {
                 int m0, n0;
-                lq_tile_origin(tile, mt, nt, BN, m0, n0);
+                lq_tile_origin<CG>(tile, mt, nt, BN, m0, n0);
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % NS;
                     if (it >= NS && !lq_mbar_wait(empty(s), ((it / NS) - 1) & 1)) {
                         ok = false;
                         break;
                     }
-                    mbar_expect_tx(full(s), STAGE);
-                    tma_load_2d(base + s * STAGE, &map_x, kb * LQ_BK, m0, full(s));
-                    tma_load_2d(base + s * STAGE + LQ_A_BYTES, &map_w, kb * LQ_BK, n0, full(s));
+                    if (CG == 2) {
+                        if (rank == 0) mbar_expect_tx(full(s), 2 * STAGE);
+                        const uint32_t bar = lq_peer(full(s), 0);
+                        lq_load<2, KB>(base + s * STAGE, &map_x, kb, m0 + (int)rank * LQ_BM, bar);
+                        lq_load<2, KB>(base + s * STAGE + KB * LQ_A_BYTES, &map_w, kb, n0 + (int)rank * (BN / 2), bar);
+                    } else {
+                        mbar_expect_tx(full(s), (uint32_t)(KB * p.x_rows) * (LQ_BK * 2) + KB * lq_b_bytes(BN, CG));
+                        lq_load<1, KB>(base + s * STAGE, &map_x, kb, m0, full(s));
+                        lq_load<1, KB>(base + s * STAGE + KB * LQ_A_BYTES, &map_w, kb, n0, full(s));
+                    }
                 }
             }
-            if (!ok)  // giving up: let the copies already issued land before the block's shared memory is released
-                for (int j = it > NS ? it - NS : 0; j < it; ++j) (void)lq_mbar_wait(full(j % NS), (j / NS) & 1);
+            const int last = it > NS ? it - NS : 0;
+            if (!ok && rank == 0)  // giving up: let the copies already issued (a pair's: both blocks') land before the shared memory is released
+                for (int j = last; j < it; ++j) (void)lq_mbar_wait(full(j % NS), (j / NS) & 1);
+            if (CG == 2 && ok)  // the first block's MMA warp still arrives at the other's barriers: neither may end before
+                for (int j = last; j < it; ++j) ok = ok && lq_mbar_wait(empty(j % NS), (j / NS) & 1);
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = lq_instr_desc(BN);
-            int it = 0, n_tile = 0;
-            for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++n_tile) {
-                const int b = n_tile & 1;
-                // the epilogue must have drained this accumulator (used two tiles ago)
-                if (n_tile >= 2 && !lq_mbar_wait(acc_empty(b), ((n_tile >> 1) - 1) & 1)) {
-                    ok = false;
-                    break;
-                }
+        // The whole warp walks the loop and one elected lane issues: with the issuing lane picked by a comparison of
+        // its index the compiler cannot know that a single thread is active, and every MMA's operands (which the
+        // instruction takes from uniform registers) cost a loop over the lanes.
+        constexpr uint32_t idesc = lq_instr_desc(BN, CG);
+        const uint64_t desc0 = lq_smem_desc(base);
+        const uint32_t x_kb = CG == 2 ? LQ_A_BYTES >> 4 : (uint32_t)p.x_rows * (LQ_BK * 2 >> 4);  // from one k-block of x to the next
+        int it = 0, n_tile = 0;
+        for (int tile = rank == 0 ? first_tile : tiles; tile < tiles && ok; tile += tile_step, ++n_tile) {
+            const int b = n_tile & 1;
+            // the epilogue must have drained this accumulator (used two tiles ago)
+            if (n_tile >= 2) ok = __all_sync(0xffffffffu, lq_mbar_wait(acc_empty(b), ((n_tile >> 1) - 1) & 1));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d = tmem + (uint32_t)(b * BN);
+            for (int kb = 0; kb < nkb; ++kb, ++it) {
+                const int s = it % NS;
+                ok = __all_sync(0xffffffffu, lq_mbar_wait(full(s), (it / NS) & 1));
+                if (!ok) break;
                 tc_fence_after();
-                const uint32_t d = tmem + (uint32_t)(b * BN);
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % NS;
-                    if (!lq_mbar_wait(full(s), (it / NS) & 1)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t a = base + s * STAGE, bb = a + LQ_A_BYTES;
+                if (lq_elect()) {
+                    const uint64_t a = desc0 + (uint64_t)((uint32_t)s * (STAGE >> 4));
 #pragma unroll
-                    for (int k4 = 0; k4 < LQ_BK / 16; ++k4)
-                        tc_mma_bf16(d, lq_smem_desc(a + k4 * 32), lq_smem_desc(bb + k4 * 32), idesc, (kb | k4) != 0);
-                    tc_commit(empty(s));  // arrives when the MMAs above have read the stage
+                    for (int k4 = 0; k4 < KB * (LQ_BK / 16); ++k4) {
+                        const uint64_t ka = (uint64_t)((k4 / 4) * x_kb + 2 * (k4 % 4));
+                        const uint64_t kw = (uint64_t)((KB * LQ_A_BYTES + (k4 / 4) * lq_b_bytes(BN, CG)) >> 4) + 2 * (k4 % 4);
+                        tc_mma_bf16<CG>(d, a + ka, a + kw, idesc, (kb | k4) != 0);
+                    }
+                    tc_commit<CG>(empty(s));  // arrives when the MMAs above have read the stage
+                    if (kb == nkb - 1) tc_commit<CG>(acc_full(b));  // arrives when the tile's accumulator is complete
                 }
-                if (ok) tc_commit(acc_full(b));  // arrives when the tile's accumulator is complete
+                __syncwarp();
             }
         }
-        __syncwarp();
     } else {
         // ---------------- epilogue: tile i is drained while the tensor cores work on tile i + 1
         const int q = warp & 3, et = tid - 64;
         uint32_t *const lp_out = reinterpret_cast<uint32_t *>(p.payload);
         uint16_t *const hp_out = reinterpret_cast<uint16_t *>(p.payload + p.lp_bytes);
         int n_tile = 0;
-        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++n_tile) {
+        for (int tile = first_tile; tile < tiles; tile += tile_step, ++n_tile) {
             const int b = n_tile & 1;
             int m0, n0;
-            lq_tile_origin(tile, mt, nt, BN, m0, n0);
+            lq_tile_origin<CG>(tile, mt, nt, BN, m0, n0);
+            m0 += (int)rank * LQ_BM;
             float *const inv_tile = inv_tiles + b * BN;
             for (int c = et; c < BN; c += 128) {  // the tile's reciprocal steps in slot order
                 const int col = n0 + c;
@@ -300,7 +407,7 @@ linear_quantize(const LQParams p, const __grid_constant__ CUtensorMap map_x, con
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
                     const int col = n0 + c0 + 8 * g;
-                    if (col >= p.E) break;
+                    if (col >= p.E || c0 + 8 * g >= BN) break;
                     uint32_t h[4];  // the 8 sums rounded to BF16 (the layer's output type), packed in pairs
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -330,7 +437,12 @@ linear_quantize(const LQParams p, const __grid_constant__ CUtensorMap map_x, con
             // this warp has read its quadrant of the accumulator: hand it back to the MMA thread
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(b)) : "memory");
+            if (lane == 0) {
+                if (CG == 2)
+                    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(lq_peer(acc_empty(b), 0)) : "memory");
+                else
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(b)) : "memory");
+            }
         }
         // zero padding of the code section (its size is rounded up to 16 bytes)
         if (blockIdx.x == 0 && warp == 2) {
@@ -341,10 +453,11 @@ linear_quantize(const LQParams p, const __grid_constant__ CUtensorMap map_x, con
     if (!ok) atomicExch(p.status, (int)TPQ_ERR_TIMEOUT);
     tc_fence_before();
     __syncthreads();
+    if (CG == 2) lq_cluster_sync();  // neither block's shared or tensor memory is in use by the other any more
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        tc_dealloc(tmem, TCOLS);
+        tc_dealloc<CG>(tmem, TCOLS);
     }
 }
 
@@ -366,31 +479,47 @@ __global__ void __launch_bounds__(256) permute_weight(const uint16_t *__restrict
 }
 
 
-// [rows][K] BF16, row-major -> boxes of box_rows x 64 elements with the 128-byte swizzle; out-of-range reads give 0
-bool lq_map(const void *ptr, int64_t rows, int64_t K, int box_rows, CUtensorMap *out)
+// [rows][K] BF16, row-major -> boxes of box_rows rows x kb k-blocks of 64 elements with the 128-byte swizzle;
+// out-of-range reads give 0.  Several k-blocks per box (K a multiple of 64): the row is cut into 64-value pieces, a third dimension.
+bool lq_map(const void *ptr, int64_t rows, int64_t K, int box_rows, int kb, CUtensorMap *out)
 {
     tpq_encode_tiled_fn fn = tpq_tensor_map_encoder();
     if (!fn) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)LQ_BK, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+    const cuuint64_t dims2[2] = {(cuuint64_t)K, (cuuint64_t)rows}, dims3[3] = {LQ_BK, (cuuint64_t)rows, (cuuint64_t)(K / LQ_BK)};
+    const cuuint64_t strides[2] = {(cuuint64_t)K * 2, LQ_BK * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)LQ_BK, (cuuint32_t)box_rows, (cuuint32_t)kb};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, kb > 1 ? 3 : 2, const_cast<void *>(ptr), kb > 1 ? dims3 : dims2, strides, box,
+              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
-cudaError_t lq_launch(const LQParams &p, const void *x, const void *w, int sm_count, cudaStream_t st)
+template <int BN, int CG, int KB>
+cudaError_t lq_launch(LQParams p, const void *x, const void *w, int sm_count, cudaStream_t st)
 {
+    p.x_rows = CG == 1 && p.T < LQ_BM ? (int)(p.T + 7) / 8 * 8 : LQ_BM;
     CUtensorMap mx, mw;
-    if (!lq_map(x, p.T, p.K, LQ_BM, &mx) || !lq_map(w, p.E, p.K, BN, &mw)) return cudaErrorNotSupported;
-    const size_t smem = lq_smem_bytes(BN);
-    cudaError_t e = cudaFuncSetAttribute(linear_quantize<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (!lq_map(x, p.T, p.K, p.x_rows, KB, &mx) || !lq_map(w, p.E, p.K, BN / CG, KB, &mw)) return cudaErrorNotSupported;
+    const size_t smem = lq_smem_bytes(BN, CG, KB);
+    cudaError_t e = cudaFuncSetAttribute(linear_quantize<BN, CG, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int64_t tiles = ((p.T + LQ_BM - 1) / LQ_BM) * ((p.E + BN - 1) / BN);
-    const dim3 grid((unsigned)(tiles < sm_count ? tiles : sm_count));  // persistent: a block walks tiles b, b + grid, ...
-    return tpq_launch_pdl(linear_quantize<BN>, grid, dim3(LQ_THREADS), smem, st, p, mx, mw);
+    const int64_t tiles = ((p.T + CG * LQ_BM - 1) / (CG * LQ_BM)) * ((p.E + BN - 1) / BN);
+    const int64_t places = sm_count / CG;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(CG * (tiles < places ? tiles : places)));  // persistent: a block (pair) walks tiles b, b + places, ...
+    cfg.blockDim = dim3(LQ_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = CG;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CG == 2 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, linear_quantize<BN, CG, KB>, p, mx, mw);
 }
 
 }  // namespace
@@ -401,7 +530,7 @@ bool tpq_linear_ok(const tpq_ctx *c, int64_t T, int64_t K)
     if (c->E % 8 || c->k % 8 || c->E - c->k < 8) return false;
     if (T < 1 || K < 8 || K % 8) return false;  // 16-byte row pitch for the tensor maps
     if (T > (int64_t)1 << 31 || K > (int64_t)1 << 31) return false;
-    return lq_smem_bytes(256) <= (size_t)c->smem_optin;
+    return lq_smem_bytes(192, 2, 2) <= (size_t)c->smem_optin;
 }
 
 cudaError_t tpq_launch_permute_weight(const tpq_ctx *c, const void *w, void *out, int64_t K, cudaStream_t st, int64_t *launches)
@@ -423,25 +552,44 @@ cudaError_t tpq_launch_linear_quantize(const tpq_ctx *c, int shard, const void *
     p.payload = static_cast<uint8_t *>(payload);
     p.y_slots = static_cast<uint16_t *>(y_slots);
     p.status = c->t.status;
-    // Tile width.  A block's time is (tiles it walks) x (k-blocks per tile) x (time per k-block), and the time
-    // per k-block barely depends on the width (the operand pipeline, not the tensor pipe, sets it: measured
-    // 385 / 376 / 344 ns for 256 / 192 / 128 columns), so the widest tile wins unless a narrower one saves a
-    // whole wave of the persistent grid.
-    const int64_t mt = (T + LQ_BM - 1) / LQ_BM;
-    int best = 256;
-    double best_cost = 0.0;
-    for (int bn : {256, 192, 128}) {
-        const int64_t tiles = mt * ((c->E + bn - 1) / bn);
-        const int64_t waves = (tiles + c->sm_count - 1) / c->sm_count;
-        const double cost = (double)waves * (bn == 256 ? 385.0 : bn == 192 ? 376.0 : 344.0);
-        if (best_cost == 0.0 || cost < best_cost - 1e-9) {
+    // Tile shape.  What bounds a place is its shared memory, 128 bytes a clock for the copies that write the operands and
+    // the MMAs that read them: per 64-wide k-block a single block writes and reads 16 KB of x and BN / 8 KB of weights, one
+    // of a pair writes 16 + BN / 16 KB and reads 16 + BN / 8 KB.  (Measured, ns per k-block against that sum: pairs of
+    // 256 / 192 / 160 / 128 columns 307 / 259 / 232 / 230 for 80 / 68 / 62 / 56 KB, single blocks of 256 / 128 / 64 / 48 / 32
+    // columns 385 / 260 / 207 / 186 / 180 for 96 / 64 / 48 / 44 / 40 KB; the MMAs alone would take 260 at 256 columns.)  The
+    // shape with the least of waves x that sum wins, the earlier one of equals.  2048 x 3456 x 5120: 59.9 us with single
+    // blocks of 192 columns, 51.0 us with pairs of 192 (256: 55.8, 160: 55.0); 8192 tokens 208 -> 180 us (pairs of 256);
+    // 64 x 1280 x 5120 9.2 -> 6.6 us (single blocks of 48: 107 of them instead of 40); 1 x 1280 x 5120 11.9 -> 6.6 us (x boxes of 8
+    // rows instead of 128); 128 x 8192 x 8192 42.5 -> 29.7 us.
+    struct Shape { int bn, cg; };
+    constexpr Shape shapes[] = {{256, 2}, {192, 2}, {160, 2}, {128, 2}, {128, 1}, {64, 1}, {48, 1}, {32, 1}};
+    int best = 0;
+    int64_t best_cost = 0;
+    for (int j = 0; j < (int)(sizeof shapes / sizeof *shapes); ++j) {
+        const int bn = shapes[j].bn, cg = shapes[j].cg;
+        const int64_t tiles = ((T + cg * LQ_BM - 1) / (cg * LQ_BM)) * ((c->E + bn - 1) / bn), places = c->sm_count / cg;
+        const int64_t cost = (tiles + places - 1) / places * (cg == 2 ? 512 + 3 * bn : 512 + 4 * bn);  // KB x 16
+        if (j == 0 || cost < best_cost) {
             best_cost = cost;
-            best = bn;
+            best = j;
         }
     }
-    cudaError_t e = best == 256 ? lq_launch<256>(p, x, w_slots, c->sm_count, st)
-                  : best == 192 ? lq_launch<192>(p, x, w_slots, c->sm_count, st)
-                                : lq_launch<128>(p, x, w_slots, c->sm_count, st);
+    // Stages of 128 values of K where its 64-value pieces are whole: half as many copies and barrier rounds (48-column
+    // blocks 186 against 250 ns per k-block), except where such a stage leaves room for three only (pairs of 256).
+    const bool k2 = K % LQ_BK == 0 && K >= 2 * LQ_BK;
+    cudaError_t e;
+#define LQ_GO(BN, CG) e = k2 ? lq_launch<BN, CG, 2>(p, x, w_slots, c->sm_count, st) : lq_launch<BN, CG, 1>(p, x, w_slots, c->sm_count, st)
+    switch (best) {
+    case 0: e = lq_launch<256, 2, 1>(p, x, w_slots, c->sm_count, st); break;
+    case 1: LQ_GO(192, 2); break;
+    case 2: LQ_GO(160, 2); break;
+    case 3: LQ_GO(128, 2); break;
+    case 4: LQ_GO(128, 1); break;
+    case 5: LQ_GO(64, 1); break;
+    case 6: LQ_GO(48, 1); break;
+    default: LQ_GO(32, 1); break;
+    }
+#undef LQ_GO
     if (e == cudaSuccess) ++*launches;
     return e;
 }

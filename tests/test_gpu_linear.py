@@ -180,3 +180,13 @@ def test_fused_layer_and_push_on_random_shapes():
             assert gu.guards_intact(wh, P) and np.array_equal(v.cpu().numpy(), want), tag
         assert bool((words == 9).all()), tag
         t.close()
+
+
+@pytest.mark.parametrize("T,K,E,k", [
+    (3, 128, 768, 8), (9, 200, 800, 16), (127, 192, 640, 8), (70, 64, 4864, 72), (121, 1280, 4864, 0), (140, 128, 3584, 56),
+    (129, 256, 4864, 72), (257, 200, 4864, 72), (300, 192, 5120, 80), (513, 72, 4096, 64), (601, 128, 4096, 64), (601, 320, 4864, 72),
+    (1100, 64, 5120, 80), (1301, 136, 4864, 72)])
+def test_fused_layer_tile_shapes(T, K, E, k):
+    """Every tile shape of the kernel (single blocks of 32 to 128 columns with x tiles of 8 rows and more, pairs of blocks of
+    128 to 256), one and two tiles per place, an odd number of 64-value pieces of K, K that is no multiple of 64."""
+    test_fused_layer(1, T, K, E, k)
