@@ -56,49 +56,102 @@ __device__ __forceinline__ uint32_t qs_code(float x, float inv)
     return __float_as_uint(__fadd_rn(u, 12582912.0f));  // + 1.5 * 2^23: nearest even, the code in the low bits
 }
 
-// 8 values (one uint4 of BF16) -> 4 codes in each of two 32-bit halves, packed from bit 0.  As in the Int4
-// kernels the patterns 0x4B400000 + code are summed with one shift-add each and the constant part is removed at
-// the end: what is left is the sum of the signed codes times their weights, and adding the weights' 2^(B-1)
-// makes the digits non-negative, so that they do not borrow from one another.
-template <int B>
-__device__ __forceinline__ void qs_quant8(const uint4 v, const float2 (&inv)[4], uint32_t (&half)[2])
+// 8 values -> 8 codes of B bits, four in each of two halves (two's complement, packed from bit 0).  inv: the reciprocal
+// steps in pairs (i, i + 4): the two halves run side by side in packed instructions.
+//
+// Per value u = fl(x * inv), clamped, r = fl(u + 1.5 * 2^23): nearest even, an integer code on top of the magic number.
+// From 6 bits on both clamps are minima and maxima and the shifted patterns are summed as integers.  Up to 5 bits the
+// upper clamp and the packing move to the FMA pipe, which runs at twice the integer pipe's rate: t = sat(r / 2^B + c) with
+// c such that t = 1 at the highest code (exact: every value in range is a multiple of 2^-B); 2^B t - 1 = code + 2^(B-1) is
+// the code's digit with the sign bit flipped, and four digits are put together by FMAs as an integer below 2^20 on
+// top of 2^23.  (18 integer-pipe instructions per 8 codes instead of 34; 4 x 2048 x 5120, 51 selected: 26.9 -> 26.3 us;
+// at 8 bits, where pairs of digits would be needed, 29.7 -> 30.2 us.)  NaN gives the lowest code (the lower clamp drops
+// it), infinities saturate.
+__device__ __forceinline__ float qs_sat_fma(float a, float b, float c)
 {
-    constexpr float lo = -(float)(1 << (B - 1)), hi = (float)((1 << (B - 1)) - 1);
+    float d;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+template <int B>
+__device__ __forceinline__ void qs_quant_halves(const uint4 v, const float2 (&inv)[4], uint32_t (&half)[2])
+{
+    constexpr float lo = -(float)(1 << (B - 1)), hi = (float)((1 << (B - 1)) - 1), scale = 1.0f / (float)(1 << B);
+    constexpr float c = 1.0f - (12582912.0f + hi) * scale;
     constexpr uint32_t ones = 1u + (1u << B) + (1u << (2 * B)) + (1u << (3 * B));
     constexpr uint32_t sign = ones << (B - 1);
+    constexpr float base = 8388608.0f - (float)ones;
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    float2 s = make_float2(base, base);
+    uint32_t n[2] = {0u, 0u};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        uint32_t acc = 0;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const uint32_t x = w[2 * h + i];
-            float2 u = __fmul2_rn(make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u)), inv[2 * h + i]);
-            u.x = fminf(fmaxf(u.x, lo), hi);
-            u.y = fminf(fmaxf(u.y, lo), hi);
-            const float2 r = __fadd2_rn(u, make_float2(12582912.0f, 12582912.0f));
-            acc += __float_as_uint(r.x) << (2 * i * B);
-            acc += __float_as_uint(r.y) << ((2 * i + 1) * B);
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t a = w[i >> 1], b = w[2 + (i >> 1)];
+        const float2 x = (i & 1) ? make_float2(__uint_as_float(a & 0xFFFF0000u), __uint_as_float(b & 0xFFFF0000u))
+                                 : make_float2(__uint_as_float(a << 16), __uint_as_float(b << 16));
+        float2 u = __fmul2_rn(x, inv[i]);
+        u.x = fmaxf(u.x, lo);
+        u.y = fmaxf(u.y, lo);
+        if constexpr (B > 5) {
+            u.x = fminf(u.x, hi);
+            u.y = fminf(u.y, hi);
         }
-        half[h] = (acc - 0x4B400000u * ones + sign) ^ sign;
+        const float2 r = __fadd2_rn(u, make_float2(12582912.0f, 12582912.0f));
+        if constexpr (B <= 5) {
+            constexpr float unit = (float)(1 << B);
+            const float at = unit * (float)(1 << (i * B));  // (the digit's place, times 2^B)
+            s = __ffma2_rn(make_float2(qs_sat_fma(r.x, scale, c), qs_sat_fma(r.y, scale, c)), make_float2(at, at), s);
+        } else {
+            n[0] += __float_as_uint(r.x) << (i * B);
+            n[1] += __float_as_uint(r.y) << (i * B);
+        }
     }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        half[h] = B <= 5 ? __float_as_uint(h ? s.y : s.x) ^ (0x4B000000u | sign)  // the exponent goes, the sign bits flip
+                         : (n[h] - 0x4B400000u * ones + sign) ^ sign;            // likewise, with the patterns' constant part
 }
 
-// B bytes of codes (the two halves of a group) -> shared memory, B-byte aligned
+// A group's 8 codes in registers: one word of 8B bits up to 4 bits, else two words of 4B bits.
+__host__ __device__ constexpr int qs_group_words(int B) { return B <= 4 ? 1 : 2; }
 template <int B>
-__device__ __forceinline__ void qs_store_group(uint8_t *dst, const uint32_t (&half)[2])
+__device__ __forceinline__ void qs_quant8(const uint4 v, const float2 (&inv)[4], uint32_t (&w)[qs_group_words(B)])
 {
-    const uint64_t bits = (uint64_t)half[0] | ((uint64_t)half[1] << (4 * B));
-    if (B == 8) {
-        *reinterpret_cast<uint2 *>(dst) = make_uint2(half[0], half[1]);
-    } else if (B == 4) {
-        *reinterpret_cast<uint32_t *>(dst) = (uint32_t)bits;
-    } else if (B == 2 || B == 6) {
-#pragma unroll
-        for (int j = 0; j < B / 2; ++j) reinterpret_cast<uint16_t *>(dst)[j] = (uint16_t)(bits >> (16 * j));
+    uint32_t half[2];
+    qs_quant_halves<B>(v, inv, half);
+    if constexpr (B == 4) {
+        w[0] = __byte_perm(half[0], half[1], 0x5410);
+    } else if constexpr (B < 4) {
+        w[0] = half[0] | half[1] << (4 * B);
     } else {
+        w[0] = half[0];
+        w[1] = half[1];
+    }
+}
+// code n of a group: which word, and its field there
+template <int B>
+__device__ __forceinline__ uint32_t qs_field_shift(int n) { return (uint32_t)((B <= 4 ? n : n & 3) * B); }
+template <int B>
+__device__ __forceinline__ bool qs_field_in(int n, int word) { return B <= 4 || (n >> 2) == word; }
+
+// B bytes of codes -> shared memory, B-byte aligned
+template <int B>
+__device__ __forceinline__ void qs_store_group(uint8_t *dst, const uint32_t (&w)[qs_group_words(B)])
+{
+    if constexpr (B == 8) {
+        *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
+    } else if constexpr (B == 4) {
+        *reinterpret_cast<uint32_t *>(dst) = w[0];
+    } else {
+        uint64_t bits = w[0];
+        if constexpr (B > 4) bits |= (uint64_t)w[1] << (4 * B);
+        if constexpr (B % 2 == 0) {
 #pragma unroll
-        for (int j = 0; j < B; ++j) dst[j] = (uint8_t)(bits >> (8 * j));
+            for (int j = 0; j < B / 2; ++j) reinterpret_cast<uint16_t *>(dst)[j] = (uint16_t)(bits >> (16 * j));
+        } else {
+#pragma unroll
+            for (int j = 0; j < B; ++j) dst[j] = (uint8_t)(bits >> (8 * j));
+        }
     }
 }
 
@@ -177,13 +230,12 @@ __global__ void __launch_bounds__(QS_THREADS, VEC ? 4 : 2) quantize_stream_tile(
         if (VEC) {
             const float4 a = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g));
             const float4 b = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g + 4));
-            inv[0] = make_float2(a.x, a.y); inv[1] = make_float2(a.z, a.w);
-            inv[2] = make_float2(b.x, b.y); inv[3] = make_float2(b.z, b.w);
+            inv[0] = make_float2(a.x, b.x); inv[1] = make_float2(a.y, b.y);
+            inv[2] = make_float2(a.z, b.z); inv[3] = make_float2(a.w, b.w);
         } else {
 #pragma unroll
             for (int n = 0; n < 4; ++n)
-                inv[n] = make_float2(8 * g + 2 * n < E ? __ldg(inv_s + 8 * g + 2 * n) : 0.0f,
-                                     8 * g + 2 * n + 1 < E ? __ldg(inv_s + 8 * g + 2 * n + 1) : 0.0f);
+                inv[n] = make_float2(8 * g + n < E ? __ldg(inv_s + 8 * g + n) : 0.0f, 8 * g + n + 4 < E ? __ldg(inv_s + 8 * g + n + 4) : 0.0f);
         }
         const uint32_t mask = __ldg(p.grp + g) & 0xFFu;
         const uint16_t *src = y + 8 * g;
@@ -206,14 +258,14 @@ __global__ void __launch_bounds__(QS_THREADS, VEC ? 4 : 2) quantize_stream_tile(
             }
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                uint32_t half[2];
-                qs_quant8<B>(v[r], inv, half);
+                uint32_t w[qs_group_words(B)];
+                qs_quant8<B>(v[r], inv, w);
                 if (mask) {  // the holes' codes come later
 #pragma unroll
                     for (int n = 0; n < 8; ++n)
-                        if (mask & (1u << n)) half[n >> 2] &= ~(((1u << B) - 1u) << ((n & 3) * B));
+                        if (mask & (1u << n)) w[B <= 4 ? 0 : n >> 2] &= ~(((1u << B) - 1u) << qs_field_shift<B>(n));
                 }
-                qs_store_group<B>(dst + (r0 + r) * RW * 4, half);
+                qs_store_group<B>(dst + (r0 + r) * RW * 4, w);
             }
         }
     }
@@ -262,8 +314,10 @@ cudaError_t launch_quantize_tile(const QSParams &p, bool vec, int threads, dim3 
 //   and 16 of its first, or-ed together), for every row of the block and the row ahead of it.
 // A block may therefore start at any row.  (Built before this and measured at 4 x 2048 x 5120, 51 selected: strings of
 // whole tiles with a barrier of all consumers per 4 rows 43 us; one tile of 8 rows per block, four blocks per SM, 29.5 us;
-// this kernel 26.9 us against 15.9 us for its bytes at 6.65 TB/s; the shape-generic kernel 114 us.
-// 3 bits 41.1 -> 28.4 us, 8 x 1000 x 4608 at 8 bits 39.5 -> 29.7 us.  115 warp instructions per 32 groups: the ALU pipe.)
+// this kernel 23.9 us against 15.9 us for its bytes at 6.65 TB/s; the shape-generic kernel 114 us.
+// 3 bits 41.1 -> 25.0 us, 8 x 1000 x 4608 at 8 bits 39.5 -> 29.7 us.  Bound by instruction issue: 115 warp instructions
+// per 32 groups took 26.9 us; with one word per group up to 4 bits, field masks worked out once and the second hole's
+// shuffle only in warps that have one, 23.9 us.)
 constexpr int QS_STAGE = 4;             // rows of a stage
 constexpr int QS_MAX_THREADS = 768;     // 80 registers a thread
 constexpr int QS_MAX_GPT = 2;           // groups of a consumer lane
@@ -446,10 +500,11 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
     // ---------------- consumers: constants (see quantize_tiled)
     const int warp = tid >> 5;  // consumer warp
     float2 inv[GPT][4];
-    uint32_t mask[GPT], w_off[GPT], f_sh[GPT][2], h_in[GPT][2], keep[GPT][2];
+    constexpr int NW = qs_group_words(B);
+    uint32_t mask[GPT], w_off[GPT], f_sh[GPT][2], field[GPT][2][NW], keep[GPT][NW];
     int hb[GPT], n_wh[GPT], src0[GPT];
     float w_inv[GPT];
-    bool serial[GPT];
+    bool serial[GPT], two[GPT];
     const int my_hp = tid < k ? __ldg(p.hp_idx + tid) : 0;
 #pragma unroll
     for (int a = 0; a < GPT; ++a) {
@@ -462,8 +517,8 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
             const float4 i0 = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g));
             const float4 i1 = __ldg(reinterpret_cast<const float4 *>(inv_s + 8 * g + 4));
             const uint32_t gd = __ldg(p.grp + g);
-            inv[a][0] = make_float2(i0.x, i0.y); inv[a][1] = make_float2(i0.z, i0.w);
-            inv[a][2] = make_float2(i1.x, i1.y); inv[a][3] = make_float2(i1.z, i1.w);
+            inv[a][0] = make_float2(i0.x, i1.x); inv[a][1] = make_float2(i0.y, i1.y);  // (pairs: see qs_quant_halves)
+            inv[a][2] = make_float2(i0.z, i1.z); inv[a][3] = make_float2(i0.w, i1.w);
             mask[a] = gd & 0xFFu;
             if (8 * g + 8 > L) mask[a] &= (1u << (L - 8 * g)) - 1u;  // (features at or above L have no slot)
             hb[a] = (int)(gd >> 8);
@@ -479,6 +534,7 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
         n_wh[a] = __shfl_sync(0xffffffffu, incl, 31);
         const int hb_warp = __shfl_sync(0xffffffffu, hb[a], 0);
         serial[a] = n_wh[a] > 32 || __any_sync(0xffffffffu, nh > 2);
+        two[a] = __any_sync(0xffffffffu, nh > 1);  // some group of the warp has a second hole
         w_off[a] = 0;
         w_inv[a] = 0.0f;
         if (lane < n_wh[a] && !serial[a]) {
@@ -486,19 +542,18 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
             w_off[a] = (uint32_t)f * 2u;
             w_inv[a] = __ldg(inv_s + f);
         }
-        keep[a][0] = keep[a][1] = 0xFFFFFFFFu;
-        f_sh[a][0] = f_sh[a][1] = 0;
-        h_in[a][0] = h_in[a][1] = 0;
         uint32_t m = mask[a];
 #pragma unroll
+        for (int j = 0; j < NW; ++j) keep[a][j] = 0xFFFFFFFFu;
+#pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (!m) break;
-            const int n = __ffs(m) - 1;
-            const uint32_t sh = (uint32_t)((n & 3) * B), field = ((1u << B) - 1u) << sh;
-            f_sh[a][h] = sh;
-            h_in[a][h] = n < 4 ? 1u : 2u;  // 0: no such hole, 1: in the lower half, 2: in the upper one
-            keep[a][0] &= n < 4 ? ~field : 0xFFFFFFFFu;
-            keep[a][1] &= n < 4 ? 0xFFFFFFFFu : ~field;
+            const int n = m ? __ffs(m) - 1 : 0;
+            f_sh[a][h] = qs_field_shift<B>(n);
+#pragma unroll
+            for (int j = 0; j < NW; ++j) {
+                field[a][h][j] = m && qs_field_in<B>(n, j) ? ((1u << B) - 1u) << f_sh[a][h] : 0u;
+                keep[a][j] &= ~field[a][h][j];
+            }
             m &= m - 1;
         }
     }
@@ -533,13 +588,13 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
             };
             auto row_o = [&](int r) { return 31 - ((in0 + r * LB + a0 + 31) & 31); };
             // a row's codes: at 4 bits a group is a word, so its neighbour's comes by a shuffle; else to the bit string
-            auto emit = [&](int r, const uint32_t (&half)[2], bool store) {
-                if (B == 4) {
-                    const uint32_t own = half[0] | half[1] << 16, next = __shfl_down_sync(0xffffffffu, own, 1);
+            auto emit = [&](int r, const uint32_t (&wd)[NW], bool store) {
+                if constexpr (B == 4) {
+                    const uint32_t next = __shfl_down_sync(0xffffffffu, wd[0], 1);
                     const int o = row_o(r);
-                    if (store) put(r, 0, o, __funnelshift_r(own, next, o));
+                    if (store) put(r, 0, o, __funnelshift_r(wd[0], next, o));
                 } else {
-                    qs_store_group<B>(reinterpret_cast<uint8_t *>(ws + r * WW) + lane * B, half);
+                    qs_store_group<B>(reinterpret_cast<uint8_t *>(ws + r * WW) + lane * B, wd);
                 }
             };
             if (!serial[a]) {
@@ -553,21 +608,25 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
                 }
 #pragma unroll
                 for (int r = 0; r < QS_STAGE; ++r) {
-                    uint32_t half[2];
-                    qs_quant8<B>(v[r], inv[a], half);
-                    if (n_wh[a]) {  // uniform over the warp
+                    uint32_t wd[NW];
+                    qs_quant8<B>(v[r], inv[a], wd);
+                    if (n_wh[a]) {  // uniform over the warp, as is two
                         const uint32_t qv = qs_code<B>(__uint_as_float(fx[r] << 16), w_inv[a]) & ((1u << B) - 1u);
                         const uint32_t c0 = __shfl_sync(0xffffffffu, qv, src0[a]) << f_sh[a][0];
-                        const uint32_t c1 = __shfl_sync(0xffffffffu, qv, src0[a] + 1) << f_sh[a][1];
-                        half[0] = (half[0] & keep[a][0]) | (h_in[a][0] == 1u ? c0 : 0u) | (h_in[a][1] == 1u ? c1 : 0u);
-                        half[1] = (half[1] & keep[a][1]) | (h_in[a][0] == 2u ? c0 : 0u) | (h_in[a][1] == 2u ? c1 : 0u);
+#pragma unroll
+                        for (int j = 0; j < NW; ++j) wd[j] = (wd[j] & keep[a][j]) | (c0 & field[a][0][j]);
+                        if (two[a]) {
+                            const uint32_t c1 = __shfl_sync(0xffffffffu, qv, src0[a] + 1) << f_sh[a][1];
+#pragma unroll
+                            for (int j = 0; j < NW; ++j) wd[j] |= c1 & field[a][1][j];
+                        }
                     }
-                    emit(r, half, r < rows);
+                    emit(r, wd, r < rows);
                 }
             } else {
                 for (int r = 0; r < rows; ++r) {  // a warp on the serial path: every hole patched by its owner
-                    uint32_t half[2];
-                    qs_quant8<B>(*reinterpret_cast<const uint4 *>(src + r * row_bytes), inv[a], half);
+                    uint32_t wd[NW];
+                    qs_quant8<B>(*reinterpret_cast<const uint4 *>(src + r * row_bytes), inv[a], wd);
                     uint32_t m = mask[a];
                     for (int h = 0; m; ++h) {
                         const int n = __ffs(m) - 1;
@@ -575,12 +634,15 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
                         const int f = __ldg(p.filler + hb[a] + h);
                         const uint32_t x = *reinterpret_cast<const uint16_t *>(stage8 + r * row_bytes + 2 * f);
                         const uint32_t c = qs_code<B>(__uint_as_float(x << 16), __ldg(inv_s + f)) & ((1u << B) - 1u);
-                        const uint32_t sh = (uint32_t)((n & 3) * B);
-                        if (n < 4) half[0] = (half[0] & ~(((1u << B) - 1u) << sh)) | (c << sh);
-                        else half[1] = (half[1] & ~(((1u << B) - 1u) << sh)) | (c << sh);
+                        const uint32_t sh = qs_field_shift<B>(n);
+#pragma unroll
+                        for (int j = 0; j < NW; ++j) {
+                            const uint32_t fm = qs_field_in<B>(n, j) ? ((1u << B) - 1u) << sh : 0u;
+                            wd[j] = (wd[j] & ~fm) | (c << sh & fm);
+                        }
                     }
                     __syncwarp();
-                    emit(r, half, true);
+                    emit(r, wd, true);
                 }
             }
             if (B != 4) {
