@@ -440,11 +440,14 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
     }
     if constexpr (PUSH) {
         // Publication.  The block's consumer threads meet (their stores happen-before the fence below), one
-        // thread orders them before its count at system scope; the block that counts last has thereby
-        // observed every other block's stores and releases the arrival words to the destinations' owners.
+        // thread orders them before its count at GPU scope (a release to the counting blocks); the block that counts
+        // last has thereby observed every other block's stores and releases them, with its own, to the destinations'
+        // owners at system scope.  Release is cumulative, so one fence at system scope per launch is enough: it costs a
+        // block about 2 us, and with one in every block, ahead of its count, the last block's came on top of the slowest's
+        // (512 x 5120, one destination: 8.4 -> 5.3 us a launch; the plain quantiser takes 2.7 us).
         asm volatile("bar.sync 2, %0;" ::"r"(NT) : "memory");
         if (tid == 0) {
-            __threadfence_system();
+            __threadfence();
             // a block whose waits ran out counts in the upper half as well: the payload is then incomplete,
             // the words are not written, and the receivers' own bounded waits flag the step
             const unsigned int prev = atomicAdd(p.done, s_failed ? 0x10001u : 1u);

@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
         // publication, as quantize_tiled: the block that counts last has observed every block's stores
         asm volatile("bar.sync 2, %0;" ::"r"(NT + 32) : "memory");
         if (tid == 0) {
-            __threadfence_system();
+            __threadfence();
             const unsigned int prev = atomicAdd(pp.done, s_failed ? 0x10001u : 1u);
             if ((prev & 0xFFFFu) == gridDim.x - 1) {
                 *pp.done = 0u;
