@@ -8,6 +8,7 @@ if the library cannot be loaded the import of :func:`lib` raises.
 from __future__ import annotations
 
 import ctypes
+import struct
 from ctypes import POINTER, byref, c_char_p, c_double, c_float, c_int, c_int32, c_int64, c_size_t, c_void_p
 from pathlib import Path
 
@@ -51,17 +52,17 @@ SIGNATURES = {
     "tpq_payload_bytes_for_bits": (c_size_t, [c_int64, c_int64, c_int64, c_int]),
     "tpq_comm_bytes": (c_int, [c_void_p, c_int64, POINTER(CommReport)]),
     "tpq_quantize_pack": (c_int, [c_void_p, c_int, c_void_p, c_int64, c_int64, c_void_p, c_size_t, c_void_p]),
-    "tpq_quantize_pack_batch": (c_int, [c_void_p, c_int, c_int, POINTER(c_void_p), c_int64, c_int64, POINTER(c_void_p),
+    "tpq_quantize_pack_batch": (c_int, [c_void_p, c_int, c_int, c_void_p, c_int64, c_int64, c_void_p,
                                         c_size_t, c_void_p]),
-    "tpq_dequant_reduce": (c_int, [c_void_p, POINTER(c_void_p), c_int, c_int64, c_void_p, c_int, c_int64, c_void_p]),
-    "tpq_dequant_reduce_bias": (c_int, [c_void_p, POINTER(c_void_p), c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
+    "tpq_dequant_reduce": (c_int, [c_void_p, c_void_p, c_int, c_int64, c_void_p, c_int, c_int64, c_void_p]),
+    "tpq_dequant_reduce_bias": (c_int, [c_void_p, c_void_p, c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
                                         c_void_p]),
     "tpq_permute_weight": (c_int, [c_void_p, c_void_p, c_int64, c_void_p, c_void_p]),
     "tpq_linear_quantize_pack": (c_int, [c_void_p, c_int, c_void_p, c_void_p, c_int64, c_int64, c_void_p, c_size_t, c_void_p,
                                          c_void_p]),
-    "tpq_quantize_pack_push": (c_int, [c_void_p, c_int, c_void_p, c_int64, c_int64, POINTER(c_void_p), POINTER(c_void_p),
+    "tpq_quantize_pack_push": (c_int, [c_void_p, c_int, c_void_p, c_int64, c_int64, c_void_p, c_void_p,
                                        c_int, c_size_t, ctypes.c_uint32, c_void_p]),
-    "tpq_dequant_reduce_arrivals": (c_int, [c_void_p, POINTER(c_void_p), c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
+    "tpq_dequant_reduce_arrivals": (c_int, [c_void_p, c_void_p, c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
                                             c_void_p, ctypes.c_uint32, ctypes.c_uint64, c_void_p]),
     "tpq_wait_arrivals": (c_int, [c_void_p, c_void_p, c_int, ctypes.c_uint32, ctypes.c_uint64, c_void_p]),
     "tpq_get_state": (c_int, [c_void_p, c_void_p, POINTER(c_size_t)]),
@@ -96,6 +97,26 @@ class TpqError(RuntimeError):
     def __init__(self, status: int, message: str):
         super().__init__(f"tpq status {status} ({lib().tpq_status_string(status).decode()}): {message}")
         self.status = status
+
+
+_packers = {}   # number of pointers -> struct.Struct
+
+
+def _ptrs(ptrs):
+    """A host array of device pointers: ctypes arrays as they are, sequences of addresses packed into bytes (a fifth of
+    the time that building and passing a ctypes array takes)."""
+    if isinstance(ptrs, (list, tuple)):
+        n = len(ptrs)
+        pack = _packers.get(n)
+        if pack is None:
+            pack = _packers[n] = struct.Struct(f"{n}Q")
+        try:
+            return pack.pack(*ptrs)
+        except struct.error:   # None or c_void_p among them
+            pass
+    elif isinstance(ptrs, ctypes.Array):
+        return ptrs
+    return (c_void_p * len(ptrs))(*ptrs)
 
 
 def _fp(a: np.ndarray):
@@ -207,49 +228,57 @@ class Tpq:
 
     def quantize_pack(self, shard: int, y_ptr: int, T: int, payload_ptr: int, payload_capacity: int,
                       row_stride: int | None = None, stream: int = 0):
-        self._check(lib().tpq_quantize_pack(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride,
-                                            payload_ptr, payload_capacity, stream))
+        st = _lib.tpq_quantize_pack(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride, payload_ptr,
+                                    payload_capacity, stream)
+        if st:
+            self._check(st)
 
     def quantize_pack_batch(self, first_shard: int, y_ptrs, T: int, payload_ptrs, payload_capacity: int,
                             row_stride: int | None = None, stream: int = 0):
         n = len(y_ptrs)
         assert len(payload_ptrs) == n
-        ya = y_ptrs if isinstance(y_ptrs, ctypes.Array) else (c_void_p * n)(*y_ptrs)
-        pa = payload_ptrs if isinstance(payload_ptrs, ctypes.Array) else (c_void_p * n)(*payload_ptrs)
-        self._check(lib().tpq_quantize_pack_batch(self._h, first_shard, n, ya, T,
-                                                  self.E if row_stride is None else row_stride, pa,
-                                                  payload_capacity, stream))
+        ya = _ptrs(y_ptrs)
+        pa = _ptrs(payload_ptrs)
+        st = _lib.tpq_quantize_pack_batch(self._h, first_shard, n, ya, T, self.E if row_stride is None else row_stride, pa,
+                                          payload_capacity, stream)
+        if st:
+            self._check(st)
 
     def dequant_reduce(self, payload_ptrs, T: int, out_ptr: int, out_dtype: int = TPQ_OUT_BF16,
                        out_row_stride: int | None = None, stream: int = 0, bias_ptr: int | None = None,
                        arrived_ptr: int | None = None, epoch: int = 0, timeout_ns: int = 0):
-        arr = payload_ptrs if isinstance(payload_ptrs, ctypes.Array) else (c_void_p * len(payload_ptrs))(*payload_ptrs)
+        arr = _ptrs(payload_ptrs)
         stride = self.E if out_row_stride is None else out_row_stride
         if arrived_ptr is not None:
-            self._check(lib().tpq_dequant_reduce_arrivals(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride,
-                                                          bias_ptr, arrived_ptr, epoch & 0xFFFFFFFF, timeout_ns, stream))
+            st = _lib.tpq_dequant_reduce_arrivals(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr,
+                                                  arrived_ptr, epoch & 0xFFFFFFFF, timeout_ns, stream)
         elif bias_ptr is None:
-            self._check(lib().tpq_dequant_reduce(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, stream))
+            st = _lib.tpq_dequant_reduce(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, stream)
         else:
-            self._check(lib().tpq_dequant_reduce_bias(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride,
-                                                      bias_ptr, stream))
+            st = _lib.tpq_dequant_reduce_bias(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr, stream)
+        if st:
+            self._check(st)
 
     def permute_weight(self, w_ptr: int, K: int, w_slots_ptr: int, stream: int = 0):
         self._check(lib().tpq_permute_weight(self._h, w_ptr, K, w_slots_ptr, stream))
 
     def linear_quantize_pack(self, shard: int, x_ptr: int, w_slots_ptr: int, T: int, K: int, payload_ptr: int,
                              payload_capacity: int, y_slots_ptr: int | None = None, stream: int = 0):
-        self._check(lib().tpq_linear_quantize_pack(self._h, shard, x_ptr, w_slots_ptr, T, K, payload_ptr, payload_capacity,
-                                                   y_slots_ptr, stream))
+        st = _lib.tpq_linear_quantize_pack(self._h, shard, x_ptr, w_slots_ptr, T, K, payload_ptr, payload_capacity,
+                                           y_slots_ptr, stream)
+        if st:
+            self._check(st)
 
     def quantize_pack_push(self, shard: int, y_ptr: int, T: int, dst_ptrs, arrived_ptrs, dst_capacity: int, epoch: int,
                            row_stride: int | None = None, stream: int = 0):
         n = len(dst_ptrs)
         assert len(arrived_ptrs) == n
-        da = dst_ptrs if isinstance(dst_ptrs, ctypes.Array) else (c_void_p * n)(*dst_ptrs)
-        aa = arrived_ptrs if isinstance(arrived_ptrs, ctypes.Array) else (c_void_p * n)(*arrived_ptrs)
-        self._check(lib().tpq_quantize_pack_push(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride,
-                                                 da, aa, n, dst_capacity, epoch & 0xFFFFFFFF, stream))
+        da = _ptrs(dst_ptrs)
+        aa = _ptrs(arrived_ptrs)
+        st = _lib.tpq_quantize_pack_push(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride, da, aa, n,
+                                         dst_capacity, epoch & 0xFFFFFFFF, stream)
+        if st:
+            self._check(st)
 
     def wait_arrivals(self, arrived_ptr: int, n: int, epoch: int, timeout_ns: int = 0, stream: int = 0):
         self._check(lib().tpq_wait_arrivals(self._h, arrived_ptr, n, epoch & 0xFFFFFFFF, timeout_ns, stream))
