@@ -1079,6 +1079,329 @@ cudaError_t launch_dequant_stream(const DSParams &p, int fp32_out, cudaStream_t 
     return tpq_launch_pdl(kern, dim3((unsigned)(p.panels * p.gy)), dim3(DS_THREADS), smem, st, p);
 }
 
+// ----------------------------------------------------------------------------------------------
+// Dequantise + reduce for up to four devices: the row kernel (dequant.cu) at bit granularity.
+//
+// One persistent block per SM on a run of adjacent rows, DW_ROWS at a time.  Warp 0 streams the devices' code rows
+// into a ring (one bulk copy per device and stage, from the 16-byte boundary at or below the first bit).  A main
+// thread owns a group of 8 features with the steps of all devices in registers (0 at selected features), funnels its bits
+// out of two (three) words, stores the whole group and then overwrites the lanes of selected features with the sums
+// the auxiliary warps left in shared memory (same thread, same address: ordered).  An auxiliary thread per rank h adds up
+// the devices' BF16 values of selected feature h, loaded from memory a stage ahead (the BF16 rows are not aligned for bulk
+// copies and end with the payload), and decodes column L + h of the output where that is a filler feature.
+// No warp waits for another's global stores.  Measured against the panel kernel above it: XXDW
+// ----------------------------------------------------------------------------------------------
+constexpr int DW_ROWS = 4, DW_MAX_DEV = 4, DW_MAIN = 640, DW_AUX = 96, DW_MAX_K = 384;
+
+struct DWParams {
+    DSParams d;
+    const float *s_k;      // [N][E] steps, 0 at selected features
+    const int32_t *pos;    // [E]
+    int nstage;
+    uint32_t dev_bytes;    // a device's part of a stage
+    int64_t rows_per_block;
+    int *status;
+};
+
+__host__ __device__ inline uint32_t dw_dev_bytes(int L, int B) { return (uint32_t)(((DW_ROWS * L * B + 127 + 127) / 128 + 1) * 16); }
+inline size_t dw_smem_bytes(int N, uint32_t dev_bytes, int k, int nstage)
+{
+    return (size_t)nstage * ((size_t)N * dev_bytes + (size_t)DW_ROWS * k * 4 + 24) + 16;
+}
+
+template <int B, bool FP32OUT, bool HAS_BIAS>
+__global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(const DWParams pp)
+{
+    extern __shared__ __align__(128) uint8_t dw_smem[];
+    const DSParams &p = pp.d;
+    const int N = p.N, E = p.E, k = p.k, L = p.L, G = (L + 7) >> 3, nstage = pp.nstage;
+    const uint32_t LB = (uint32_t)L * B;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t stage_bytes = (uint32_t)N * pp.dev_bytes;
+    uint32_t *const sums = reinterpret_cast<uint32_t *>(dw_smem + (size_t)nstage * stage_bytes);  // [nstage][DW_ROWS][k]
+    uint64_t *const full = reinterpret_cast<uint64_t *>(dw_smem + (((size_t)nstage * (stage_bytes + (size_t)DW_ROWS * k * 4) + 15) & ~(size_t)15));
+    uint64_t *const empty = full + nstage, *const sums_ready = empty + nstage;
+    const int64_t t_begin = (int64_t)blockIdx.x * pp.rows_per_block;
+    const int rows_mine = (int)(p.T - t_begin < pp.rows_per_block ? p.T - t_begin : pp.rows_per_block);
+
+    tpq_grid_dep_launch();
+    if (p.arr.words) {
+        tpq_block_wait_arrivals(p.arr);
+        __syncthreads();
+    }
+    if (tid < 32) {
+        // ---------------- producer warp: lane i copies device i's rows
+        if (lane == 0) {
+            for (int s = 0; s < nstage; ++s) {
+                mbar_init(smem_u32(&full[s]), 1);
+                mbar_init(smem_u32(&empty[s]), (blockDim.x - 32) / 32);
+                mbar_init(smem_u32(&sums_ready[s]), DW_AUX / 32);
+            }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");  // the barriers exist
+        tpq_grid_dep_wait();  // the payloads and the output buffer may still be in use by the kernel ahead
+        int st = 0;
+        uint32_t parity = 1;
+        for (int it = 0, r0 = 0; r0 < rows_mine; ++it, r0 += DW_ROWS) {
+            const int rows = rows_mine - r0 < DW_ROWS ? rows_mine - r0 : DW_ROWS;
+            const int64_t bit = (t_begin + r0) * (int64_t)LB, from = (bit >> 3) & ~(int64_t)15;
+            const int64_t to = ((bit + (int64_t)rows * LB + 127) >> 7) << 4;  // (the code section is a multiple of 16 bytes)
+            const uint32_t bytes = (uint32_t)(to - from), bar = smem_u32(&full[st]);
+            int ok = 1;
+            if (lane == 0) {
+                if (it >= nstage && !mbar_wait(smem_u32(&empty[st]), parity)) {
+                    atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
+                    ok = 0;
+                } else {
+                    mbar_expect_tx(bar, (uint32_t)N * bytes);
+                }
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            if (!ok) break;
+            if (lane < N) bulk_g2s(smem_u32(dw_smem) + (uint32_t)st * stage_bytes + (uint32_t)lane * pp.dev_bytes, p.pl[lane] + from, bytes, bar);
+            if (++st == nstage) {
+                st = 0;
+                parity ^= 1u;
+            }
+        }
+        return;
+    }
+    int st = 0;
+    uint32_t parity = 0;
+    if (tid < 32 + DW_AUX) {
+        // ---------------- auxiliary warps
+        const int at = tid - 32;
+        const bool on = at < k;
+        const int s_col = on ? __ldg(p.hp_idx + at) : 0;                       // rank `at`: its feature
+        const int ps = on ? __ldg(pp.pos + L + at) : -1;                       // column L + at: its slot (< 0: selected)
+        float c_s[DW_MAX_DEV];
+#pragma unroll
+        for (int i = 0; i < DW_MAX_DEV; ++i) c_s[i] = i < N && ps >= 0 ? __ldg(pp.s_k + (size_t)i * E + L + at) : 0.0f;
+        const float s_b = HAS_BIAS && on ? __ldg(p.bias + s_col) : 0.0f, c_b = HAS_BIAS && on ? __ldg(p.bias + L + at) : 0.0f;
+        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+        tpq_grid_dep_wait();  // the BF16 values are read and columns written without waiting for a copy
+        uint16_t v[DW_ROWS][DW_MAX_DEV];
+        auto load = [&](int r0) {
+            if (on) {
+#pragma unroll
+                for (int r = 0; r < DW_ROWS; ++r)
+#pragma unroll
+                    for (int i = 0; i < DW_MAX_DEV; ++i)
+                        if (r0 + r < rows_mine && i < N)
+                            v[r][i] = __ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + p.lp_bytes) + (t_begin + r0 + r) * k + at);
+            }
+        };
+        // the code of slot `slot` in the row whose first bit is bit `row_bit` of a device's part of the stage
+        auto code = [&](const uint32_t *dev, uint32_t row_bit, int slot) {
+            const uint32_t bit = row_bit + (uint32_t)slot * B;
+            const uint32_t w = __funnelshift_r(dev[bit >> 5], dev[(bit >> 5) + 1], bit & 31u) & ((1u << B) - 1u);
+            return (float)((int)(w ^ (1u << (B - 1))) - (1 << (B - 1)));
+        };
+        auto put = [&](int r, int64_t t, int rank, int col, float sum) {  // a selected feature's sum
+            if (col < L)
+                sums[((size_t)st * DW_ROWS + r) * k + rank] =
+                    FP32OUT ? __float_as_uint(sum) : (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(sum));
+            else
+                ds_store_one<FP32OUT>(p.out, t * p.out_stride + col, sum);
+        };
+        load(0);
+        for (int r0 = 0; r0 < rows_mine; r0 += DW_ROWS) {
+            const int rows = rows_mine - r0 < DW_ROWS ? rows_mine - r0 : DW_ROWS;
+            const int64_t t0 = t_begin + r0;
+            // the stage's previous sums have been read by everybody when its next copies land: wait for those first
+            if (!mbar_wait(smem_u32(&full[st]), parity)) {
+                atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
+                break;
+            }
+            if (on) {
+#pragma unroll
+                for (int r = 0; r < DW_ROWS; ++r) {
+                    if (r >= rows) break;
+                    float sum = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < DW_MAX_DEV; ++i)
+                        if (i < N) sum = __fadd_rn(sum, __uint_as_float((uint32_t)v[r][i] << 16));
+                    put(r, t0 + r, at, s_col, HAS_BIAS ? __fadd_rn(sum, s_b) : sum);
+                }
+            }
+            for (int h = at + DW_AUX; h < k; h += DW_AUX) {  // more selected features than threads
+                const int col = __ldg(p.hp_idx + h);
+                for (int r = 0; r < rows; ++r) {
+                    float sum = 0.0f;
+                    for (int i = 0; i < N; ++i)
+                        sum = __fadd_rn(sum, __uint_as_float((uint32_t)__ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + p.lp_bytes) + (t0 + r) * k + h) << 16));
+                    put(r, t0 + r, h, col, HAS_BIAS ? __fadd_rn(sum, __ldg(p.bias + col)) : sum);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sums_ready[st]));  // (release: the sums are visible to whoever waits)
+            if (r0 + DW_ROWS < rows_mine) load(r0 + DW_ROWS);
+            // the last k columns: filler features, decoded from the holes' slots that carry them
+            const uint8_t *const stage = dw_smem + (size_t)st * stage_bytes;
+            const uint32_t rem = (uint32_t)((t0 * (int64_t)LB) & 127);
+            for (int h = at; h < k; h += DW_AUX) {
+                const int slot = h == at ? ps : __ldg(pp.pos + L + h);
+                if (slot < 0) continue;
+#pragma unroll 1
+                for (int r = 0; r < rows; ++r) {
+                    float acc = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < DW_MAX_DEV; ++i)
+                        if (i < N)
+                            acc = __fmaf_rn(code(reinterpret_cast<const uint32_t *>(stage + (size_t)i * pp.dev_bytes), rem + (uint32_t)r * LB, slot),
+                                            h == at ? c_s[i] : __ldg(pp.s_k + (size_t)i * E + L + h), acc);
+                    if (HAS_BIAS) acc = __fadd_rn(acc, h == at ? c_b : __ldg(p.bias + L + h));
+                    ds_store_one<FP32OUT>(p.out, (t0 + r) * p.out_stride + L + h, acc);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
+            if (++st == nstage) {
+                st = 0;
+                parity ^= 1u;
+            }
+        }
+        return;
+    }
+    // ---------------- main warps
+    const int g = tid - 32 - DW_AUX;
+    const int lanes = L - 8 * g < 8 ? L - 8 * g : 8;  // slots of the group (the last one may be short, idle threads have none)
+    float2 sc[DW_MAX_DEV][4], b[4];
+    uint32_t mask = 0;
+    int hb = 0;
+#pragma unroll
+    for (int i = 0; i < DW_MAX_DEV; ++i)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) sc[i][h] = make_float2(0.0f, 0.0f);
+    if (lanes > 0) {
+        const uint32_t gd = __ldg(p.grp + g);
+        mask = gd & 0xFFu;
+        if (lanes < 8) mask &= (1u << lanes) - 1u;
+        hb = (int)(gd >> 8);
+#pragma unroll
+        for (int i = 0; i < DW_MAX_DEV; ++i)
+            if (i < N) {
+                const float4 u = __ldg(reinterpret_cast<const float4 *>(pp.s_k + (size_t)i * E + 8 * g));
+                const float4 w = __ldg(reinterpret_cast<const float4 *>(pp.s_k + (size_t)i * E + 8 * g + 4));
+                const float s8[8] = {u.x, u.y, u.z, u.w, w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    sc[i][h] = make_float2(s8[2 * h] * (1.0f / (float)(1u << ds_pos(B, 2 * h))),
+                                           s8[2 * h + 1] * (1.0f / (float)(1u << ds_pos(B, 2 * h + 1))));
+            }
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+        b[h] = HAS_BIAS && lanes > 0 ? make_float2(__ldg(p.bias + 8 * g + 2 * h), __ldg(p.bias + 8 * g + 2 * h + 1)) : make_float2(0.0f, 0.0f);
+    asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+    for (int r0 = 0; r0 < rows_mine; r0 += DW_ROWS) {
+        const int rows = rows_mine - r0 < DW_ROWS ? rows_mine - r0 : DW_ROWS;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), parity))) {
+            atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
+            break;
+        }
+        const int64_t t0 = t_begin + r0;
+        const uint8_t *const stage = dw_smem + (size_t)st * stage_bytes;
+        const uint32_t rem = (uint32_t)((t0 * (int64_t)LB) & 127);
+        int64_t o = t0 * p.out_stride + 8 * (int64_t)g;
+#pragma unroll
+        for (int r = 0; r < DW_ROWS; ++r, o += p.out_stride) {
+            if (r >= rows) break;
+            const uint32_t bit = rem + (uint32_t)r * LB + (uint32_t)(lanes > 0 ? g : 0) * (8 * B);
+            const uint8_t *w = stage + (bit >> 5) * 4;
+            float2 acc[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) acc[h] = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int i = 0; i < DW_MAX_DEV; ++i, w += pp.dev_bytes)
+                if (i < N) {
+                    const uint32_t *const q = reinterpret_cast<const uint32_t *>(w);
+                    const uint32_t lo = __funnelshift_r(q[0], q[1], bit & 31u);
+                    uint32_t hi;
+                    if (B <= 4)
+                        hi = lo >> (B < 8 ? 4 * B : 0);
+                    else {
+                        const uint32_t up = __funnelshift_r(q[1], q[2], bit & 31u);
+                        hi = B == 8 ? up : __funnelshift_r(lo, up, 4 * B & 31);
+                    }
+                    ds_decode4<B>(lo, sc[i][0], sc[i][1], acc[0], acc[1]);
+                    ds_decode4<B>(hi, sc[i][2], sc[i][3], acc[2], acc[3]);
+                }
+            if (HAS_BIAS) {  // (a selected feature's lane is overwritten below)
+#pragma unroll
+                for (int h = 0; h < 4; ++h) acc[h] = __fadd2_rn(acc[h], b[h]);
+            }
+            if (lanes >= 8) {
+                if (FP32OUT) {
+                    float4 *const dst = reinterpret_cast<float4 *>(static_cast<float *>(p.out) + o);
+                    __stcs(dst, make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y));
+                    __stcs(dst + 1, make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y));
+                } else {
+                    uint32_t x[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const __nv_bfloat162 t = __floats2bfloat162_rn(acc[h].x, acc[h].y);
+                        x[h] = *reinterpret_cast<const uint32_t *>(&t);
+                    }
+                    __stcs(reinterpret_cast<uint4 *>(static_cast<uint16_t *>(p.out) + o), make_uint4(x[0], x[1], x[2], x[3]));
+                }
+            } else {
+#pragma unroll
+                for (int n = 0; n < 8; ++n)
+                    if (n < lanes) ds_store_one<FP32OUT>(p.out, o + n, (n & 1) ? acc[n >> 1].y : acc[n >> 1].x);
+            }
+        }
+        if (__any_sync(0xffffffffu, mask != 0)) {  // the selected features' lanes
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sums_ready[st]), parity))) {
+                atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
+                break;
+            }
+            uint32_t m = mask;
+            for (int h = hb; m; ++h) {
+                const int n = __ffs(m) - 1;
+                m &= m - 1;
+                const uint32_t *sum = sums + (size_t)st * DW_ROWS * k + h;
+                int64_t at = t0 * p.out_stride + 8 * (int64_t)g + n;
+                for (int r = 0; r < rows; ++r, sum += k, at += p.out_stride) {
+                    if (FP32OUT)
+                        static_cast<uint32_t *>(p.out)[at] = *sum;
+                    else
+                        static_cast<uint16_t *>(p.out)[at] = (uint16_t)*sum;
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
+        if (++st == nstage) {
+            st = 0;
+            parity ^= 1u;
+        }
+    }
+}
+
+// ring depth; 0: the shape is the panel kernel's
+int dw_stages(const tpq_ctx *c, int64_t out_stride)
+{
+    const int L = c->E - c->k, G = (L + 7) / 8;
+    if (c->N > DW_MAX_DEV || c->E % 8 || out_stride % 8 || G > DW_MAIN || c->k > DW_MAX_K) return 0;
+    int n = 4;
+    while (n > 1 && dw_smem_bytes(c->N, dw_dev_bytes(L, c->bits), c->k, n) > (size_t)c->smem_optin) --n;
+    return n > 1 ? n : 0;
+}
+
+template <int B>
+cudaError_t launch_dequant_rows(const DWParams &pp, int fp32_out, unsigned grid, int threads, size_t smem, cudaStream_t st)
+{
+    auto kern = pp.d.bias ? (fp32_out ? dequant_stream_rows<B, true, true> : dequant_stream_rows<B, false, true>)
+                          : (fp32_out ? dequant_stream_rows<B, true, false> : dequant_stream_rows<B, false, false>);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return tpq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, pp);
+}
+
 }  // namespace
 
 // Rows of at least 32 bits (a word of the stream spans two rows at most), bit strings that fit in shared memory,
@@ -1191,6 +1514,28 @@ cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *paylo
     p.filler = c->t.filler; p.n_holes = c->n_holes;
     p.vec = E % 8 == 0 && out_stride % 8 == 0;
     p.out = out; p.bias = c->call_bias; p.arr = c->call_arr;
+    cudaError_t e;
+    if (const int nstage = dw_stages(c, out_stride)) {
+        DWParams pp;
+        pp.d = p;
+        pp.s_k = c->t.s_k; pp.pos = c->t.pos; pp.nstage = nstage; pp.status = c->t.status;
+        pp.dev_bytes = dw_dev_bytes(L, c->bits);
+        pp.rows_per_block = (T + c->sm_count - 1) / c->sm_count;
+        const unsigned grid = (unsigned)((T + pp.rows_per_block - 1) / pp.rows_per_block);
+        const int threads = 32 + DW_AUX + (G + 31) / 32 * 32;
+        const size_t smem = dw_smem_bytes(c->N, pp.dev_bytes, k, nstage);
+        switch (c->bits) {
+        case 2: e = launch_dequant_rows<2>(pp, fp32_out, grid, threads, smem, st); break;
+        case 3: e = launch_dequant_rows<3>(pp, fp32_out, grid, threads, smem, st); break;
+        case 4: e = launch_dequant_rows<4>(pp, fp32_out, grid, threads, smem, st); break;
+        case 5: e = launch_dequant_rows<5>(pp, fp32_out, grid, threads, smem, st); break;
+        case 6: e = launch_dequant_rows<6>(pp, fp32_out, grid, threads, smem, st); break;
+        case 7: e = launch_dequant_rows<7>(pp, fp32_out, grid, threads, smem, st); break;
+        default: e = launch_dequant_rows<8>(pp, fp32_out, grid, threads, smem, st); break;
+        }
+        if (e == cudaSuccess) ++*launches;
+        return e;
+    }
     constexpr int RC = DS_THREADS / DS_CG * DS_R;
     p.panels = (G + DS_CG - 1) / DS_CG;
     p.n_chunks = (T + RC - 1) / RC;
@@ -1199,7 +1544,6 @@ cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *paylo
     if (gy > p.n_chunks) gy = p.n_chunks;
     if (gy < 1) gy = 1;
     p.gy = (int)gy;
-    cudaError_t e;
     switch (c->bits) {
     case 2: e = launch_dequant_stream<2>(p, fp32_out, st); break;
     case 3: e = launch_dequant_stream<3>(p, fp32_out, st); break;

@@ -19,6 +19,8 @@ CASES = [  # N, T, E, k, bits, row padding, bias
     (8, 40, 2304, 36, 4, 0, False), (8, 129, 4608, 72, 8, 0, True), (5, 31, 5120, 80, 5, 8, False),
     (3, 65, 1041, 17, 7, 0, True), (3, 24, 1047, 23, 6, 1, False), (16, 50, 832, 13, 5, 0, True),
     (33, 18, 520, 9, 4, 0, False), (64, 70, 264, 8, 8, 0, True), (2, 20, 8192, 128, 8, 0, False), (2, 11, 16384, 9, 8, 0, False),
+    (4, 147, 5120, 0, 8, 0, True), (3, 297, 2048, 33, 6, 64, True), (4, 5, 1024, 380, 4, 0, True), (2, 149, 4096, 400, 4, 8, False),
+    (1, 2, 64, 7, 7, 0, True), (4, 595, 512, 40, 2, 0, False),
     (1, 300, 5121, 5000, 4, 0, False), (2, 600, 200, 3, 3, 0, False), (1, 2500, 1000, 15, 4, 0, True),
 ]
 
