@@ -111,16 +111,17 @@ struct QPParams {
     unsigned int *done;                 // blocks that have finished their stores (returns to 0)
 };
 
-// Dynamic shared memory layout (byte offsets).
+// Dynamic shared memory layout (byte offsets).  A pushing block's failure flag lies behind the barriers: a static
+// variable would count against the block's limit beside the ring, which may fill it to the last byte.
 struct QPLayout {
     size_t ring, bars, total;
 };
-__host__ __device__ inline QPLayout qp_layout(int E, int G, int nstage)
+__host__ __device__ inline QPLayout qp_layout(int E, int G, int nstage, bool push)
 {
     QPLayout l;
     l.ring = 0;
     l.bars = (size_t)nstage * G * E * 2;
-    l.total = l.bars + (size_t)nstage * 16;
+    l.total = l.bars + (size_t)nstage * 16 + (push ? 16 : 0);
     return l;
 }
 
@@ -163,10 +164,8 @@ template <int GPT, int G, int TB, bool PUSH>  // TB: upper bound of the block si
 __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ int s_failed;  // (push mode) a wait of this block ran out
     const int tid = threadIdx.x;
     const int NT = blockDim.x - 32;  // consumer threads
-    if (PUSH && tid == 0) s_failed = 0;  // (ordered before any use by the named barrier of the prologue)
     // this block's shard of the batch, its index among the shard's blocks, and the shard's buffers
     const int sb = blockIdx.x / p.cps;
     const int bx = blockIdx.x - sb * p.cps;
@@ -178,10 +177,12 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
     const int E8 = E >> 3, L8 = (E - k) >> 3;
     const uint32_t row_bytes = (uint32_t)E * 2u;
     const uint32_t stage_bytes = (uint32_t)G * row_bytes;
-    const QPLayout lay = qp_layout(E, G, nstage);
+    const QPLayout lay = qp_layout(E, G, nstage, PUSH);
     uint8_t *ring = smem + lay.ring;
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + lay.bars);
     uint64_t *empty = full + nstage;
+    int *const failed = reinterpret_cast<int *>(empty + nstage);  // (push mode) a wait of this block ran out
+    if (PUSH && tid == 0) *failed = 0;  // (ordered before any use by the named barrier of the prologue)
 
     // this block's rows
     const int64_t t_begin = (int64_t)bx * p.rows_per_block;
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
         const int rows = stage_rows(it, r0s);
         if (!mbar_wait(smem_u32(&full[st]), parity)) {
             atomicExch(p.status, (int)TPQ_ERR_TIMEOUT);
-            if constexpr (PUSH) s_failed = 1;  // this block's part of the payload is incomplete
+            if constexpr (PUSH) *failed = 1;  // this block's part of the payload is incomplete
             break;
         }
         const int64_t t0 = t_begin + r0s;
@@ -450,10 +451,10 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
             __threadfence();
             // a block whose waits ran out counts in the upper half as well: the payload is then incomplete,
             // the words are not written, and the receivers' own bounded waits flag the step
-            const unsigned int prev = atomicAdd(p.done, s_failed ? 0x10001u : 1u);
+            const unsigned int prev = atomicAdd(p.done, *failed ? 0x10001u : 1u);
             if ((prev & 0xFFFFu) == gridDim.x - 1) {
                 *p.done = 0u;  // the next launch in the stream starts from zero
-                if ((prev >> 16) == 0 && !s_failed) {
+                if ((prev >> 16) == 0 && !*failed) {
                     // one fence (acquire side of the counts above, release side of the words below), then the
                     // words as relaxed system-scope stores: together a release of everything observed so far
                     __threadfence_system();
@@ -495,7 +496,7 @@ __global__ void wait_arrivals(const uint32_t *arrived, int n, uint32_t epoch, un
     }
 }
 
-size_t qp_smem_bytes(int E, int G, int nstage) { return qp_layout(E, G, nstage).total; }
+size_t qp_smem_bytes(int E, int G, int nstage, bool push) { return qp_layout(E, G, nstage, push).total; }
 
 }  // namespace
 
@@ -506,7 +507,7 @@ bool tpq_quantize_tiled_ok(const tpq_ctx *c, int64_t T, int64_t stride)
     if (E % 8 || k % 8 || stride % 8 || T <= 0) return false;
     if (E - k < 8) return false;
     if (E / 8 > QP_MAX_CONSUMERS * QP_MAX_GPT) return false;
-    if (qp_smem_bytes(E, 1, 2) > (size_t)c->smem_optin) return false;
+    if (qp_smem_bytes(E, 1, 2, true) > (size_t)c->smem_optin) return false;
     return true;
 }
 
@@ -569,13 +570,13 @@ cudaError_t launch_tiled(const tpq_ctx *c, int shard0, int n, const void *const 
     const int64_t rpb = (T + cps - 1) / cps;
     cps = (int)((T + rpb - 1) / rpb);
     int G = 4;
-    while (G > 1 && (rpb < G || qp_smem_bytes(E, G, 3) > (size_t)c->smem_optin)) G >>= 1;
+    while (G > 1 && (rpb < G || qp_smem_bytes(E, G, 3, push != nullptr) > (size_t)c->smem_optin)) G >>= 1;
     const int first = (G == 4 && rpb > 4) ? 2 : G;
     const int64_t grid = (int64_t)cps * n;
     const int64_t per_block = (rpb + G - 1) / G + (first < G ? 1 : 0);
     int nstage = (int)(per_block < 8 ? per_block : 8);
     if (nstage < 2) nstage = 2;
-    while (nstage > 2 && qp_smem_bytes(E, G, nstage) > (size_t)c->smem_optin) --nstage;
+    while (nstage > 2 && qp_smem_bytes(E, G, nstage, push != nullptr) > (size_t)c->smem_optin) --nstage;
 
     QPParams p;
     const int64_t lpb = tpq_lp_bytes_i(T, E, k);
@@ -597,7 +598,7 @@ cudaError_t launch_tiled(const tpq_ctx *c, int shard0, int n, const void *const 
     p.prefetch_rows = QP_PREFETCH_ROWS;
     p.inv_s = c->t.inv_s + (size_t)shard0 * E; p.grp = c->t.grp; p.filler = c->t.filler; p.hp_idx = c->t.hp_idx;
     p.lp_words = lpb / 4; p.status = c->t.status;
-    const size_t smem = qp_smem_bytes(E, G, nstage);
+    const size_t smem = qp_smem_bytes(E, G, nstage, push != nullptr);
 
     cudaError_t e = cudaSuccess;
 #define TPQ_QP_LAUNCH(GPT, GG, TB)                                                                                   \

@@ -350,7 +350,7 @@ inline int qs_warps(int G, int B, int gpt)
 inline size_t qs_pipe_bytes(int E, int B, int warps, int gpt, int nstage)
 {
     return (size_t)nstage * QS_STAGE * E * 2 + (size_t)warps * gpt * QS_STAGE * qs_warp_words(B) * 4 + (size_t)nstage * 16 +
-           256;  // (lanes with no word to write may look up to 64 words past their string's start)
+           256;  // (the failure flag; lanes with no word to write may look up to 64 words past their string's start)
 }
 
 template <int B, int GPT, bool PUSH>
@@ -358,13 +358,11 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
 {
     constexpr int OWN = 32 - qs_ahead(B), WW = qs_warp_words(B);
     extern __shared__ __align__(128) uint8_t qs_pipe[];
-    __shared__ int s_failed;  // (push mode) a wait of this block ran out
     const QSParams &p = pp.q;
     // warp 0 is the producer, warp 1 the edge warp, then come the NT consumers: where several warps of a scheduler can
     // issue, the first goes first, and the few instructions of these two must not wait behind the consumers' many
     // (as last warps 27.3 us at 4 x 2048 x 5120, 51 selected; 27.0 us so)
     const int NT = blockDim.x - 64, tid = (int)threadIdx.x - 64;
-    if (PUSH && threadIdx.x == 0) s_failed = 0;  // (ordered before any use by the barrier of the prologue)
     const int E = p.E, k = p.k, L = p.L, G = (L + 7) >> 3, nstage = pp.nstage;
     const int LB = L * B;  // bits of a row
     const int sb = blockIdx.x / pp.bps, bx = blockIdx.x - sb * pp.bps;
@@ -375,6 +373,10 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
     uint32_t *const strings = reinterpret_cast<uint32_t *>(ring + (size_t)nstage * stage_bytes);
     uint64_t *const full = reinterpret_cast<uint64_t *>(strings + (size_t)(NT / 32) * GPT * QS_STAGE * WW);
     uint64_t *const empty = full + nstage;
+    // (push mode) a wait of this block ran out; in the slack behind the barriers, not a static variable: that would count
+    // against the block's limit beside a ring that may fill it to the last byte
+    int *const failed = reinterpret_cast<int *>(empty + nstage);
+    if (PUSH && threadIdx.x == 0) *failed = 0;  // (ordered before any use by the barrier of the prologue)
     const int64_t t_begin = (int64_t)bx * pp.rows_per_block;
     const int rows_mine = (int)(p.T - t_begin < pp.rows_per_block ? p.T - t_begin : pp.rows_per_block);
     const int lane = threadIdx.x & 31;
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
             const int rows = rows_mine - r0 < QS_STAGE ? rows_mine - r0 : QS_STAGE;
             if (!mbar_wait(smem_u32(&full[st]), parity)) {
                 atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
-                if (PUSH) s_failed = 1;
+                if (PUSH) *failed = 1;
                 dead = true;
             }
             if (__any_sync(0xffffffffu, dead)) {
@@ -563,7 +565,7 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
         const int rows = rows_mine - r0 < QS_STAGE ? rows_mine - r0 : QS_STAGE;
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), parity))) {
             atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
-            if (PUSH) s_failed = 1;
+            if (PUSH) *failed = 1;
             break;
         }
         const uint8_t *const stage8 = ring + (size_t)st * stage_bytes;
@@ -679,10 +681,10 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
         asm volatile("bar.sync 2, %0;" ::"r"(NT + 32) : "memory");
         if (tid == 0) {
             __threadfence();
-            const unsigned int prev = atomicAdd(pp.done, s_failed ? 0x10001u : 1u);
+            const unsigned int prev = atomicAdd(pp.done, *failed ? 0x10001u : 1u);
             if ((prev & 0xFFFFu) == gridDim.x - 1) {
                 *pp.done = 0u;
-                if ((prev >> 16) == 0 && !s_failed) {
+                if ((prev >> 16) == 0 && !*failed) {
                     __threadfence_system();
                     for (int d = 0; d < pp.n_dst; ++d)
                         asm volatile("st.relaxed.sys.global.u32 [%0], %1;" ::"l"(pp.arrived[d]), "r"(pp.epoch) : "memory");

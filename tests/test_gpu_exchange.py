@@ -61,6 +61,24 @@ def test_push_writes_every_destination_and_publishes(N, T, E, k, bits, n_dst):
     t.close()
 
 
+@pytest.mark.parametrize("bits,T,E,k", [(8, 40, 5248, 82), (2, 40, 9216, 144), (3, 9, 6864, 107), (4, 40, 6776, 105),
+                                        (4, 5000, 4840, 72), (4, 2000, 5808, 88), (4, 700, 9680, 152), (4, 700, 23232, 360)])
+def test_push_where_the_ring_fills_shared_memory(bits, T, E, k):
+    """Shapes whose ring of stages ends within 127 bytes of the most shared memory a block can have (the last four of the
+    Int4 kernel for multiples of 8, with 6, 5 and 3 stages of 4 rows and 5 of 1): the push is launched and publishes the plain call's payload."""
+    t, _, ys = _ctx(1, T, E, k, bits)
+    P = t.payload_bytes(T)
+    y = gu.dev_bf16(ys[0])
+    want, got = (torch.zeros(P, dtype=torch.uint8, device="cuda") for _ in range(2))
+    f, f0 = _words(1)
+    t.quantize_pack(0, y.data_ptr(), T, want.data_ptr(), P)
+    t.quantize_pack_push(0, y.data_ptr(), T, [got.data_ptr()], [f.data_ptr() + 4 * f0], P, 3)
+    torch.cuda.synchronize()
+    assert t.device_status() == 0 and int(f[f0]) == 3
+    assert torch.equal(got, want)
+    t.close()
+
+
 @pytest.mark.parametrize("N,T,E,k", [(4, 150, 1024, 16), (2, 2048, 5120, 80), (8, 64, 2048, 32)])
 def test_emulated_ranks_exchange_and_reduce(N, T, E, k):
     """Every rank pushes its shard into its slot of every rank's receive buffer; every rank waits for its N
