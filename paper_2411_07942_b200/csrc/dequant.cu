@@ -266,14 +266,14 @@ __device__ __forceinline__ void dp_store_rows(const DQParams &p, const int32_t *
         for (int h = 0; h < 4; ++h) acc[r][h] = acc_in[r][h];
     if (p.bias) {
         // lane n belongs to feature 8g+n, or, at a hole, to the filler feature whose codes sit in the slot
-        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p.bias + 8 * g));
-        const float4 b1 = __ldg(reinterpret_cast<const float4 *>(p.bias + 8 * g + 4));
+        const float4 b0 = *reinterpret_cast<const float4 *>(p.bias + 8 * g);
+        const float4 b1 = *reinterpret_cast<const float4 *>(p.bias + 8 * g + 4);
         float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
         const uint32_t holes = __ldg(p.grp + g) & 0xFFu;
         if (holes) {
 #pragma unroll
             for (int n = 0; n < 8; ++n)
-                if (holes & (1u << n)) b[n] = __ldg(p.bias + __ldg(lp_idx + 8 * g + n));
+                if (holes & (1u << n)) b[n] = p.bias[__ldg(lp_idx + 8 * g + n)];
         }
 #pragma unroll
         for (int r = 0; r < DP_R; ++r)
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(DP_THREADS, 1) dequant_panels(const DPParams p
                 static_cast<uint16_t *>(p.out)[orow + filler_col] =
                     __ldcg(static_cast<const uint16_t *>(p.out) + orow + sel_col);
         }
-        store_one<FP32OUT>(p.out, orow + sel_col, p.bias ? __fadd_rn(v, __ldg(p.bias + sel_col)) : v);
+        store_one<FP32OUT>(p.out, orow + sel_col, p.bias ? __fadd_rn(v, p.bias[sel_col]) : v);
     };
     // the items of the chunk whose first row is tcp: this thread's pipelined one (sum v) and, in panels with
     // more items than threads, the rest
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(DP_THREADS, 1) dequant_panels(const DPParams p
                 else
                     static_cast<uint16_t *>(p.out)[fl_row + my_fcol] = (uint16_t)__float_as_uint(fl_f);
             }
-            store_one<FP32OUT>(p.out, fl_row + my_col, p.bias ? __fadd_rn(fl_v, __ldg(p.bias + my_col)) : fl_v);
+            store_one<FP32OUT>(p.out, fl_row + my_col, p.bias ? __fadd_rn(fl_v, p.bias[my_col]) : fl_v);
             fl_on = false;
         }
     };
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) dequant_tpanels(const DTParams 
                     static_cast<uint16_t *>(p.out)[orow + filler_col] =
                         __ldcg(static_cast<const uint16_t *>(p.out) + orow + sel_col);
             }
-            store_one<FP32OUT>(p.out, orow + sel_col, p.bias ? __fadd_rn(v, __ldg(p.bias + sel_col)) : v);
+            store_one<FP32OUT>(p.out, orow + sel_col, p.bias ? __fadd_rn(v, p.bias[sel_col]) : v);
         };
 
         for (int64_t ch = chb; ch < che; ch += cstep) {
@@ -1012,9 +1012,9 @@ __global__ void __launch_bounds__(MAXT + DAUX + 32, 1) dequant_rows(const DRPara
 
     // Order of the prologue.  The producer warp sets up the barriers, waits for the kernel ahead in the stream
     // and issues the first stages' copies at once: the other warps' table loads then run in the shadow of the
-    // first stage's flight instead of ahead of it.  Only the producer executes griddepcontrol.wait: every
-    // other access to the payloads, and every store to the output, follows a "full" barrier that one of the
-    // producer's copies completes, i.e. follows that wait.
+    // first stage's flight instead of ahead of it.  Besides the loads of the bias, only the producer executes
+    // griddepcontrol.wait: every other access to the payloads, and every store to the output, follows a "full"
+    // barrier that one of the producer's copies completes, i.e. follows that wait.
     tpq_grid_dep_launch();  // the next kernel in the stream may start its own prologue as SMs free up
     if constexpr (HAS_WAIT) {  // (an instantiation of its own: the plain call's prologue stays short)
         tpq_block_wait_arrivals(p.arr);
@@ -1139,8 +1139,9 @@ __global__ void __launch_bounds__(MAXT + DAUX + 32, 1) dequant_rows(const DRPara
             for (int i = 0; i < NMAX; ++i)
                 c_s[i] = (do_dec && i < N) ? __ldg(p.s_k + (size_t)i * E + col) * (1.0f / (float)(1 << shl)) : 0.0f;
             float c_b = 0.0f;  // the column's bias
-            if (HAS_BIAS && do_dec) c_b = __ldg(p.bias + col);
-            if (HAS_BIAS && do_sum) c_b = __ldg(p.bias + __ldg(x.hp_idx + rank));
+            if (HAS_BIAS) tpq_grid_dep_wait();  // (the kernel ahead may be writing it)
+            if (HAS_BIAS && do_dec) c_b = p.bias[col];
+            if (HAS_BIAS && do_sum) c_b = p.bias[__ldg(x.hp_idx + rank)];
             uint32_t h_off = (uint32_t)rank * 2u, s_off = (uint32_t)rank * 4u;
             keep(do_sum); keep(do_dec); keep(to_out); keep(c_off); keep(c_hi); keep(c_mask); keep(c_nb); keep(c_b);
             keep(h_off); keep(s_off);
@@ -1203,11 +1204,11 @@ __global__ void __launch_bounds__(MAXT + DAUX + 32, 1) dequant_rows(const DRPara
                                 for (int i = 0; i < N; ++i)
                                     v = __fmaf_rn(code_at(lds32(stage + (uint32_t)i * lp_b + (uint32_t)(r * L8 + (pc >> 3)) * 4u), (pc & 7) * 4),
                                                   __ldg(p.s_k + (size_t)i * E + cl), v);
-                                if (HAS_BIAS) v = __fadd_rn(v, __ldg(p.bias + cl));
+                                if (HAS_BIAS) v = __fadd_rn(v, p.bias[cl]);
                             } else {
                                 for (int i = 0; i < N; ++i)
                                     v = __fadd_rn(v, __uint_as_float(lds16(hp_s + (uint32_t)i * hp_b + (uint32_t)(r * k + rk) * 2u) << 16));
-                                if (HAS_BIAS) v = __fadd_rn(v, __ldg(p.bias + __ldg(x.hp_idx + rk)));
+                                if (HAS_BIAS) v = __fadd_rn(v, p.bias[__ldg(x.hp_idx + rk)]);
                             }
                             if (q < nc) store_bits<FP32OUT>(obase + r * out_row_bytes + (int64_t)cl * ESIZE, out_bits<FP32OUT>(v));
                             else sts32(sums + (uint32_t)(r * k + rk) * 4u, out_bits<FP32OUT>(v));
@@ -1249,8 +1250,9 @@ __global__ void __launch_bounds__(MAXT + DAUX + 32, 1) dequant_rows(const DRPara
 #pragma unroll
         for (int i = 0; i < NMAX; ++i)
             c_s[i] = (on && ps >= 0 && i < N) ? __ldg(p.s_k + (size_t)i * E + col) * (1.0f / (float)(1 << shl)) : 0.0f;
-        float c_b = (HAS_BIAS && on && ps >= 0) ? __ldg(p.bias + col) : 0.0f;
-        float h_b = (HAS_BIAS && on) ? __ldg(p.bias + __ldg(x.hp_idx + at)) : 0.0f;
+        if (HAS_BIAS) tpq_grid_dep_wait();  // (the kernel ahead may be writing the bias)
+        float c_b = (HAS_BIAS && on && ps >= 0) ? p.bias[col] : 0.0f;
+        float h_b = (HAS_BIAS && on) ? p.bias[__ldg(x.hp_idx + at)] : 0.0f;
         keep(sel); keep(c_off); keep(c_sum); keep(c_hi); keep(c_mask); keep(c_nb); keep(c_b); keep(h_b);
 #pragma unroll
         for (int i = 0; i < NMAX; ++i) keep(c_s[i]);
@@ -1284,7 +1286,7 @@ __global__ void __launch_bounds__(MAXT + DAUX + 32, 1) dequant_rows(const DRPara
                 }
             }
             for (int c = at + DR_AUX; c < k; c += DR_AUX) {  // (more selected features than threads)
-                const float hb = HAS_BIAS ? __ldg(p.bias + __ldg(x.hp_idx + c)) : 0.0f;
+                const float hb = HAS_BIAS ? p.bias[__ldg(x.hp_idx + c)] : 0.0f;
                 for (int r = 0; r < rows; ++r) {
                     float v = 0.0f;
                     for (int i = 0; i < N; ++i)
@@ -1329,7 +1331,7 @@ __global__ void __launch_bounds__(MAXT + DAUX + 32, 1) dequant_rows(const DRPara
                         for (int i = 0; i < N; ++i)
                             v = __fmaf_rn(code_at(lds32(stage + (uint32_t)i * lp_b + (uint32_t)(r * L8 + (pc >> 3)) * 4u), (pc & 7) * 4),
                                           __ldg(p.s_k + (size_t)i * E + cl), v);
-                        if (HAS_BIAS) v = __fadd_rn(v, __ldg(p.bias + cl));
+                        if (HAS_BIAS) v = __fadd_rn(v, p.bias[cl]);
                         bits = out_bits<FP32OUT>(v);
                     } else {
                         bits = lds32(sums + (uint32_t)(r * k + (-pc - 1)) * 4u);
@@ -1371,8 +1373,9 @@ __global__ void __launch_bounds__(MAXT + DAUX + 32, 1) dequant_rows(const DRPara
 #pragma unroll
     for (int h = 0; h < 4; ++h) b[h] = make_float2(0.0f, 0.0f);
     if (HAS_BIAS) {
-        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(p.bias + 8 * g_ld));
-        const float4 b1 = __ldg(reinterpret_cast<const float4 *>(p.bias + 8 * g_ld + 4));
+        tpq_grid_dep_wait();  // (the kernel ahead may be writing it)
+        const float4 b0 = *reinterpret_cast<const float4 *>(p.bias + 8 * g_ld);
+        const float4 b1 = *reinterpret_cast<const float4 *>(p.bias + 8 * g_ld + 4);
         b[0] = make_float2(b0.x, b0.y); b[1] = make_float2(b0.z, b0.w);
         b[2] = make_float2(b1.x, b1.y); b[3] = make_float2(b1.z, b1.w);
     }

@@ -929,7 +929,7 @@ __global__ void __launch_bounds__(DS_THREADS, 2) dequant_stream(const DSParams p
     auto flush = [&]() {
         if (fl_on) {
             if (my_fcol >= 0) write_out(fl_row + my_fcol, fl_f);
-            ds_store_one<FP32OUT>(p.out, fl_row + my_col, p.bias ? __fadd_rn(fl_v, __ldg(p.bias + my_col)) : fl_v);
+            ds_store_one<FP32OUT>(p.out, fl_row + my_col, p.bias ? __fadd_rn(fl_v, p.bias[my_col]) : fl_v);
             fl_on = false;
         }
     };
@@ -949,7 +949,7 @@ __global__ void __launch_bounds__(DS_THREADS, 2) dequant_stream(const DSParams p
                 u = __fadd_rn(u, __uint_as_float((uint32_t)__ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + off)) << 16));
             const int col = __ldg(p.hp_idx + h);
             if (h < n_holes) write_out(orow + __ldg(p.filler + h), read_out(orow + col));
-            ds_store_one<FP32OUT>(p.out, orow + col, p.bias ? __fadd_rn(u, __ldg(p.bias + col)) : u);
+            ds_store_one<FP32OUT>(p.out, orow + col, p.bias ? __fadd_rn(u, p.bias[col]) : u);
         }
     };
     bool pend = false, pend_on = false;
@@ -1027,7 +1027,7 @@ __global__ void __launch_bounds__(DS_THREADS, 2) dequant_stream(const DSParams p
             float b[8];  // lane n belongs to feature 8g+n, or, at a hole, to the filler whose codes sit in the slot
 #pragma unroll
             for (int n = 0; n < 8; ++n)
-                b[n] = n < lanes ? __ldg(p.bias + ((holes & (1u << n)) ? __ldg(p.lp_idx + 8 * g + n) : 8 * g + n)) : 0.0f;
+                b[n] = n < lanes ? p.bias[(holes & (1u << n)) ? __ldg(p.lp_idx + 8 * g + n) : 8 * g + n] : 0.0f;
 #pragma unroll
             for (int r = 0; r < DS_R; ++r)
 #pragma unroll
@@ -1189,9 +1189,9 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
         float c_s[DW_MAX_DEV];
 #pragma unroll
         for (int i = 0; i < DW_MAX_DEV; ++i) c_s[i] = i < N && ps >= 0 ? __ldg(pp.s_k + (size_t)i * E + L + at) : 0.0f;
-        const float s_b = HAS_BIAS && on ? __ldg(p.bias + s_col) : 0.0f, c_b = HAS_BIAS && on ? __ldg(p.bias + L + at) : 0.0f;
         asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
-        tpq_grid_dep_wait();  // the BF16 values are read and columns written without waiting for a copy
+        tpq_grid_dep_wait();  // the bias and the BF16 values are read, and columns written, without waiting for a copy
+        const float s_b = HAS_BIAS && on ? p.bias[s_col] : 0.0f, c_b = HAS_BIAS && on ? p.bias[L + at] : 0.0f;
         uint16_t v[DW_ROWS][DW_MAX_DEV];
         auto load = [&](int r0) {
             if (on) {
@@ -1242,7 +1242,7 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
                     float sum = 0.0f;
                     for (int i = 0; i < N; ++i)
                         sum = __fadd_rn(sum, __uint_as_float((uint32_t)__ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + p.lp_bytes) + (t0 + r) * k + h) << 16));
-                    put(r, t0 + r, h, col, HAS_BIAS ? __fadd_rn(sum, __ldg(p.bias + col)) : sum);
+                    put(r, t0 + r, h, col, HAS_BIAS ? __fadd_rn(sum, p.bias[col]) : sum);
                 }
             }
             __syncwarp();
@@ -1262,7 +1262,7 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
                         if (i < N)
                             acc = __fmaf_rn(code(reinterpret_cast<const uint32_t *>(stage + (size_t)i * pp.dev_bytes), rem + (uint32_t)r * LB, slot),
                                             h == at ? c_s[i] : __ldg(pp.s_k + (size_t)i * E + L + h), acc);
-                    if (HAS_BIAS) acc = __fadd_rn(acc, h == at ? c_b : __ldg(p.bias + L + h));
+                    if (HAS_BIAS) acc = __fadd_rn(acc, h == at ? c_b : p.bias[L + h]);
                     ds_store_one<FP32OUT>(p.out, (t0 + r) * p.out_stride + L + h, acc);
                 }
             }
@@ -1302,9 +1302,10 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
                                            s8[2 * h + 1] * (1.0f / (float)(1u << ds_pos(B, 2 * h + 1))));
             }
     }
+    if (HAS_BIAS) tpq_grid_dep_wait();  // (the kernel ahead may be writing it)
 #pragma unroll
     for (int h = 0; h < 4; ++h)
-        b[h] = HAS_BIAS && lanes > 0 ? make_float2(__ldg(p.bias + 8 * g + 2 * h), __ldg(p.bias + 8 * g + 2 * h + 1)) : make_float2(0.0f, 0.0f);
+        b[h] = HAS_BIAS && lanes > 0 ? make_float2(p.bias[8 * g + 2 * h], p.bias[8 * g + 2 * h + 1]) : make_float2(0.0f, 0.0f);
     // (opaque: the compiler, short of registers, would otherwise load the steps again at every use)
 #pragma unroll
     for (int i = 0; i < DW_MAX_DEV; ++i)

@@ -148,7 +148,9 @@ cudaError_t tpq_launch_dequant_tiled(const tpq_ctx *c, const void *const *payloa
 // ---- programmatic dependent launch: a kernel launched this way may start (and run its prologue: barrier
 // set-up, loads of the context's tables, which no kernel in flight writes) before the kernel ahead of it in
 // the stream has drained; it must execute tpq_grid_dep_wait() before it touches memory that earlier work in
-// the stream may still read or write.
+// the stream may still read or write: the caller's buffers (inputs, payloads, the bias, the output) and scratch.  Such
+// memory is read with coherent loads (plain, .cs, .cg, bulk copies): __ldg and const __restrict__ parameters promise
+// that nobody writes it while the kernel runs, and it may have been written after this kernel's start.
 #ifdef __CUDACC__
 __device__ __forceinline__ void tpq_grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void tpq_grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -723,3 +723,36 @@ def test_batched_quantize_equals_per_shard_calls(N, T, E, k, path):
             assert np.array_equal(bufs2[j][1].cpu().numpy(), bufs[1 + j][1].cpu().numpy())
     assert t.raw("tpq_quantize_pack_batch", N - 1, 2, None, T, E, None, P, None) == binding.TPQ_ERR_INVALID_ARG
     t.close()
+
+
+@pytest.mark.parametrize("N,T,E,k,bits", [(2, 297, 1024, 16, 4), (6, 40, 1024, 16, 4), (9, 2400, 1024, 32, 4), (9, 100, 1040, 8, 4),
+                                          (2, 297, 1024, 16, 3), (6, 300, 1033, 16, 4), (2, 3, 65, 1, 4)])
+def test_bias_from_the_call_ahead(N, T, E, k, bits):
+    """The bias is a row that the reduction right ahead in the stream writes (its own FP32 output): dependent launches may
+    start ahead of that kernel's end, but must not read the row before.  Every reduction kernel; the row kernels' first
+    calls leave SMs idle, on which the second call's blocks start at once.  fl(sum + bias) is exact to state."""
+    w = _workload(N, T, E, 41 * E + T + bits, calib=(2, 8))
+    scale = synth.column_scales(w)
+    t = binding.Tpq(N, E, bits=bits)
+    gu.calibrate_both(t, [synth.calibration_np(w, i, scale=scale) for i in range(N)])
+    t.select_features(k)
+    P, stride = t.payload_bytes(T), (E + 3) // 4 * 4
+    pls = [torch.zeros(P, dtype=torch.uint8, device="cuda") for _ in range(N)]
+    for i in range(N):
+        y = gu.dev_bf16(synth.activations_np(w, i, T, scale=scale))
+        t.quantize_pack(i, y.data_ptr(), T, pls[i].data_ptr(), P)
+        torch.cuda.synchronize()
+    ptrs = [p.data_ptr() for p in pls]
+    a, b = (torch.empty((T, stride), dtype=torch.float32, device="cuda") for _ in range(2))
+    side = torch.cuda.Stream()
+    for _ in range(5):
+        with torch.cuda.stream(side):
+            a.fill_(1e9)
+            torch.cuda._sleep(1 << 20)      # both launches are queued when the first one starts
+            for out, bias in ((a, None), (b, a[T - 1].data_ptr())):
+                t.dequant_reduce(ptrs, T, out.data_ptr(), binding.TPQ_OUT_FP32, out_row_stride=stride, stream=side.cuda_stream,
+                                 bias_ptr=bias)
+        torch.cuda.synchronize()
+        assert torch.equal(b[:, :E], a[:, :E] + a[T - 1, :E])
+    assert t.device_status() == 0
+    t.close()
