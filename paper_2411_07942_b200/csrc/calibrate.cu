@@ -39,13 +39,16 @@ __device__ __forceinline__ float key_to_float(int16_t key)
 constexpr uint32_t KEY_MAX2 = 0x7FFF7FFFu;  // identity of min
 constexpr uint32_t KEY_MIN2 = 0x80008000u;  // identity of max
 
+// (No pointer of these kernels is __restrict__: they are dependent launches, and what they read -- the sequences, the partial
+// extremes, the running ranges -- may still be written by a kernel of this library after they have started, up to the
+// wait.  The compiler must neither load it through the read-only path nor move a load ahead of the wait.)
+//
 // Tiled extremes: thread = 8 adjacent features (one 128-bit load per row), 8 row lanes per block,
 // eight independent loads in flight per thread.  grid = (feature chunks of 256, row splits, sequences).
 constexpr int CM_BLOCKS_PER_SM = 4;  // resident blocks (64 registers a thread)
 
-__global__ void __launch_bounds__(256, CM_BLOCKS_PER_SM) colminmax_tiled(const uint16_t *__restrict__ y, int64_t S, int64_t stride, int E,
-                                                       int n_split, int16_t *__restrict__ part_lo,
-                                                       int16_t *__restrict__ part_hi)
+__global__ void __launch_bounds__(256, CM_BLOCKS_PER_SM) colminmax_tiled(const uint16_t *y, int64_t S, int64_t stride, int E,
+                                                                         int n_split, int16_t *part_lo, int16_t *part_hi)
 {
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int g = blockIdx.x * 32 + tx;  // group of 8 features
@@ -125,9 +128,8 @@ __global__ void __launch_bounds__(256, CM_BLOCKS_PER_SM) colminmax_tiled(const u
 }
 
 // Shape-generic extremes: thread = one feature, any E and stride.
-__global__ void __launch_bounds__(256) colminmax_generic(const uint16_t *__restrict__ y, int64_t S, int64_t stride,
-                                                         int E, int n_split, int16_t *__restrict__ part_lo,
-                                                         int16_t *__restrict__ part_hi)
+__global__ void __launch_bounds__(256) colminmax_generic(const uint16_t *y, int64_t S, int64_t stride, int E, int n_split,
+                                                         int16_t *part_lo, int16_t *part_hi)
 {
     tpq_grid_dep_launch();
     tpq_grid_dep_wait();
@@ -159,10 +161,8 @@ __global__ void __launch_bounds__(256) colminmax_generic(const uint16_t *__restr
 // memory, and the first thread row then runs the moving average over them in sequence order.
 constexpr int EF_X = 32, EF_Y = 8, EF_Q = 64;
 
-__global__ void __launch_bounds__(EF_X *EF_Y) ema_fold(const int16_t *__restrict__ part_lo,
-                                                       const int16_t *__restrict__ part_hi, int64_t n_seq, int n_split,
-                                                       int E, float *__restrict__ m, float *__restrict__ M,
-                                                       int64_t count0, float gamma)
+__global__ void __launch_bounds__(EF_X *EF_Y) ema_fold(const int16_t *part_lo, const int16_t *part_hi, int64_t n_seq, int n_split,
+                                                       int E, float *m, float *M, int64_t count0, float gamma)
 {
     __shared__ int16_t s_lo[EF_Q][EF_X], s_hi[EF_Q][EF_X];
     const int x = threadIdx.x & (EF_X - 1), yl = threadIdx.x / EF_X;

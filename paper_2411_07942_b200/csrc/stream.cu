@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(QS_THREADS, VEC ? 4 : 2) quantize_stream_tile(
 #pragma unroll
             for (int r = 0; r < 4; ++r) {  // all loads first; rows past the end re-read the last row
                 if (VEC) {
-                    v[r] = __ldg(reinterpret_cast<const uint4 *>(src));
+                    v[r] = *reinterpret_cast<const uint4 *>(src);  // (not __ldg: the kernel ahead may have written it)
                 } else {
                     uint32_t x[8];
 #pragma unroll
@@ -467,8 +467,10 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
                 dead = true;
                 break;
             }
-            // (the copies of this stage were issued behind the dependency wait, so this read is as well)
-            if (r0 == 0 && t_begin > 0) last = code(y[(t_begin - 1) * p.stride + f]);
+            if (r0 == 0 && t_begin > 0) {
+                tpq_grid_dep_wait();  // (the kernel ahead may have written the row: a load of this warp's own, so a wait of its own)
+                last = code(y[(t_begin - 1) * p.stride + f]);
+            }
             const uint16_t *const stage = reinterpret_cast<const uint16_t *>(ring + (size_t)st * stage_bytes);
             const int64_t bit0 = (t_begin + r0) * LB, w_stage = bit0 >> 5;
             const int in0 = (int)(bit0 & 31);

@@ -756,3 +756,45 @@ def test_bias_from_the_call_ahead(N, T, E, k, bits):
         assert torch.equal(b[:, :E], a[:, :E] + a[T - 1, :E])
     assert t.device_status() == 0
     t.close()
+
+
+@pytest.mark.parametrize("T,E,k,bits", [(64, 1000, 15, 4), (300, 1033, 9, 4), (297, 1024, 16, 3), (200, 1024, 16, 4), (40, 11264, 11, 4)])
+def test_inputs_from_the_call_ahead(T, E, k, bits):
+    """Quantisation and calibration of what the reduction right ahead in the stream writes, with all launches queued when the
+    first one starts, give the bytes and ranges that synchronised calls give."""
+    N = 2
+    w = _workload(N, T, E, 43 * E + T + bits, calib=(2, 8))
+    scale = synth.column_scales(w)
+    cal = [synth.calibration_np(w, i, scale=scale) for i in range(N)]
+    ys = [gu.dev_bf16(synth.activations_np(w, i, T, scale=scale)) for i in range(N)]
+    side = torch.cuda.Stream()
+    got = []
+    for queued in (False, True, True):
+        t = binding.Tpq(N, E, bits=bits)
+        gu.calibrate_both(t, cal)
+        t.select_features(k)
+        P = t.payload_bytes(T)
+        pls = [torch.zeros(P, dtype=torch.uint8, device="cuda") for _ in range(N)]
+        out = torch.full((T, E), 3e38, dtype=torch.bfloat16, device="cuda")
+        again = torch.zeros(P, dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        st = side.cuda_stream
+        calls = [lambda: t.quantize_pack_batch(0, [y.data_ptr() for y in ys], T, [p.data_ptr() for p in pls], P, stream=st),
+                 lambda: t.dequant_reduce([p.data_ptr() for p in pls], T, out.data_ptr(), binding.TPQ_OUT_BF16, stream=st),
+                 lambda: t.quantize_pack_batch(1, [out.data_ptr()], T, [again.data_ptr()], P, stream=st),
+                 lambda: t.calibrate_ranges(1, out.data_ptr(), 1, T, stream=st),
+                 lambda: t.calibrate_ranges(1, out.data_ptr(), T, 1, stream=st)]
+        with torch.cuda.stream(side):
+            if queued:
+                torch.cuda._sleep(1 << 20)
+            for call in calls:
+                call()
+                if not queued:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert t.device_status() == 0
+        got.append([out.view(torch.int16).cpu().numpy(), again.cpu().numpy(), *t.get_ranges(with_R=False)])
+        t.close()
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.array_equal(a, b)
