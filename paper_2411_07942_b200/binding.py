@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import struct
+import types
 from ctypes import POINTER, byref, c_char_p, c_double, c_float, c_int, c_int32, c_int64, c_size_t, c_void_p
 from pathlib import Path
 
@@ -52,17 +53,17 @@ SIGNATURES = {
     "tpq_payload_bytes_for_bits": (c_size_t, [c_int64, c_int64, c_int64, c_int]),
     "tpq_comm_bytes": (c_int, [c_void_p, c_int64, POINTER(CommReport)]),
     "tpq_quantize_pack": (c_int, [c_void_p, c_int, c_void_p, c_int64, c_int64, c_void_p, c_size_t, c_void_p]),
-    "tpq_quantize_pack_batch": (c_int, [c_void_p, c_int, c_int, c_void_p, c_int64, c_int64, c_void_p,
+    "tpq_quantize_pack_batch": (c_int, [c_void_p, c_int, c_int, POINTER(c_void_p), c_int64, c_int64, POINTER(c_void_p),
                                         c_size_t, c_void_p]),
-    "tpq_dequant_reduce": (c_int, [c_void_p, c_void_p, c_int, c_int64, c_void_p, c_int, c_int64, c_void_p]),
-    "tpq_dequant_reduce_bias": (c_int, [c_void_p, c_void_p, c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
+    "tpq_dequant_reduce": (c_int, [c_void_p, POINTER(c_void_p), c_int, c_int64, c_void_p, c_int, c_int64, c_void_p]),
+    "tpq_dequant_reduce_bias": (c_int, [c_void_p, POINTER(c_void_p), c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
                                         c_void_p]),
     "tpq_permute_weight": (c_int, [c_void_p, c_void_p, c_int64, c_void_p, c_void_p]),
     "tpq_linear_quantize_pack": (c_int, [c_void_p, c_int, c_void_p, c_void_p, c_int64, c_int64, c_void_p, c_size_t, c_void_p,
                                          c_void_p]),
-    "tpq_quantize_pack_push": (c_int, [c_void_p, c_int, c_void_p, c_int64, c_int64, c_void_p, c_void_p,
+    "tpq_quantize_pack_push": (c_int, [c_void_p, c_int, c_void_p, c_int64, c_int64, POINTER(c_void_p), POINTER(c_void_p),
                                        c_int, c_size_t, ctypes.c_uint32, c_void_p]),
-    "tpq_dequant_reduce_arrivals": (c_int, [c_void_p, c_void_p, c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
+    "tpq_dequant_reduce_arrivals": (c_int, [c_void_p, POINTER(c_void_p), c_int, c_int64, c_void_p, c_int, c_int64, c_void_p,
                                             c_void_p, ctypes.c_uint32, ctypes.c_uint64, c_void_p]),
     "tpq_wait_arrivals": (c_int, [c_void_p, c_void_p, c_int, ctypes.c_uint32, ctypes.c_uint64, c_void_p]),
     "tpq_get_state": (c_int, [c_void_p, c_void_p, POINTER(c_size_t)]),
@@ -75,6 +76,9 @@ SIGNATURES = {
 }
 
 _lib = None
+_fast = types.SimpleNamespace()   # the calls below that take pointer arrays, as functions that take what _ptrs returns
+_FAST = ("tpq_quantize_pack_batch", "tpq_dequant_reduce", "tpq_dequant_reduce_bias", "tpq_quantize_pack_push",
+         "tpq_dequant_reduce_arrivals")
 
 
 def lib() -> ctypes.CDLL:
@@ -89,6 +93,11 @@ def lib() -> ctypes.CDLL:
             fn = getattr(L, name)
             fn.restype = res
             fn.argtypes = args
+        for name in _FAST:
+            fn = L[name]   # a function object of its own: lib()'s keep the types of SIGNATURES
+            fn.restype, args = SIGNATURES[name]
+            fn.argtypes = [c_void_p if a is POINTER(c_void_p) else a for a in args]
+            setattr(_fast, name, fn)
         _lib = L
     return _lib
 
@@ -99,23 +108,26 @@ class TpqError(RuntimeError):
         self.status = status
 
 
-_packers = {}   # number of pointers -> struct.Struct
+_PACK = [struct.Struct(f"{n}Q").pack for n in range(65)]   # by the number of pointers (a context has at most 64 devices)
 
 
 def _ptrs(ptrs):
-    """A host array of device pointers: ctypes arrays as they are, sequences of addresses packed into bytes (a fifth of
-    the time that building and passing a ctypes array takes)."""
+    """A host array of device pointers.  Sequences of plain integers are packed into bytes (a quarter of the time that
+    building a ctypes array takes); what else c_void_p takes (None, c_void_p) goes into a ctypes array, and ctypes arrays
+    must be of c_void_p: other objects, numbers that are no addresses among them, are refused as the C signature refuses
+    them."""
     if isinstance(ptrs, (list, tuple)):
-        n = len(ptrs)
-        pack = _packers.get(n)
-        if pack is None:
-            pack = _packers[n] = struct.Struct(f"{n}Q")
         try:
-            return pack.pack(*ptrs)
-        except struct.error:   # None or c_void_p among them
+            # (the sum of integers is an integer; struct alone would take whatever has an __index__, a tensor for instance)
+            if type(sum(ptrs)) is int:
+                return _PACK[len(ptrs)](*ptrs)
+        except (TypeError, struct.error, IndexError):   # not all of them numbers, negative or above 64 bits, more than 64
             pass
     elif isinstance(ptrs, ctypes.Array):
-        return ptrs
+        try:
+            return POINTER(c_void_p).from_param(ptrs)
+        except TypeError as e:
+            raise ctypes.ArgumentError(str(e)) from None
     return (c_void_p * len(ptrs))(*ptrs)
 
 
@@ -239,7 +251,7 @@ class Tpq:
         assert len(payload_ptrs) == n
         ya = _ptrs(y_ptrs)
         pa = _ptrs(payload_ptrs)
-        st = _lib.tpq_quantize_pack_batch(self._h, first_shard, n, ya, T, self.E if row_stride is None else row_stride, pa,
+        st = _fast.tpq_quantize_pack_batch(self._h, first_shard, n, ya, T, self.E if row_stride is None else row_stride, pa,
                                           payload_capacity, stream)
         if st:
             self._check(st)
@@ -250,12 +262,12 @@ class Tpq:
         arr = _ptrs(payload_ptrs)
         stride = self.E if out_row_stride is None else out_row_stride
         if arrived_ptr is not None:
-            st = _lib.tpq_dequant_reduce_arrivals(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr,
+            st = _fast.tpq_dequant_reduce_arrivals(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr,
                                                   arrived_ptr, epoch & 0xFFFFFFFF, timeout_ns, stream)
         elif bias_ptr is None:
-            st = _lib.tpq_dequant_reduce(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, stream)
+            st = _fast.tpq_dequant_reduce(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, stream)
         else:
-            st = _lib.tpq_dequant_reduce_bias(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr, stream)
+            st = _fast.tpq_dequant_reduce_bias(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr, stream)
         if st:
             self._check(st)
 
@@ -275,7 +287,7 @@ class Tpq:
         assert len(arrived_ptrs) == n
         da = _ptrs(dst_ptrs)
         aa = _ptrs(arrived_ptrs)
-        st = _lib.tpq_quantize_pack_push(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride, da, aa, n,
+        st = _fast.tpq_quantize_pack_push(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride, da, aa, n,
                                          dst_capacity, epoch & 0xFFFFFFFF, stream)
         if st:
             self._check(st)

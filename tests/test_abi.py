@@ -80,3 +80,44 @@ def test_product_never_imports_the_oracle():
             if f.endswith((".py", ".cu", ".h", ".cuh")):
                 src = open(os.path.join(dirpath, f)).read()
                 assert "import oracle" not in src and "from oracle" not in src and "tpqo_" not in src, f
+
+
+def test_pointer_arrays_are_checked_like_the_c_signature(lib):
+    """What stands for a host array of addresses: sequences of addresses, None or c_void_p, and arrays of c_void_p.  Arrays
+    of other elements (a 32-bit one is half as long as the library reads), numbers that are no plain integers (a
+    one-element tensor has an __index__) and single addresses are refused."""
+    import ctypes
+
+    import numpy as np
+    import torch
+
+    from paper_2411_07942_b200 import binding
+
+    def read(obj, n):
+        return list((ctypes.c_uint64 * n).from_buffer_copy(bytes(obj)))
+
+    assert read(binding._ptrs([4096, 2 ** 47]), 2) == [4096, 2 ** 47]
+    assert read(binding._ptrs((1, None, ctypes.c_void_p(7))), 3) == [1, 0, 7]
+    assert read(binding._ptrs((ctypes.c_void_p * 2)(5, 6)), 2) == [5, 6]
+    assert read(binding._ptrs([-1]), 1) == [2 ** 64 - 1]
+    for bad in ((ctypes.c_uint32 * 2)(1, 2), (ctypes.c_uint64 * 2)(1, 2), (ctypes.c_float * 2)()):
+        with pytest.raises(ctypes.ArgumentError):
+            binding._ptrs(bad)
+    for bad in ([torch.tensor(4096)], [np.int64(4096)], [4096.0], ["x"]):
+        with pytest.raises(TypeError):
+            binding._ptrs(bad)
+    ok = (ctypes.c_void_p * 2)()
+    for name, args in (("tpq_quantize_pack_batch", (0, 2, None, 1, 8, None, 0, None)), ("tpq_dequant_reduce", (None, 2, 1, None, 0, 8, None)),
+                       ("tpq_quantize_pack_push", (0, None, 1, 8, None, None, 2, 0, 1, None))):
+        fn, types = getattr(lib, name), binding.SIGNATURES[name][1]
+        for j, kind in enumerate(types):
+            if kind is not ctypes.POINTER(ctypes.c_void_p):
+                continue
+            with_ok = [None, *args]
+            with_ok[j] = ok
+            assert fn(*with_ok) == binding.TPQ_ERR_INVALID_ARG          # (no context)
+            for bad in (4096, b"12345678", (ctypes.c_uint32 * 2)()):
+                wrong = [None, *args]
+                wrong[j] = bad
+                with pytest.raises(ctypes.ArgumentError):
+                    fn(*wrong)
