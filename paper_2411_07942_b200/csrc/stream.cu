@@ -1512,6 +1512,39 @@ bool tpq_stream_pipe_ok(const tpq_ctx *c, int64_t T, int64_t stride)
     return tpq_stream_ok(c, T) && qs_pipe_plan(c, stride, &gpt, &warps, &nstage);
 }
 
+// One block per SM has a warp for 31 or 62 groups.  Rows of up to 256 groups leave it so few warps that the copies'
+// latency shows once a block has several rows: 512 features (3 warps an SM against the group kernel's 8 and more) level at
+// 1000 rows of a launch, 1.5 times as long at 2000, 2.4 at 32768; 2048 features 0.8 at 512 rows, 1.05 at 1000, 1.2 to 1.5
+// beyond; 2112 features level at 5000 rows, 1.1 at 9600; from 2304 on 0.5 to 1.0.  Two groups a lane: up to three tokens (a
+// thread of the group kernel takes four) 1.0 to 1.4 times as long; 0.7 to 0.9 at 30 rows, 0.9 to 1.1 at 100 to 300 and 0.7 to
+// 1.0 at 9600 of 5376 to 8256 features (1.2 at 600 or 1200 rows of 6144, whose last stage of four holds one row); above
+// 8704 features only up to 3 bits and from 500 rows on less (0.8 to 0.95).  Rows too long for the ring are the tile
+// kernel's, a block to 8 rows: 0.8 to 0.9 times as long with 4000 rows at 2 and 3 bits, 1.0 to 2.2 at more, 1.1 to 5.8 with fewer.
+bool tpq_stream_ahead(const tpq_ctx *c, int n, int64_t T, int64_t stride)
+{
+    int gpt, warps, nstage;
+    const int G = (c->E - c->k + 7) / 8, sm = c->sm_count;
+    const int64_t rows = (n < QS_MAX_BATCH ? n : QS_MAX_BATCH) * T;  // of a launch
+    if (!tpq_stream_ok(c, T)) return false;
+    if (!qs_pipe_plan(c, stride, &gpt, &warps, &nstage)) return c->bits <= 3 && rows >= 24 * sm;
+    if (gpt > 1) return T >= 4 && (c->E <= 8704 || (c->bits <= 3 && rows >= 3 * sm));
+    return G > 280 || rows < (G > 256 ? 32 : 7) * sm;
+}
+
+// The copies and the publishing kernel cost the other way about 4 us and 1 us more per destination (16 destinations of few
+// rows 25 us against 5 to 10), the push mode stores every word n_dst times.  Narrow rows: one destination 0.8 times as
+// long at 256 rows, 1.2 at 1000, 1.5 to 1.8 at 2048; two 0.75, 1.1, 1.4; four 0.55, 0.8, 1.1.  Two groups a lane: one
+// destination 0.8 to 1.1 at up to 256 rows, 1.2 at 1000, 1.4 at 2048 (1.2 at one row above 8704 features); two 0.9 and 1.2;
+// sixteen 0.4 and 1.1.
+bool tpq_stream_push_ahead(const tpq_ctx *c, int n_dst, int64_t T, int64_t stride)
+{
+    int gpt, warps, nstage;
+    if (!qs_pipe_plan(c, stride, &gpt, &warps, &nstage)) return false;
+    const int sm = c->sm_count;
+    if (gpt > 1) return n_dst > 1 ? T < 10 * sm : T < 3 * sm && (c->E <= 8704 || T >= 24);
+    return (c->E - c->k + 7) / 8 > 256 || T < 3 * sm * n_dst;
+}
+
 cudaError_t tpq_launch_quantize_stream_push(const tpq_ctx *c, int shard, const void *y, int64_t T, int64_t stride, void *const *dst,
                                             uint32_t *const *arrived, int n_dst, uint32_t epoch, cudaStream_t st, int64_t *launches)
 {

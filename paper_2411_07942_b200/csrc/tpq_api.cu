@@ -76,17 +76,44 @@ tpq_status build_tables(tpq_ctx *c, int k, bool topk)
     return TPQ_OK;
 }
 
-// Shapes that option TPQ_OPT_KERNEL_PATH = 2 accepts at code widths other than 4 bits.
-bool widths_ok(const tpq_ctx *c, int64_t stride)
-{
-    return c->bits != 4 && c->E % 8 == 0 && c->k % 8 == 0 && stride % 8 == 0 && c->E - c->k >= 8;
-}
-
 // Calls below this many values (T*E) stay with the shape-generic kernels where the bit-stream kernels' longer prologue
 // costs more than it brings: the reduction (E = 700 to 5120, N = 4 to 16: generic 2.4 to 3.9 us against 2.8 to 8.5 us below
 // the line, 4.0 to 12.5 against 3.4 to 8.7 us above it) and one shard whose rows bulk copies cannot fetch (E = 700:
 // 3.6 against 4.0 us below, within 0.5 us of one another around it, 28 against 14 us at 2048 x 5120).
 constexpr int64_t SMALL_VALUES = 1 << 18;
+
+// The kernels that quantise n shards of T rows.
+enum class Quantiser { TILED, STREAM, GROUPS, GENERIC };
+Quantiser pick_quantiser(const tpq_ctx *c, int n, int64_t T, int64_t stride)
+{
+    if (c->kernel_path == 1) return Quantiser::GENERIC;
+    if (tpq_quantize_tiled_ok(c, T, stride)) return Quantiser::TILED;
+    if (tpq_groups_ok(c, T, stride)) return tpq_stream_ahead(c, n, T, stride) ? Quantiser::STREAM : Quantiser::GROUPS;
+    const bool stream = tpq_stream_ok(c, T), pipe = tpq_stream_pipe_ok(c, T, stride);
+    return stream && (pipe || n > 1 || T * c->E >= SMALL_VALUES) ? Quantiser::STREAM : Quantiser::GENERIC;
+}
+
+cudaError_t quantize(tpq_ctx *c, Quantiser q, int first_shard, int n, const void *const *ys, int64_t T, int64_t stride,
+                     void *const *payloads, cudaStream_t st)
+{
+    switch (q) {
+    case Quantiser::TILED: return tpq_launch_quantize_tiled_batch(c, first_shard, n, ys, T, stride, payloads, st, &c->launches);
+    case Quantiser::STREAM: return tpq_launch_quantize_stream(c, first_shard, n, ys, T, stride, payloads, st, &c->launches);
+    case Quantiser::GROUPS: return tpq_launch_quantize_groups(c, first_shard, n, ys, T, stride, payloads, st, &c->launches);
+    default: break;
+    }
+    cudaError_t e = cudaSuccess;
+    for (int b = 0; b < n && e == cudaSuccess; ++b)
+        e = tpq_launch_quantize_generic(c, first_shard + b, static_cast<const uint16_t *>(ys[b]), T, stride,
+                                        static_cast<uint8_t *>(payloads[b]), st, &c->launches);
+    return e;
+}
+
+// Shapes that option TPQ_OPT_KERNEL_PATH = 2 accepts of a quantiser.
+bool forced_ok(const tpq_ctx *c, int64_t T, int64_t stride)
+{
+    return tpq_quantize_tiled_ok(c, T, stride) || tpq_groups_ok(c, T, stride);
+}
 
 struct StateHeader {
     char magic[8];
@@ -416,20 +443,9 @@ tpq_status tpq_quantize_pack(tpq_ctx *c, int shard, const void *y, int64_t T, in
     if (!aligned16(y) || !aligned16(payload)) return fail(c, TPQ_ERR_ALIGN, "y and payload must be 16-byte aligned");
     if (cap < tpq_payload_bytes(c, T))
         return fail(c, TPQ_ERR_SIZE, "payload capacity %zu < %zu", cap, tpq_payload_bytes(c, T));
-    const bool tiled_ok = tpq_quantize_tiled_ok(c, T, stride);
-    if (c->kernel_path == 2 && !tiled_ok && !widths_ok(c, stride))
+    if (c->kernel_path == 2 && !forced_ok(c, T, stride))
         return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the tiled kernel");
-    cudaError_t e;
-    if (tiled_ok && c->kernel_path != 1)
-        e = tpq_launch_quantize_tiled(c, shard, static_cast<const uint16_t *>(y), T, stride,
-                                      static_cast<uint8_t *>(payload), static_cast<cudaStream_t>(stream), &c->launches);
-    else if (c->kernel_path != 1 && tpq_stream_ok(c, T) && (tpq_stream_pipe_ok(c, T, stride) || T * c->E >= SMALL_VALUES))
-        e = tpq_launch_quantize_stream(c, shard, 1, &y, T, stride, &payload, static_cast<cudaStream_t>(stream),
-                                       &c->launches);
-    else
-        e = tpq_launch_quantize_generic(c, shard, static_cast<const uint16_t *>(y), T, stride,
-                                        static_cast<uint8_t *>(payload), static_cast<cudaStream_t>(stream),
-                                        &c->launches);
+    const cudaError_t e = quantize(c, pick_quantiser(c, 1, T, stride), shard, 1, &y, T, stride, &payload, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "quantize_pack kernel");
     return TPQ_OK;
 }
@@ -453,22 +469,9 @@ tpq_status tpq_quantize_pack_batch(tpq_ctx *c, int first_shard, int n, const voi
         if (!aligned16(ys[b]) || !aligned16(payloads[b]))
             return fail(c, TPQ_ERR_ALIGN, "y and payload of shard %d must be 16-byte aligned", first_shard + b);
     }
-    const bool tiled_ok = tpq_quantize_tiled_ok(c, T, stride);
-    if (c->kernel_path == 2 && !tiled_ok && !widths_ok(c, stride))
+    if (c->kernel_path == 2 && !forced_ok(c, T, stride))
         return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the tiled kernel");
-    cudaError_t e = cudaSuccess;
-    if (tiled_ok && c->kernel_path != 1) {
-        e = tpq_launch_quantize_tiled_batch(c, first_shard, n, ys, T, stride, payloads, static_cast<cudaStream_t>(stream),
-                                            &c->launches);
-    } else if (c->kernel_path != 1 && tpq_stream_ok(c, T)) {
-        e = tpq_launch_quantize_stream(c, first_shard, n, ys, T, stride, payloads, static_cast<cudaStream_t>(stream),
-                                       &c->launches);
-    } else {
-        for (int b = 0; b < n && e == cudaSuccess; ++b)
-            e = tpq_launch_quantize_generic(c, first_shard + b, static_cast<const uint16_t *>(ys[b]), T, stride,
-                                            static_cast<uint8_t *>(payloads[b]), static_cast<cudaStream_t>(stream),
-                                            &c->launches);
-    }
+    const cudaError_t e = quantize(c, pick_quantiser(c, n, T, stride), first_shard, n, ys, T, stride, payloads, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "quantize_pack kernel");
     return TPQ_OK;
 }
@@ -503,7 +506,8 @@ tpq_status tpq_quantize_pack_push(tpq_ctx *c, int shard, const void *y, int64_t 
         if (e != cudaSuccess) return cuda_fail(c, e, "quantize_pack_push kernel");
         return TPQ_OK;
     }
-    if (c->kernel_path != 1 && tpq_stream_pipe_ok(c, T, stride)) {
+    const bool groups = tpq_groups_ok(c, T, stride);
+    if (c->kernel_path != 1 && tpq_stream_pipe_ok(c, T, stride) && (!groups || tpq_stream_push_ahead(c, n_dst, T, stride))) {
         e = tpq_launch_quantize_stream_push(c, shard, y, T, stride, dst, arrived, n_dst, epoch, st, &c->launches);
         if (e != cudaSuccess) return cuda_fail(c, e, "quantize_pack_push kernel");
         return TPQ_OK;
@@ -511,11 +515,9 @@ tpq_status tpq_quantize_pack_push(tpq_ctx *c, int shard, const void *y, int64_t 
     // other shapes: quantise into the first destination, copy it to the others in stream
     // order, then publish the arrival words
     void *first = dst[0];
-    if (c->kernel_path != 1 && tpq_stream_ok(c, T))
-        e = tpq_launch_quantize_stream(c, shard, 1, &y, T, stride, &first, st, &c->launches);
-    else
-        e = tpq_launch_quantize_generic(c, shard, static_cast<const uint16_t *>(y), T, stride,
-                                        static_cast<uint8_t *>(first), st, &c->launches);
+    const Quantiser q = c->kernel_path == 1 ? Quantiser::GENERIC : groups ? Quantiser::GROUPS
+                      : tpq_stream_ok(c, T) ? Quantiser::STREAM : Quantiser::GENERIC;
+    e = quantize(c, q, shard, 1, &y, T, stride, &first, st);
     const size_t bytes = tpq_payload_bytes(c, T);
     for (int d = 1; d < n_dst && e == cudaSuccess; ++d)
         if (dst[d] != first) e = cudaMemcpyAsync(dst[d], first, bytes, cudaMemcpyDefault, st);
@@ -637,14 +639,17 @@ static tpq_status dequant_reduce_impl(tpq_ctx *c, const void *const *payloads, i
     if (!aligned16(out)) return fail(c, TPQ_ERR_ALIGN, "out must be 16-byte aligned");
     const int fp32 = dt == TPQ_OUT_FP32;
     const bool tiled_ok = tpq_dequant_tiled_ok(c, T, out_stride, fp32);
-    if (c->kernel_path == 2 && !tiled_ok && !widths_ok(c, out_stride))
-        return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the tiled kernel");
+    const bool groups_ok = tpq_groups_ok(c, T, out_stride);
+    if (c->kernel_path == 2 && !tiled_ok && !groups_ok) return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the tiled kernel");
     cudaError_t e;
     if (tiled_ok && c->kernel_path != 1)
         e = tpq_launch_dequant_tiled(c, payloads, T, out, fp32, out_stride, static_cast<cudaStream_t>(stream),
                                      &c->launches);
     else if (c->kernel_path != 1 && tpq_stream_ok(c, T) && T * c->E >= SMALL_VALUES)
         e = tpq_launch_dequant_stream(c, payloads, T, out, fp32, out_stride, static_cast<cudaStream_t>(stream),
+                                      &c->launches);
+    else if (c->kernel_path != 1 && groups_ok && T * c->E >= SMALL_VALUES)
+        e = tpq_launch_dequant_groups(c, payloads, T, out, fp32, out_stride, static_cast<cudaStream_t>(stream),
                                       &c->launches);
     else
         e = tpq_launch_dequant_generic(c, payloads, T, out, fp32, out_stride, static_cast<cudaStream_t>(stream),

@@ -127,11 +127,22 @@ cudaError_t tpq_launch_permute_weight(const tpq_ctx *c, const void *w, void *out
 cudaError_t tpq_launch_linear_quantize(const tpq_ctx *c, int shard, const void *x, const void *w_slots, int64_t T, int64_t K,
                                        void *payload, void *y_slots, cudaStream_t st, int64_t *launches);
 
+// Group kernels (groups.cu): code widths other than 4 bits on shapes that are multiples of 8.
+bool tpq_groups_ok(const tpq_ctx *c, int64_t T, int64_t stride);
+cudaError_t tpq_launch_quantize_groups(const tpq_ctx *c, int shard0, int n, const void *const *ys, int64_t T,
+                                       int64_t stride, void *const *payloads, cudaStream_t st, int64_t *launches);
+cudaError_t tpq_launch_dequant_groups(const tpq_ctx *c, const void *const *payloads, int64_t T, void *out, int fp32_out,
+                                      int64_t out_stride, cudaStream_t st, int64_t *launches);
+
 // Bit-stream kernels (stream.cu): code widths other than 4 bits, and any E, k or stride.
 bool tpq_stream_ok(const tpq_ctx *c, int64_t T);
 cudaError_t tpq_launch_quantize_stream(const tpq_ctx *c, int shard0, int n, const void *const *ys, int64_t T,
                                        int64_t stride, void *const *payloads, cudaStream_t st, int64_t *launches);
 bool tpq_stream_pipe_ok(const tpq_ctx *c, int64_t T, int64_t stride);  // (its quantiser is the pipelined one; push mode needs it)
+// of a shape of the group kernels: whether the bit-stream quantiser is ahead on n shards of T rows, and its push mode of the
+// group kernel, n_dst - 1 copies and a publishing kernel
+bool tpq_stream_ahead(const tpq_ctx *c, int n, int64_t T, int64_t stride);
+bool tpq_stream_push_ahead(const tpq_ctx *c, int n_dst, int64_t T, int64_t stride);
 cudaError_t tpq_launch_quantize_stream_push(const tpq_ctx *c, int shard, const void *y, int64_t T, int64_t stride, void *const *dst,
                                             uint32_t *const *arrived, int n_dst, uint32_t epoch, cudaStream_t st, int64_t *launches);
 cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *payloads, int64_t T, void *out, int fp32_out,

@@ -70,3 +70,37 @@ def test_stream_kernels_equal_generic(N, T, E, k, bits, pad, with_bias):
             for x, y in zip(a, b):
                 assert np.array_equal(x, y), (hp, np.nonzero(x != y)[0][:8])
     t.close()
+
+
+@pytest.mark.parametrize("N,T,E,k,bits,pad,with_bias", [
+    (4, 300, 512, 8, 3, 0, True), (3, 37, 64, 8, 2, 8, False), (2, 9, 11264, 176, 5, 0, False), (2, 5, 9216, 144, 7, 16, True),
+    (2, 3, 32768, 512, 8, 0, True), (2, 1, 131072, 2048, 2, 8, False), (16, 60, 2048, 32, 6, 0, False), (17, 130, 256, 248, 8, 0, False)])
+def test_group_kernels_equal_generic(N, T, E, k, bits, pad, with_bias):
+    """Other code widths where the group kernels quantise: narrow rows, rows too long for the ring or of two groups a lane; the
+    two longest are also theirs to reduce."""
+    test_stream_kernels_equal_generic(N, T, E, k, bits, pad, with_bias)
+
+
+@pytest.mark.parametrize("T,E,k,bits,n_dst", [(1000, 512, 8, 3, 1), (1900, 1024, 16, 5, 3), (70, 8192, 128, 8, 1), (1500, 8192, 128, 7, 2),
+                                              (40, 16384, 256, 6, 2)])
+def test_pushes_through_the_group_kernels(T, E, k, bits, n_dst):
+    """The quantise, copy and publish form of a push: every destination and word, against the shape-generic quantiser."""
+    t = binding.Tpq(1, E, bits=bits)
+    g = torch.Generator(device="cuda").manual_seed(T + E)
+    y = (torch.randn((T + 16, E), generator=g, device="cuda") * 2).to(torch.bfloat16)
+    t.calibrate_ranges(0, y.data_ptr(), 1, 16)
+    torch.cuda.synchronize()
+    t.select_features(k)
+    P = t.payload_bytes(T)
+    want = torch.zeros(P, dtype=torch.uint8, device="cuda")
+    t.set_option(binding.TPQ_OPT_KERNEL_PATH, binding.PATH_GENERIC)
+    t.quantize_pack(0, y.data_ptr(), T, want.data_ptr(), P)
+    t.set_option(binding.TPQ_OPT_KERNEL_PATH, binding.PATH_AUTO)
+    bufs = [gu.guarded(P) for _ in range(n_dst)]
+    words = torch.zeros(n_dst, dtype=torch.int32, device="cuda")
+    t.quantize_pack_push(0, y.data_ptr(), T, [v.data_ptr() for _, v in bufs], [words.data_ptr() + 4 * d for d in range(n_dst)], P, 11)
+    torch.cuda.synchronize()
+    assert t.device_status() == 0 and bool((words == 11).all())
+    for whole, v in bufs:
+        assert gu.guards_intact(whole, P) and torch.equal(v, want)
+    t.close()
