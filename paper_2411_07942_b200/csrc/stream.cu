@@ -1531,6 +1531,22 @@ bool tpq_stream_ahead(const tpq_ctx *c, int n, int64_t T, int64_t stride)
     return G > 280 || rows < (G > 256 ? 32 : 7) * sm;
 }
 
+// The tile kernel against n launches of the shape-generic one.  A block takes 8 rows from end to end, 320 groups at a
+// time, so however few rows there are the launch takes as long as a block: 3.6 us + 1.1 ns a feature (1.3 ns from 5 bits
+// on), 2 us + 0.85 ns up to 4 rows, 0.5 ns for one.  The generic kernel takes 3.4 us a launch (6 at 2 bits, 5 at 3) and from
+// about 400 000 values on 3 us + 2.5 ps a value (4.7 at 2 bits, 3.6 at 3).  Measured at 4 bits, generic against tile: one shard of 5121
+// features 4.4 and 9.4 us at 64 rows, 6.3 and 9.5 at 256, 15.8 and 12.8 at 1024; of 16385 4.4 and 22.7 at 16, 23.7 and 25.4 at 512; two
+// shards 8.4 and 22.8, 46 and 33; 16 of 1033 features 58 and 4.5 at 16 rows.
+bool tpq_stream_tile_ahead(const tpq_ctx *c, int n, int64_t T)
+{
+    const int b = c->bits;
+    const double E = c->E, values = (double)T * E;
+    const double tile = T > 4 ? 3600.0 + (b > 4 ? 1.3 : 1.1) * E : 2000.0 + (T > 1 ? 0.85 : 0.5) * E;
+    const double least = b == 2 ? 6000.0 : b == 3 ? 5000.0 : 3400.0;
+    const double generic = (b <= 3 ? 3500.0 : 3000.0) + (b == 2 ? 4.7e-3 : b == 3 ? 3.6e-3 : 2.5e-3) * values;
+    return tile < n * (generic > least ? generic : least);
+}
+
 // The copies and the publishing kernel cost the other way about 4 us and 1 us more per destination (16 destinations of few
 // rows 25 us against 5 to 10), the push mode stores every word n_dst times.  Narrow rows: one destination 0.8 times as
 // long at 256 rows, 1.2 at 1000, 1.5 to 1.8 at 2048; two 0.75, 1.1, 1.4; four 0.55, 0.8, 1.1.  Two groups a lane: one

@@ -76,10 +76,9 @@ tpq_status build_tables(tpq_ctx *c, int k, bool topk)
     return TPQ_OK;
 }
 
-// Calls below this many values (T*E) stay with the shape-generic kernels where the bit-stream kernels' longer prologue
-// costs more than it brings: the reduction (E = 700 to 5120, N = 4 to 16: generic 2.4 to 3.9 us against 2.8 to 8.5 us below
-// the line, 4.0 to 12.5 against 3.4 to 8.7 us above it) and one shard whose rows bulk copies cannot fetch (E = 700:
-// 3.6 against 4.0 us below, within 0.5 us of one another around it, 28 against 14 us at 2048 x 5120).
+// Reductions below this many values (T*E) stay with the shape-generic kernel, where the bit-stream kernels' longer prologue
+// costs more than it brings (E = 700 to 5120, N = 4 to 16: generic 2.4 to 3.9 us against 2.8 to 8.5 us below the line, 4.0 to
+// 12.5 against 3.4 to 8.7 us above it; at 64 devices it takes 13 to 28 us below the line).
 constexpr int64_t SMALL_VALUES = 1 << 18;
 
 // The kernels that quantise n shards of T rows.
@@ -90,7 +89,7 @@ Quantiser pick_quantiser(const tpq_ctx *c, int n, int64_t T, int64_t stride)
     if (tpq_quantize_tiled_ok(c, T, stride)) return Quantiser::TILED;
     if (tpq_groups_ok(c, T, stride)) return tpq_stream_ahead(c, n, T, stride) ? Quantiser::STREAM : Quantiser::GROUPS;
     const bool stream = tpq_stream_ok(c, T), pipe = tpq_stream_pipe_ok(c, T, stride);
-    return stream && (pipe || n > 1 || T * c->E >= SMALL_VALUES) ? Quantiser::STREAM : Quantiser::GENERIC;
+    return pipe || (stream && tpq_stream_tile_ahead(c, n, T)) ? Quantiser::STREAM : Quantiser::GENERIC;
 }
 
 cudaError_t quantize(tpq_ctx *c, Quantiser q, int first_shard, int n, const void *const *ys, int64_t T, int64_t stride,
@@ -515,8 +514,7 @@ tpq_status tpq_quantize_pack_push(tpq_ctx *c, int shard, const void *y, int64_t 
     // other shapes: quantise into the first destination, copy it to the others in stream
     // order, then publish the arrival words
     void *first = dst[0];
-    const Quantiser q = c->kernel_path == 1 ? Quantiser::GENERIC : groups ? Quantiser::GROUPS
-                      : tpq_stream_ok(c, T) ? Quantiser::STREAM : Quantiser::GENERIC;
+    const Quantiser q = groups && c->kernel_path != 1 ? Quantiser::GROUPS : pick_quantiser(c, 1, T, stride);
     e = quantize(c, q, shard, 1, &y, T, stride, &first, st);
     const size_t bytes = tpq_payload_bytes(c, T);
     for (int d = 1; d < n_dst && e == cudaSuccess; ++d)

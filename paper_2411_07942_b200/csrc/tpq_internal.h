@@ -143,6 +143,8 @@ bool tpq_stream_pipe_ok(const tpq_ctx *c, int64_t T, int64_t stride);  // (its q
 // group kernel, n_dst - 1 copies and a publishing kernel
 bool tpq_stream_ahead(const tpq_ctx *c, int n, int64_t T, int64_t stride);
 bool tpq_stream_push_ahead(const tpq_ctx *c, int n_dst, int64_t T, int64_t stride);
+// of a shape that is neither theirs nor the ring's: whether its tile kernel is ahead of n launches of the shape-generic one
+bool tpq_stream_tile_ahead(const tpq_ctx *c, int n, int64_t T);
 cudaError_t tpq_launch_quantize_stream_push(const tpq_ctx *c, int shard, const void *y, int64_t T, int64_t stride, void *const *dst,
                                             uint32_t *const *arrived, int n_dst, uint32_t epoch, cudaStream_t st, int64_t *launches);
 cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *payloads, int64_t T, void *out, int fp32_out,

@@ -104,3 +104,32 @@ def test_pushes_through_the_group_kernels(T, E, k, bits, n_dst):
     for whole, v in bufs:
         assert gu.guards_intact(whole, P) and torch.equal(v, want)
     t.close()
+
+
+@pytest.mark.parametrize("E,k,bits", [(5121, 51, 4), (16385, 3, 2), (1033, 16, 8), (5121, 5000, 4), (65, 1, 3)])
+def test_rows_that_bulk_copies_cannot_fetch(E, k, bits):
+    """The tile kernel and the shape-generic one share these shapes by size: token counts on both sides of the line, tiles of
+    less than 4 and less than 8 rows, one shard and three."""
+    N = 3
+    g = torch.Generator(device="cuda").manual_seed(E + bits)
+    t = binding.Tpq(N, E, bits=bits)
+    c = torch.randn((32, E), generator=g, device="cuda").to(torch.bfloat16)
+    for i in range(N):
+        t.calibrate_ranges(i, c.data_ptr(), 1, 32)
+    torch.cuda.synchronize()
+    t.select_features(k)
+    for T in (1, 4, 5, 64, 167, 601, 2049 if E < 6000 else 900):
+        ys = [(1.5 * torch.randn((T, E), generator=g, device="cuda")).to(torch.bfloat16) for _ in range(N)]
+        P = t.payload_bytes(T)
+        got = []
+        for path, n in ((binding.PATH_GENERIC, 1), (binding.PATH_AUTO, 1), (binding.PATH_AUTO, N)):
+            t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+            bufs = [gu.guarded(P) for _ in range(N)]
+            for i in range(0, N, n):
+                t.quantize_pack_batch(i, [y.data_ptr() for y in ys[i:i + n]], T, [v.data_ptr() for _, v in bufs[i:i + n]], P)
+            torch.cuda.synchronize()
+            assert t.device_status() == 0 and all(gu.guards_intact(w, P) for w, _ in bufs)
+            got.append([v for _, v in bufs])
+        for other in got[1:]:
+            assert all(torch.equal(a, b) for a, b in zip(got[0], other)), T
+    t.close()
