@@ -59,9 +59,10 @@ typedef enum { TPQ_OUT_BF16 = 0, TPQ_OUT_FP32 = 1 } tpq_out_dtype;
 
 /* Options for tpq_set_option. */
 typedef enum {
-    /* 0 = automatic (default); 1 = always the shape-generic kernels; 2 = the tiled kernels,
-     * TPQ_ERR_INVALID_ARG from the call if the shape does not admit them (E, k and strides
-     * multiples of 8, 4-bit codes). */
+    /* 0 = automatic (default); 1 = always the shape-generic kernels; 2 = never those: the kernels
+     * for E, k and strides that are multiples of 8, whatever the size (the Int4 kernels; at other
+     * code widths the bit-stream or group kernels, chosen as by 0), TPQ_ERR_INVALID_ARG from the
+     * call if the shape does not admit them. */
     TPQ_OPT_KERNEL_PATH = 0,
     /* Which tiled kernel tpq_dequant_reduce uses when the tiled path is taken: 0 = chosen from the
      * shape (default); 1 = row kernel (needs N <= 4 and (E-k)/8 <= 768, or N <= 8 and (E-k)/8 <= 640); 2 = tensor-map panel kernel

@@ -443,7 +443,7 @@ tpq_status tpq_quantize_pack(tpq_ctx *c, int shard, const void *y, int64_t T, in
     if (cap < tpq_payload_bytes(c, T))
         return fail(c, TPQ_ERR_SIZE, "payload capacity %zu < %zu", cap, tpq_payload_bytes(c, T));
     if (c->kernel_path == 2 && !forced_ok(c, T, stride))
-        return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the tiled kernel");
+        return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the kernels for multiples of 8");
     const cudaError_t e = quantize(c, pick_quantiser(c, 1, T, stride), shard, 1, &y, T, stride, &payload, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "quantize_pack kernel");
     return TPQ_OK;
@@ -469,7 +469,7 @@ tpq_status tpq_quantize_pack_batch(tpq_ctx *c, int first_shard, int n, const voi
             return fail(c, TPQ_ERR_ALIGN, "y and payload of shard %d must be 16-byte aligned", first_shard + b);
     }
     if (c->kernel_path == 2 && !forced_ok(c, T, stride))
-        return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the tiled kernel");
+        return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the kernels for multiples of 8");
     const cudaError_t e = quantize(c, pick_quantiser(c, n, T, stride), first_shard, n, ys, T, stride, payloads, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(c, e, "quantize_pack kernel");
     return TPQ_OK;
@@ -638,15 +638,16 @@ static tpq_status dequant_reduce_impl(tpq_ctx *c, const void *const *payloads, i
     const int fp32 = dt == TPQ_OUT_FP32;
     const bool tiled_ok = tpq_dequant_tiled_ok(c, T, out_stride, fp32);
     const bool groups_ok = tpq_groups_ok(c, T, out_stride);
-    if (c->kernel_path == 2 && !tiled_ok && !groups_ok) return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the tiled kernel");
+    if (c->kernel_path == 2 && !tiled_ok && !groups_ok) return fail(c, TPQ_ERR_INVALID_ARG, "shape does not admit the kernels for multiples of 8");
+    const bool fast = c->kernel_path == 2 || (c->kernel_path == 0 && T * c->E >= SMALL_VALUES);
     cudaError_t e;
     if (tiled_ok && c->kernel_path != 1)
         e = tpq_launch_dequant_tiled(c, payloads, T, out, fp32, out_stride, static_cast<cudaStream_t>(stream),
                                      &c->launches);
-    else if (c->kernel_path != 1 && tpq_stream_ok(c, T) && T * c->E >= SMALL_VALUES)
+    else if (fast && tpq_stream_ok(c, T))
         e = tpq_launch_dequant_stream(c, payloads, T, out, fp32, out_stride, static_cast<cudaStream_t>(stream),
                                       &c->launches);
-    else if (c->kernel_path != 1 && groups_ok && T * c->E >= SMALL_VALUES)
+    else if (fast && groups_ok)
         e = tpq_launch_dequant_groups(c, payloads, T, out, fp32, out_stride, static_cast<cudaStream_t>(stream),
                                       &c->launches);
     else

@@ -133,3 +133,41 @@ def test_rows_that_bulk_copies_cannot_fetch(E, k, bits):
         for other in got[1:]:
             assert all(torch.equal(a, b) for a, b in zip(got[0], other)), T
     t.close()
+
+
+def _kernels(call):
+    from torch.profiler import ProfilerActivity, profile
+
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as p:
+        call()
+        torch.cuda.synchronize()
+    return " ".join(e.name for e in p.events())
+
+
+@pytest.mark.parametrize("N,T,E,k,bits,quantiser,reducer", [
+    (3, 37, 512, 8, 3, "quantize_stream<", "dequant_stream_rows<"), (6, 9, 520, 16, 8, "quantize_stream<", "dequant_stream<"),
+    (2, 3, 32768, 512, 8, "quantize_groups<", "dequant_groups<"), (2, 5, 16, 8, 2, "quantize_groups<", "dequant_groups<"),
+    (2, 3, 512, 8, 4, "quantize_tiled<", "dequant_rows<")])
+def test_forced_path_runs_no_generic_kernel(N, T, E, k, bits, quantiser, reducer):
+    """Path 2 at sizes that the automatic choice leaves to the shape-generic reduction: every width's own kernels, and the
+    same bytes and sums as path 1."""
+    t = binding.Tpq(N, E, bits=bits)
+    g = torch.Generator(device="cuda").manual_seed(E + bits)
+    ys = [(2 * torch.randn((T, E), generator=g, device="cuda")).to(torch.bfloat16) for _ in range(N)]
+    for i in range(N):
+        t.calibrate_ranges(i, ys[i].data_ptr(), 1, T)
+    torch.cuda.synchronize()
+    t.select_features(k)
+    P = t.payload_bytes(T)
+    got = []
+    for path, kernels in ((binding.PATH_GENERIC, ("quantize_generic", "dequant_generic")), (binding.PATH_TILED, (quantiser, reducer))):
+        t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+        pls = [torch.zeros(P, dtype=torch.uint8, device="cuda") for _ in range(N)]
+        out = torch.empty((T, E), dtype=torch.float32, device="cuda")
+        ptrs = [p.data_ptr() for p in pls]
+        assert kernels[0] in _kernels(lambda: t.quantize_pack_batch(0, [y.data_ptr() for y in ys], T, ptrs, P))
+        assert kernels[1] in _kernels(lambda: t.dequant_reduce(ptrs, T, out.data_ptr(), binding.TPQ_OUT_FP32))
+        assert t.device_status() == 0
+        got.append([*pls, out])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    t.close()
