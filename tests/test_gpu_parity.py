@@ -798,3 +798,23 @@ def test_inputs_from_the_call_ahead(T, E, k, bits):
     for other in got[1:]:
         for a, b in zip(got[0], other):
             assert np.array_equal(a, b)
+
+
+def test_few_blocks_share_the_rows():
+    """512 rows of 100 features take about as long as one sequence as they do as eight of 64 rows (whose blocks are eight
+    in any case): a call of few blocks splits its rows."""
+    y = torch.randn((512, 100), device="cuda").to(torch.bfloat16)
+    t = binding.Tpq(1, 100)
+    times = {}
+    for n_seq in (1, 8):
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        for _ in range(20):
+            torch.cuda._sleep(1 << 17)      # the launches are queued before the first one starts
+            e[0].record()
+            for _ in range(8):
+                t.calibrate_ranges(0, y.data_ptr(), n_seq, 512 // n_seq)
+            e[1].record()
+            torch.cuda.synchronize()
+            times[n_seq] = min(times.get(n_seq, 1e9), e[0].elapsed_time(e[1]))
+    t.close()
+    assert times[1] < 2.0 * times[8], times
