@@ -109,7 +109,8 @@ tpq_status tpq_set_option(tpq_ctx *ctx, tpq_option opt, int value);
  *   y_bf16_dev : [n_seq][S][E] BF16, row stride row_stride_elems (>= E), the
  *                sequences back to back (sequence q starts at row q*S).
  * Enqueues on cuda_stream.  May grow a context-owned scratch buffer
- * (cudaMalloc) when n_seq*S exceeds every earlier call.
+ * (cudaMalloc) when n_seq*S exceeds every earlier call, or when there are more
+ * sequences than it has room for (4 * n_seq * E bytes).
  * n_seq == 0 is a no-op.  Errors: INVALID_ARG, ALIGN, NOMEM, CUDA. */
 tpq_status tpq_calibrate_ranges(tpq_ctx *ctx, int shard, const void *y_bf16_dev, int64_t n_seq, int64_t S,
                                 int64_t row_stride_elems, void *cuda_stream);

@@ -249,7 +249,12 @@ tpq_status tpq_calibrate_ranges(tpq_ctx *c, int shard, const void *y, int64_t n_
     if (n_seq * S > (int64_t)1 << 40) return fail(c, TPQ_ERR_INVALID_ARG, "calibration set too large");
     int n_split = 1;
     const size_t need = tpq_calib_scratch_bytes(n_seq, S, c->E, c->sm_count, &n_split);
-    if (need > c->scratch_bytes) {
+    // The number of splits goes up and down with the shape (8 sequences of 2048 x 4608: 4, 7: 9).  A call of no more tokens
+    // than an earlier one takes the splits that fit rather than allocate: it may be one that is captured.
+    const size_t per_split = need / n_split;
+    if (need > c->scratch_bytes && n_seq * S <= c->scratch_tokens && per_split <= c->scratch_bytes) {
+        n_split = (int)(c->scratch_bytes / per_split);
+    } else if (need > c->scratch_bytes) {
         TPQ_CUDA(c, cudaFree(c->scratch));  // waits for work that still uses it
         c->scratch = nullptr;
         c->scratch_bytes = 0;
@@ -257,6 +262,7 @@ tpq_status tpq_calibrate_ranges(tpq_ctx *c, int shard, const void *y, int64_t n_
         if (e != cudaSuccess) return cuda_fail(c, e, "calibration scratch");
         c->scratch_bytes = need;
     }
+    if (n_seq * S > c->scratch_tokens) c->scratch_tokens = n_seq * S;
     float *m = c->t.m + (size_t)shard * c->E, *M = c->t.M + (size_t)shard * c->E;
     cudaError_t e = tpq_launch_calibrate(static_cast<const uint16_t *>(y), n_seq, S, stride, c->E, m, M,
                                          c->counts[shard], c->gamma, c->scratch, n_split,

@@ -53,6 +53,7 @@ struct tpq_ctx {
     tpq_tables t;
     void *scratch;      // calibration partial extremes
     size_t scratch_bytes;
+    int64_t scratch_tokens;  // most tokens (n_seq * S) of a calibration call so far
     int64_t launches;
     void *dq_cache;     // tensor maps of recently used payloads (dequant.cu)
     const float *call_bias;  // bias of the tpq_dequant_reduce_bias call in progress (NULL otherwise)

@@ -818,3 +818,20 @@ def test_few_blocks_share_the_rows():
             times[n_seq] = min(times.get(n_seq, 1e9), e[0].elapsed_time(e[1]))
     t.close()
     assert times[1] < 2.0 * times[8], times
+
+
+def test_a_smaller_call_needs_no_more_scratch():
+    """After a call with 8 sequences, calls with fewer of them (and shorter ones) allocate nothing: they can be captured."""
+    E, S = 4608, 2048
+    y = torch.randn((8 * S, E), device="cuda").to(torch.bfloat16)
+    t = binding.Tpq(1, E)
+    t.calibrate_ranges(0, y.data_ptr(), 8, S)
+    torch.cuda.synchronize()
+    for n_seq, rows in [(n, S) for n in range(1, 9)] + [(8, 100), (5, 1000), (3, 2000)]:
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            t.calibrate_ranges(0, y.data_ptr(), n_seq, rows, stream=torch.cuda.current_stream().cuda_stream)
+        g.replay()
+        torch.cuda.synchronize()
+    assert t.device_status() == 0
+    t.close()
