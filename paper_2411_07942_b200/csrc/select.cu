@@ -60,57 +60,47 @@ __global__ void __launch_bounds__(32 * TK_WARPS) topk_flags_kernel(const float *
     if (lane == 0) flag[j] = beats < k ? 1 : 0;
 }
 
-// One block: exclusive scan of the flags -> selected list, hole / filler lists.  A thread scans an even share of
-// adjacent features, so there is one block-wide scan whatever E is.
+// One block: exclusive scan of the flags -> selected list, hole / filler lists.  A warp takes an even share of adjacent
+// features, 32 at a time (its lanes' loads and stores are adjacent), first to count, then to place; one block-wide scan
+// of the warps' counts lies between, whatever E is.
 __global__ void __launch_bounds__(1024) scan_kernel(tpq_tables t, int E, int k)
 {
-    __shared__ int warp_sums[32];
-    __shared__ int s_below;  // selected features below L
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    __shared__ int2 warp_sums[32];  // a warp's selected features, those of them below L
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int L = E - k;
-    const int per = (E + 1023) / 1024, j0 = tid * per < E ? tid * per : E, j1 = j0 + per < E ? j0 + per : E;
-    int mine = 0;
-    for (int j = j0; j < j1; ++j) mine += t.flag[j];
-    int incl = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += o;
-    }
-    if (lane == 31) warp_sums[wid] = incl;
-    if (tid == 0) s_below = k;  // (L == E: every selected feature -- there is none -- is below L)
-    __syncthreads();
-    if (wid == 0) {
-        const int w = warp_sums[lane];
-        int wi = w;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int o = __shfl_up_sync(0xffffffffu, wi, d);
-            if (lane >= d) wi += o;
-        }
-        warp_sums[lane] = wi - w;  // exclusive
-    }
-    __syncthreads();
-    const int start = warp_sums[wid] + incl - mine;  // selected features before j0
-    int before = start;
-    for (int j = j0; j < j1; ++j) {
+    const int per = ((E + 31) / 32 + 31) / 32 * 32;  // features of a warp
+    const int j0 = wid * per < E ? wid * per : E, j1 = j0 + per < E ? j0 + per : E;
+    int all = 0, below = 0;
+#pragma unroll 4
+    for (int j = j0 + lane; j < j1; j += 32) {
         const int f = t.flag[j];
-        t.hpre[j] = before;
-        if (j == L) s_below = before;
-        if (f) {
-            t.hp_idx[before] = j;
-            if (j < L) t.hole[before] = j;
-        }
-        before += f;
+        all += f;
+        below += j < L ? f : 0;
     }
+    all = __reduce_add_sync(0xffffffffu, all);
+    below = __reduce_add_sync(0xffffffffu, below);
+    if (lane == 0) warp_sums[wid] = make_int2(all, below);
     __syncthreads();
-    // holes: selected features below L; fillers: unselected features at or above L (equally many)
-    const int m = s_below;
-    before = start;
-    for (int j = j0; j < j1; ++j) {
-        const int f = t.flag[j];
-        if (!f && j >= L) t.filler[(j - L) - (before - m)] = j;
-        before += f;
+    const int2 w = warp_sums[lane];
+    const int m = __reduce_add_sync(0xffffffffu, w.y);                       // selected features below L
+    int run = __reduce_add_sync(0xffffffffu, lane < wid ? w.x : 0);          // selected features before the warp's next 32
+#pragma unroll 4
+    for (int base = j0; base < j1; base += 32) {
+        const int j = base + lane;
+        const int f = j < j1 ? t.flag[j] : 0;
+        const uint32_t set = __ballot_sync(0xffffffffu, f != 0);
+        const int before = run + __popc(set & ((1u << lane) - 1u));
+        run += __popc(set);
+        if (j < j1) {
+            t.hpre[j] = before;
+            // holes: selected features below L; fillers: unselected features at or above L (equally many)
+            if (f) {
+                t.hp_idx[before] = j;
+                if (j < L) t.hole[before] = j;
+            } else if (j >= L) {
+                t.filler[(j - L) - (before - m)] = j;
+            }
+        }
     }
 }
 

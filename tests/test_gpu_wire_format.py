@@ -145,3 +145,22 @@ def test_library_payload_is_decoded_by_hand(E, selected, T):
     hp = b[lp_bytes:].view(np.uint16).reshape(T, k)
     assert np.array_equal(hp, yb[:, selected])
     t.close()
+
+
+@pytest.mark.parametrize("E,k", [(31, 5), (33, 33), (1024, 0), (1025, 300), (5001, 51), (40000, 1), (131072 + 17, 2048), (1 << 20, 1 << 19)])
+def test_tables_of_any_number_of_features(E, k):
+    """The selected list and the slot order for feature counts around the scan's shares of 32 warps x 32 lanes: random sets
+    with a run at either end."""
+    rng = np.random.default_rng(E + k)
+    t = binding.Tpq(1, E)
+    t.set_ranges(np.full((1, E), -1.0, np.float32), np.full((1, E), 1.0, np.float32), [1])
+    picked = rng.permutation(E)[:k]
+    for hp in (np.sort(picked), np.arange(k), np.arange(E - k, E)):
+        t.set_features(hp)
+        assert np.array_equal(t.get_features(), hp)
+        L, flag = E - k, np.zeros(E, bool)
+        flag[hp] = True
+        want = np.arange(L)
+        want[flag[:L]] = L + np.nonzero(~flag[L:])[0]
+        assert np.array_equal(t.get_slot_order(), want)
+    t.close()
