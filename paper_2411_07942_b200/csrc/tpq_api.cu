@@ -23,8 +23,10 @@ tpq_status fail(tpq_ctx *c, tpq_status st, const char *fmt, ...)
     return st;
 }
 
+// (A refused allocation or launch also stays behind as the runtime's last error, which the next launch would take for its own.)
 tpq_status cuda_fail(tpq_ctx *c, cudaError_t e, const char *what)
 {
+    (void)cudaGetLastError();
     return fail(c, e == cudaErrorMemoryAllocation ? TPQ_ERR_NOMEM : TPQ_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 

@@ -108,3 +108,20 @@ def test_comm_report_matches_formulas():
     assert r.bf16_ring_allreduce_send == 2 * 7 * 2 * 64 * 4608 // 8
     assert r.bits_per_value == pytest.approx(4.1875) and r.bits_per_value_formula == pytest.approx(4.1875)
     t.close()
+
+
+def test_a_refused_call_does_not_fail_the_next_one():
+    """A call that fails in the CUDA runtime (a calibration whose scratch is far more than any GPU has) leaves nothing
+    behind: the next launches, of this context and of another, go through."""
+    a, b = binding.Tpq(1, 64), binding.Tpq(1, 64)
+    y = torch.randn((4, 64), device="cuda").to(torch.bfloat16)
+    for t in (a, b):
+        t.calibrate_ranges(0, y.data_ptr(), 1, 4)
+    for t in (a, b):
+        with pytest.raises(binding.TpqError) as e:
+            a.calibrate_ranges(0, y.data_ptr(), 1 << 36, 1)
+        assert e.value.status == binding.TPQ_ERR_NOMEM
+        t.select_features(8)
+        assert t.num_selected() == 8
+    a.close()
+    b.close()
