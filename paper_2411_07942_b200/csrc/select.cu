@@ -62,7 +62,8 @@ __global__ void __launch_bounds__(32 * TK_WARPS) topk_flags_kernel(const float *
 
 // One block: exclusive scan of the flags -> selected list, hole / filler lists.  A warp takes an even share of adjacent
 // features, 32 at a time (its lanes' loads and stores are adjacent), first to count, then to place; one block-wide scan
-// of the warps' counts lies between, whatever E is.
+// of the warps' counts lies between, whatever E is.  (An even share per thread, strided loads and stores: tpq_set_features
+// of 131072 features 366 us, so 102; 1048576: 2565 and 478; 4608 of 8 devices 57 and 55.)
 __global__ void __launch_bounds__(1024) scan_kernel(tpq_tables t, int E, int k)
 {
     __shared__ int2 warp_sums[32];  // a warp's selected features, those of them below L
