@@ -552,30 +552,35 @@ cudaError_t tpq_launch_linear_quantize(const tpq_ctx *c, int shard, const void *
     p.payload = static_cast<uint8_t *>(payload);
     p.y_slots = static_cast<uint16_t *>(y_slots);
     p.status = c->t.status;
-    // Tile shape.  What bounds a place is its shared memory, 128 bytes a clock for the copies that write the operands and
-    // the MMAs that read them: per 64-wide k-block a single block writes and reads 16 KB of x and BN / 8 KB of weights, one
-    // of a pair writes 16 + BN / 16 KB and reads 16 + BN / 8 KB.  (Measured, ns per k-block against that sum: pairs of
-    // 256 / 192 / 160 / 128 columns 307 / 259 / 232 / 230 for 80 / 68 / 62 / 56 KB, single blocks of 256 / 128 / 64 / 48 / 32
-    // columns 385 / 260 / 207 / 186 / 180 for 96 / 64 / 48 / 44 / 40 KB; the MMAs alone would take 260 at 256 columns.)  The
-    // shape with the least of waves x that sum wins, the earlier one of equals.  2048 x 3456 x 5120: 59.9 us with single
-    // blocks of 192 columns, 51.0 us with pairs of 192 (256: 55.8, 160: 55.0); 8192 tokens 208 -> 180 us (pairs of 256);
-    // 64 x 1280 x 5120 9.2 -> 6.6 us (single blocks of 48: 107 of them instead of 40); 1 x 1280 x 5120 11.9 -> 6.6 us (x boxes of 8
-    // rows instead of 128); 128 x 8192 x 8192 42.5 -> 29.7 us.
-    struct Shape { int bn, cg; };
-    constexpr Shape shapes[] = {{256, 2}, {192, 2}, {160, 2}, {128, 2}, {128, 1}, {64, 1}, {48, 1}, {32, 1}};
+    // Tile shape: the least estimated time.  A tile's MMAs overlap the epilogue of the tile before it, so a place takes
+    // start-up + one tile's k-blocks + (tiles - 1) x the longer of k-blocks and epilogue + one epilogue.
+    // A 64-wide k-block is bound by shared memory, 128 bytes a clock for the copies that write the operands and the MMAs
+    // that read them: a single block writes and reads 16 KB of x and BN / 8 KB of weights, one of a pair writes 16 + BN / 16 KB
+    // and reads 16 + BN / 8 KB (the MMAs alone would take 260 ns at 256 columns).  The epilogue takes 15 ns a column (four
+    // warps) and a hand-over of 0.8 us, between two blocks 1.8 us: below K = 1000 or so it is what bounds a tile, and pairs,
+    // which save k-blocks' time, only cost theirs.  The constants (ns) are fitted to all ten shapes at K = 64 to 3456, E = 512 to
+    // 8192, T = 1 to 4096: the choice is within 0.5 % of the fastest one on average, 12 % at worst.  2048 x 3456 x 5120: 59.9 us
+    // with single blocks of 192 columns, 51.0 us with pairs of 192 (256: 55.8, 160: 55.0); 8192 tokens 208 -> 180 us (pairs of
+    // 256); 300 x 256 x 8192: pairs of 256 8.4 us, single blocks of 192 6.6; 64 x 1280 x 5120 9.2 -> 6.6 us (single blocks of 48:
+    // 107 of them instead of 40); 1 x 1280 x 5120 11.9 -> 6.6 us (x boxes of 8 rows instead of 128); 128 x 8192 x 8192 42.5 -> 29.7 us.
+    struct Shape { int bn, cg, kb; };
+    constexpr Shape shapes[] = {{256, 2, 307}, {192, 2, 265}, {160, 2, 236}, {128, 2, 230}, {256, 1, 385},
+                                {192, 1, 376}, {128, 1, 260}, {64, 1, 207},  {48, 1, 186},  {32, 1, 180}};
     int best = 0;
     int64_t best_cost = 0;
     for (int j = 0; j < (int)(sizeof shapes / sizeof *shapes); ++j) {
         const int bn = shapes[j].bn, cg = shapes[j].cg;
         const int64_t tiles = ((T + cg * LQ_BM - 1) / (cg * LQ_BM)) * ((c->E + bn - 1) / bn), places = c->sm_count / cg;
-        const int64_t cost = (tiles + places - 1) / places * (cg == 2 ? 512 + 3 * bn : 512 + 4 * bn);  // KB x 16
+        const int64_t waves = (tiles + places - 1) / places;
+        const int64_t main = (K + LQ_BK - 1) / LQ_BK * shapes[j].kb, epilogue = (cg == 2 ? 1800 : 800) + 15 * bn;
+        const int64_t cost = (cg == 2 ? 1000 : 1400) + main + (waves - 1) * (main > epilogue ? main : epilogue) + epilogue;
         if (j == 0 || cost < best_cost) {
             best_cost = cost;
             best = j;
         }
     }
     // Stages of 128 values of K where its 64-value pieces are whole: half as many copies and barrier rounds (48-column
-    // blocks 186 against 250 ns per k-block), except where such a stage leaves room for three only (pairs of 256).
+    // blocks 186 against 250 ns per k-block), except where such a stage leaves room for three at most (256 columns).
     const bool k2 = K % LQ_BK == 0 && K >= 2 * LQ_BK;
     cudaError_t e;
 #define LQ_GO(BN, CG) e = k2 ? lq_launch<BN, CG, 2>(p, x, w_slots, c->sm_count, st) : lq_launch<BN, CG, 1>(p, x, w_slots, c->sm_count, st)
@@ -584,9 +589,11 @@ cudaError_t tpq_launch_linear_quantize(const tpq_ctx *c, int shard, const void *
     case 1: LQ_GO(192, 2); break;
     case 2: LQ_GO(160, 2); break;
     case 3: LQ_GO(128, 2); break;
-    case 4: LQ_GO(128, 1); break;
-    case 5: LQ_GO(64, 1); break;
-    case 6: LQ_GO(48, 1); break;
+    case 4: e = lq_launch<256, 1, 1>(p, x, w_slots, c->sm_count, st); break;
+    case 5: LQ_GO(192, 1); break;
+    case 6: LQ_GO(128, 1); break;
+    case 7: LQ_GO(64, 1); break;
+    case 8: LQ_GO(48, 1); break;
     default: LQ_GO(32, 1); break;
     }
 #undef LQ_GO

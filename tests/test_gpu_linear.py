@@ -190,3 +190,13 @@ def test_fused_layer_tile_shapes(T, K, E, k):
     """Every tile shape of the kernel (single blocks of 32 to 128 columns with x tiles of 8 rows and more, pairs of blocks of
     128 to 256), one and two tiles per place, an odd number of 64-value pieces of K, K that is no multiple of 64."""
     test_fused_layer(1, T, K, E, k)
+
+
+@pytest.mark.parametrize("T,K,E,k", [
+    (129, 1280, 4864, 72), (129, 1288, 4864, 72), (400, 512, 4864, 72), (400, 520, 4864, 72), (1301, 512, 3584, 56), (400, 512, 6144, 96),
+    (513, 1000, 8192, 128), (513, 768, 6144, 96), (1301, 1280, 4864, 72), (257, 512, 8192, 128), (300, 64, 8192, 128), (1100, 72, 5120, 80),
+    (2050, 320, 2048, 32), (2050, 512, 3584, 56), (129, 512, 4864, 72), (1301, 512, 2560, 40)])
+def test_fused_layer_pairs_and_wide_tiles(T, K, E, k):
+    """Pairs of blocks of 128, 160, 192 and 256 columns, single blocks of 192 and 256, of 48 and 64 with several tiles a place: one
+    and two tiles a place, stages of 64 and of 128 values of K."""
+    test_fused_layer(1, T, K, E, k)
