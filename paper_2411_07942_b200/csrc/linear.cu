@@ -561,7 +561,7 @@ cudaError_t tpq_launch_linear_quantize(const tpq_ctx *c, int shard, const void *
     // which save k-blocks' time, only cost theirs.  The constants (ns) are fitted to all ten shapes at K = 64 to 3456, E = 512 to
     // 8192, T = 1 to 4096: the choice is within 0.5 % of the fastest one on average, 12 % at worst.  2048 x 3456 x 5120: 59.9 us
     // with single blocks of 192 columns, 51.0 us with pairs of 192 (256: 55.8, 160: 55.0); 8192 tokens 208 -> 180 us (pairs of
-    // 256); 300 x 256 x 8192: pairs of 256 8.4 us, single blocks of 192 6.6; 64 x 1280 x 5120 9.2 -> 6.6 us (single blocks of 48:
+    // 256); 300 x 256 x 8192: pairs of 256 8.4 us, single blocks of 192 6.5; 64 x 1280 x 5120 9.2 -> 6.6 us (single blocks of 48:
     // 107 of them instead of 40); 1 x 1280 x 5120 11.9 -> 6.6 us (x boxes of 8 rows instead of 128); 128 x 8192 x 8192 42.5 -> 29.7 us.
     struct Shape { int bn, cg, kb; };
     constexpr Shape shapes[] = {{256, 2, 307}, {192, 2, 265}, {160, 2, 236}, {128, 2, 230}, {256, 1, 385},

@@ -184,6 +184,63 @@ def test_reduction_with_its_own_wait_on_every_kernel(N, T, E, k, bits):
     t.close()
 
 
+@pytest.mark.parametrize("N,T,E,k,bits,path", [(2, 300, 1024, 51, 4, binding.PATH_AUTO), (4, 9, 512, 8, 8, binding.PATH_TILED),
+                                              (6, 1100, 253, 9, 4, binding.PATH_AUTO), (8, 33, 520, 8, 3, binding.PATH_TILED),
+                                              (3, 5, 16, 8, 2, binding.PATH_TILED)])
+def test_bit_stream_reductions_with_their_own_wait(N, T, E, k, bits, path):
+    """tpq_dequant_reduce_arrivals on the row kernel (the first two), the panel kernel and the group kernel: the words set,
+    and one of them missing (every block gives up after its limit); the next call runs normally."""
+    orc = oracle.c()
+    t, hp, ys = _ctx(N, T, E, k, bits)
+    s_, inv = t.get_scales()
+    host = [orc.quantize_pack(ys[i], hp, inv[i], bits) for i in range(N)]
+    pls = [torch.from_numpy(h).cuda() for h in host]
+    ptrs = [b.data_ptr() for b in pls]
+    bias = np.random.default_rng(E).normal(0, 1, E).astype(np.float32)
+    bias_d = torch.from_numpy(bias).cuda()
+    _, chain = orc.dequant_reduce(host, T, E, hp, s_, bits=bits, bias=bias)
+    t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+    words = torch.zeros(N, dtype=torch.int32, device="cuda")
+    out = torch.empty((T, E), dtype=torch.float32, device="cuda")
+    for missing in (None, 0, N - 1, None):
+        words.fill_(77)
+        if missing is not None:
+            words[missing] = 76
+        out.fill_(float("nan"))
+        t.dequant_reduce(ptrs, T, out.data_ptr(), binding.TPQ_OUT_FP32, bias_ptr=bias_d.data_ptr(), arrived_ptr=words.data_ptr(),
+                         epoch=77, timeout_ns=100_000_000 if missing is None else 3_000_000)
+        torch.cuda.synchronize()
+        assert t.device_status() == (0 if missing is None else binding.TPQ_ERR_TIMEOUT), missing
+        if missing is None:
+            assert gu.bits_equal(out.cpu().numpy(), chain)
+    t.close()
+
+
+@pytest.mark.parametrize("T,E,k,bits,pad,n_dst", [(1301, 1000, 15, 4, 0, 2), (700, 5120, 51, 4, 64, 1), (601, 8192, 128, 8, 0, 3),
+                                                  (40, 8192, 100, 5, 8, 16), (3, 512, 9, 7, 0, 4), (900, 2048, 32, 2, 0, 16)])
+def test_push_of_the_bit_stream_quantiser(T, E, k, bits, pad, n_dst):
+    """Several stages a block, runs that start inside a word, one and two groups a lane, strided rows, words by shuffle (4
+    bits) and by bit string, up to the most destinations: every payload and word, three launches back to back."""
+    orc = oracle.c()
+    t, hp, ys = _ctx(1, T, E, k, bits)
+    _, inv = t.get_scales()
+    P = t.payload_bytes(T)
+    want = torch.from_numpy(orc.quantize_pack(ys[0], hp, inv[0], bits)).cuda()
+    wide = np.full((T, E + pad), 0x7FC0, np.uint16)
+    wide[:, :E] = ys[0]
+    y = gu.dev_bf16(wide)
+    bufs = [gu.guarded(P) for _ in range(n_dst)]
+    f, f0 = _words(n_dst)
+    for epoch in (1, 2, 3):
+        t.quantize_pack_push(0, y.data_ptr(), T, [v.data_ptr() for _, v in bufs], [f.data_ptr() + 4 * (f0 + d) for d in range(n_dst)],
+                             P, epoch, row_stride=E + pad)
+    torch.cuda.synchronize()
+    assert t.device_status() == 0 and bool((f[f0: f0 + n_dst] == 3).all())
+    for whole, v in bufs:
+        assert gu.guards_intact(whole, P) and torch.equal(v, want)
+    t.close()
+
+
 def test_push_argument_checks():
     t, hp, ys = _ctx(2, 19, 512, 8)
     P = t.payload_bytes(19)

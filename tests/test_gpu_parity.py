@@ -72,10 +72,10 @@ def test_other_code_widths(bits, N, T, E, k):
 
 
 @pytest.mark.parametrize("bits", [2, 3, 5, 6, 7, 8])
-def test_other_code_widths_group_kernels_equal_generic(bits):
-    """The group kernels (shapes that are multiples of 8) against the oracle and, bit for bit, against the
-    shape-generic kernels: strided input, clustered feature sets (several holes in a group, whole groups,
-    selected features at the end)."""
+def test_other_code_widths_forced_path_equals_generic(bits):
+    """The kernels that path 2 runs at other widths (bit-stream quantiser and row kernel at this shape) against the
+    oracle and, bit for bit, against the shape-generic kernels: strided input, clustered feature sets (several holes
+    in a group, whole groups, selected features at the end)."""
     N, T, E = 3, 37, 512
     w = _workload(N, T, E, 90 + bits, calib=(2, 8))
     scale = synth.column_scales(w)

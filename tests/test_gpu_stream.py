@@ -1,14 +1,17 @@
 """The bit-stream kernels (code widths other than 4 bits; feature counts, strides and selected counts that are
-multiples of nothing) against the shape-generic kernels, which the parity tests pin to the oracle: payload bytes
-and FP32 / BF16 sums bit for bit.  The shapes sit where the layout can go wrong: rows of 32 bits and a little
-more, a last group of 1 to 7 slots, tiles of 8 rows and one row less or more, a tile that ends inside a word,
-panels of 128 and 32 groups with one group more, rows that a block takes in several rounds, one and two buffers."""
+multiples of nothing) and the group kernels against the shape-generic kernels, which the parity tests pin to the oracle:
+payload bytes and FP32 / BF16 sums bit for bit.  The shapes sit where the layout can go wrong: rows of 32 bits and a
+little more, a last group of 1 to 7 slots, stages of 4 rows and tiles of 8 with one row less or more, a run of rows that
+starts inside a word, panels of 64 groups with one group more, the row kernel's last shape (640 groups, 384 selected
+features) and the panel kernel's first, one and two groups a lane.  Some of the smaller shapes are the group kernels' or
+the shape-generic quantiser's by size."""
 import numpy as np
 import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
 
+import oracle  # noqa: E402
 from paper_2411_07942_b200 import binding, synth  # noqa: E402
 
 import gpu_util as gu  # noqa: E402
@@ -171,3 +174,49 @@ def test_forced_path_runs_no_generic_kernel(N, T, E, k, bits, quantiser, reducer
         got.append([*pls, out])
     assert all(torch.equal(a, b) for a, b in zip(*got))
     t.close()
+
+
+@pytest.mark.parametrize("N,T,E,k,bits,pad,with_bias", [
+    (2, 40, 5128, 8, 3, 0, True), (2, 40, 5128, 7, 4, 0, True), (3, 9, 2048, 384, 8, 0, False), (3, 9, 2048, 385, 4, 8, False),
+    (6, 40, 1040, 8, 5, 0, True), (7, 41, 1033, 8, 4, 0, False), (5, 80, 8712, 136, 2, 0, False)])
+def test_stream_kernels_at_the_limits_of_a_kernel(N, T, E, k, bits, pad, with_bias):
+    """640 and 641 groups, 384 and 385 selected features (row kernel, panel kernel), two panels of 64 groups and one group
+    more, whole and of one slot; the ring's last shapes of two groups a lane."""
+    test_stream_kernels_equal_generic(N, T, E, k, bits, pad, with_bias)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 5, 6, 7, 8])
+def test_every_pattern_at_every_width(bits):
+    """All BF16 patterns (steps of 1 and 0.37: exact ties, values far past the clamps, infinities) through the pipelined
+    quantiser (rows of 256 and of 264 features with 9 selected, which the other kernels cannot take at 4 bits), bit-exact
+    against the oracle; and with the NaN patterns as the shape-generic kernel has them."""
+    orc = oracle.c()
+    allp = np.arange(65536, dtype=np.uint32).astype(np.uint16)
+    nan = ((allp & 0x7F80) == 0x7F80) & ((allp & 0x007F) != 0)
+    for E, hp in ((256, []), (264, list(range(100, 109)))) if bits != 4 else ((264, list(range(100, 109))),):
+        T = 65536 // E + 1
+        steps = np.array([1.0, 0.37], np.float32)
+        t = binding.Tpq(2, E, bits=bits)
+        M = np.repeat((steps * np.float32((2 ** bits - 1) / 2))[:, None], E, axis=1)
+        t.set_ranges(-M, M, np.ones(2, np.int64))
+        t.set_features(hp)
+        _, inv = t.get_scales()
+        P = t.payload_bytes(T)
+        for with_nan in (False, True):
+            y = np.resize(allp if with_nan else allp[~nan], (T, E))
+            d = gu.dev_bf16(y)
+            for i in range(2):
+                got = []
+                for path in (binding.PATH_GENERIC, binding.PATH_AUTO):
+                    t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+                    whole, view = gu.guarded(P)
+                    t.quantize_pack(i, d.data_ptr(), T, view.data_ptr(), P)
+                    torch.cuda.synchronize()
+                    assert gu.guards_intact(whole, P)
+                    got.append(view.cpu().numpy())
+                assert np.array_equal(*got), (E, i)
+                if not with_nan:
+                    assert np.array_equal(got[1], orc.quantize_pack(y, np.asarray(hp, np.int32), inv[i], bits)), (E, i)
+        t.set_option(binding.TPQ_OPT_KERNEL_PATH, binding.PATH_AUTO)
+        assert "quantize_stream<" in _kernels(lambda: t.quantize_pack(0, d.data_ptr(), T, view.data_ptr(), P))
+        t.close()
