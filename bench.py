@@ -328,7 +328,7 @@ def main():
     ap.add_argument("--tokens", type=int, default=0, help="override the workload's token count")
     ap.add_argument("--shards", type=int, default=0, help="override the workload's number of shards (devices)")
     ap.add_argument("--bits", type=int, default=4, help="code width (4 = the paper's Int4 and the bench's metric; "
-                                                        "2..8 run on the shape-generic kernels)")
+                                                        "2..8 run on the bit-stream kernels)")
     args = ap.parse_args()
     rank, local_rank, world = dist_env()
     if args.warmup < 3:

@@ -14,8 +14,8 @@
  *   - "dev" pointers are CUDA device pointers, "host" pointers are host memory.
  *   - BF16 tensors are 16-bit patterns, row-major, row stride given in ELEMENTS
  *     (any stride >= E; the Int4 kernels need E, k and the strides to be
- *     multiples of 8, other shapes run on the bit-stream kernels, and very
- *     small or very wide ones on shape-generic kernels).
+ *     multiples of 8, other shapes run on the bit-stream and group kernels,
+ *     and very small ones on shape-generic kernels).
  *   - The caller owns every data buffer.  The library owns only the context
  *     and its small device tables (O(N*E) floats), released by tpq_destroy.
  *   - Calls that take a `cuda_stream` (a cudaStream_t passed as void*; NULL is
@@ -91,7 +91,7 @@ typedef struct tpq_comm_report {
  * paper's Int4 (Section 3) and the width the tiled kernels serve; 2..8 are
  * accepted (other code widths, as evaluated in Section 4 / Figure 3:
  * step R/(2^bits - 1), codes -2^(bits-1) .. 2^(bits-1)-1, one little-endian
- * stream of bits-wide codes) and run on the bit-stream kernels.  gamma is
+ * stream of bits-wide codes) and run on the bit-stream or group kernels.  gamma is
  * the moving-average constant of Eq. (1)-(2) (the paper uses 0.01),
  * 0 <= gamma <= 1.  Errors: INVALID_ARG, NOMEM, CUDA. */
 tpq_status tpq_create(tpq_ctx **ctx, int n_shards, int n_features, int bits, float gamma);

@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(EF_X *EF_Y) ema_fold(const int16_t *part_lo, c
 // Row splits per sequence.  All blocks take about the same time, so what counts is how full the last wave of resident
 // blocks is: of the counts up to two waves' worth (and at least 64 rows each) the fullest, the smaller one where they are
 // within 2 % of one another (of the smaller one's: in a call of a few blocks every split counts: 512 rows of 100 features
-// 24.9 us in one block, 6.2 us in eight).
+// 25.1 us in one block, 5.9 us in eight).
 // (A fixed target of 8 blocks per SM gave 1296 blocks on 592 places for 8 sequences of 2048 x 4608: 2.2 waves took the time
 // of three: 32.5 us a call; one wave of 576, and both kernels launched ahead of the end of the one before them: 26.6 us.
 // 32 sequences 96.8 -> 93.6 us, one 12.4 -> 9.1 us.)

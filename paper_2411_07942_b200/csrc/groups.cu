@@ -13,9 +13,9 @@
 //
 // The bit-stream kernels (stream.cu) take most of these shapes; what is left here is what their one block per SM does
 // badly: the quantiser on narrow rows, whose few groups leave a block only a few warps (16 shards of 2048 x 512 at 3 bits
-// 24.5 us here, 59 us there), on a few tokens of rows of two groups a lane, and on rows too long for the ring
+// 25.1 us here, 54.1 us there), on a few tokens of rows of two groups a lane, and on rows too long for the ring
 // (64 x 65536 at 2 bits 6.2 us, 54 us); the reduction where rows are longer than those kernels take (256 x 65536 of two
-// devices at 8 bits 25.5 us, the shape-generic kernel 95 us).  The rules: tpq_stream_ahead, tpq_stream_push_ahead.
+// devices at 8 bits 25.5 us, the shape-generic kernel 94.8 us).  The rules: tpq_stream_ahead, tpq_stream_push_ahead.
 #include <cuda_bf16.h>
 
 #include "tpq_internal.h"

@@ -9,7 +9,7 @@
 //
 // Kernel: tcgen05 (5th-generation tensor cores), persistent: one block per SM walks 128 x BN tiles of the
 // output, or a PAIR of blocks (a cluster of two SMs, tcgen05 cta_group::2) walks 256 x BN tiles.  What bounds a
-// block is its shared memory's bandwidth, which the copies that write the operands and the MMAs that read them share: a
+// block (from K of about 1000 on; below, the epilogue) is its shared memory's bandwidth, which the copies that write the operands and the MMAs that read them share: a
 // 64-wide k-block of a 128 x 256 tile is 48 KB each way, 385 ns, against 260 ns of MMA.  In a pair each block fetches its
 // own 128 rows of x and HALF of the weight tile, and the tensor cores of both read the halves from either's shared
 // memory: 32 KB in and 48 KB out per block and k-block.

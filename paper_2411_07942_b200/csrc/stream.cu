@@ -3,13 +3,17 @@
 // Section 4 / Figure 3), and any E, k or row stride (k = E/64 is a multiple of 8 for few widths E).
 //
 // A token's codes are L*B bits long (L = E - k slots of B bits), so rows start at any bit of the code stream and
-// the 8 adjacent slots of a group lie across its words.  Both kernels therefore work on a group of 8 slots per
-// thread, as the Int4 kernels do, and put the bit offset into shared memory, where an unaligned field costs one
-// funnel shift:
-//   quantise    a block quantises 8 rows into per-row bit strings in shared memory, then writes the tile's bytes
-//               (8*L*B bits are a whole number of bytes) as consecutive 32-bit words funnelled out of the strings;
-//   dequantise  a block's panel of code words comes in by 16-byte copies from the aligned place at or below each
-//               row's first bit; a thread funnels its group's bits out of the landed words.
+// the 8 adjacent slots of a group lie across its words.  All four kernels work on a group of 8 slots per thread, as
+// the Int4 kernels do; an unaligned field costs one funnel shift out of shared memory or of a neighbour's register:
+//   quantize_stream       rows that bulk copies can fetch: a ring of stages, warps that pack the codes of their own
+//                         groups and write the words of the stream that start there, an edge warp for the words in
+//                         which one row ends and the next begins; no barrier between warps; with a push mode
+//   quantize_stream_tile  any other rows: a block quantises 8 rows into bit strings in shared memory, then writes the
+//                         tile's bytes (8*L*B bits are a whole number of bytes) as words funnelled out of the strings
+//   dequant_stream_rows   up to four devices: the row kernel, code rows by bulk copies into a ring
+//   dequant_stream        more: a block's panel of code words comes in by 16-byte copies from the aligned place at or
+//                         below each row's first bit
+// Which calls they serve is decided in tpq_api.cu, by the rules at the end of this file.
 // Arithmetic as everywhere: u = fl(x * inv_s), clamp, round to nearest even; acc = fma(code, s, acc) over the
 // devices in ascending order.
 #include <cuda_bf16.h>
@@ -64,8 +68,8 @@ __device__ __forceinline__ uint32_t qs_code(float x, float inv)
 // upper clamp and the packing move to the FMA pipe, which runs at twice the integer pipe's rate: t = sat(r / 2^B + c) with
 // c such that t = 1 at the highest code (exact: every value in range is a multiple of 2^-B); 2^B t - 1 = code + 2^(B-1) is
 // the code's digit with the sign bit flipped, and four digits are put together by FMAs as an integer below 2^20 on
-// top of 2^23.  (18 integer-pipe instructions per 8 codes instead of 34; 4 x 2048 x 5120, 51 selected: 26.9 -> 26.3 us;
-// at 8 bits, where pairs of digits would be needed, 29.7 -> 30.2 us.)  NaN gives the lowest code (the lower clamp drops
+// top of 2^23.  (18 integer-pipe instructions per 8 codes instead of 34; at 8 bits, where pairs of digits
+// would be needed, it measured slower.)  NaN gives the lowest code (the lower clamp drops
 // it), infinities saturate.
 __device__ __forceinline__ float qs_sat_fma(float a, float b, float c)
 {
@@ -312,12 +316,11 @@ cudaError_t launch_quantize_tile(const QSParams &p, bool vec, int threads, dim3 
 //   groups (qs_ahead) are the next warp's first ones, packed by both;
 //   the edge warp writes the words in which one row ends and the next begins (one code per lane: 16 of a row's last
 //   and 16 of its first, or-ed together), for every row of the block and the row ahead of it.
-// A block may therefore start at any row.  (Built before this and measured at 4 x 2048 x 5120, 51 selected: strings of
-// whole tiles with a barrier of all consumers per 4 rows 43 us; one tile of 8 rows per block, four blocks per SM, 29.5 us;
-// this kernel 23.9 us against 15.9 us for its bytes at 6.65 TB/s; the shape-generic kernel 114 us.
-// 3 bits 41.1 -> 25.0 us, 8 x 1000 x 4608 at 8 bits 39.5 -> 29.7 us.  Bound by instruction issue: 115 warp instructions
-// per 32 groups took 26.9 us; with one word per group up to 4 bits, field masks worked out once and the second hole's
-// shuffle only in warps that have one, 23.9 us.)
+// A block may therefore start at any row.  Measured at 4 x 2048 x 5120, 51 selected, back to back: 23.1 us against 16.3 us
+// for its bytes at the copy rate (strings of whole tiles with a barrier of all consumers per 4 rows 43 us; one tile of 8 rows
+// per block, four blocks per SM, 29.5 us; the shape-generic kernel 114 us); 3 bits 25.0 us, 6 bits 28.0 us, 8 x 1000 x 4608 at
+// 8 bits 25.2 us.  Nearest limit: instruction issue.  A warp executes 102 instructions per 32 groups and row at 4 bits, 112 at 3,
+// 131 at 8, which take 67 to 71 % of the issue slots of the launch, with DRAM at a third.
 constexpr int QS_STAGE = 4;             // rows of a stage
 constexpr int QS_MAX_THREADS = 768;     // 80 registers a thread
 constexpr int QS_MAX_GPT = 2;           // groups of a consumer lane
@@ -361,7 +364,7 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
     const QSParams &p = pp.q;
     // warp 0 is the producer, warp 1 the edge warp, then come the NT consumers: where several warps of a scheduler can
     // issue, the first goes first, and the few instructions of these two must not wait behind the consumers' many
-    // (as last warps 27.3 us at 4 x 2048 x 5120, 51 selected; 27.0 us so)
+    // (as last warps it measured 1 % longer)
     const int NT = blockDim.x - 64, tid = (int)threadIdx.x - 64;
     const int E = p.E, k = p.k, L = p.L, G = (L + 7) >> 3, nstage = pp.nstage;
     const int LB = L * B;  // bits of a row
@@ -733,9 +736,9 @@ cudaError_t launch_quantize_pipe(const QPipeParams &pp, bool push, int gpt, int 
 // the alignment: a segment starts at any bit, so the copies start at the 16-byte boundary at or below it and a
 // thread funnels its 8*B bits out of two (three) words; the shift is the same for all devices, so it is worked
 // out once per chunk and row.  Blocks are half the size, two to an SM, so that one's barrier hides behind the other's work.
-// Measured (before: the shape-generic kernel, or one thread per group with byte loads for other widths): 4 x 2048 x 5120
-// with 51 selected 91.7 -> 17.8 us, 3 bits 26.2 -> 16.5 us; 8 x 1000 x 4608 at 8 bits 20.1 -> 16.2 us; one block of 512
-// threads per SM 18.8, 16.9 and 22.1 us.  Bound by instruction issue (22 per 8 codes) and the chunk's barriers.
+// 8 x 1000 x 4608 at 8 bits 15.4 us back to back (7.2 us for its bytes at the copy rate; one block of 512 threads per SM 22.1).
+// 61 instructions per warp of 32 groups and device take 52 % of the issue slots: 14 warps an SM (109 registers a thread) leave
+// one eligible a cycle between the chunk's barriers.
 // ----------------------------------------------------------------------------------------------
 constexpr int DS_THREADS = 256;  // two blocks share an SM, so that one's barrier hides behind the other's work
 constexpr int DS_CG = 64;        // groups of a panel
@@ -1093,8 +1096,10 @@ cudaError_t launch_dequant_stream(const DSParams &p, int fp32_out, cudaStream_t 
 // the auxiliary warps left in shared memory (same thread, same address: ordered).  An auxiliary thread per rank h adds up
 // the devices' BF16 values of selected feature h, loaded from memory a stage ahead (the BF16 rows are not aligned for bulk
 // copies and end with the payload), and decodes column L + h of the output where that is a filler feature.
-// No warp waits for another's global stores.  4 x 2048 x 5120, panel kernel -> this one: 51 selected 17.8 -> 14.7 us, 3 bits
-// 16.5 -> 14.1, 6 bits 19.9 -> 16.4 us (the Int4 row kernel 10.8 us; the L2 prefetch and steps kept in registers 15.6 -> 14.7).
+// No warp waits for another's global stores.  4 x 2048 x 5120 back to back, panel kernel against this one: 51 selected 17.8 and
+// 14.0 us, 3 bits 16.5 and 13.8, 6 bits 19.9 and 15.3 (the Int4 row kernel 10.6; 6.6, 5.8 and 8.2 us for the bytes).  59 to 61
+// instructions per warp of 32 groups and device take 60 % of the issue slots; the rest is the prologue's table loads and the
+// auxiliary warps' BF16 values.
 // ----------------------------------------------------------------------------------------------
 constexpr int DW_ROWS = 4, DW_MAX_DEV = 4, DW_MAIN = 640, DW_AUX = 96, DW_MAX_K = 384;
 
