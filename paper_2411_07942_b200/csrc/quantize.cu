@@ -289,11 +289,16 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
     // Holes are patched warp-cooperatively.  The holes of a warp's 32 groups are consecutive in the
     // global hole order, so lane i quantises the filler element of the warp's i-th hole (w_off / w_inv)
     // and the owner of a hole fetches the code with a shuffle (from lane src0, src0 + 1 for a second
-    // hole).  A warp with more than 32 holes, or a lane with more than two, takes the serial path.
+    // hole).  A warp that has a lane with more holes puts the others in one after the other, in code of its own.  (Of random sets
+    // of E/64 features one in seven has such a lane at E = 5120, one in five at 8192, and a block waits for its slowest
+    // warp: 8 x 2048 x 5120 61.0 us a launch with the serial path, 35.0 with this one, 34.9 for a set that has none.  One row at
+    // a time is not enough: 58 us.)  A warp with more than 32 holes takes the serial path, which reads the tables for every
+    // hole and row.
     const int lane = tid & 31;
     uint32_t w_off[GPT];     // byte offset of "my" filler element in a staged row (lane < n_wh)
     float w_inv[GPT];
     int n_wh[GPT], src0[GPT];
+    int most[GPT];           // most holes of a lane of the warp
     bool serial[GPT];
     uint32_t keep[GPT];      // word bits that are not holes
 #pragma unroll
@@ -308,7 +313,8 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
         src0[a] = incl - nh;
         n_wh[a] = __shfl_sync(0xffffffffu, incl, 31);
         const int hb_warp = __shfl_sync(0xffffffffu, hb[a], 0);
-        serial[a] = n_wh[a] > 32 || __any_sync(0xffffffffu, nh > 2);
+        most[a] = __reduce_max_sync(0xffffffffu, nh);
+        serial[a] = n_wh[a] > 32;
         w_off[a] = 0;
         w_inv[a] = 0.0f;
         if (lane < n_wh[a] && !serial[a]) {
@@ -349,8 +355,10 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
             const bool live = g < L8;
             const int g_ld = live ? g : 0;  // idle lanes load something harmless: straight-line code below
             // GR rows from row rb of the stage on: all shared loads first, then GR independent chains, no branches
-            auto rows_fast = [&](auto gr_tag, int rb) {
+            // (DEEP: a warp that has a lane with more than two holes)
+            auto rows_fast = [&](auto gr_tag, auto deep_tag, int rb) {
                 constexpr int GR = decltype(gr_tag)::value;
+                constexpr bool DEEP = decltype(deep_tag)::value;
                 uint4 v[GR];
                 uint32_t fx[GR];
 #pragma unroll
@@ -361,13 +369,25 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
                 uint32_t word[GR];
 #pragma unroll
                 for (int r = 0; r < GR; ++r) word[r] = quant8(v[r], inv[a]);
-                if (n_wh[a]) {  // uniform over the warp
+                if (DEEP || n_wh[a]) {  // uniform over the warp
+                    uint32_t qv[GR];
 #pragma unroll
                     for (int r = 0; r < GR; ++r) {
-                        const uint32_t qv = quant_bits(fx[r], w_inv[a]) & 0xFu;
-                        const uint32_t q0 = __shfl_sync(0xffffffffu, qv, src0[a]) << f_sh[a][0];
-                        const uint32_t q1 = __shfl_sync(0xffffffffu, qv, src0[a] + 1) << f_sh[a][1];
+                        qv[r] = quant_bits(fx[r], w_inv[a]) & 0xFu;
+                        const uint32_t q0 = __shfl_sync(0xffffffffu, qv[r], src0[a]) << f_sh[a][0];
+                        const uint32_t q1 = __shfl_sync(0xffffffffu, qv[r], src0[a] + 1) << f_sh[a][1];
                         word[r] = (word[r] & keep[a]) | (q0 & hmask[a][0]) | (q1 & hmask[a][1]);
+                    }
+                    if constexpr (DEEP) {  // the third and further holes
+                        uint32_t m = mask[a] & (mask[a] - 1);
+                        m &= m - 1;
+                        for (int h = 2; h < most[a]; ++h, m &= m - 1) {
+                            const int at = m ? (__ffs(m) - 1) * 4 : 0;
+                            const uint32_t field = m ? 0xFu << at : 0u;
+#pragma unroll
+                            for (int r = 0; r < GR; ++r)
+                                word[r] = (word[r] & ~field) | (__shfl_sync(0xffffffffu, qv[r], src0[a] + h) << at & field);
+                        }
                     }
                 }
                 if (live) {
@@ -383,11 +403,16 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
                     }
                 }
             };
-            if (!serial[a]) {  // (uniform over the warp, like the row counts below)
+            auto stage_fast = [&](auto deep) {
                 int rb = 0;
-                if (G >= 4 && rows - rb >= 4) { rows_fast(std::integral_constant<int, 4>(), rb); rb += 4; }
-                if (G >= 2 && rows - rb >= 2) { rows_fast(std::integral_constant<int, 2>(), rb); rb += 2; }
-                if (rows - rb >= 1) rows_fast(std::integral_constant<int, 1>(), rb);
+                if (G >= 4 && rows - rb >= 4) { rows_fast(std::integral_constant<int, 4>(), deep, rb); rb += 4; }
+                if (G >= 2 && rows - rb >= 2) { rows_fast(std::integral_constant<int, 2>(), deep, rb); rb += 2; }
+                if (rows - rb >= 1) rows_fast(std::integral_constant<int, 1>(), deep, rb);
+            };
+            if (!serial[a] && most[a] <= 2) {  // (uniform over the warp, like the row counts above)
+                stage_fast(std::false_type());
+            } else if (!serial[a]) {
+                stage_fast(std::true_type());
             } else if (live) {
                 // a warp on the serial path: every hole patched by its owner
                 for (int r = 0; r < rows; ++r) {

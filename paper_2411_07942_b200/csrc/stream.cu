@@ -20,6 +20,8 @@
 
 #include "tpq_internal.h"
 
+#include <type_traits>
+
 namespace {
 
 __device__ __forceinline__ uint32_t lop3_and_or(uint32_t x, uint32_t mask, uint32_t magic)
@@ -511,6 +513,7 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
     uint32_t mask[GPT], w_off[GPT], f_sh[GPT][2], field[GPT][2][NW], keep[GPT][NW];
     int hb[GPT], n_wh[GPT], src0[GPT];
     float w_inv[GPT];
+    int most[GPT];  // most holes of a lane of the warp
     bool serial[GPT], two[GPT];
     const int my_hp = tid < k ? __ldg(p.hp_idx + tid) : 0;
 #pragma unroll
@@ -540,8 +543,9 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
         src0[a] = incl - nh;
         n_wh[a] = __shfl_sync(0xffffffffu, incl, 31);
         const int hb_warp = __shfl_sync(0xffffffffu, hb[a], 0);
-        serial[a] = n_wh[a] > 32 || __any_sync(0xffffffffu, nh > 2);
-        two[a] = __any_sync(0xffffffffu, nh > 1);  // some group of the warp has a second hole
+        most[a] = __reduce_max_sync(0xffffffffu, nh);
+        serial[a] = n_wh[a] > 32;
+        two[a] = most[a] > 1;  // some group of the warp has a second hole
         w_off[a] = 0;
         w_inv[a] = 0.0f;
         if (lane < n_wh[a] && !serial[a]) {
@@ -604,10 +608,13 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
                     qs_store_group<B>(reinterpret_cast<uint8_t *>(ws + r * WW) + lane * B, wd);
                 }
             };
-            if (!serial[a]) {
-                // QS_STAGE independent rows (a short stage's missing ones hold old bytes and are never written)
+            // QS_STAGE independent rows (a short stage's missing ones hold old bytes and are never written)
+            // (DEEP: a warp that has a lane with more than two holes, see quantize_tiled: 4 x 2048 x 5120 of 51 selected 36.4 us a
+            // launch on the serial path, 23.2 so; 8 x 1000 x 4608 at 8 bits 38.1 and 26.6)
+            auto rows_fast = [&](auto deep_tag) {
+                constexpr bool DEEP = decltype(deep_tag)::value;
                 uint4 v[QS_STAGE];
-                uint32_t fx[QS_STAGE];
+                uint32_t fx[QS_STAGE], wd[QS_STAGE][NW];
 #pragma unroll
                 for (int r = 0; r < QS_STAGE; ++r) {
                     v[r] = *reinterpret_cast<const uint4 *>(src + r * row_bytes);
@@ -615,21 +622,45 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
                 }
 #pragma unroll
                 for (int r = 0; r < QS_STAGE; ++r) {
-                    uint32_t wd[NW];
-                    qs_quant8<B>(v[r], inv[a], wd);
-                    if (n_wh[a]) {  // uniform over the warp, as is two
+                    qs_quant8<B>(v[r], inv[a], wd[r]);
+                    if (DEEP || n_wh[a]) {  // uniform over the warp, as is two
                         const uint32_t qv = qs_code<B>(__uint_as_float(fx[r] << 16), w_inv[a]) & ((1u << B) - 1u);
                         const uint32_t c0 = __shfl_sync(0xffffffffu, qv, src0[a]) << f_sh[a][0];
 #pragma unroll
-                        for (int j = 0; j < NW; ++j) wd[j] = (wd[j] & keep[a][j]) | (c0 & field[a][0][j]);
-                        if (two[a]) {
+                        for (int j = 0; j < NW; ++j) wd[r][j] = (wd[r][j] & keep[a][j]) | (c0 & field[a][0][j]);
+                        if (DEEP || two[a]) {
                             const uint32_t c1 = __shfl_sync(0xffffffffu, qv, src0[a] + 1) << f_sh[a][1];
 #pragma unroll
-                            for (int j = 0; j < NW; ++j) wd[j] |= c1 & field[a][1][j];
+                            for (int j = 0; j < NW; ++j) wd[r][j] |= c1 & field[a][1][j];
+                        }
+                        if (DEEP) fx[r] = qv;
+                    }
+                    if (!DEEP) emit(r, wd[r], r < rows);
+                }
+                if constexpr (DEEP) {  // the third and further holes
+                    uint32_t m = mask[a] & (mask[a] - 1);
+                    m &= m - 1;
+                    for (int h = 2; h < most[a]; ++h, m &= m - 1) {
+                        const int n = m ? __ffs(m) - 1 : 0;
+                        const uint32_t sh = qs_field_shift<B>(n);
+#pragma unroll
+                        for (int r = 0; r < QS_STAGE; ++r) {
+                            const uint32_t c = __shfl_sync(0xffffffffu, fx[r], src0[a] + h);
+#pragma unroll
+                            for (int j = 0; j < NW; ++j) {
+                                const uint32_t fm = m && qs_field_in<B>(n, j) ? ((1u << B) - 1u) << sh : 0u;
+                                wd[r][j] = (wd[r][j] & ~fm) | (c << sh & fm);
+                            }
                         }
                     }
-                    emit(r, wd, r < rows);
+#pragma unroll
+                    for (int r = 0; r < QS_STAGE; ++r) emit(r, wd[r], r < rows);
                 }
+            };
+            if (!serial[a] && most[a] <= 2) {
+                rows_fast(std::false_type());
+            } else if (!serial[a]) {
+                rows_fast(std::true_type());
             } else {
                 for (int r = 0; r < rows; ++r) {  // a warp on the serial path: every hole patched by its owner
                     uint32_t wd[NW];

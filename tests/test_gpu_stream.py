@@ -220,3 +220,33 @@ def test_every_pattern_at_every_width(bits):
         t.set_option(binding.TPQ_OPT_KERNEL_PATH, binding.PATH_AUTO)
         assert "quantize_stream<" in _kernels(lambda: t.quantize_pack(0, d.data_ptr(), T, view.data_ptr(), P))
         t.close()
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 5, 8])
+def test_groups_with_many_selected_features(bits):
+    """3 to 8 selected features in one group of 8 beside groups with fewer, and a warp with 32 and with 33 of them: payloads
+    of the pipelined quantisers (at 4 bits the one for multiples of 8 too, by the set's size) against the generic kernel."""
+    N, T, E = 2, 23, 1024
+    w = synth.Workload("holes", N, T, E, 0.7, 10, 20.0, 200.0, 1, 8, 5 + bits)
+    scale = synth.column_scales(w)
+    t = binding.Tpq(N, E, bits=bits)
+    gu.calibrate_both(t, [synth.calibration_np(w, i, scale=scale) for i in range(N)])
+    ys = [gu.dev_bf16(synth.activations_np(w, i, T, scale=scale)) for i in range(N)]
+    group = lambda g, n: [8 * g + (3 * i + g) % 8 for i in range(n)]  # n features of a group, not its first ones
+    sets = [group(0, n) + group(1, 2) + group(31, 1) + group(63, n) for n in range(3, 9)]
+    sets += [group(2, 8) + group(3, 8) + group(9, 8) + group(30, n) for n in (8, 7)] + [group(2, 8) + group(3, 8) + group(9, 8) + group(30, 8) + group(11, 1)]
+    sets += [s + group(100, -len(s) % 8) for s in sets]   # sizes that are multiples of 8 as well
+    for hp in map(sorted, sets):
+        t.set_features(hp)
+        P = t.payload_bytes(T)
+        got = []
+        for path in (binding.PATH_GENERIC, binding.PATH_AUTO):
+            t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+            pls = [torch.zeros(P, dtype=torch.uint8, device="cuda") for _ in range(N)]
+            t.quantize_pack_batch(0, [y.data_ptr() for y in ys], T, [p.data_ptr() for p in pls], P)
+            torch.cuda.synchronize()
+            assert t.device_status() == 0
+            got.append([p.cpu().numpy() for p in pls])
+        for a, b in zip(*got):
+            assert np.array_equal(a, b), hp
+    t.close()
