@@ -59,8 +59,9 @@ bool all_calibrated(const tpq_ctx *c)
     return true;
 }
 
-// ranges -> (flags already on the device) -> tables; synchronises
-tpq_status build_tables(tpq_ctx *c, int k, bool topk)
+// ranges -> (flags already on the device) -> tables; synchronises.  topk: the features are chosen here and, if hp_out
+// is given, copied there; else hp holds them.
+tpq_status build_tables(tpq_ctx *c, int k, bool topk, int32_t *hp_out, const int32_t *hp)
 {
     cudaError_t e = tpq_launch_ranges(c->t, c->N, c->E, c->bits, 0, &c->launches);
     if (e != cudaSuccess) return cuda_fail(c, e, "ranges kernel");
@@ -70,10 +71,17 @@ tpq_status build_tables(tpq_ctx *c, int k, bool topk)
     }
     e = tpq_launch_tables(c->t, c->N, c->E, k, 0, &c->launches);
     if (e != cudaSuccess) return cuda_fail(c, e, "tables kernel");
+    if (topk && hp_out && k > 0) {
+        TPQ_CUDA(c, cudaMemcpy(hp_out, c->t.hp_idx, (size_t)k * sizeof(int32_t), cudaMemcpyDeviceToHost));
+        hp = hp_out;
+    }
     TPQ_CUDA(c, cudaDeviceSynchronize());
-    c->n_holes = 0;
-    if (k > 0 && k < c->E)
-        TPQ_CUDA(c, cudaMemcpy(&c->n_holes, c->t.hpre + (c->E - k), sizeof(int), cudaMemcpyDeviceToHost));
+    int holes = 0;  // selected features below E - k (the list is ascending)
+    if (hp)
+        while (holes < k && hp[holes] < c->E - k) ++holes;
+    else if (k > 0 && k < c->E)
+        TPQ_CUDA(c, cudaMemcpy(&holes, c->t.hpre + (c->E - k), sizeof(int), cudaMemcpyDeviceToHost));
+    c->n_holes = holes;
     c->k = k;
     return TPQ_OK;
 }
@@ -187,7 +195,7 @@ tpq_status tpq_create(tpq_ctx **out, int n_shards, int n_features, int bits, flo
     if (e == cudaSuccess) e = dalloc(&t.inv_s, NE);
     if (e == cudaSuccess) e = dalloc(&t.s_k, NE);
     if (e == cudaSuccess) e = dalloc(&t.s_slot, NE);
-    if (e == cudaSuccess) e = dalloc(&t.flag, E);
+    if (e == cudaSuccess) e = dalloc(&t.flag, (E + 15) / 16 * 16);  // (the scan reads 16 at a time)
     if (e == cudaSuccess) e = dalloc(&t.hpre, E);
     if (e == cudaSuccess) e = dalloc(&t.pos, E);
     if (e == cudaSuccess) e = dalloc(&t.hp_idx, E);
@@ -313,9 +321,8 @@ tpq_status tpq_select_features(tpq_ctx *c, int k, int32_t *hp_out, int *k_out)
     if (k < 0) k = c->E / 64;  // Section 4: k = floor(E/64)
     if (k > c->E) return fail(c, TPQ_ERR_INVALID_ARG, "k = %d exceeds E = %d", k, c->E);
     if (!all_calibrated(c)) return fail(c, TPQ_ERR_BAD_STATE, "every shard needs at least one calibration sequence");
-    tpq_status st = build_tables(c, k, true);
+    tpq_status st = build_tables(c, k, true, hp_out, nullptr);
     if (st != TPQ_OK) return st;
-    if (hp_out && k > 0) TPQ_CUDA(c, cudaMemcpy(hp_out, c->t.hp_idx, (size_t)k * sizeof(int32_t), cudaMemcpyDeviceToHost));
     if (k_out) *k_out = k;
     return TPQ_OK;
 }
@@ -333,7 +340,7 @@ tpq_status tpq_set_features(tpq_ctx *c, const int32_t *hp, int k)
         flag[hp[h]] = 1;
     }
     TPQ_CUDA(c, cudaMemcpy(c->t.flag, flag.data(), flag.size(), cudaMemcpyHostToDevice));
-    return build_tables(c, k, false);
+    return build_tables(c, k, false, nullptr, hp);
 }
 
 tpq_status tpq_set_ranges(tpq_ctx *c, const float *m, const float *M, const int64_t *counts)
