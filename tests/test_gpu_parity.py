@@ -835,3 +835,36 @@ def test_a_smaller_call_needs_no_more_scratch():
         torch.cuda.synchronize()
     assert t.device_status() == 0
     t.close()
+
+
+@pytest.mark.parametrize("E", [1, 15, 17, 64, 65, 1000, 4097, 32768, 32769])
+def test_slot_order_at_the_edges_of_the_scan(E):
+    """The selector's tables against the written definition of the slot order, at the edges of the scan's words, blocks and
+    of the one-launch form's range: feature sets of no, one, some and all features, at both ends and scattered."""
+    rng = np.random.default_rng(E)
+    t = binding.Tpq(2, E)
+    M = rng.permutation(E).astype(np.float32) + 1.0
+    t.set_ranges(np.stack([-M, -M]), np.stack([M, M]), [1, 1])
+    for k in sorted({0, 1, E // 64, E // 3, E - 1, E}):
+        sets = [None, list(range(k)), list(range(E - k, E)), sorted(rng.permutation(E)[:k].tolist())]
+        for hp in sets:
+            if hp is None:
+                hp = t.select_features(k).tolist()
+                assert hp == sorted(np.argsort(-M, kind="stable")[:k].tolist())
+            else:
+                t.set_features(hp)
+            L, sel = E - k, set(hp)
+            fill = iter([j for j in range(L, E) if j not in sel])
+            assert t.get_slot_order().tolist() == [next(fill) if c in sel else c for c in range(L)]
+    t.close()
+
+
+def test_selection_takes_k_features_of_ranges_that_are_not_numbers():
+    E, k = 200, 6
+    M = np.arange(1, E + 1, dtype=np.float32)
+    M[[3, 77]], M[120] = np.nan, np.inf
+    t = binding.Tpq(1, E)
+    t.set_ranges(-M[None], M[None], [1])
+    assert t.select_features(k).tolist() == [3, 77, 120, 197, 198, 199]
+    assert sorted(t.get_slot_order().tolist()) == [j for j in range(E) if j not in (3, 77, 120, 197, 198, 199)]
+    t.close()
