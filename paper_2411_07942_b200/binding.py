@@ -76,6 +76,9 @@ SIGNATURES = {
 }
 
 _lib = None
+_calls = None   # the extension module (csrc/calls.c): the calls of a step with plain arguments; it returns None for others
+_CALLS = ("tpq_calibrate_ranges", "tpq_quantize_pack", "tpq_quantize_pack_batch", "tpq_dequant_reduce", "tpq_dequant_reduce_bias",
+          "tpq_dequant_reduce_arrivals", "tpq_quantize_pack_push", "tpq_linear_quantize_pack")   # in the order of its table
 _fast = types.SimpleNamespace()   # the calls below that take pointer arrays, as functions that take what _ptrs returns
 _FAST = ("tpq_quantize_pack_batch", "tpq_dequant_reduce", "tpq_dequant_reduce_bias", "tpq_quantize_pack_push",
          "tpq_dequant_reduce_arrivals")
@@ -83,7 +86,7 @@ _FAST = ("tpq_quantize_pack_batch", "tpq_dequant_reduce", "tpq_dequant_reduce_bi
 
 def lib() -> ctypes.CDLL:
     """Load libtpq.so (built in-tree by ``paper_2411_07942_b200.build``); raises if absent."""
-    global _lib
+    global _lib, _calls
     if _lib is None:
         if not _LIB_PATH.exists():
             raise RuntimeError(f"{_LIB_PATH} is missing: run `python -m paper_2411_07942_b200.build` "
@@ -98,6 +101,12 @@ def lib() -> ctypes.CDLL:
             fn.restype, args = SIGNATURES[name]
             fn.argtypes = [c_void_p if a is POINTER(c_void_p) else a for a in args]
             setattr(_fast, name, fn)
+        try:
+            from . import _calls as calls
+        except ImportError as e:
+            raise RuntimeError("the extension module _calls is missing: run `python -m paper_2411_07942_b200.build`") from e
+        calls.bind([ctypes.cast(getattr(L, name), c_void_p).value for name in _CALLS])
+        _calls = calls
         _lib = L
     return _lib
 
@@ -144,12 +153,14 @@ class Tpq:
         if st != TPQ_OK:
             self._h = c_void_p()
             raise TpqError(st, "tpq_create failed")
+        self._p = self._h.value   # (as a plain integer, for _calls)
         self.N, self.E, self.bits = n_shards, n_features, bits
 
     def close(self):
         if getattr(self, "_h", None) and self._h.value:
             lib().tpq_destroy(self._h)
             self._h = c_void_p()
+            self._p = None
 
     def __del__(self):
         try:
@@ -170,8 +181,12 @@ class Tpq:
 
     def calibrate_ranges(self, shard: int, y_ptr: int, n_seq: int, S: int, row_stride: int | None = None,
                          stream: int = 0):
-        self._check(lib().tpq_calibrate_ranges(self._h, shard, y_ptr, n_seq, S,
-                                               self.E if row_stride is None else row_stride, stream))
+        stride = self.E if row_stride is None else row_stride
+        st = _calls.calibrate_ranges(self._p, shard, y_ptr, n_seq, S, stride, stream)
+        if st is None:   # (arguments of another form than plain integers, here and below)
+            st = _lib.tpq_calibrate_ranges(self._h, shard, y_ptr, n_seq, S, stride, stream)
+        if st:
+            self._check(st)
 
     def calibrate_ranges_noalloc(self, shard: int, y_ptr: int, n_seq: int, S: int, row_stride: int | None = None,
                                  stream: int = 0):
@@ -240,34 +255,44 @@ class Tpq:
 
     def quantize_pack(self, shard: int, y_ptr: int, T: int, payload_ptr: int, payload_capacity: int,
                       row_stride: int | None = None, stream: int = 0):
-        st = _lib.tpq_quantize_pack(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride, payload_ptr,
-                                    payload_capacity, stream)
+        stride = self.E if row_stride is None else row_stride
+        st = _calls.quantize_pack(self._p, shard, y_ptr, T, stride, payload_ptr, payload_capacity, stream)
+        if st is None:
+            st = _lib.tpq_quantize_pack(self._h, shard, y_ptr, T, stride, payload_ptr, payload_capacity, stream)
         if st:
             self._check(st)
 
     def quantize_pack_batch(self, first_shard: int, y_ptrs, T: int, payload_ptrs, payload_capacity: int,
                             row_stride: int | None = None, stream: int = 0):
-        n = len(y_ptrs)
-        assert len(payload_ptrs) == n
-        ya = _ptrs(y_ptrs)
-        pa = _ptrs(payload_ptrs)
-        st = _fast.tpq_quantize_pack_batch(self._h, first_shard, n, ya, T, self.E if row_stride is None else row_stride, pa,
-                                          payload_capacity, stream)
+        stride = self.E if row_stride is None else row_stride
+        st = _calls.quantize_pack_batch(self._p, first_shard, y_ptrs, T, stride, payload_ptrs, payload_capacity, stream)
+        if st is None:
+            n = len(y_ptrs)
+            assert len(payload_ptrs) == n
+            st = _fast.tpq_quantize_pack_batch(self._h, first_shard, n, _ptrs(y_ptrs), T, stride, _ptrs(payload_ptrs),
+                                              payload_capacity, stream)
         if st:
             self._check(st)
 
     def dequant_reduce(self, payload_ptrs, T: int, out_ptr: int, out_dtype: int = TPQ_OUT_BF16,
                        out_row_stride: int | None = None, stream: int = 0, bias_ptr: int | None = None,
                        arrived_ptr: int | None = None, epoch: int = 0, timeout_ns: int = 0):
-        arr = _ptrs(payload_ptrs)
         stride = self.E if out_row_stride is None else out_row_stride
         if arrived_ptr is not None:
-            st = _fast.tpq_dequant_reduce_arrivals(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr,
-                                                  arrived_ptr, epoch & 0xFFFFFFFF, timeout_ns, stream)
-        elif bias_ptr is None:
-            st = _fast.tpq_dequant_reduce(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, stream)
+            epoch &= 0xFFFFFFFF
+            st = _calls.dequant_reduce_arrivals(self._p, payload_ptrs, T, out_ptr, out_dtype, stride, bias_ptr, arrived_ptr, epoch,
+                                                timeout_ns, stream)
         else:
-            st = _fast.tpq_dequant_reduce_bias(self._h, arr, len(payload_ptrs), T, out_ptr, out_dtype, stride, bias_ptr, stream)
+            st = _calls.dequant_reduce(self._p, payload_ptrs, T, out_ptr, out_dtype, stride, bias_ptr, stream)
+        if st is None:
+            arr, n = _ptrs(payload_ptrs), len(payload_ptrs)
+            if arrived_ptr is not None:
+                st = _fast.tpq_dequant_reduce_arrivals(self._h, arr, n, T, out_ptr, out_dtype, stride, bias_ptr, arrived_ptr, epoch,
+                                                      timeout_ns, stream)
+            elif bias_ptr is None:
+                st = _fast.tpq_dequant_reduce(self._h, arr, n, T, out_ptr, out_dtype, stride, stream)
+            else:
+                st = _fast.tpq_dequant_reduce_bias(self._h, arr, n, T, out_ptr, out_dtype, stride, bias_ptr, stream)
         if st:
             self._check(st)
 
@@ -276,19 +301,23 @@ class Tpq:
 
     def linear_quantize_pack(self, shard: int, x_ptr: int, w_slots_ptr: int, T: int, K: int, payload_ptr: int,
                              payload_capacity: int, y_slots_ptr: int | None = None, stream: int = 0):
-        st = _lib.tpq_linear_quantize_pack(self._h, shard, x_ptr, w_slots_ptr, T, K, payload_ptr, payload_capacity,
-                                           y_slots_ptr, stream)
+        st = _calls.linear_quantize_pack(self._p, shard, x_ptr, w_slots_ptr, T, K, payload_ptr, payload_capacity, y_slots_ptr, stream)
+        if st is None:
+            st = _lib.tpq_linear_quantize_pack(self._h, shard, x_ptr, w_slots_ptr, T, K, payload_ptr, payload_capacity,
+                                               y_slots_ptr, stream)
         if st:
             self._check(st)
 
     def quantize_pack_push(self, shard: int, y_ptr: int, T: int, dst_ptrs, arrived_ptrs, dst_capacity: int, epoch: int,
                            row_stride: int | None = None, stream: int = 0):
-        n = len(dst_ptrs)
-        assert len(arrived_ptrs) == n
-        da = _ptrs(dst_ptrs)
-        aa = _ptrs(arrived_ptrs)
-        st = _fast.tpq_quantize_pack_push(self._h, shard, y_ptr, T, self.E if row_stride is None else row_stride, da, aa, n,
-                                         dst_capacity, epoch & 0xFFFFFFFF, stream)
+        stride = self.E if row_stride is None else row_stride
+        epoch &= 0xFFFFFFFF
+        st = _calls.quantize_pack_push(self._p, shard, y_ptr, T, stride, dst_ptrs, arrived_ptrs, dst_capacity, epoch, stream)
+        if st is None:
+            n = len(dst_ptrs)
+            assert len(arrived_ptrs) == n
+            st = _fast.tpq_quantize_pack_push(self._h, shard, y_ptr, T, stride, _ptrs(dst_ptrs), _ptrs(arrived_ptrs), n,
+                                             dst_capacity, epoch, stream)
         if st:
             self._check(st)
 

@@ -1,15 +1,17 @@
-"""Build libtpq.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Build libtpq.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the extension module _calls.so."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 INCLUDE = PKG.parent / "include"
 LIB = PKG / "libtpq.so"
+CALLS = PKG / "_calls.so"   # csrc/calls.c: the step's calls for Python (binding.py)
 
 OBJ = PKG / "build"   # object files (git-ignored)
 
@@ -32,12 +34,27 @@ def _stale(target: Path, deps) -> bool:
 
 
 def needs_build() -> bool:
-    return _stale(LIB, list(CSRC.glob("*")) + [INCLUDE / "tpq.h", Path(__file__)])
+    return _stale(LIB, [f for f in CSRC.glob("*") if f.suffix != ".c"] + [INCLUDE / "tpq.h", Path(__file__)])
+
+
+def build_calls(force: bool = False) -> Path:
+    src = CSRC / "calls.c"
+    if not force and not _stale(CALLS, [src, INCLUDE / "tpq.h", Path(__file__)]):
+        return CALLS
+    tmp = CALLS.with_suffix(f".{os.getpid()}.tmp")
+    cmd = [os.environ.get("CC", "gcc"), "-std=c11", "-O2", "-Wall", "-fPIC", "-shared", f"-I{sysconfig.get_paths()['include']}",
+           f"-I{INCLUDE}", "-o", str(tmp), str(src)]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("calls.c:\n" + res.stdout + res.stderr)
+    os.replace(tmp, CALLS)
+    return CALLS
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
     """Compile every translation unit to an object file (only the stale ones unless ``force``), side by side,
-    and link them into libtpq.so."""
+    and link them into libtpq.so; build the extension module."""
+    build_calls(force)
     if not force and not needs_build():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

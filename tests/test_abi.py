@@ -121,3 +121,66 @@ def test_pointer_arrays_are_checked_like_the_c_signature(lib):
                 wrong[j] = bad
                 with pytest.raises(ctypes.ArgumentError):
                     fn(*wrong)
+
+
+def test_extension_calls_pass_on_what_ctypes_would(lib):
+    """Every call of the extension module, bound to recorders: plain arguments arrive as the C signature types them (64-bit
+    addresses, 32-bit tags, sizes, None for an optional pointer); any other form is left to ctypes without a call."""
+    import ctypes
+
+    from paper_2411_07942_b200 import binding
+
+    seen, keep, addresses = [], [], []
+    for name in binding._CALLS:
+        res, types = binding.SIGNATURES[name]
+        plain = [ctypes.c_void_p if isinstance(a, type) and issubclass(a, ctypes._Pointer) else a for a in types]
+
+        def record(*args, _name=name):
+            lists = {i: n for i, a in enumerate(binding.SIGNATURES[_name][1]) if a is ctypes.POINTER(ctypes.c_void_p) for n in [2]}
+            seen.append((_name, [[(ctypes.c_uint64 * n).from_address(x)[j] for j in range(n)] if (n := lists.get(i)) else x
+                                 for i, x in enumerate(args)]))
+            return 7
+
+        fn = ctypes.CFUNCTYPE(res, *plain)(record)
+        keep.append(fn)
+        addresses.append(ctypes.cast(fn, ctypes.c_void_p).value)
+    c, ctx, big, st = binding._calls, 2 ** 47 + 8, 2 ** 64 - 16, 2 ** 63 + 64
+    calls = [  # function, arguments, what the library's entry point receives
+        (c.calibrate_ranges, (ctx, 1, big, 3, 4, 8, st), "tpq_calibrate_ranges", [ctx, 1, big, 3, 4, 8, st]),
+        (c.quantize_pack, (ctx, -1, big, 2 ** 40, 8, 32, 2 ** 63, 0), "tpq_quantize_pack", [ctx, -1, big, 2 ** 40, 8, 32, 2 ** 63, None]),
+        (c.quantize_pack_batch, (ctx, 5, [16, big], -3, 8, (48, 64), 9, st), "tpq_quantize_pack_batch", [ctx, 5, 2, [16, big], -3, 8, [48, 64], 9, st]),
+        (c.dequant_reduce, (ctx, [16, big], 4, 48, 1, 8, None, st), "tpq_dequant_reduce", [ctx, [16, big], 2, 4, 48, 1, 8, st]),
+        (c.dequant_reduce, (ctx, (16, big), 4, 48, 0, 8, 80, st), "tpq_dequant_reduce_bias", [ctx, [16, big], 2, 4, 48, 0, 8, 80, st]),
+        (c.dequant_reduce_arrivals, (ctx, [16, big], 4, 48, 1, 8, None, 96, 2 ** 32 - 1, 2 ** 64 - 1, st), "tpq_dequant_reduce_arrivals",
+         [ctx, [16, big], 2, 4, 48, 1, 8, None, 96, 2 ** 32 - 1, 2 ** 64 - 1, st]),
+        (c.quantize_pack_push, (ctx, 0, 32, 4, 8, [16, big], [20, 24], 2 ** 63, 2 ** 32 - 1, st), "tpq_quantize_pack_push",
+         [ctx, 0, 32, 4, 8, [16, big], [20, 24], 2, 2 ** 63, 2 ** 32 - 1, st]),
+        (c.linear_quantize_pack, (ctx, 2, 32, 48, 4, 8, 64, 9, None, st), "tpq_linear_quantize_pack", [ctx, 2, 32, 48, 4, 8, 64, 9, None, st]),
+        (c.linear_quantize_pack, (ctx, 2, 32, 48, 4, 8, 64, 9, 80, st), "tpq_linear_quantize_pack", [ctx, 2, 32, 48, 4, 8, 64, 9, 80, st]),
+    ]
+    try:
+        c.bind(addresses)
+        for fn, args, name, want in calls:
+            assert fn(*args) == 7
+            assert seen.pop() == (name, want)
+            for i, a in enumerate(args):
+                if isinstance(a, (list, tuple)):
+                    others = [list(a[:1]) + [None], [1.0, 2], [True, 2], [-1, 2], [2 ** 64, 2], (ctypes.c_void_p * 2)(1, 2), 4096, [1] * 65, "12"]
+                    if fn in (c.quantize_pack_batch, c.quantize_pack_push):
+                        others.append(list(a) + [1])   # (not as long as the other list)
+                else:
+                    others = [True, 1.0, "1", ctypes.c_void_p(1), 2 ** 64, [1]] + ([] if i in (6, 8) else [None])
+                for other in others:
+                    assert fn(*args[:i], other, *args[i + 1:]) is None, (name, i, other)
+            assert fn(*args[:-1]) is None and fn(*args, 0) is None
+        assert not seen
+        t = binding.Tpq.__new__(binding.Tpq)   # a closed context: refused by the library, as through ctypes
+        t._h, t._p, t.N, t.E = ctypes.c_void_p(), None, 2, 8
+    finally:
+        c.bind([ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in binding._CALLS])
+    for call in (lambda: t.quantize_pack_batch(0, [16, 16], 1, [16, 16], 9), lambda: t.dequant_reduce([16, 16], 1, 16), lambda: t.quantize_pack(0, 16, 1, 16, 9)):
+        with pytest.raises(binding.TpqError) as e:
+            call()
+        assert e.value.status == binding.TPQ_ERR_INVALID_ARG
+    with pytest.raises(AssertionError):
+        t.quantize_pack_batch(0, [16, 16], 1, [16], 9)
