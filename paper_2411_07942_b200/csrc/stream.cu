@@ -803,30 +803,76 @@ __host__ __device__ constexpr size_t ds_smem_bytes(int B, int N)
 }
 
 // bit position, inside the float's mantissa, at which code n of a half is decoded
-__host__ __device__ constexpr int ds_pos(int B, int n) { return (B <= 5 ? (n & 3) : (n & 1)) * B; }
+__host__ __device__ constexpr int ds_pos(int B, int n) { return (B <= 5 ? (n & 3) : B == 8 ? 0 : (n & 1)) * B; }
 
 // 4 codes of a half (x: the half's bits from bit 0 on, more above), accumulated: (x & mask) | 0x4B000000 is the
 // float 2^23 + (code + 2^(B-1)) 2^pos once the sign bits are flipped; subtracting 2^23 + 2^(B-1+pos) is exact and the
 // steps are pre-divided by 2^pos, so the FMA rounds exactly like fma(code, s, acc).  A code must end below bit 23:
-// up to 5 bits all four do, wider ones take codes 2 and 3 from the half shifted down.
+// up to 5 bits all four do, 6 and 7 bits take codes 2 and 3 from the half shifted down, and at 8 bits a byte permute
+// puts every code at bit 0 in one instruction.
+//
+// DSConsts: masks, exponent pattern and bias pairs.  KEEP makes them opaque to the compiler, which then keeps them in
+// registers instead of rebuilding them at every use (where the kernel has the registers for it).
 template <int B>
-__device__ __forceinline__ void ds_decode4(uint32_t x, const float2 s01, const float2 s23, float2 &a01, float2 &a23)
+struct DSConsts {
+    uint32_t magic, mask[4];
+    float2 bias[2];
+    template <bool KEEP>
+    __device__ __forceinline__ void init()
+    {
+        magic = 0x4B000000u;
+#pragma unroll
+        for (int n = 0; n < 4; ++n) mask[n] = ((1u << B) - 1u) << ds_pos(B, n);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            bias[h] = make_float2(-(8388608.0f + (float)(1u << (B - 1 + ds_pos(B, 2 * h)))),
+                                  -(8388608.0f + (float)(1u << (B - 1 + ds_pos(B, 2 * h + 1)))));
+        if (KEEP) {
+            asm volatile("" : "+r"(magic));
+#pragma unroll
+            for (int n = 0; n < (B == 8 ? 0 : B <= 5 ? 4 : 2); ++n) asm volatile("" : "+r"(mask[n]));
+#pragma unroll
+            for (int h = 0; h < (B <= 5 ? 2 : 1); ++h) asm volatile("" : "+f"(bias[h].x), "+f"(bias[h].y));
+        }
+    }
+};
+// FIRST: the accumulators start here (what fma(code, step, +0) gives, but for the sign of a zero where a step is 0: the lane
+// of a selected feature, whose sum is never kept)
+template <int B, bool FIRST = false>
+__device__ __forceinline__ void ds_decode4(uint32_t x, const float2 s01, const float2 s23, float2 &a01, float2 &a23, const DSConsts<B> &c)
 {
-    constexpr uint32_t m = (1u << B) - 1u;
     constexpr uint32_t sign = (1u << (B - 1)) * (1u + (1u << B) + (1u << (2 * B)) + (1u << (3 * B)));
-    constexpr float b0 = -(8388608.0f + (float)(1u << (B - 1)));
-    constexpr float b1 = -(8388608.0f + (float)(1u << (2 * B - 1)));
     x ^= sign;
-    const uint32_t x2 = B <= 5 ? x : x >> (2 * B);
-    constexpr int p2 = ds_pos(B, 2), p3 = ds_pos(B, 3);
-    constexpr float b2 = -(8388608.0f + (float)(1u << (B - 1 + p2)));
-    constexpr float b3 = -(8388608.0f + (float)(1u << (B - 1 + p3)));
-    const float2 f01 = make_float2(__uint_as_float(lop3_and_or(x, m, 0x4B000000u)),
-                                   __uint_as_float(lop3_and_or(x, m << B, 0x4B000000u)));
-    const float2 f23 = make_float2(__uint_as_float(lop3_and_or(x2, m << p2, 0x4B000000u)),
-                                   __uint_as_float(lop3_and_or(x2, m << p3, 0x4B000000u)));
-    a01 = __ffma2_rn(__fadd2_rn(f01, make_float2(b0, b1)), s01, a01);
-    a23 = __ffma2_rn(__fadd2_rn(f23, make_float2(b2, b3)), s23, a23);
+    float2 f01, f23;
+    if constexpr (B == 8) {
+        f01 = make_float2(__uint_as_float(__byte_perm(x, c.magic, 0x7440)), __uint_as_float(__byte_perm(x, c.magic, 0x7441)));
+        f23 = make_float2(__uint_as_float(__byte_perm(x, c.magic, 0x7442)), __uint_as_float(__byte_perm(x, c.magic, 0x7443)));
+    } else {
+        const uint32_t x2 = B <= 5 ? x : x >> (2 * B);
+        constexpr int m2 = B <= 5 ? 2 : 0;
+        f01 = make_float2(__uint_as_float(lop3_and_or(x, c.mask[0], c.magic)), __uint_as_float(lop3_and_or(x, c.mask[1], c.magic)));
+        f23 = make_float2(__uint_as_float(lop3_and_or(x2, c.mask[m2], c.magic)), __uint_as_float(lop3_and_or(x2, c.mask[m2 + 1], c.magic)));
+    }
+    const float2 d01 = __fadd2_rn(f01, c.bias[0]), d23 = __fadd2_rn(f23, c.bias[B <= 5 ? 1 : 0]);
+    a01 = FIRST ? __fmul2_rn(d01, s01) : __ffma2_rn(d01, s01, a01);
+    a23 = FIRST ? __fmul2_rn(d23, s23) : __ffma2_rn(d23, s23, a23);
+}
+
+// the 8 codes that begin at bit sh of the first of a group's words (w1: the second one, w2: the third, read from 5 bits on)
+template <int B, bool FIRST = false>
+__device__ __forceinline__ void ds_decode8(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t sh, const float2 (&sc)[4], float2 (&acc)[4],
+                                           const DSConsts<B> &c)
+{
+    const uint32_t lo = __funnelshift_r(w0, w1, sh);
+    uint32_t hi;  // codes 4..7
+    if constexpr (B <= 4) {
+        hi = lo >> (4 * B);
+    } else {
+        const uint32_t up = __funnelshift_r(w1, w2, sh);
+        hi = B == 8 ? up : __funnelshift_r(lo, up, 4 * B & 31);
+    }
+    ds_decode4<B, FIRST>(lo, sc[0], sc[1], acc[0], acc[1], c);
+    ds_decode4<B, FIRST>(hi, sc[2], sc[3], acc[2], acc[3], c);
 }
 
 __device__ __forceinline__ void ds_cp16(uint32_t dst, const void *src)
@@ -991,6 +1037,8 @@ __global__ void __launch_bounds__(DS_THREADS, 2) dequant_stream(const DSParams p
     bool pend = false, pend_on = false;
     float pend_v = 0.0f;
     int64_t pend_tc = 0;
+    DSConsts<B> dc;
+    dc.template init<false>();  // (in registers: 18.1 us instead of 17.8 at 16 x 500 x 4416)
 
     for (int64_t ch = by; ch < p.n_chunks; ch += p.gy) {
         const int64_t tc = ch * RC, t0 = tc + rs * DS_R;
@@ -1034,19 +1082,11 @@ __global__ void __launch_bounds__(DS_THREADS, 2) dequant_stream(const DSParams p
             for (int i = 0; i < NB; ++i) {
                 if (i0 + i >= N) break;
                 const float4 a = st4[(2 * i) * CG], b = st4[(2 * i + 1) * CG];
+                const float2 sc[4] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y), make_float2(b.z, b.w)};
 #pragma unroll
                 for (int r = 0; r < DS_R; ++r) {
                     const uint32_t *const s = sw + i * RC * SEGW + wofs[r];
-                    const uint32_t lo = __funnelshift_r(s[0], s[1], wsh[r]);
-                    uint32_t hi;  // codes 4..7
-                    if (B <= 4)
-                        hi = lo >> (B < 8 ? 4 * B : 0);
-                    else {
-                        const uint32_t up = __funnelshift_r(s[1], s[2], wsh[r]);
-                        hi = B == 8 ? up : __funnelshift_r(lo, up, 4 * B & 31);
-                    }
-                    ds_decode4<B>(lo, make_float2(a.x, a.y), make_float2(a.z, a.w), acc[r][0], acc[r][1]);
-                    ds_decode4<B>(hi, make_float2(b.x, b.y), make_float2(b.z, b.w), acc[r][2], acc[r][3]);
+                    ds_decode8<B>(s[0], s[1], B > 4 ? s[2] : 0u, wsh[r], sc, acc[r], dc);
                 }
             }
             sw += STAGE_BYTES / 4;
@@ -1120,17 +1160,19 @@ cudaError_t launch_dequant_stream(const DSParams &p, int fp32_out, cudaStream_t 
 // ----------------------------------------------------------------------------------------------
 // Dequantise + reduce for up to four devices: the row kernel (dequant.cu) at bit granularity.
 //
-// One persistent block per SM on a run of adjacent rows, DW_ROWS at a time.  Warp 0 streams the devices' code rows
-// into a ring (one bulk copy per device and stage, from the 16-byte boundary at or below the first bit).  A main
-// thread owns a group of 8 features with the steps of all devices in registers (0 at selected features), funnels its bits
-// out of two (three) words, stores the whole group and then overwrites the lanes of selected features with the sums
-// the auxiliary warps left in shared memory (same thread, same address: ordered).  An auxiliary thread per rank h adds up
-// the devices' BF16 values of selected feature h, loaded from memory a stage ahead (the BF16 rows are not aligned for bulk
-// copies and end with the payload), and decodes column L + h of the output where that is a filler feature.
-// No warp waits for another's global stores.  4 x 2048 x 5120 back to back, panel kernel against this one: 51 selected 17.8 and
-// 14.0 us, 3 bits 16.5 and 13.8, 6 bits 19.9 and 15.3 (the Int4 row kernel 10.6; 6.6, 5.8 and 8.2 us for the bytes).  59 to 61
-// instructions per warp of 32 groups and device take 60 % of the issue slots; the rest is the prologue's table loads and the
-// auxiliary warps' BF16 values.
+// One persistent block per SM on a run of adjacent rows, DW_ROWS at a time (two in the first stage, which lands sooner).
+// Warp 0 streams the devices' code rows and BF16 rows into a ring (two bulk copies per device and stage, between 16-byte
+// boundaries).  A main thread owns a group of 8 features with the steps of all devices in registers (0 at selected
+// features), funnels its bits out of two (three) words, stores the whole group and then overwrites the lanes of selected
+// features with the sums the auxiliary warps left in shared memory (same thread, same address: ordered).  An auxiliary
+// thread per rank h adds up the devices' BF16 values of selected feature h and decodes column L + h of the output where that
+// is a filler feature.  No warp waits for another's global stores.
+// What bounds it is the auxiliary warps' latency per stage (without selected features 9.6 us at 4 x 2048 x 5120, 3 bits), then
+// the decode.  Back to back, with the BF16 values loaded from memory a stage ahead, general loops in the auxiliary warps
+// and a device count read at run time, against this form: 4 x 2048 x 5120, 51 selected 14.9 and 12.0 us, 3 bits 14.5 and
+// 11.9, 6 bits 16.4 and 13.5; two devices 11.2 and 8.5; three 12.7 and 11.5 (6.6, 5.8, 8.2, 4.9 and 5.8 us for the bytes; the
+// Int4 row kernel 10.8).  Either half alone loses: the staged values behind general loops take 15.9 us, the compile-time
+// device count without them 15.2.
 // ----------------------------------------------------------------------------------------------
 constexpr int DW_ROWS = 4, DW_MAX_DEV = 4, DW_MAIN = 640, DW_AUX = 96, DW_MAX_K = 384;
 
@@ -1139,18 +1181,81 @@ struct DWParams {
     const float *s_k;      // [N][E] steps, 0 at selected features
     const int32_t *pos;    // [E]
     int nstage;
-    uint32_t dev_bytes;    // a device's part of a stage
+    uint32_t dev_bytes;    // a device's code words in a stage ...
+    uint32_t hp_bytes;     // ... and its BF16 values
+    int first;             // rows of a block's first stage
     int64_t rows_per_block;
     int *status;
 };
 
 __host__ __device__ inline uint32_t dw_dev_bytes(int L, int B) { return (uint32_t)(((DW_ROWS * L * B + 127 + 127) / 128 + 1) * 16); }
-inline size_t dw_smem_bytes(int N, uint32_t dev_bytes, int k, int nstage)
+__host__ __device__ inline uint32_t dw_hp_bytes(int k) { return k ? (uint32_t)(DW_ROWS * k * 2 + 14 + 15) & ~15u : 0u; }
+inline size_t dw_smem_bytes(int nd, uint32_t dev_bytes, int k, int nstage)
 {
-    return (size_t)nstage * ((size_t)N * dev_bytes + (size_t)DW_ROWS * k * 4 + 24) + 16;
+    return (size_t)nstage * ((size_t)nd * (dev_bytes + dw_hp_bytes(k)) + (size_t)DW_ROWS * k * 4 + 24) + 16;
 }
 
-template <int B, bool FP32OUT, bool HAS_BIAS>
+__device__ __forceinline__ uint32_t dw_lds32(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t dw_lds16(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void dw_sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+
+// ROWS rows of a stage for one main thread.  stage: its address, bit: the first bit of the thread's group in the first row.
+// ND devices, a number that the compiler knows: straight-line code, every device's words at the same place in its part.
+template <int B, int ND, int ROWS, bool FP32OUT, bool HAS_BIAS>
+__device__ __forceinline__ void dw_rows(const uint8_t *stage, uint32_t dev_bytes, uint32_t bit, uint32_t LB, const float2 (&sc)[ND][4],
+                                        const float2 (&b)[4], const DSConsts<B> &dc, uint8_t *out, int64_t out_row_bytes, int lanes)
+{
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r, bit += LB, out += out_row_bytes) {
+        const uint8_t *w = stage + (bit >> 5) * 4;
+        float2 acc[4];
+#pragma unroll
+        for (int i = 0; i < ND; ++i, w += dev_bytes) {
+            const uint32_t *const q = reinterpret_cast<const uint32_t *>(w);
+            if (i == 0) ds_decode8<B, true>(q[0], q[1], B > 4 ? q[2] : 0u, bit & 31u, sc[i], acc, dc);
+            else ds_decode8<B>(q[0], q[1], B > 4 ? q[2] : 0u, bit & 31u, sc[i], acc, dc);
+        }
+        if (HAS_BIAS) {  // (a selected feature's lane is overwritten later)
+#pragma unroll
+            for (int h = 0; h < 4; ++h) acc[h] = __fadd2_rn(acc[h], b[h]);
+        }
+        if (lanes >= 8) {
+            if (FP32OUT) {
+                __stcs(reinterpret_cast<float4 *>(out), make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y));
+                __stcs(reinterpret_cast<float4 *>(out) + 1, make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y));
+            } else {
+                uint32_t x[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const __nv_bfloat162 t = __floats2bfloat162_rn(acc[h].x, acc[h].y);
+                    x[h] = *reinterpret_cast<const uint32_t *>(&t);
+                }
+                __stcs(reinterpret_cast<uint4 *>(out), make_uint4(x[0], x[1], x[2], x[3]));
+            }
+        } else {
+#pragma unroll
+            for (int n = 0; n < 8; ++n)
+                if (n < lanes) ds_store_one<FP32OUT>(out, n, (n & 1) ? acc[n >> 1].y : acc[n >> 1].x);
+        }
+    }
+}
+
+// first row (within the block's run) of the block's it-th stage: a short first stage lands sooner
+__device__ __forceinline__ int dw_stage_row(int it, int first) { return it == 0 ? 0 : first + (it - 1) * DW_ROWS; }
+
+// ND: 2 or 4, at least the number of devices.  A stage has room for ND; where there are fewer, the last ones have steps of 0
+// and whatever bits lie in their part: every pattern decodes to a finite code, and fma(code, 0, acc) is acc (never -0).
+template <int B, int ND, bool FP32OUT, bool HAS_BIAS>
 __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(const DWParams pp)
 {
     extern __shared__ __align__(128) uint8_t dw_smem[];
@@ -1158,7 +1263,7 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
     const int N = p.N, E = p.E, k = p.k, L = p.L, G = (L + 7) >> 3, nstage = pp.nstage;
     const uint32_t LB = (uint32_t)L * B;
     const int tid = threadIdx.x, lane = tid & 31;
-    const uint32_t stage_bytes = (uint32_t)N * pp.dev_bytes;
+    const uint32_t stage_bytes = (uint32_t)ND * (pp.dev_bytes + pp.hp_bytes);
     uint32_t *const sums = reinterpret_cast<uint32_t *>(dw_smem + (size_t)nstage * stage_bytes);  // [nstage][DW_ROWS][k]
     uint64_t *const full = reinterpret_cast<uint64_t *>(dw_smem + (((size_t)nstage * (stage_bytes + (size_t)DW_ROWS * k * 4) + 15) & ~(size_t)15));
     uint64_t *const empty = full + nstage, *const sums_ready = empty + nstage;
@@ -1171,7 +1276,9 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
         __syncthreads();
     }
     if (tid < 32) {
-        // ---------------- producer warp: lane i copies device i's rows
+        // ---------------- producer warp: lane i copies device i's code rows, lane ND + i its BF16 rows.  Those begin and
+        // end anywhere: the copy runs between 16-byte boundaries, and what the payload's last, incomplete 16 bytes hold is
+        // read by the auxiliary threads themselves
         if (lane == 0) {
             for (int s = 0; s < nstage; ++s) {
                 mbar_init(smem_u32(&full[s]), 1);
@@ -1192,23 +1299,32 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
         tpq_grid_dep_wait();  // the payloads and the output buffer may still be in use by the kernel ahead
         int st = 0;
         uint32_t parity = 1;
-        for (int it = 0, r0 = 0; r0 < rows_mine; ++it, r0 += DW_ROWS) {
-            const int rows = rows_mine - r0 < DW_ROWS ? rows_mine - r0 : DW_ROWS;
+        for (int it = 0, r0 = 0; r0 < rows_mine; r0 = dw_stage_row(++it, pp.first)) {
+            const int cap = it == 0 ? pp.first : DW_ROWS, rows = rows_mine - r0 < cap ? rows_mine - r0 : cap;
             const int64_t bit = (t_begin + r0) * (int64_t)LB, from = (bit >> 3) & ~(int64_t)15;
             const int64_t to = ((bit + (int64_t)rows * LB + 127) >> 7) << 4;  // (the code section is a multiple of 16 bytes)
             const uint32_t bytes = (uint32_t)(to - from), bar = smem_u32(&full[st]);
+            const int64_t h_from = ((t_begin + r0) * k * 2) & ~(int64_t)15, h_all = (p.T * k * 2) & ~(int64_t)15;
+            int64_t h_to = ((t_begin + r0 + rows) * k * 2 + 15) & ~(int64_t)15;
+            if (h_to > h_all) h_to = h_all;
+            const uint32_t h_bytes = h_to > h_from ? (uint32_t)(h_to - h_from) : 0u;
             int ok = 1;
             if (lane == 0) {
                 if (it >= nstage && !mbar_wait(smem_u32(&empty[st]), parity)) {
                     atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
                     ok = 0;
                 } else {
-                    mbar_expect_tx(bar, (uint32_t)N * bytes);
+                    mbar_expect_tx(bar, (uint32_t)N * (bytes + h_bytes));
                 }
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
-            if (lane < N) bulk_g2s(smem_u32(dw_smem) + (uint32_t)st * stage_bytes + (uint32_t)lane * pp.dev_bytes, p.pl[lane] + from, bytes, bar);
+            const uint32_t stage = smem_u32(dw_smem) + (uint32_t)st * stage_bytes;
+            const int h_lane = lane - ND;
+            if (lane < N)
+                bulk_g2s(stage + (uint32_t)lane * pp.dev_bytes, p.pl[lane] + from, bytes, bar);
+            else if (h_lane >= 0 && h_lane < N && h_bytes)
+                bulk_g2s(stage + ND * pp.dev_bytes + (uint32_t)h_lane * pp.hp_bytes, p.pl[h_lane] + p.lp_bytes + h_from, h_bytes, bar);
             if (++st == nstage) {
                 st = 0;
                 parity ^= 1u;
@@ -1219,89 +1335,103 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
     int st = 0;
     uint32_t parity = 0;
     if (tid < 32 + DW_AUX) {
-        // ---------------- auxiliary warps
+        // ---------------- auxiliary warps: thread `at` adds up selected feature `at` and decodes column L + at, row by row in
+        // short rolled loops over what it has loaded once (this code runs once per stage and nobody else runs it, so that
+        // straight-line code would pay an instruction fetch for every few instructions)
         const int at = tid - 32;
         const bool on = at < k;
         const int s_col = on ? __ldg(p.hp_idx + at) : 0;                       // rank `at`: its feature
         const int ps = on ? __ldg(pp.pos + L + at) : -1;                       // column L + at: its slot (< 0: selected)
-        float c_s[DW_MAX_DEV];
+        float c_s[ND];
 #pragma unroll
-        for (int i = 0; i < DW_MAX_DEV; ++i) c_s[i] = i < N && ps >= 0 ? __ldg(pp.s_k + (size_t)i * E + L + at) : 0.0f;
+        for (int i = 0; i < ND; ++i) c_s[i] = i < N && ps >= 0 ? __ldg(pp.s_k + (size_t)i * E + L + at) : 0.0f;
         asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
-        tpq_grid_dep_wait();  // the bias and the BF16 values are read, and columns written, without waiting for a copy
-        const float s_b = HAS_BIAS && on ? p.bias[s_col] : 0.0f, c_b = HAS_BIAS && on ? p.bias[L + at] : 0.0f;
-        uint16_t v[DW_ROWS][DW_MAX_DEV];
-        auto load = [&](int r0) {
-            if (on) {
+        if (HAS_BIAS) tpq_grid_dep_wait();  // (the kernel ahead may be writing it)
+        float s_b = HAS_BIAS && on ? p.bias[s_col] : 0.0f, c_b = HAS_BIAS && on ? p.bias[L + at] : 0.0f;
+        uint32_t c_bit = (uint32_t)(ps >= 0 ? ps : 0) * B;
+        asm volatile("" : "+r"(c_bit), "+f"(s_b), "+f"(c_b));
 #pragma unroll
-                for (int r = 0; r < DW_ROWS; ++r)
-#pragma unroll
-                    for (int i = 0; i < DW_MAX_DEV; ++i)
-                        if (r0 + r < rows_mine && i < N)
-                            v[r][i] = __ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + p.lp_bytes) + (t_begin + r0 + r) * k + at);
-            }
+        for (int i = 0; i < ND; ++i) asm volatile("" : "+f"(c_s[i]));
+        constexpr int ESIZE = FP32OUT ? 4 : 2;
+        const int64_t out_row_bytes = p.out_stride * ESIZE;
+        auto bits_of = [&](float v) { return FP32OUT ? __float_as_uint(v) : (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v)); };
+        // the code of the slot whose first bit is bit `bit` of a device's part of the stage
+        auto code = [&](uint32_t dev, uint32_t bit) {
+            const uint32_t a = dev + (bit >> 5) * 4u;
+            const uint32_t w = __funnelshift_r(dw_lds32(a), dw_lds32(a + 4u), bit & 31u) & ((1u << B) - 1u);
+            return __fsub_rn(__uint_as_float((w ^ (1u << (B - 1))) | 0x4B000000u), 8388608.0f + (float)(1 << (B - 1)));
         };
-        // the code of slot `slot` in the row whose first bit is bit `row_bit` of a device's part of the stage
-        auto code = [&](const uint32_t *dev, uint32_t row_bit, int slot) {
-            const uint32_t bit = row_bit + (uint32_t)slot * B;
-            const uint32_t w = __funnelshift_r(dev[bit >> 5], dev[(bit >> 5) + 1], bit & 31u) & ((1u << B) - 1u);
-            return (float)((int)(w ^ (1u << (B - 1))) - (1 << (B - 1)));
-        };
-        auto put = [&](int r, int64_t t, int rank, int col, float sum) {  // a selected feature's sum
-            if (col < L)
-                sums[((size_t)st * DW_ROWS + r) * k + rank] =
-                    FP32OUT ? __float_as_uint(sum) : (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(sum));
-            else
-                ds_store_one<FP32OUT>(p.out, t * p.out_stride + col, sum);
-        };
-        load(0);
-        for (int r0 = 0; r0 < rows_mine; r0 += DW_ROWS) {
-            const int rows = rows_mine - r0 < DW_ROWS ? rows_mine - r0 : DW_ROWS;
+        for (int it = 0, r0 = 0; r0 < rows_mine; r0 = dw_stage_row(++it, pp.first)) {
+            const int cap = it == 0 ? pp.first : DW_ROWS, rows = rows_mine - r0 < cap ? rows_mine - r0 : cap;
             const int64_t t0 = t_begin + r0;
-            // the stage's previous sums have been read by everybody when its next copies land: wait for those first
+            // (the stage's previous sums have been read by everybody when its next copies land)
             if (!mbar_wait(smem_u32(&full[st]), parity)) {
                 atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
                 break;
             }
-            if (on) {
+            const uint32_t stage = smem_u32(dw_smem) + (uint32_t)st * stage_bytes;
+            const uint32_t sum0 = smem_u32(sums) + (uint32_t)(st * DW_ROWS * k) * 4u;  // the stage's sums
+            uint8_t *const out0 = static_cast<uint8_t *>(p.out) + t0 * out_row_bytes;
+            // the sums of the selected features, out of the stage; `have`: values of a device that lie there
+            const int64_t h_first = t0 * k, h_left = ((p.T * k) & ~(int64_t)7) - h_first;
+            const bool whole = h_left >= (int64_t)rows * k;
+            const uint32_t hp = stage + ND * pp.dev_bytes + (uint32_t)((h_first * 2) & 15);
+            if (on && whole) {
+                uint32_t a = hp + 2u * at, o = sum0 + 4u * at;
+                uint8_t *og = out0 + (int64_t)s_col * ESIZE;
+#pragma unroll 1
+                for (int r = 0; r < rows; ++r, a += 2u * k, o += 4u * k, og += out_row_bytes) {
+                    float v = 0.0f;
 #pragma unroll
-                for (int r = 0; r < DW_ROWS; ++r) {
-                    if (r >= rows) break;
-                    float sum = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < DW_MAX_DEV; ++i)
-                        if (i < N) sum = __fadd_rn(sum, __uint_as_float((uint32_t)v[r][i] << 16));
-                    put(r, t0 + r, at, s_col, HAS_BIAS ? __fadd_rn(sum, s_b) : sum);
+                    for (int i = 0; i < ND; ++i)
+                        if (i < N) v = __fadd_rn(v, __uint_as_float(dw_lds16(a + (uint32_t)i * pp.hp_bytes) << 16));
+                    if (HAS_BIAS) v = __fadd_rn(v, s_b);
+                    if (s_col < L) dw_sts32(o, bits_of(v));
+                    else ds_store_one<FP32OUT>(og, 0, v);
                 }
             }
-            for (int h = at + DW_AUX; h < k; h += DW_AUX) {  // more selected features than threads
+            // more selected features than threads, and the payload's last rows (a value that no copy brought is read here)
+            for (int h = whole ? at + DW_AUX : at; h < k; h += DW_AUX) {
                 const int col = __ldg(p.hp_idx + h);
                 for (int r = 0; r < rows; ++r) {
-                    float sum = 0.0f;
-                    for (int i = 0; i < N; ++i)
-                        sum = __fadd_rn(sum, __uint_as_float((uint32_t)__ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + p.lp_bytes) + (t0 + r) * k + h) << 16));
-                    put(r, t0 + r, h, col, HAS_BIAS ? __fadd_rn(sum, p.bias[col]) : sum);
+                    const int e = r * k + h;
+                    float v = 0.0f;
+                    for (int i = 0; i < N; ++i) {
+                        const uint32_t x = e < h_left ? dw_lds16(hp + (uint32_t)i * pp.hp_bytes + 2u * e)
+                                                      : (uint32_t)__ldcs(reinterpret_cast<const uint16_t *>(p.pl[i] + p.lp_bytes) + h_first + e);
+                        v = __fadd_rn(v, __uint_as_float(x << 16));
+                    }
+                    if (HAS_BIAS) v = __fadd_rn(v, p.bias[col]);
+                    if (col < L) dw_sts32(sum0 + 4u * e, bits_of(v));
+                    else ds_store_one<FP32OUT>(out0 + r * out_row_bytes, col, v);
                 }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sums_ready[st]));  // (release: the sums are visible to whoever waits)
-            if (r0 + DW_ROWS < rows_mine) load(r0 + DW_ROWS);
             // the last k columns: filler features, decoded from the holes' slots that carry them
-            const uint8_t *const stage = dw_smem + (size_t)st * stage_bytes;
             const uint32_t rem = (uint32_t)((t0 * (int64_t)LB) & 127);
-            for (int h = at; h < k; h += DW_AUX) {
-                const int slot = h == at ? ps : __ldg(pp.pos + L + h);
-                if (slot < 0) continue;
+            if (ps >= 0) {
+                uint32_t bit = rem + c_bit;
+                uint8_t *og = out0 + (int64_t)(L + at) * ESIZE;
 #pragma unroll 1
-                for (int r = 0; r < rows; ++r) {
-                    float acc = 0.0f;
+                for (int r = 0; r < rows; ++r, bit += LB, og += out_row_bytes) {
+                    float v = 0.0f;
 #pragma unroll
-                    for (int i = 0; i < DW_MAX_DEV; ++i)
-                        if (i < N)
-                            acc = __fmaf_rn(code(reinterpret_cast<const uint32_t *>(stage + (size_t)i * pp.dev_bytes), rem + (uint32_t)r * LB, slot),
-                                            h == at ? c_s[i] : __ldg(pp.s_k + (size_t)i * E + L + h), acc);
-                    if (HAS_BIAS) acc = __fadd_rn(acc, h == at ? c_b : p.bias[L + h]);
-                    ds_store_one<FP32OUT>(p.out, (t0 + r) * p.out_stride + L + h, acc);
+                    for (int i = 0; i < ND; ++i) v = __fmaf_rn(code(stage + (uint32_t)i * pp.dev_bytes, bit), c_s[i], v);
+                    if (HAS_BIAS) v = __fadd_rn(v, c_b);
+                    ds_store_one<FP32OUT>(og, 0, v);
+                }
+            }
+            for (int h = at + DW_AUX; h < k; h += DW_AUX) {  // (more columns than threads)
+                const int slot = __ldg(pp.pos + L + h);
+                if (slot < 0) continue;
+                for (int r = 0; r < rows; ++r) {
+                    float v = 0.0f;
+                    for (int i = 0; i < N; ++i)
+                        v = __fmaf_rn(code(stage + (uint32_t)i * pp.dev_bytes, rem + (uint32_t)r * LB + (uint32_t)slot * B),
+                                      __ldg(pp.s_k + (size_t)i * E + L + h), v);
+                    if (HAS_BIAS) v = __fadd_rn(v, p.bias[L + h]);
+                    ds_store_one<FP32OUT>(out0 + r * out_row_bytes, L + h, v);
                 }
             }
             __syncwarp();
@@ -1316,11 +1446,11 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
     // ---------------- main warps
     const int g = tid - 32 - DW_AUX;
     const int lanes = L - 8 * g < 8 ? L - 8 * g : 8;  // slots of the group (the last one may be short, idle threads have none)
-    float2 sc[DW_MAX_DEV][4], b[4];
+    float2 sc[ND][4], b[4];
     uint32_t mask = 0;
     int hb = 0;
 #pragma unroll
-    for (int i = 0; i < DW_MAX_DEV; ++i)
+    for (int i = 0; i < ND; ++i)
 #pragma unroll
         for (int h = 0; h < 4; ++h) sc[i][h] = make_float2(0.0f, 0.0f);
     if (lanes > 0) {
@@ -1329,7 +1459,7 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
         if (lanes < 8) mask &= (1u << lanes) - 1u;
         hb = (int)(gd >> 8);
 #pragma unroll
-        for (int i = 0; i < DW_MAX_DEV; ++i)
+        for (int i = 0; i < ND; ++i)
             if (i < N) {
                 const float4 u = __ldg(reinterpret_cast<const float4 *>(pp.s_k + (size_t)i * E + 8 * g));
                 const float4 w = __ldg(reinterpret_cast<const float4 *>(pp.s_k + (size_t)i * E + 8 * g + 4));
@@ -1346,68 +1476,33 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
         b[h] = HAS_BIAS && lanes > 0 ? make_float2(p.bias[8 * g + 2 * h], p.bias[8 * g + 2 * h + 1]) : make_float2(0.0f, 0.0f);
     // (opaque: the compiler, short of registers, would otherwise load the steps again at every use)
 #pragma unroll
-    for (int i = 0; i < DW_MAX_DEV; ++i)
+    for (int i = 0; i < ND; ++i)
 #pragma unroll
         for (int h = 0; h < 4; ++h) asm volatile("" : "+f"(sc[i][h].x), "+f"(sc[i][h].y));
     asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
-    for (int r0 = 0; r0 < rows_mine; r0 += DW_ROWS) {
-        const int rows = rows_mine - r0 < DW_ROWS ? rows_mine - r0 : DW_ROWS;
+    DSConsts<B> dc;
+    dc.template init<true>();
+    constexpr int ESIZE = FP32OUT ? 4 : 2;
+    const int64_t out_row_bytes = p.out_stride * ESIZE;
+    uint8_t *out = static_cast<uint8_t *>(p.out) + t_begin * out_row_bytes + (lanes > 0 ? g : 0) * (8 * ESIZE);
+    const uint32_t g_bit = (uint32_t)(lanes > 0 ? g : 0) * (8 * B);
+    const bool warp_holes = __any_sync(0xffffffffu, mask != 0);
+    for (int it = 0, r0 = 0; r0 < rows_mine; r0 = dw_stage_row(++it, pp.first)) {
+        const int cap = it == 0 ? pp.first : DW_ROWS, rows = rows_mine - r0 < cap ? rows_mine - r0 : cap;
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), parity))) {
             atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
             break;
         }
-        const int64_t t0 = t_begin + r0;
         const uint8_t *const stage = dw_smem + (size_t)st * stage_bytes;
-        const uint32_t rem = (uint32_t)((t0 * (int64_t)LB) & 127);
-        int64_t o = t0 * p.out_stride + 8 * (int64_t)g;
-#pragma unroll
-        for (int r = 0; r < DW_ROWS; ++r, o += p.out_stride) {
-            if (r >= rows) break;
-            const uint32_t bit = rem + (uint32_t)r * LB + (uint32_t)(lanes > 0 ? g : 0) * (8 * B);
-            const uint8_t *w = stage + (bit >> 5) * 4;
-            float2 acc[4];
-#pragma unroll
-            for (int h = 0; h < 4; ++h) acc[h] = make_float2(0.0f, 0.0f);
-#pragma unroll
-            for (int i = 0; i < DW_MAX_DEV; ++i, w += pp.dev_bytes)
-                if (i < N) {
-                    const uint32_t *const q = reinterpret_cast<const uint32_t *>(w);
-                    const uint32_t lo = __funnelshift_r(q[0], q[1], bit & 31u);
-                    uint32_t hi;
-                    if (B <= 4)
-                        hi = lo >> (B < 8 ? 4 * B : 0);
-                    else {
-                        const uint32_t up = __funnelshift_r(q[1], q[2], bit & 31u);
-                        hi = B == 8 ? up : __funnelshift_r(lo, up, 4 * B & 31);
-                    }
-                    ds_decode4<B>(lo, sc[i][0], sc[i][1], acc[0], acc[1]);
-                    ds_decode4<B>(hi, sc[i][2], sc[i][3], acc[2], acc[3]);
-                }
-            if (HAS_BIAS) {  // (a selected feature's lane is overwritten below)
-#pragma unroll
-                for (int h = 0; h < 4; ++h) acc[h] = __fadd2_rn(acc[h], b[h]);
-            }
-            if (lanes >= 8) {
-                if (FP32OUT) {
-                    float4 *const dst = reinterpret_cast<float4 *>(static_cast<float *>(p.out) + o);
-                    __stcs(dst, make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y));
-                    __stcs(dst + 1, make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y));
-                } else {
-                    uint32_t x[4];
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        const __nv_bfloat162 t = __floats2bfloat162_rn(acc[h].x, acc[h].y);
-                        x[h] = *reinterpret_cast<const uint32_t *>(&t);
-                    }
-                    __stcs(reinterpret_cast<uint4 *>(static_cast<uint16_t *>(p.out) + o), make_uint4(x[0], x[1], x[2], x[3]));
-                }
-            } else {
-#pragma unroll
-                for (int n = 0; n < 8; ++n)
-                    if (n < lanes) ds_store_one<FP32OUT>(p.out, o + n, (n & 1) ? acc[n >> 1].y : acc[n >> 1].x);
-            }
+        const uint32_t bit = (uint32_t)(((t_begin + r0) * (int64_t)LB) & 127) + g_bit;
+        if (rows == DW_ROWS) {
+            dw_rows<B, ND, DW_ROWS, FP32OUT, HAS_BIAS>(stage, pp.dev_bytes, bit, LB, sc, b, dc, out, out_row_bytes, lanes);
+        } else {
+#pragma unroll 1
+            for (int r = 0; r < rows; ++r)
+                dw_rows<B, ND, 1, FP32OUT, HAS_BIAS>(stage, pp.dev_bytes, bit + (uint32_t)r * LB, LB, sc, b, dc, out + r * out_row_bytes, out_row_bytes, lanes);
         }
-        if (__any_sync(0xffffffffu, mask != 0)) {  // the selected features' lanes
+        if (warp_holes) {  // the selected features' lanes
             if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sums_ready[st]), parity))) {
                 atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
                 break;
@@ -1417,15 +1512,16 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
                 const int n = __ffs(m) - 1;
                 m &= m - 1;
                 const uint32_t *sum = sums + (size_t)st * DW_ROWS * k + h;
-                int64_t at = t0 * p.out_stride + 8 * (int64_t)g + n;
-                for (int r = 0; r < rows; ++r, sum += k, at += p.out_stride) {
+                uint8_t *at = out + n * ESIZE;
+                for (int r = 0; r < rows; ++r, sum += k, at += out_row_bytes) {
                     if (FP32OUT)
-                        static_cast<uint32_t *>(p.out)[at] = *sum;
+                        *reinterpret_cast<uint32_t *>(at) = *sum;
                     else
-                        static_cast<uint16_t *>(p.out)[at] = (uint16_t)*sum;
+                        *reinterpret_cast<uint16_t *>(at) = (uint16_t)*sum;
                 }
             }
         }
+        out += rows * out_row_bytes;
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
         if (++st == nstage) {
@@ -1435,24 +1531,33 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
     }
 }
 
+int dw_nd(int N) { return N <= 2 ? 2 : 4; }
+
 // ring depth; 0: the shape is the panel kernel's
 int dw_stages(const tpq_ctx *c, int64_t out_stride)
 {
     const int L = c->E - c->k, G = (L + 7) / 8;
     if (c->N > DW_MAX_DEV || c->E % 8 || out_stride % 8 || G > DW_MAIN || c->k > DW_MAX_K) return 0;
     int n = 4;
-    while (n > 1 && dw_smem_bytes(c->N, dw_dev_bytes(L, c->bits), c->k, n) > (size_t)c->smem_optin) --n;
+    while (n > 1 && dw_smem_bytes(dw_nd(c->N), dw_dev_bytes(L, c->bits), c->k, n) > (size_t)c->smem_optin) --n;
     return n > 1 ? n : 0;
+}
+
+template <int B, int ND>
+cudaError_t launch_dequant_rows_nd(const DWParams &pp, int fp32_out, unsigned grid, int threads, size_t smem, cudaStream_t st)
+{
+    auto kern = pp.d.bias ? (fp32_out ? dequant_stream_rows<B, ND, true, true> : dequant_stream_rows<B, ND, false, true>)
+                          : (fp32_out ? dequant_stream_rows<B, ND, true, false> : dequant_stream_rows<B, ND, false, false>);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return tpq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, pp);
 }
 
 template <int B>
 cudaError_t launch_dequant_rows(const DWParams &pp, int fp32_out, unsigned grid, int threads, size_t smem, cudaStream_t st)
 {
-    auto kern = pp.d.bias ? (fp32_out ? dequant_stream_rows<B, true, true> : dequant_stream_rows<B, false, true>)
-                          : (fp32_out ? dequant_stream_rows<B, true, false> : dequant_stream_rows<B, false, false>);
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return tpq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, pp);
+    return pp.d.N <= 2 ? launch_dequant_rows_nd<B, 2>(pp, fp32_out, grid, threads, smem, st)
+                       : launch_dequant_rows_nd<B, 4>(pp, fp32_out, grid, threads, smem, st);
 }
 
 }  // namespace
@@ -1622,10 +1727,12 @@ cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *paylo
         pp.d = p;
         pp.s_k = c->t.s_k; pp.pos = c->t.pos; pp.nstage = nstage; pp.status = c->t.status;
         pp.dev_bytes = dw_dev_bytes(L, c->bits);
+        pp.hp_bytes = dw_hp_bytes(k);
         pp.rows_per_block = (T + c->sm_count - 1) / c->sm_count;
+        pp.first = pp.rows_per_block > DW_ROWS ? 2 : DW_ROWS;
         const unsigned grid = (unsigned)((T + pp.rows_per_block - 1) / pp.rows_per_block);
         const int threads = 32 + DW_AUX + (G + 31) / 32 * 32;
-        const size_t smem = dw_smem_bytes(c->N, pp.dev_bytes, k, nstage);
+        const size_t smem = dw_smem_bytes(dw_nd(c->N), pp.dev_bytes, k, nstage);
         switch (c->bits) {
         case 2: e = launch_dequant_rows<2>(pp, fp32_out, grid, threads, smem, st); break;
         case 3: e = launch_dequant_rows<3>(pp, fp32_out, grid, threads, smem, st); break;
