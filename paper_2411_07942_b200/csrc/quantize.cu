@@ -297,9 +297,8 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
     const int lane = tid & 31;
     uint32_t w_off[GPT];     // byte offset of "my" filler element in a staged row (lane < n_wh)
     float w_inv[GPT];
-    int n_wh[GPT], src0[GPT];
-    int most[GPT];           // most holes of a lane of the warp
-    bool serial[GPT];
+    int src0[GPT];
+    int most[GPT];           // most holes of a lane of the warp; above 8: the warp's holes outnumber its lanes (serial path)
     uint32_t keep[GPT];      // word bits that are not holes
 #pragma unroll
     for (int a = 0; a < GPT; ++a) {
@@ -311,13 +310,12 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
             if (lane >= d) incl += o;
         }
         src0[a] = incl - nh;
-        n_wh[a] = __shfl_sync(0xffffffffu, incl, 31);
+        const int n_wh = __shfl_sync(0xffffffffu, incl, 31);  // holes of the warp
         const int hb_warp = __shfl_sync(0xffffffffu, hb[a], 0);
-        most[a] = __reduce_max_sync(0xffffffffu, nh);
-        serial[a] = n_wh[a] > 32;
+        most[a] = n_wh > 32 ? 9 : __reduce_max_sync(0xffffffffu, nh);
         w_off[a] = 0;
         w_inv[a] = 0.0f;
-        if (lane < n_wh[a] && !serial[a]) {
+        if (lane < n_wh && n_wh <= 32) {
             const int f = __ldg(p.filler + hb_warp + lane);
             w_off[a] = (uint32_t)f * 2u;
             w_inv[a] = __ldg(inv_s + f);
@@ -369,7 +367,7 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
                 uint32_t word[GR];
 #pragma unroll
                 for (int r = 0; r < GR; ++r) word[r] = quant8(v[r], inv[a]);
-                if (DEEP || n_wh[a]) {  // uniform over the warp
+                if (DEEP || most[a]) {  // uniform over the warp
                     uint32_t qv[GR];
 #pragma unroll
                     for (int r = 0; r < GR; ++r) {
@@ -409,9 +407,9 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
                 if (G >= 2 && rows - rb >= 2) { rows_fast(std::integral_constant<int, 2>(), deep, rb); rb += 2; }
                 if (rows - rb >= 1) rows_fast(std::integral_constant<int, 1>(), deep, rb);
             };
-            if (!serial[a] && most[a] <= 2) {  // (uniform over the warp, like the row counts above)
+            if (most[a] <= 2) {  // (uniform over the warp, like the row counts above)
                 stage_fast(std::false_type());
-            } else if (!serial[a]) {
+            } else if (most[a] <= 8) {
                 stage_fast(std::true_type());
             } else if (live) {
                 // a warp on the serial path: every hole patched by its owner

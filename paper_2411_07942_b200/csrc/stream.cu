@@ -511,10 +511,9 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
     float2 inv[GPT][4];
     constexpr int NW = qs_group_words(B);
     uint32_t mask[GPT], w_off[GPT], f_sh[GPT][2], field[GPT][2][NW], keep[GPT][NW];
-    int hb[GPT], n_wh[GPT], src0[GPT];
+    int hb[GPT], src0[GPT];
     float w_inv[GPT];
-    int most[GPT];  // most holes of a lane of the warp
-    bool serial[GPT], two[GPT];
+    int most[GPT];  // most holes of a lane of the warp; above 8: the warp's holes outnumber its lanes (serial path)
     const int my_hp = tid < k ? __ldg(p.hp_idx + tid) : 0;
 #pragma unroll
     for (int a = 0; a < GPT; ++a) {
@@ -541,14 +540,12 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
             if (lane >= d) incl += o;
         }
         src0[a] = incl - nh;
-        n_wh[a] = __shfl_sync(0xffffffffu, incl, 31);
+        const int n_wh = __shfl_sync(0xffffffffu, incl, 31);  // holes of the warp
         const int hb_warp = __shfl_sync(0xffffffffu, hb[a], 0);
-        most[a] = __reduce_max_sync(0xffffffffu, nh);
-        serial[a] = n_wh[a] > 32;
-        two[a] = most[a] > 1;  // some group of the warp has a second hole
+        most[a] = n_wh > 32 ? 9 : __reduce_max_sync(0xffffffffu, nh);
         w_off[a] = 0;
         w_inv[a] = 0.0f;
-        if (lane < n_wh[a] && !serial[a]) {
+        if (lane < n_wh && n_wh <= 32) {
             const int f = __ldg(p.filler + hb_warp + lane);
             w_off[a] = (uint32_t)f * 2u;
             w_inv[a] = __ldg(inv_s + f);
@@ -623,12 +620,12 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
 #pragma unroll
                 for (int r = 0; r < QS_STAGE; ++r) {
                     qs_quant8<B>(v[r], inv[a], wd[r]);
-                    if (DEEP || n_wh[a]) {  // uniform over the warp, as is two
+                    if (DEEP || most[a]) {  // uniform over the warp
                         const uint32_t qv = qs_code<B>(__uint_as_float(fx[r] << 16), w_inv[a]) & ((1u << B) - 1u);
                         const uint32_t c0 = __shfl_sync(0xffffffffu, qv, src0[a]) << f_sh[a][0];
 #pragma unroll
                         for (int j = 0; j < NW; ++j) wd[r][j] = (wd[r][j] & keep[a][j]) | (c0 & field[a][0][j]);
-                        if (DEEP || two[a]) {
+                        if (DEEP || most[a] > 1) {
                             const uint32_t c1 = __shfl_sync(0xffffffffu, qv, src0[a] + 1) << f_sh[a][1];
 #pragma unroll
                             for (int j = 0; j < NW; ++j) wd[r][j] |= c1 & field[a][1][j];
@@ -657,9 +654,9 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
                     for (int r = 0; r < QS_STAGE; ++r) emit(r, wd[r], r < rows);
                 }
             };
-            if (!serial[a] && most[a] <= 2) {
+            if (most[a] <= 2) {
                 rows_fast(std::false_type());
-            } else if (!serial[a]) {
+            } else if (most[a] <= 8) {
                 rows_fast(std::true_type());
             } else {
                 for (int r = 0; r < rows; ++r) {  // a warp on the serial path: every hole patched by its owner
