@@ -1171,7 +1171,9 @@ cudaError_t launch_dequant_stream(const DSParams &p, int fp32_out, cudaStream_t 
 // Int4 row kernel 10.8).  Either half alone loses: the staged values behind general loops take 15.9 us, the compile-time
 // device count without them 15.2.
 // ----------------------------------------------------------------------------------------------
-constexpr int DW_ROWS = 4, DW_MAX_DEV = 4, DW_MAIN = 640, DW_AUX = 96, DW_MAX_K = 384;
+constexpr int DW_ROWS = 4, DW_AUX = 96, DW_MAX_K = 384;
+// most groups of a row, by the devices whose steps a main thread keeps in registers
+__host__ __device__ constexpr int dw_main(int nd) { return nd > 4 ? 320 : 640; }
 
 struct DWParams {
     DSParams d;
@@ -1250,10 +1252,10 @@ __device__ __forceinline__ void dw_rows(const uint8_t *stage, uint32_t dev_bytes
 // first row (within the block's run) of the block's it-th stage: a short first stage lands sooner
 __device__ __forceinline__ int dw_stage_row(int it, int first) { return it == 0 ? 0 : first + (it - 1) * DW_ROWS; }
 
-// ND: 2 or 4, at least the number of devices.  A stage has room for ND; where there are fewer, the last ones have steps of 0
+// ND: 2, 4 or 8, at least the number of devices.  A stage has room for ND; where there are fewer, the last ones have steps of 0
 // and whatever bits lie in their part: every pattern decodes to a finite code, and fma(code, 0, acc) is acc (never -0).
 template <int B, int ND, bool FP32OUT, bool HAS_BIAS>
-__global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(const DWParams pp)
+__global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_rows(const DWParams pp)
 {
     extern __shared__ __align__(128) uint8_t dw_smem[];
     const DSParams &p = pp.d;
@@ -1528,13 +1530,17 @@ __global__ void __launch_bounds__(DW_MAIN + DW_AUX + 32, 1) dequant_stream_rows(
     }
 }
 
-int dw_nd(int N) { return N <= 2 ? 2 : 4; }
+int dw_nd(int N) { return N <= 2 ? 2 : N <= 4 ? 4 : 8; }
 
-// ring depth; 0: the shape is the panel kernel's
+// Ring depth; 0: the shape is the panel kernel's.  Five to eight devices: the 320 groups that a block has registers for, and rows
+// wide enough to give it warps (panel kernel and this one, us: 8 devices 1000 x 2304 11.5 and 7.3, 4000 x 2304 25.8 and 20.6,
+// 2000 x 2560 at 8 bits 20.1 and 13.2; 5 devices 15.2 and 12.2; 8 x 8000 x 1088 30.7 and 29.3, 5 devices 24.8 and 29.1; 8 x
+// 1000 x 576 4.9 and 5.9).
 int dw_stages(const tpq_ctx *c, int64_t out_stride)
 {
     const int L = c->E - c->k, G = (L + 7) / 8;
-    if (c->N > DW_MAX_DEV || c->E % 8 || out_stride % 8 || G > DW_MAIN || c->k > DW_MAX_K) return 0;
+    if (c->N > 4 && G < 160) return 0;
+    if (c->N > 8 || c->E % 8 || out_stride % 8 || G > dw_main(dw_nd(c->N)) || c->k > DW_MAX_K) return 0;
     int n = 4;
     while (n > 1 && dw_smem_bytes(dw_nd(c->N), dw_dev_bytes(L, c->bits), c->k, n) > (size_t)c->smem_optin) --n;
     return n > 1 ? n : 0;
@@ -1553,8 +1559,11 @@ cudaError_t launch_dequant_rows_nd(const DWParams &pp, int fp32_out, unsigned gr
 template <int B>
 cudaError_t launch_dequant_rows(const DWParams &pp, int fp32_out, unsigned grid, int threads, size_t smem, cudaStream_t st)
 {
-    return pp.d.N <= 2 ? launch_dequant_rows_nd<B, 2>(pp, fp32_out, grid, threads, smem, st)
-                       : launch_dequant_rows_nd<B, 4>(pp, fp32_out, grid, threads, smem, st);
+    switch (dw_nd(pp.d.N)) {
+    case 2: return launch_dequant_rows_nd<B, 2>(pp, fp32_out, grid, threads, smem, st);
+    case 4: return launch_dequant_rows_nd<B, 4>(pp, fp32_out, grid, threads, smem, st);
+    default: return launch_dequant_rows_nd<B, 8>(pp, fp32_out, grid, threads, smem, st);
+    }
 }
 
 }  // namespace

@@ -25,6 +25,9 @@ CASES = [  # N, T, E, k, bits, row padding, bias
     (4, 147, 5120, 0, 8, 0, True), (3, 297, 2048, 33, 6, 64, True), (4, 5, 1024, 380, 4, 0, True), (2, 149, 4096, 400, 4, 8, False),
     (1, 2, 64, 7, 7, 0, True), (4, 595, 512, 40, 2, 0, False),
     (1, 300, 5121, 5000, 4, 0, False), (2, 600, 200, 3, 3, 0, False), (1, 2500, 1000, 15, 4, 0, True),
+    # five to eight devices on the row kernel: its narrowest and widest rows and one group more or less, more than 96 selected
+    (5, 33, 1296, 17, 4, 0, True), (8, 149, 1272, 8, 3, 0, False), (8, 31, 2600, 40, 8, 8, True), (6, 20, 2608, 40, 6, 0, False),
+    (7, 13, 2312, 105, 5, 0, True), (8, 150, 2304, 0, 2, 0, False),
 ]
 
 
