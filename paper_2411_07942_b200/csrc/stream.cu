@@ -1180,6 +1180,7 @@ struct DWParams {
     const float *s_k;      // [N][E] steps, 0 at selected features
     const int32_t *pos;    // [E]
     int nstage;
+    int half_groups;       // (two blocks to a run of rows) groups of the first block
     uint32_t dev_bytes;    // a device's code words in a stage ...
     uint32_t hp_bytes;     // ... and its BF16 values
     int first;             // rows of a block's first stage
@@ -1188,6 +1189,8 @@ struct DWParams {
 };
 
 __host__ __device__ inline uint32_t dw_dev_bytes(int L, int B) { return (uint32_t)(((DW_ROWS * L * B + 127 + 127) / 128 + 1) * 16); }
+// (two blocks to a run of rows) a row's half in a stage
+__host__ __device__ inline uint32_t dw_pitch(int half_groups, int B) { return (uint32_t)((half_groups * 8 * B + 127 + 127) / 128 * 16); }
 __host__ __device__ inline uint32_t dw_hp_bytes(int k) { return k ? (uint32_t)(DW_ROWS * k * 2 + 14 + 15) & ~15u : 0u; }
 inline size_t dw_smem_bytes(int nd, uint32_t dev_bytes, int k, int nstage)
 {
@@ -1208,14 +1211,24 @@ __device__ __forceinline__ uint32_t dw_lds16(uint32_t a)
 }
 __device__ __forceinline__ void dw_sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 
-// ROWS rows of a stage for one main thread.  stage: its address, bit: the first bit of the thread's group in the first row.
+// ROWS rows of a stage, from its row r0 on, for one main thread.  stage: its address, rem: the bit of its first 16 bytes at which
+// its first row begins, g_bit: the first bit of the thread's group in a row.
 // ND devices, a number that the compiler knows: straight-line code, every device's words at the same place in its part.
-template <int B, int ND, int ROWS, bool FP32OUT, bool HAS_BIAS>
-__device__ __forceinline__ void dw_rows(const uint8_t *stage, uint32_t dev_bytes, uint32_t bit, uint32_t LB, const float2 (&sc)[ND][4],
-                                        const float2 (&b)[4], const DSConsts<B> &dc, uint8_t *out, int64_t out_row_bytes, int lanes)
+// SPLIT: a row's half lies by itself, DW_ROWS of them `pitch` bytes apart.
+template <bool SPLIT>
+__device__ __forceinline__ uint32_t dw_row_bit(uint32_t rem, int r, uint32_t LB, uint32_t pitch)
+{
+    return SPLIT ? (uint32_t)r * pitch * 8u + ((rem + (uint32_t)r * LB) & 127u) : rem + (uint32_t)r * LB;
+}
+
+template <int B, int ND, bool SPLIT, int ROWS, bool FP32OUT, bool HAS_BIAS>
+__device__ __forceinline__ void dw_rows(const uint8_t *stage, uint32_t dev_bytes, uint32_t rem, int r0, uint32_t LB, uint32_t pitch, uint32_t g_bit,
+                                        const float2 (&sc)[ND][4], const float2 (&b)[4], const DSConsts<B> &dc, uint8_t *out,
+                                        int64_t out_row_bytes, int lanes)
 {
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r, bit += LB, out += out_row_bytes) {
+    for (int r = 0; r < ROWS; ++r, out += out_row_bytes) {
+        const uint32_t bit = dw_row_bit<SPLIT>(rem, r0 + r, LB, pitch) + g_bit;
         const uint8_t *w = stage + (bit >> 5) * 4;
         float2 acc[4];
 #pragma unroll
@@ -1254,7 +1267,11 @@ __device__ __forceinline__ int dw_stage_row(int it, int first) { return it == 0 
 
 // ND: 2, 4 or 8, at least the number of devices.  A stage has room for ND; where there are fewer, the last ones have steps of 0
 // and whatever bits lie in their part: every pattern decodes to a finite code, and fma(code, 0, acc) is acc (never -0).
-template <int B, int ND, bool FP32OUT, bool HAS_BIAS>
+//
+// SPLIT (five to eight devices on rows of more than 320 groups): two blocks share a run of rows.  Each stages its half of every row (a
+// copy per device and row) and the BF16 rows, decodes its groups, adds up the selected features that lie among them (the
+// second block also those at or above L) and decodes the columns whose codes lie there.
+template <int B, int ND, bool SPLIT, bool FP32OUT, bool HAS_BIAS>
 __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_rows(const DWParams pp)
 {
     extern __shared__ __align__(128) uint8_t dw_smem[];
@@ -1266,8 +1283,12 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
     uint32_t *const sums = reinterpret_cast<uint32_t *>(dw_smem + (size_t)nstage * stage_bytes);  // [nstage][DW_ROWS][k]
     uint64_t *const full = reinterpret_cast<uint64_t *>(dw_smem + (((size_t)nstage * (stage_bytes + (size_t)DW_ROWS * k * 4) + 15) & ~(size_t)15));
     uint64_t *const empty = full + nstage, *const sums_ready = empty + nstage;
-    const int64_t t_begin = (int64_t)blockIdx.x * pp.rows_per_block;
+    const int64_t t_begin = (int64_t)(SPLIT ? blockIdx.x >> 1 : blockIdx.x) * pp.rows_per_block;
     const int rows_mine = (int)(p.T - t_begin < pp.rows_per_block ? p.T - t_begin : pp.rows_per_block);
+    const int half = SPLIT ? (int)(blockIdx.x & 1u) : 0;
+    const int g0 = half * pp.half_groups, g1 = SPLIT ? (half ? G : pp.half_groups) : G;  // this block's groups
+    const uint32_t bit0 = SPLIT ? (uint32_t)g0 * (8 * B) : 0u;                              // their first bit in a row
+    const uint32_t pitch = SPLIT ? dw_pitch(pp.half_groups, B) : 0u;
 
     tpq_grid_dep_launch();
     if (p.arr.words) {
@@ -1303,6 +1324,17 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
             const int64_t bit = (t_begin + r0) * (int64_t)LB, from = (bit >> 3) & ~(int64_t)15;
             const int64_t to = ((bit + (int64_t)rows * LB + 127) >> 7) << 4;  // (the code section is a multiple of 16 bytes)
             const uint32_t bytes = (uint32_t)(to - from), bar = smem_u32(&full[st]);
+            // SPLIT: lane 8 r + i copies device i's half of row r
+            uint32_t c_bytes = 0;
+            int64_t c_from = 0;
+            const int c_dev = lane & 7, c_row = lane >> 3;
+            if (SPLIT && c_dev < N && c_row < rows) {
+                const int64_t b0 = (t_begin + r0 + c_row) * (int64_t)LB + bit0;
+                const uint32_t n = half ? LB - bit0 : (uint32_t)pp.half_groups * (8 * B);
+                c_from = (b0 >> 3) & ~(int64_t)15;
+                c_bytes = (uint32_t)((((b0 + n + 127) >> 7) << 4) - c_from);
+            }
+            const uint32_t all = SPLIT ? __reduce_add_sync(0xffffffffu, c_bytes) : (uint32_t)N * bytes;
             const int64_t h_from = ((t_begin + r0) * k * 2) & ~(int64_t)15, h_all = (p.T * k * 2) & ~(int64_t)15;
             int64_t h_to = ((t_begin + r0 + rows) * k * 2 + 15) & ~(int64_t)15;
             if (h_to > h_all) h_to = h_all;
@@ -1313,16 +1345,19 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
                     atomicExch(pp.status, (int)TPQ_ERR_TIMEOUT);
                     ok = 0;
                 } else {
-                    mbar_expect_tx(bar, (uint32_t)N * (bytes + h_bytes));
+                    mbar_expect_tx(bar, all + (uint32_t)N * h_bytes);
                 }
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             const uint32_t stage = smem_u32(dw_smem) + (uint32_t)st * stage_bytes;
-            const int h_lane = lane - ND;
-            if (lane < N)
+            const int h_lane = SPLIT ? lane : lane - ND;
+            if (SPLIT) {
+                if (c_bytes) bulk_g2s(stage + (uint32_t)c_dev * pp.dev_bytes + (uint32_t)c_row * pitch, p.pl[c_dev] + c_from, c_bytes, bar);
+            } else if (lane < N) {
                 bulk_g2s(stage + (uint32_t)lane * pp.dev_bytes, p.pl[lane] + from, bytes, bar);
-            else if (h_lane >= 0 && h_lane < N && h_bytes)
+            }
+            if (h_lane >= 0 && h_lane < N && h_bytes)
                 bulk_g2s(stage + ND * pp.dev_bytes + (uint32_t)h_lane * pp.hp_bytes, p.pl[h_lane] + p.lp_bytes + h_from, h_bytes, bar);
             if (++st == nstage) {
                 st = 0;
@@ -1338,16 +1373,19 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
         // short rolled loops over what it has loaded once (this code runs once per stage and nobody else runs it, so that
         // straight-line code would pay an instruction fetch for every few instructions)
         const int at = tid - 32;
-        const bool on = at < k;
-        const int s_col = on ? __ldg(p.hp_idx + at) : 0;                       // rank `at`: its feature
-        const int ps = on ? __ldg(pp.pos + L + at) : -1;                       // column L + at: its slot (< 0: selected)
+        // (SPLIT: whether a feature below L, or a slot, lies among this block's groups; the second block takes the features above)
+        auto mine = [&](int c) { return !SPLIT || (c < L ? (c >> 3) >= g0 && (c >> 3) < g1 : half == 1); };
+        const int s_col = at < k ? __ldg(p.hp_idx + at) : 0;                    // rank `at`: its feature
+        const bool on = at < k && mine(s_col);
+        int ps = at < k ? __ldg(pp.pos + L + at) : -1;                          // column L + at: its slot (< 0: selected)
+        if (ps >= 0 && !mine(ps)) ps = -1;
         float c_s[ND];
 #pragma unroll
         for (int i = 0; i < ND; ++i) c_s[i] = i < N && ps >= 0 ? __ldg(pp.s_k + (size_t)i * E + L + at) : 0.0f;
         asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
         if (HAS_BIAS) tpq_grid_dep_wait();  // (the kernel ahead may be writing it)
-        float s_b = HAS_BIAS && on ? p.bias[s_col] : 0.0f, c_b = HAS_BIAS && on ? p.bias[L + at] : 0.0f;
-        uint32_t c_bit = (uint32_t)(ps >= 0 ? ps : 0) * B;
+        float s_b = HAS_BIAS && on ? p.bias[s_col] : 0.0f, c_b = HAS_BIAS && ps >= 0 ? p.bias[L + at] : 0.0f;
+        uint32_t c_bit = ps >= 0 ? (uint32_t)ps * B - bit0 : 0u;
         asm volatile("" : "+r"(c_bit), "+f"(s_b), "+f"(c_b));
 #pragma unroll
         for (int i = 0; i < ND; ++i) asm volatile("" : "+f"(c_s[i]));
@@ -1392,6 +1430,7 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
             // more selected features than threads, and the payload's last rows (a value that no copy brought is read here)
             for (int h = whole ? at + DW_AUX : at; h < k; h += DW_AUX) {
                 const int col = __ldg(p.hp_idx + h);
+                if (!mine(col)) continue;
                 for (int r = 0; r < rows; ++r) {
                     const int e = r * k + h;
                     float v = 0.0f;
@@ -1408,12 +1447,12 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sums_ready[st]));  // (release: the sums are visible to whoever waits)
             // the last k columns: filler features, decoded from the holes' slots that carry them
-            const uint32_t rem = (uint32_t)((t0 * (int64_t)LB) & 127);
+            const uint32_t rem = (uint32_t)((t0 * (int64_t)LB + bit0) & 127);
             if (ps >= 0) {
-                uint32_t bit = rem + c_bit;
                 uint8_t *og = out0 + (int64_t)(L + at) * ESIZE;
 #pragma unroll 1
-                for (int r = 0; r < rows; ++r, bit += LB, og += out_row_bytes) {
+                for (int r = 0; r < rows; ++r, og += out_row_bytes) {
+                    const uint32_t bit = dw_row_bit<SPLIT>(rem, r, LB, pitch) + c_bit;
                     float v = 0.0f;
 #pragma unroll
                     for (int i = 0; i < ND; ++i) v = __fmaf_rn(code(stage + (uint32_t)i * pp.dev_bytes, bit), c_s[i], v);
@@ -1423,11 +1462,11 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
             }
             for (int h = at + DW_AUX; h < k; h += DW_AUX) {  // (more columns than threads)
                 const int slot = __ldg(pp.pos + L + h);
-                if (slot < 0) continue;
+                if (slot < 0 || !mine(slot)) continue;
                 for (int r = 0; r < rows; ++r) {
                     float v = 0.0f;
                     for (int i = 0; i < N; ++i)
-                        v = __fmaf_rn(code(stage + (uint32_t)i * pp.dev_bytes, rem + (uint32_t)r * LB + (uint32_t)slot * B),
+                        v = __fmaf_rn(code(stage + (uint32_t)i * pp.dev_bytes, dw_row_bit<SPLIT>(rem, r, LB, pitch) + (uint32_t)slot * B - bit0),
                                       __ldg(pp.s_k + (size_t)i * E + L + h), v);
                     if (HAS_BIAS) v = __fadd_rn(v, p.bias[L + h]);
                     ds_store_one<FP32OUT>(out0 + r * out_row_bytes, L + h, v);
@@ -1443,8 +1482,8 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
         return;
     }
     // ---------------- main warps
-    const int g = tid - 32 - DW_AUX;
-    const int lanes = L - 8 * g < 8 ? L - 8 * g : 8;  // slots of the group (the last one may be short, idle threads have none)
+    const int g = g0 + tid - 32 - DW_AUX;
+    const int lanes = g >= g1 ? 0 : L - 8 * g < 8 ? L - 8 * g : 8;  // slots of the group (the last one may be short, idle threads have none)
     float2 sc[ND][4], b[4];
     uint32_t mask = 0;
     int hb = 0;
@@ -1484,7 +1523,7 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
     constexpr int ESIZE = FP32OUT ? 4 : 2;
     const int64_t out_row_bytes = p.out_stride * ESIZE;
     uint8_t *out = static_cast<uint8_t *>(p.out) + t_begin * out_row_bytes + (lanes > 0 ? g : 0) * (8 * ESIZE);
-    const uint32_t g_bit = (uint32_t)(lanes > 0 ? g : 0) * (8 * B);
+    const uint32_t g_bit = (uint32_t)(lanes > 0 ? g - g0 : 0) * (8 * B);
     const bool warp_holes = __any_sync(0xffffffffu, mask != 0);
     for (int it = 0, r0 = 0; r0 < rows_mine; r0 = dw_stage_row(++it, pp.first)) {
         const int cap = it == 0 ? pp.first : DW_ROWS, rows = rows_mine - r0 < cap ? rows_mine - r0 : cap;
@@ -1493,13 +1532,13 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
             break;
         }
         const uint8_t *const stage = dw_smem + (size_t)st * stage_bytes;
-        const uint32_t bit = (uint32_t)(((t_begin + r0) * (int64_t)LB) & 127) + g_bit;
+        const uint32_t rem = (uint32_t)(((t_begin + r0) * (int64_t)LB + bit0) & 127);
         if (rows == DW_ROWS) {
-            dw_rows<B, ND, DW_ROWS, FP32OUT, HAS_BIAS>(stage, pp.dev_bytes, bit, LB, sc, b, dc, out, out_row_bytes, lanes);
+            dw_rows<B, ND, SPLIT, DW_ROWS, FP32OUT, HAS_BIAS>(stage, pp.dev_bytes, rem, 0, LB, pitch, g_bit, sc, b, dc, out, out_row_bytes, lanes);
         } else {
 #pragma unroll 1
             for (int r = 0; r < rows; ++r)
-                dw_rows<B, ND, 1, FP32OUT, HAS_BIAS>(stage, pp.dev_bytes, bit + (uint32_t)r * LB, LB, sc, b, dc, out + r * out_row_bytes, out_row_bytes, lanes);
+                dw_rows<B, ND, SPLIT, 1, FP32OUT, HAS_BIAS>(stage, pp.dev_bytes, rem, r, LB, pitch, g_bit, sc, b, dc, out + r * out_row_bytes, out_row_bytes, lanes);
         }
         if (warp_holes) {  // the selected features' lanes
             if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sums_ready[st]), parity))) {
@@ -1532,25 +1571,36 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
 
 int dw_nd(int N) { return N <= 2 ? 2 : N <= 4 ? 4 : 8; }
 
+// two blocks to a run of rows
+bool dw_split(const tpq_ctx *c) { return (c->E - c->k + 7) / 8 > dw_main(dw_nd(c->N)); }
+// a device's code words in a stage
+uint32_t dw_part_bytes(const tpq_ctx *c)
+{
+    const int L = c->E - c->k, G = (L + 7) / 8;
+    return dw_split(c) ? DW_ROWS * dw_pitch((G + 1) / 2, c->bits) : dw_dev_bytes(L, c->bits);
+}
+
 // Ring depth; 0: the shape is the panel kernel's.  Five to eight devices: the 320 groups that a block has registers for, and rows
 // wide enough to give it warps (panel kernel and this one, us: 8 devices 1000 x 2304 11.5 and 7.3, 4000 x 2304 25.8 and 20.6,
 // 2000 x 2560 at 8 bits 20.1 and 13.2; 5 devices 15.2 and 12.2; 8 x 8000 x 1088 30.7 and 29.3, 5 devices 24.8 and 29.1; 8 x
-// 1000 x 576 4.9 and 5.9).
-int dw_stages(const tpq_ctx *c, int64_t out_stride)
+// 1000 x 576 4.9 and 5.9).  Wider rows, two blocks to a run: six devices or more and up to 8 rows an SM (8 devices 64 x 4608 4.5
+// and 3.0, 1000 x 4608 13.3 and 12.9, at 8 bits 15.4 and 13.4; 6 devices 200 x 3008 4.2 and 3.9; 4000 x 4608 40.9 and 41.8; 5
+// devices 1000 x 4416 11.0 and 11.8).
+int dw_stages(const tpq_ctx *c, int64_t T, int64_t out_stride)
 {
     const int L = c->E - c->k, G = (L + 7) / 8;
-    if (c->N > 4 && G < 160) return 0;
-    if (c->N > 8 || c->E % 8 || out_stride % 8 || G > dw_main(dw_nd(c->N)) || c->k > DW_MAX_K) return 0;
+    if (c->N > 8 || c->E % 8 || out_stride % 8 || G > 640 || c->k > DW_MAX_K || (c->N > 4 && G < 160)) return 0;
+    if (dw_split(c) && (c->N < 6 || T > 8 * c->sm_count)) return 0;
     int n = 4;
-    while (n > 1 && dw_smem_bytes(dw_nd(c->N), dw_dev_bytes(L, c->bits), c->k, n) > (size_t)c->smem_optin) --n;
+    while (n > 1 && dw_smem_bytes(dw_nd(c->N), dw_part_bytes(c), c->k, n) > (size_t)c->smem_optin) --n;
     return n > 1 ? n : 0;
 }
 
-template <int B, int ND>
+template <int B, int ND, bool SPLIT>
 cudaError_t launch_dequant_rows_nd(const DWParams &pp, int fp32_out, unsigned grid, int threads, size_t smem, cudaStream_t st)
 {
-    auto kern = pp.d.bias ? (fp32_out ? dequant_stream_rows<B, ND, true, true> : dequant_stream_rows<B, ND, false, true>)
-                          : (fp32_out ? dequant_stream_rows<B, ND, true, false> : dequant_stream_rows<B, ND, false, false>);
+    auto kern = pp.d.bias ? (fp32_out ? dequant_stream_rows<B, ND, SPLIT, true, true> : dequant_stream_rows<B, ND, SPLIT, false, true>)
+                          : (fp32_out ? dequant_stream_rows<B, ND, SPLIT, true, false> : dequant_stream_rows<B, ND, SPLIT, false, false>);
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return tpq_launch_pdl(kern, dim3(grid), dim3(threads), smem, st, pp);
@@ -1560,10 +1610,12 @@ template <int B>
 cudaError_t launch_dequant_rows(const DWParams &pp, int fp32_out, unsigned grid, int threads, size_t smem, cudaStream_t st)
 {
     switch (dw_nd(pp.d.N)) {
-    case 2: return launch_dequant_rows_nd<B, 2>(pp, fp32_out, grid, threads, smem, st);
-    case 4: return launch_dequant_rows_nd<B, 4>(pp, fp32_out, grid, threads, smem, st);
-    default: return launch_dequant_rows_nd<B, 8>(pp, fp32_out, grid, threads, smem, st);
+    case 2: return launch_dequant_rows_nd<B, 2, false>(pp, fp32_out, grid, threads, smem, st);
+    case 4: return launch_dequant_rows_nd<B, 4, false>(pp, fp32_out, grid, threads, smem, st);
+    default: break;
     }
+    return pp.half_groups ? launch_dequant_rows_nd<B, 8, true>(pp, fp32_out, grid, threads, smem, st)
+                          : launch_dequant_rows_nd<B, 8, false>(pp, fp32_out, grid, threads, smem, st);
 }
 
 }  // namespace
@@ -1728,16 +1780,19 @@ cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *paylo
     p.vec = E % 8 == 0 && out_stride % 8 == 0;
     p.out = out; p.bias = c->call_bias; p.arr = c->call_arr;
     cudaError_t e;
-    if (const int nstage = dw_stages(c, out_stride)) {
+    if (const int nstage = dw_stages(c, T, out_stride)) {
         DWParams pp;
         pp.d = p;
         pp.s_k = c->t.s_k; pp.pos = c->t.pos; pp.nstage = nstage; pp.status = c->t.status;
-        pp.dev_bytes = dw_dev_bytes(L, c->bits);
+        pp.dev_bytes = dw_part_bytes(c);
         pp.hp_bytes = dw_hp_bytes(k);
-        pp.rows_per_block = (T + c->sm_count - 1) / c->sm_count;
+        pp.half_groups = dw_split(c) ? (G + 1) / 2 : 0;
+        const int per_run = pp.half_groups ? 2 : 1;
+        const int64_t runs = c->sm_count / per_run;
+        pp.rows_per_block = (T + runs - 1) / runs;
         pp.first = pp.rows_per_block > DW_ROWS ? 2 : DW_ROWS;
-        const unsigned grid = (unsigned)((T + pp.rows_per_block - 1) / pp.rows_per_block);
-        const int threads = 32 + DW_AUX + (G + 31) / 32 * 32;
+        const unsigned grid = (unsigned)((T + pp.rows_per_block - 1) / pp.rows_per_block * per_run);
+        const int threads = 32 + DW_AUX + ((pp.half_groups ? pp.half_groups : G) + 31) / 32 * 32;
         const size_t smem = dw_smem_bytes(dw_nd(c->N), pp.dev_bytes, k, nstage);
         switch (c->bits) {
         case 2: e = launch_dequant_rows<2>(pp, fp32_out, grid, threads, smem, st); break;
