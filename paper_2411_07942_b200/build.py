@@ -2,9 +2,11 @@
 from __future__ import annotations
 
 import os
+import shlex
 import subprocess
 import sys
 import sysconfig
+import warnings
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
@@ -38,23 +40,40 @@ def needs_build() -> bool:
 
 
 def build_calls(force: bool = False) -> Path:
+    """Compile the extension module.  Raises RuntimeError if that fails, and then leaves none behind: an older one might call the
+    library by another table."""
     src = CSRC / "calls.c"
     if not force and not _stale(CALLS, [src, INCLUDE / "tpq.h", Path(__file__)]):
         return CALLS
     tmp = CALLS.with_suffix(f".{os.getpid()}.tmp")
-    cmd = [os.environ.get("CC", "gcc"), "-std=c11", "-O2", "-Wall", "-fPIC", "-shared", f"-I{sysconfig.get_paths()['include']}",
-           f"-I{INCLUDE}", "-o", str(tmp), str(src)]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("calls.c:\n" + res.stdout + res.stderr)
+    cmd = [*shlex.split(os.environ.get("CC", "gcc")), "-std=c11", "-O2", "-Wall", "-fPIC", "-shared",
+           f"-I{sysconfig.get_paths()['include']}", f"-I{INCLUDE}", "-o", str(tmp), str(src)]
+    try:
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        failed = f"status {res.returncode}\n{res.stdout}{res.stderr}" if res.returncode != 0 else None
+    except OSError as e:   # no such compiler
+        failed = str(e)
+    if failed is not None:
+        CALLS.unlink(missing_ok=True)
+        raise RuntimeError("calls.c: " + failed)
     os.replace(tmp, CALLS)
     return CALLS
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
+    """Build the library, then the extension module.  The library needs no C compiler and no Python headers, and every call
+    can go through ctypes: where the module cannot be compiled, that is a warning."""
+    build_lib(force, verbose)
+    try:
+        build_calls(force)
+    except RuntimeError as e:
+        warnings.warn(f"the extension module is not built (the calls of a step will go through ctypes): {e}", RuntimeWarning)
+    return LIB
+
+
+def build_lib(force: bool = False, verbose: bool = False) -> Path:
     """Compile every translation unit to an object file (only the stale ones unless ``force``), side by side,
-    and link them into libtpq.so; build the extension module."""
-    build_calls(force)
+    and link them into libtpq.so."""
     if not force and not needs_build():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -184,3 +184,22 @@ def test_extension_calls_pass_on_what_ctypes_would(lib):
         assert e.value.status == binding.TPQ_ERR_INVALID_ARG
     with pytest.raises(AssertionError):
         t.quantize_pack_batch(0, [16, 16], 1, [16], 9)
+
+
+@pytest.mark.parametrize("cc", ["no-such-compiler", "false", "sh -c 'exit 1'"])
+def test_library_is_built_without_a_compiler_for_the_extension(lib, monkeypatch, tmp_path, cc):
+    """The C library needs neither a C compiler nor the Python headers: build() brings it about and warns; an extension module
+    that is out of date does not stay behind."""
+    from paper_2411_07942_b200 import build
+
+    order = []
+    monkeypatch.setattr(build, "build_lib", lambda force=False, verbose=False: order.append("lib"), raising=False)
+    compile_calls = build.build_calls
+    monkeypatch.setattr(build, "build_calls", lambda force=False: (order.append("calls"), compile_calls(force)))
+    monkeypatch.setenv("CC", cc)
+    monkeypatch.setattr(build, "CALLS", tmp_path / build.CALLS.name)
+    build.CALLS.write_bytes(b"built from another source")
+    os.utime(build.CALLS, (0, 0))
+    with pytest.warns(RuntimeWarning, match="calls.c"):
+        assert build.build() == build.LIB
+    assert order == ["lib", "calls"] and not build.CALLS.exists()
