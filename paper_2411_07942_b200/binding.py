@@ -1,5 +1,7 @@
-"""ctypes front end of libtpq.so: the same names as include/tpq.h, argument
+"""Python front end of libtpq.so: the same names as include/tpq.h, argument
 marshalling only.  Every step of the method runs in the library's CUDA kernels.
+The calls of a step with plain arguments go through the extension module
+_calls (csrc/calls.c) where it is built, everything else through ctypes.
 
 torch is used by callers for device memory and streams; this module only needs
 ``tensor.data_ptr()`` values and raw stream handles.  There is no CPU fallback:
@@ -10,6 +12,7 @@ from __future__ import annotations
 import ctypes
 import struct
 import types
+import warnings
 from ctypes import POINTER, byref, c_char_p, c_double, c_float, c_int, c_int32, c_int64, c_size_t, c_void_p
 from pathlib import Path
 
@@ -79,6 +82,10 @@ _lib = None
 _calls = None   # the extension module (csrc/calls.c): the calls of a step with plain arguments; it returns None for others
 _CALLS = ("tpq_calibrate_ranges", "tpq_quantize_pack", "tpq_quantize_pack_batch", "tpq_dequant_reduce", "tpq_dequant_reduce_bias",
           "tpq_dequant_reduce_arrivals", "tpq_quantize_pack_push", "tpq_linear_quantize_pack")   # in the order of its table
+# where that module cannot be loaded: every call of its functions is left to ctypes
+_ctypes_only = types.SimpleNamespace(**{f: lambda *args: None for f in (
+    "calibrate_ranges", "quantize_pack", "quantize_pack_batch", "dequant_reduce", "dequant_reduce_arrivals", "quantize_pack_push",
+    "linear_quantize_pack")})
 _fast = types.SimpleNamespace()   # the calls below that take pointer arrays, as functions that take what _ptrs returns
 _FAST = ("tpq_quantize_pack_batch", "tpq_dequant_reduce", "tpq_dequant_reduce_bias", "tpq_quantize_pack_push",
          "tpq_dequant_reduce_arrivals")
@@ -103,9 +110,11 @@ def lib() -> ctypes.CDLL:
             setattr(_fast, name, fn)
         try:
             from . import _calls as calls
-        except ImportError as e:
-            raise RuntimeError("the extension module _calls is missing: run `python -m paper_2411_07942_b200.build`") from e
-        calls.bind([ctypes.cast(getattr(L, name), c_void_p).value for name in _CALLS])
+            calls.bind([ctypes.cast(getattr(L, name), c_void_p).value for name in _CALLS])
+        except (ImportError, ValueError) as e:   # not built, or built for another interpreter or table
+            warnings.warn(f"the extension module _calls cannot be used ({e}): every call goes through ctypes, 1 to 2 us slower "
+                          "each; `python -m paper_2411_07942_b200.build` builds it", RuntimeWarning)
+            calls = _ctypes_only
         _calls = calls
         _lib = L
     return _lib
@@ -121,7 +130,7 @@ _PACK = [struct.Struct(f"{n}Q").pack for n in range(65)]   # by the number of po
 
 
 def _ptrs(ptrs):
-    """A host array of device pointers.  Sequences of plain integers are packed into bytes (a quarter of the time that
+    """A host array of device pointers, for the calls that ctypes makes.  Sequences of plain integers are packed into bytes (a quarter of the time that
     building a ctypes array takes); what else c_void_p takes (None, c_void_p) goes into a ctypes array, and ctypes arrays
     must be of c_void_p: other objects, numbers that are no addresses among them, are refused as the C signature refuses
     them."""

@@ -203,3 +203,35 @@ def test_library_is_built_without_a_compiler_for_the_extension(lib, monkeypatch,
     with pytest.warns(RuntimeWarning, match="calls.c"):
         assert build.build() == build.LIB
     assert order == ["lib", "calls"] and not build.CALLS.exists()
+
+
+def test_library_loads_without_the_extension_module(lib):
+    """Where the extension module is not there, a warning says so and every call goes through ctypes."""
+    import subprocess
+    import sys
+
+    code = """
+import sys, warnings
+sys.modules["paper_2411_07942_b200._calls"] = None   # (an import of it fails)
+from paper_2411_07942_b200 import binding
+with warnings.catch_warnings(record=True) as w:
+    warnings.simplefilter("always")
+    binding.lib()
+assert [x.category for x in w] == [RuntimeWarning] and "_calls" in str(w[0].message)
+import ctypes
+t = binding.Tpq.__new__(binding.Tpq)   # a closed context: what the library itself answers
+t._h, t._p, t.N, t.E = ctypes.c_void_p(), None, 2, 8
+calls = [lambda: t.calibrate_ranges(0, 16, 1, 1), lambda: t.quantize_pack(0, 16, 1, 16, 9),
+         lambda: t.quantize_pack_batch(0, [16, 16], 1, [16, 16], 9), lambda: t.dequant_reduce([16, 16], 1, 16),
+         lambda: t.dequant_reduce([16, 16], 1, 16, bias_ptr=16), lambda: t.dequant_reduce([16, 16], 1, 16, arrived_ptr=16, epoch=1),
+         lambda: t.quantize_pack_push(0, 16, 1, [16], [16], 9, 1), lambda: t.linear_quantize_pack(0, 16, 16, 1, 8, 16, 9)]
+for call in calls:
+    try:
+        call()
+    except binding.TpqError as e:
+        assert e.status == binding.TPQ_ERR_INVALID_ARG
+    else:
+        raise AssertionError("no error")
+"""
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
