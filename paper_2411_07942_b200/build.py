@@ -1,4 +1,4 @@
-"""Build libtpq.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the extension module _calls.so."""
+"""Build libtpq.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the extension module _calls."""
 from __future__ import annotations
 
 import os
@@ -13,7 +13,9 @@ PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 INCLUDE = PKG.parent / "include"
 LIB = PKG / "libtpq.so"
-CALLS = PKG / "_calls.so"   # csrc/calls.c: the step's calls for Python (binding.py)
+# csrc/calls.c: the step's calls for Python (binding.py).  Its name says which interpreter it is built for, so that no other one
+# takes it for its own.
+CALLS = PKG / f"_calls{sysconfig.get_config_var('EXT_SUFFIX')}"
 
 OBJ = PKG / "build"   # object files (git-ignored)
 
@@ -43,6 +45,7 @@ def build_calls(force: bool = False) -> Path:
     """Compile the extension module.  Raises RuntimeError if that fails, and then leaves none behind: an older one might call the
     library by another table."""
     src = CSRC / "calls.c"
+    (CALLS.parent / "_calls.so").unlink(missing_ok=True)   # (without a tag: any interpreter would load it)
     if not force and not _stale(CALLS, [src, INCLUDE / "tpq.h", Path(__file__)]):
         return CALLS
     tmp = CALLS.with_suffix(f".{os.getpid()}.tmp")

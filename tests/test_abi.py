@@ -235,3 +235,17 @@ for call in calls:
 """
     res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert res.returncode == 0, res.stderr
+
+
+def test_extension_module_is_of_this_interpreter(lib, monkeypatch, tmp_path):
+    """Its file name carries the interpreter's tag, that file is the one loaded, and one without a tag does not stay."""
+    import sysconfig
+
+    from paper_2411_07942_b200 import binding, build
+
+    assert build.CALLS.name == "_calls" + sysconfig.get_config_var("EXT_SUFFIX") != "_calls.so"
+    assert os.path.samefile(binding._calls.__file__, build.CALLS)
+    monkeypatch.setattr(build, "CALLS", tmp_path / build.CALLS.name)
+    (tmp_path / "_calls.so").write_bytes(b"built for another interpreter")
+    build.build_calls()
+    assert sorted(os.listdir(tmp_path)) == [build.CALLS.name]
