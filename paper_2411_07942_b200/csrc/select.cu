@@ -10,8 +10,16 @@ namespace {
 // RG_N devices are in flight together, and blocks of 64 features spread them over the GPU.)
 constexpr int RG_THREADS = 64, RG_N = 8;
 
+// The order of aggregated ranges as integers: -0 and +0 are equal, and a NaN (calibrated on or restored) has a place, ahead of
+// the infinities, so that exactly k features are selected whatever the ranges are; the tables rely on that.
+__device__ __forceinline__ int order_key(float x)
+{
+    const int i = __float_as_int(__fadd_rn(x, 0.0f));  // (-0 -> +0, any NaN -> the positive one)
+    return i ^ ((i >> 31) & 0x7FFFFFFF);
+}
+
 __global__ void __launch_bounds__(RG_THREADS) ranges_kernel(const float *m, const float *M, int N, int E, float levels, float *R,
-                                                            float *Rbar, float *s, float *inv_s)
+                                                            float *Rbar, int32_t *key, float *s, float *inv_s)
 {
     tpq_grid_dep_launch();
     tpq_grid_dep_wait();
@@ -42,39 +50,35 @@ __global__ void __launch_bounds__(RG_THREADS) ranges_kernel(const float *m, cons
             }
     }
     Rbar[j] = acc;
+    key[j] = order_key(acc);
 }
 
 // Feature j is selected iff fewer than k features beat it, where a beats j when
 // Rbar_a > Rbar_j, or Rbar_a == Rbar_j and a < j.  O(E^2) comparisons, a warp per feature: its lanes compare side by
-// side, four values per load (Rbar is a few tens of KB, so the loads hit L1).  (One thread per feature, the values
+// side, four values per load (a few tens of KB, so the loads hit L1).  (One thread per feature, the values
 // through shared memory, left all but 18 SMs idle: 68 us at E = 4608.)
-// The values are compared as integers of the same order, which also gives a NaN (calibrated on or restored) a place, ahead
-// of the infinities: exactly k features are selected whatever the ranges are, and the tables rely on that.
+// The keys are made once, by the kernel ahead, and those ahead of j's own four are compared with one less: a comparison and an
+// addition each.  (With the key made anew at every comparison, us per call: 2 x 32768 380 and now 203, 2 x 131072 5250 and
+// 2460; as comparisons of the values and their places 310 and 4100.)
 constexpr int TK_WARPS = 8;
 
-__device__ __forceinline__ int order_key(float x)
-{
-    const int i = __float_as_int(__fadd_rn(x, 0.0f));  // (-0 -> +0, any NaN -> the positive one)
-    return i ^ ((i >> 31) & 0x7FFFFFFF);
-}
-
-__global__ void __launch_bounds__(32 * TK_WARPS) topk_flags_kernel(const float *Rbar, int E, int k, uint8_t *flag)
+__global__ void __launch_bounds__(32 * TK_WARPS) topk_flags_kernel(const int32_t *key, int E, int k, uint8_t *flag)
 {
     tpq_grid_dep_launch();
-    tpq_grid_dep_wait();  // (the ranges are the kernel ahead's)
+    tpq_grid_dep_wait();  // (the keys are the kernel ahead's)
     const int j = blockIdx.x * TK_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= E) return;
-    const int mine = order_key(Rbar[j]);
+    const int mine = key[j], least = mine - 1;  // (no key is the least integer)
     int beats = 0;
-    const int E4 = E >> 2;
-    auto beaten = [&](float v, int a) { return order_key(v) > mine - (a < j) ? 1 : 0; };
+    const int E4 = E >> 2, jq = j >> 2;
 #pragma unroll 4
     for (int q = lane; q < E4; q += 32) {
-        const float4 v = reinterpret_cast<const float4 *>(Rbar)[q];
-        const int a = 4 * q;
-        beats += beaten(v.x, a) + beaten(v.y, a + 1) + beaten(v.z, a + 2) + beaten(v.w, a + 3);
+        const int4 v = reinterpret_cast<const int4 *>(key)[q];
+        const int than = q < jq ? least : mine;
+        beats += (v.x > than) + (v.y > than) + (v.z > than) + (v.w > than);
     }
-    if (lane < (E & 3)) beats += beaten(Rbar[4 * E4 + lane], 4 * E4 + lane);
+    if (lane < (E & 3)) beats += key[4 * E4 + lane] > mine;
+    if (lane < (j & 3)) beats += key[4 * jq + lane] == mine;  // j's own four
     beats = __reduce_add_sync(0xffffffffu, beats);
     if (lane == 0) flag[j] = beats < k ? 1 : 0;
 }
@@ -252,13 +256,13 @@ cudaError_t tpq_launch_ranges(const tpq_tables &t, int N, int E, int bits, cudaS
 {
     ++*launches;
     return tpq_launch_pdl(ranges_kernel, dim3((E + RG_THREADS - 1) / RG_THREADS), dim3(RG_THREADS), 0, st, t.m, t.M, N, E,
-                          (float)((1 << bits) - 1), t.R, t.Rbar, t.s, t.inv_s);
+                          (float)((1 << bits) - 1), t.R, t.Rbar, t.key, t.s, t.inv_s);
 }
 
 cudaError_t tpq_launch_topk_flags(const tpq_tables &t, int E, int k, cudaStream_t st, int64_t *launches)
 {
     ++*launches;
-    return tpq_launch_pdl(topk_flags_kernel, dim3((E + TK_WARPS - 1) / TK_WARPS), dim3(32 * TK_WARPS), 0, st, t.Rbar, E, k, t.flag);
+    return tpq_launch_pdl(topk_flags_kernel, dim3((E + TK_WARPS - 1) / TK_WARPS), dim3(32 * TK_WARPS), 0, st, t.key, E, k, t.flag);
 }
 
 cudaError_t tpq_launch_tables(const tpq_tables &t, int N, int E, int k, cudaStream_t st, int64_t *launches)

@@ -14,6 +14,7 @@ struct tpq_tables {
     float *m, *M;        // [N][E] running minimum / maximum, Eq. (1)-(2)
     float *R;            // [N][E] symmetric range 2 max(-m, M)
     float *Rbar;         // [E]    aggregated range
+    int32_t *key;        // [E]    the same as an integer of the same order (select.cu)
     float *s, *inv_s;    // [N][E] Int4 step and its reciprocal
     float *s_k;          // [N][E] step with 0 at selected features (dequantiser's copy)
     float *s_slot;       // [N][E] step of the feature held by code slot c (slot order; 0 for c >= E-k)

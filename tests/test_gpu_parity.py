@@ -868,3 +868,16 @@ def test_selection_takes_k_features_of_ranges_that_are_not_numbers():
     assert t.select_features(k).tolist() == [3, 77, 120, 197, 198, 199]
     assert sorted(t.get_slot_order().tolist()) == [j for j in range(E) if j not in (3, 77, 120, 197, 198, 199)]
     t.close()
+
+
+@pytest.mark.parametrize("E", [1, 5, 8, 33, 1000, 4097])
+def test_selection_among_equal_ranges(E):
+    """Few distinct ranges, zeros of both signs and negative ones among them: ties go to the lower feature wherever they lie
+    among the groups of four that the selector compares."""
+    rng = np.random.default_rng(E)
+    M = rng.choice(np.array([-1.5, -0.0, 0.0, 2.0, 2.5], np.float32), E)
+    t = binding.Tpq(1, E)
+    t.set_ranges(-M[None], M[None], [1])
+    for k in sorted({0, 1, E // 3, E // 2, E - 1, E}):
+        assert t.select_features(k).tolist() == sorted(np.argsort(-M, kind="stable")[:k].tolist())
+    t.close()
