@@ -607,7 +607,9 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
             };
             // QS_STAGE independent rows (a short stage's missing ones hold old bytes and are never written)
             // (DEEP: a warp that has a lane with more than two holes, see quantize_tiled: 4 x 2048 x 5120 of 51 selected 36.4 us a
-            // launch on the serial path, 23.2 so; 8 x 1000 x 4608 at 8 bits 38.1 and 26.6)
+            // launch on the serial path, 23.2 so; 8 x 1000 x 4608 at 8 bits 38.1 and 26.6.  What it works out of the mask is kept
+            // from the compiler: moved out of the loop over the stages it cost every warp of two groups a lane its registers,
+            // 8 x 2048 x 8192 at 8 bits 99.7 us without this path, 106.9 with it, 101 so)
             auto rows_fast = [&](auto deep_tag) {
                 constexpr bool DEEP = decltype(deep_tag)::value;
                 uint4 v[QS_STAGE];
@@ -635,14 +637,17 @@ __global__ void __launch_bounds__(QS_MAX_THREADS, 1) quantize_stream(const QPipe
                     if (!DEEP) emit(r, wd[r], r < rows);
                 }
                 if constexpr (DEEP) {  // the third and further holes
-                    uint32_t m = mask[a] & (mask[a] - 1);
+                    uint32_t m = mask[a];
+                    int s0 = src0[a];
+                    asm volatile("" : "+r"(m), "+r"(s0));
+                    m &= m - 1;
                     m &= m - 1;
                     for (int h = 2; h < most[a]; ++h, m &= m - 1) {
                         const int n = m ? __ffs(m) - 1 : 0;
                         const uint32_t sh = qs_field_shift<B>(n);
 #pragma unroll
                         for (int r = 0; r < QS_STAGE; ++r) {
-                            const uint32_t c = __shfl_sync(0xffffffffu, fx[r], src0[a] + h);
+                            const uint32_t c = __shfl_sync(0xffffffffu, fx[r], s0 + h);
 #pragma unroll
                             for (int j = 0; j < NW; ++j) {
                                 const uint32_t fm = m && qs_field_in<B>(n, j) ? ((1u << B) - 1u) << sh : 0u;
