@@ -377,14 +377,17 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
                         word[r] = (word[r] & keep[a]) | (q0 & hmask[a][0]) | (q1 & hmask[a][1]);
                     }
                     if constexpr (DEEP) {  // the third and further holes
-                        uint32_t m = mask[a] & (mask[a] - 1);
+                        uint32_t m = mask[a];
+                        int s0 = src0[a];
+                        asm volatile("" : "+r"(m), "+r"(s0));  // (what follows from them stays here, out of every warp's registers)
+                        m &= m - 1;
                         m &= m - 1;
                         for (int h = 2; h < most[a]; ++h, m &= m - 1) {
                             const int at = m ? (__ffs(m) - 1) * 4 : 0;
                             const uint32_t field = m ? 0xFu << at : 0u;
 #pragma unroll
                             for (int r = 0; r < GR; ++r)
-                                word[r] = (word[r] & ~field) | (__shfl_sync(0xffffffffu, qv[r], src0[a] + h) << at & field);
+                                word[r] = (word[r] & ~field) | (__shfl_sync(0xffffffffu, qv[r], s0 + h) << at & field);
                         }
                     }
                 }
@@ -393,11 +396,13 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
                         for (int d = 0; d < p.n_dst; ++d) {
                             uint32_t *const o = reinterpret_cast<uint32_t *>(p.payload[d]) + (t0 + rb) * L8 + g;
 #pragma unroll
-                            for (int r = 0; r < GR; ++r) o[r * L8] = word[r];
+                            for (int r = 0; r < GR; ++r)
+                                if (!DEEP || rb + r < rows) o[r * L8] = word[r];
                         }
                     } else {
 #pragma unroll
-                        for (int r = 0; r < GR; ++r) lp_out[(t0 + rb + r) * L8 + g] = word[r];
+                        for (int r = 0; r < GR; ++r)
+                            if (!DEEP || rb + r < rows) lp_out[(t0 + rb + r) * L8 + g] = word[r];
                     }
                 }
             };
@@ -410,7 +415,12 @@ __global__ void __launch_bounds__(TB, 1) quantize_tiled(const QPParams p)
             if (most[a] <= 2) {  // (uniform over the warp, like the row counts above)
                 stage_fast(std::false_type());
             } else if (most[a] <= 8) {
-                stage_fast(std::true_type());
+                // (One group a lane: one copy of this code for any number of rows -- a short stage's missing ones hold old bytes
+                // and are not stored -- because a copy per row count cost the warps that never run it up to 5 %: 8 x 2048 x 6144
+                // 42.4 us without this path, 44.7 with three copies, 43.3 with one.  Two groups a lane the other way round:
+                // 16 x 2048 x 8192 112.4, 112.9 and 115.0.)
+                if constexpr (GPT == 1) rows_fast(std::integral_constant<int, G>(), std::true_type(), 0);
+                else stage_fast(std::true_type());
             } else if (live) {
                 // a warp on the serial path: every hole patched by its owner
                 for (int r = 0; r < rows; ++r) {
