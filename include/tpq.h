@@ -139,7 +139,8 @@ tpq_status tpq_calibrate_ranges_noalloc(tpq_ctx *ctx, int shard, const void *y_b
 
 /* Section 3 "Selecting High Precision Features": R^(i)_j = 2 max(-m, M),
  * aggregated range Rbar_j = sum_i R^(i)_j (binary32, devices ascending), the
- * k features with the largest Rbar_j (ties: lower index) become the BF16 set;
+ * k features with the largest Rbar_j (ties: lower index; a NaN ranks above
+ * every number) become the BF16 set;
  * every other feature gets its static Int4 step s = R/15 (floored at 2^-23)
  * and reciprocal.  k < 0 selects the paper's k = floor(E/64) (Section 4).
  * Every device must have been calibrated with at least one sequence

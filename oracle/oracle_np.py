@@ -98,10 +98,10 @@ def calibrate(m, M, count: int, y_bits: np.ndarray, gamma):
 
 
 def ranges(m: np.ndarray, M: np.ndarray):
-    """R^(i)_j = 2 max(-m, M) and R-bar_j = sum over devices (ascending, float32)."""
+    """R^(i)_j = 2 max(-m, M), where -m > M decides, and R-bar_j = sum over devices (ascending, float32)."""
     m = np.asarray(m, dtype=F32)
     M = np.asarray(M, dtype=F32)
-    R = (F32(2.0) * np.maximum(-m, M)).astype(F32)
+    R = (F32(2.0) * np.where(-m > M, -m, M)).astype(F32)
     Rbar = R[0].copy()
     for i in range(1, R.shape[0]):
         Rbar = (Rbar + R[i]).astype(F32)
@@ -114,9 +114,9 @@ def default_k(E: int) -> int:
 
 
 def select(Rbar: np.ndarray, k: int) -> np.ndarray:
-    """Top-k features by R-bar; ties to the lower index; returned ascending."""
+    """Top-k features by R-bar (a NaN ranks above every number); ties to the lower index; returned ascending."""
     E = Rbar.shape[0]
-    order = sorted(range(E), key=lambda j: (-float(Rbar[j]), j))
+    order = sorted(range(E), key=lambda j: (0.0, 0.0, j) if np.isnan(Rbar[j]) else (1.0, -float(Rbar[j]), j))
     return np.array(sorted(order[:k]), dtype=np.int32)
 
 

@@ -170,9 +170,13 @@ void tpqo_ranges(const float *m, const float *M, int64_t N, int64_t E,
 
 /* Section 3 "Selecting High Precision Features": the k features with the
  * largest R-bar_j; the set is the same for every sequence and device.
- * Reading: equal R-bar -> the lower feature index wins; the set is returned
- * sorted by feature index, ascending.  Written as k rounds of "take the best
- * remaining feature" so that it is visibly the definition of top-k. */
+ * Reading: equal R-bar -> the lower feature index wins; an R-bar that is NaN
+ * (no step can be made of it) ranks above every number, NaNs among themselves
+ * as equals; the set is returned sorted by feature index, ascending.  Written
+ * as k rounds of "take the best remaining feature" so that it is visibly the
+ * definition of top-k. */
+static int ranks_above(float a, float b) { return isnan(a) ? !isnan(b) : a > b; }
+
 void tpqo_select(const float *Rbar, int64_t E, int64_t k, int32_t *hp_idx)
 {
     unsigned char *taken = (unsigned char *)calloc((size_t)E, 1);
@@ -180,7 +184,7 @@ void tpqo_select(const float *Rbar, int64_t E, int64_t k, int32_t *hp_idx)
         int64_t best = -1;
         for (int64_t j = 0; j < E; ++j) {
             if (taken[j]) continue;
-            if (best < 0 || Rbar[j] > Rbar[best]) best = j;  /* strict: lower j wins ties */
+            if (best < 0 || ranks_above(Rbar[j], Rbar[best])) best = j;  /* strict: lower j wins ties */
         }
         if (best < 0) break;          /* k > E: everything is taken already */
         taken[best] = 1;

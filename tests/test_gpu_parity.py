@@ -758,6 +758,13 @@ def test_bias_from_the_call_ahead(N, T, E, k, bits):
     t.close()
 
 
+@pytest.mark.parametrize("N,T,E,k,bits", [(3, 297, 1024, 15, 4), (6, 147, 2304, 37, 4), (8, 147, 2304, 36, 3), (6, 64, 4608, 70, 6),
+                                         (8, 64, 4608, 72, 8)])
+def test_bias_from_the_call_ahead_of_more_devices(N, T, E, k, bits):
+    """As above on the bit-stream row kernel for three and for five to eight devices, one and (the last two) two blocks to a run."""
+    test_bias_from_the_call_ahead(N, T, E, k, bits)
+
+
 @pytest.mark.parametrize("T,E,k,bits", [(64, 1000, 15, 4), (300, 1033, 9, 4), (297, 1024, 16, 3), (200, 1024, 16, 4), (40, 11264, 11, 4)])
 def test_inputs_from_the_call_ahead(T, E, k, bits):
     """Quantisation and calibration of what the reduction right ahead in the stream writes, with all launches queued when the
@@ -880,4 +887,20 @@ def test_selection_among_equal_ranges(E):
     t.set_ranges(-M[None], M[None], [1])
     for k in sorted({0, 1, E // 3, E // 2, E - 1, E}):
         assert t.select_features(k).tolist() == sorted(np.argsort(-M, kind="stable")[:k].tolist())
+    t.close()
+
+
+@pytest.mark.parametrize("E,N", [(200, 1), (1033, 3), (33000, 2)])
+def test_selection_of_any_ranges_is_the_oracles(E, N):
+    """NaNs in the minima, the maxima or both, infinities, zeros and equal values: the oracle's ranges and set."""
+    rng = np.random.default_rng(E)
+    special = np.array([np.nan, np.inf, -np.inf, 0.0, -0.0, 1.0], np.float32)
+    m, M = (np.where(rng.random((N, E)) < 0.1, rng.choice(special, (N, E)), rng.normal(0, 1, (N, E))).astype(np.float32) for _ in range(2))
+    orc, t = oracle.c(), binding.Tpq(N, E)
+    t.set_ranges(m, M, np.ones(N, np.int64))
+    R, Rbar = orc.ranges(m, M)
+    for k in (1, E // 64, E // 5, E // 2, E - 1):
+        assert t.select_features(k).tolist() == orc.select(Rbar, k).tolist(), k
+    got = t.get_ranges()
+    assert np.array_equal(got[2], R, equal_nan=True) and np.array_equal(got[3], Rbar, equal_nan=True)
     t.close()

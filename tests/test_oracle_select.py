@@ -37,6 +37,16 @@ def test_ties_lower_index_wins(corc, norc):
         assert orc.select(np.zeros(6, np.float32), 2).tolist() == [0, 1]
 
 
+def test_ranges_that_are_not_numbers_rank_first(corc, norc):
+    nan, inf = np.nan, np.inf
+    Rbar = np.array([1, nan, inf, 5, nan, -inf, 0], np.float32)
+    R = np.array([[2, 3, nan], [1, nan, 4]], np.float32)   # (m, M): -m > M decides, so a NaN minimum gives way to the maximum
+    for orc in (corc, norc):
+        for k, want in enumerate([[], [1], [1, 4], [1, 2, 4], [1, 2, 3, 4], [0, 1, 2, 3, 4], [0, 1, 2, 3, 4, 6], list(range(7))]):
+            assert orc.select(Rbar, k).tolist() == want
+        assert np.array_equal(orc.ranges(-R[:1], R[1:])[1], np.array([4, nan, 8], np.float32), equal_nan=True)
+
+
 def test_permuting_features_permutes_the_set(corc):
     rng = np.random.default_rng(9)
     Rbar = rng.lognormal(0, 1, 128).astype(np.float32)
