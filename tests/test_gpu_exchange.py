@@ -216,6 +216,13 @@ def test_bit_stream_reductions_with_their_own_wait(N, T, E, k, bits, path):
     t.close()
 
 
+@pytest.mark.parametrize("N,T,E,k,bits", [(3, 300, 1024, 51, 4), (6, 150, 2304, 37, 4), (8, 150, 2304, 36, 3), (6, 64, 4608, 70, 6),
+                                         (8, 64, 4608, 72, 8)])
+def test_row_reductions_of_more_devices_with_their_own_wait(N, T, E, k, bits):
+    """The bit-stream row kernel for three and for five to eight devices, one and (the last two) two blocks to a run of rows."""
+    test_bit_stream_reductions_with_their_own_wait(N, T, E, k, bits, binding.PATH_AUTO)
+
+
 @pytest.mark.parametrize("T,E,k,bits,pad,n_dst", [(1301, 1000, 15, 4, 0, 2), (700, 5120, 51, 4, 64, 1), (601, 8192, 128, 8, 0, 3),
                                                   (40, 8192, 100, 5, 8, 16), (3, 512, 9, 7, 0, 4), (900, 2048, 32, 2, 0, 16)])
 def test_push_of_the_bit_stream_quantiser(T, E, k, bits, pad, n_dst):

@@ -253,3 +253,88 @@ def test_groups_with_many_selected_features(bits):
         for a, b in zip(*got):
             assert np.array_equal(a, b), hp
     t.close()
+
+
+def _row_case(N, rows, short, E, k, bits, pad, split=False):
+    """A context with an arbitrary set (both ends of the feature range in it), its payloads (shape-generic quantiser) and T: `rows`
+    to a block of the row kernel, the last block `short` rows less."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    T = rows * (sms // 2 if split else sms) - short
+    rng = np.random.default_rng(E + T + k)
+    g = torch.Generator(device="cuda").manual_seed(E + T + k)
+    t = binding.Tpq(N, E, bits=bits)
+    M = rng.lognormal(0, 1, (N, E)).astype(np.float32)
+    t.set_ranges(-M, M, np.ones(N, np.int64))
+    ends = sorted({0, E - 1, E - k - 1, E - k} & set(range(E)))[:k]
+    t.set_features(sorted(ends + rng.permutation(sorted(set(range(E)) - set(ends)))[:k - len(ends)].tolist()))
+    P = t.payload_bytes(T)
+    t.set_option(binding.TPQ_OPT_KERNEL_PATH, binding.PATH_GENERIC)
+    pls = [torch.zeros(P, dtype=torch.uint8, device="cuda") for _ in range(N)]
+    for i in range(N):
+        y = (torch.randn((T, E), generator=g, device="cuda") * 2).to(torch.bfloat16)
+        t.quantize_pack(i, y.data_ptr(), T, pls[i].data_ptr(), P)
+    return t, T, pls
+
+
+@pytest.mark.parametrize("N,rows,short,E,k,bits,pad,with_bias,split", [
+    # rows of a block: whole stages, a short first or last one, more stages than the ring has, a last block with fewer;
+    # selected: none, one (its last values lie in the last rows of several blocks), more than the auxiliary threads, the most
+    (1, 9, 3, 1024, 7, 4, 0, True, False), (2, 14, 5, 2048, 1, 3, 8, False, False), (3, 7, 2, 1032, 105, 8, 0, True, False),
+    (3, 30, 1, 640, 3, 4, 64, False, False), (4, 6, 4, 5120, 80, 2, 0, True, False), (4, 21, 7, 512, 384, 5, 0, False, False),
+    (4, 2, 1, 1024, 1, 7, 0, True, False), (5, 5, 1, 2304, 37, 6, 0, True, False), (5, 14, 0, 1792, 0, 3, 8, False, False),
+    (6, 30, 11, 1808, 105, 8, 0, True, False), (6, 8, 3, 2048, 2, 4, 0, False, False), (7, 5, 2, 2600, 41, 5, 0, True, False),
+    (7, 18, 5, 2312, 384, 7, 0, False, False), (8, 14, 1, 2304, 36, 4, 0, True, False), (8, 30, 3, 1304, 1, 8, 8, False, False),
+    (6, 4, 2, 2608, 40, 6, 0, True, True), (6, 16, 3, 4608, 105, 8, 8, False, True), (7, 14, 5, 5120, 384, 5, 0, True, True),
+    (8, 14, 2, 4608, 72, 8, 0, True, True), (8, 9, 0, 5120, 51, 4, 0, False, True), (8, 2, 1, 3008, 1, 8, 0, True, True),
+    (8, 15, 5, 4608, 0, 6, 8, False, True)])
+def test_row_kernel_stages(N, rows, short, E, k, bits, pad, with_bias, split):
+    """The bit-stream row kernel for one to eight devices, one and two blocks to a run of rows, against the shape-generic kernel,
+    bit for bit."""
+    t, T, pls = _row_case(N, rows, short, E, k, bits, pad, split)
+    bias = torch.randn(E, generator=torch.Generator(device="cuda").manual_seed(k), device="cuda")
+    ptrs = [p.data_ptr() for p in pls]
+    for dt, size in ((binding.TPQ_OUT_FP32, 4), (binding.TPQ_OUT_BF16, 2)):
+        got = []
+        for path in (binding.PATH_GENERIC, binding.PATH_AUTO):
+            t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+            whole, out = gu.guarded(T * (E + pad) * size)
+            call = lambda: t.dequant_reduce(ptrs, T, out.data_ptr(), dt, out_row_stride=E + pad, bias_ptr=bias.data_ptr() if with_bias else None)
+            if path == binding.PATH_AUTO:
+                assert "dequant_stream_rows<" in _kernels(call)
+            else:
+                call()
+            torch.cuda.synchronize()
+            assert t.device_status() == 0 and gu.guards_intact(whole, T * (E + pad) * size)
+            got.append(out)
+        assert torch.equal(*got)
+    t.close()
+
+
+@pytest.mark.parametrize("N,rows,short,E,k,bits,split", [(4, 3, 1, 1024, 3, 4, False), (2, 7, 0, 2048, 1, 3, False), (6, 5, 2, 2304, 35, 4, False),
+                                                         (8, 9, 1, 4608, 5, 8, True)])
+def test_row_kernel_on_payloads_written_by_the_call_ahead(N, rows, short, E, k, bits, split):
+    """Steps in one stream over the same payload buffers, all queued when the first one starts: each sum is of its own step's
+    payloads, to the last value (the BF16 values end inside 16 bytes)."""
+    t, T, pls = _row_case(N, rows, short, E, k, bits, 0, split)
+    assert T * k % 8
+    g = torch.Generator(device="cuda").manual_seed(T)
+    steps = [[(torch.randn((T, E), generator=g, device="cuda") * 2).to(torch.bfloat16) for _ in range(N)] for _ in range(4)]
+    ptrs, P = [p.data_ptr() for p in pls], t.payload_bytes(T)
+    got = []
+    for path in (binding.PATH_GENERIC, binding.PATH_AUTO):
+        t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+        outs = [torch.empty((T, E), dtype=torch.float32, device="cuda") for _ in steps]
+        side = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(1 << 20)
+        for ys, out in zip(steps, outs):
+            t.quantize_pack_batch(0, [y.data_ptr() for y in ys], T, ptrs, P, stream=side.cuda_stream)
+            t.dequant_reduce(ptrs, T, out.data_ptr(), binding.TPQ_OUT_FP32, stream=side.cuda_stream)
+            if path == binding.PATH_GENERIC:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert t.device_status() == 0
+        got.append(outs)
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    t.close()
