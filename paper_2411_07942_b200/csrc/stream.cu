@@ -1162,7 +1162,7 @@ cudaError_t launch_dequant_stream(const DSParams &p, int fp32_out, cudaStream_t 
 // ----------------------------------------------------------------------------------------------
 // Dequantise + reduce for up to four devices: the row kernel (dequant.cu) at bit granularity.
 //
-// One persistent block per SM on a run of adjacent rows, DW_ROWS at a time (two in the first stage, which lands sooner).
+// One persistent block per SM on a run of adjacent rows, DW_ROWS at a time (fewer in the first stage, which lands sooner).
 // Warp 0 streams the devices' code rows and BF16 rows into a ring (two bulk copies per device and stage, between 16-byte
 // boundaries).  A main thread owns a group of 8 features with the steps of all devices in registers (0 at selected
 // features), funnels its bits out of two (three) words, stores the whole group and then overwrites the lanes of selected
@@ -1809,10 +1809,18 @@ cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *paylo
         const int per_run = pp.half_groups ? 2 : 1;
         const int64_t runs = c->sm_count / per_run;
         pp.rows_per_block = (T + runs - 1) / runs;
-        pp.first = pp.rows_per_block > DW_ROWS ? 2 : DW_ROWS;
+        // A short first stage lands sooner: it takes the rows that do not fill a stage, at least two, so that there are no more
+        // stages for it.  (Always two: 1000 rows of 1280 to 5120 features, 2 + 4 + 1 a block, 3.9 to 8.3 us, so 3.5 to 7.5 for one
+        // to four devices.)  A block of one
+        // stage has no ring: fewer barriers to set up, and shared memory left to the next launch's (148 x 3072 at 8 bits 2.2 to 3.0
+        // and 2.1 to 2.7 us).  (A ring of two stages where there are two is no gain: 1000 x 2048 at 8 bits 5.0 to 5.5 us, 5.6 to 5.9
+        // so, blocks of the next launch sharing an SM.)
+        const int odd = (int)((pp.rows_per_block - 1) % DW_ROWS) + 1;
+        pp.first = pp.rows_per_block <= DW_ROWS ? DW_ROWS : odd < 2 ? 2 : odd;
+        if (pp.rows_per_block <= DW_ROWS) pp.nstage = 1;
         const unsigned grid = (unsigned)((T + pp.rows_per_block - 1) / pp.rows_per_block * per_run);
         const int threads = 32 + DW_AUX + ((pp.half_groups ? pp.half_groups : G) + 31) / 32 * 32;
-        const size_t smem = dw_smem_bytes(dw_nd(c->N), pp.dev_bytes, k, nstage);
+        const size_t smem = dw_smem_bytes(dw_nd(c->N), pp.dev_bytes, k, pp.nstage);
         switch (c->bits) {
         case 2: e = launch_dequant_rows<2>(pp, fp32_out, grid, threads, smem, st); break;
         case 3: e = launch_dequant_rows<3>(pp, fp32_out, grid, threads, smem, st); break;
