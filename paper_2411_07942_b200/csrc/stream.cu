@@ -1270,7 +1270,7 @@ __device__ __forceinline__ void dw_rows(const uint8_t *stage, uint32_t dev_bytes
 // first row (within the block's run) of the block's it-th stage: a short first stage lands sooner
 __device__ __forceinline__ int dw_stage_row(int it, int first) { return it == 0 ? 0 : first + (it - 1) * DW_ROWS; }
 
-// ND: 2, 4 or 8, at least the number of devices.  A stage has room for ND; where there are fewer, the last ones have steps of 0
+// ND: 2, 3, 4, 6 or 8, at least the number of devices.  A stage has room for ND; where there are fewer, the last ones have steps of 0
 // and whatever bits lie in their part: every pattern decodes to a finite code, and fma(code, 0, acc) is acc (never -0).
 //
 // SPLIT (five to eight devices on rows of more than 320 groups): two blocks share a run of rows.  Each stages its half of every row (a
@@ -1588,7 +1588,9 @@ __global__ void __launch_bounds__(dw_main(ND) + DW_AUX + 32, 1) dequant_stream_r
     }
 }
 
-int dw_nd(int N) { return N <= 2 ? 2 : N <= 4 ? 4 : 8; }
+// (Three as four: 1000 x 2048 to 5120, 4 bits, 5.0 to 7.8 us, as three 4.7 to 6.6; 8192 x 2048 31 and 26.  Five as eight: 4000 x
+// 2560 22 us, as six 18; 8192 x 2048 32 and 26.)
+int dw_nd(int N) { return N <= 2 ? 2 : N <= 4 ? N : N <= 6 ? 6 : 8; }
 
 // two blocks to a run of rows
 bool dw_split(const tpq_ctx *c) { return (c->E - c->k + 7) / 8 > dw_main(dw_nd(c->N)); }
@@ -1630,7 +1632,10 @@ cudaError_t launch_dequant_rows(const DWParams &pp, int fp32_out, unsigned grid,
 {
     switch (dw_nd(pp.d.N)) {
     case 2: return launch_dequant_rows_nd<B, 2, false>(pp, fp32_out, grid, threads, smem, st);
+    case 3: return launch_dequant_rows_nd<B, 3, false>(pp, fp32_out, grid, threads, smem, st);
     case 4: return launch_dequant_rows_nd<B, 4, false>(pp, fp32_out, grid, threads, smem, st);
+    case 6: return pp.half_groups ? launch_dequant_rows_nd<B, 6, true>(pp, fp32_out, grid, threads, smem, st)
+                                  : launch_dequant_rows_nd<B, 6, false>(pp, fp32_out, grid, threads, smem, st);
     default: break;
     }
     return pp.half_groups ? launch_dequant_rows_nd<B, 8, true>(pp, fp32_out, grid, threads, smem, st)
