@@ -1273,7 +1273,7 @@ __device__ __forceinline__ int dw_stage_row(int it, int first) { return it == 0 
 // ND: 2, 3, 4, 6 or 8, at least the number of devices.  A stage has room for ND; where there are fewer, the last ones have steps of 0
 // and whatever bits lie in their part: every pattern decodes to a finite code, and fma(code, 0, acc) is acc (never -0).
 //
-// SPLIT (five to eight devices on rows of more than 320 groups): two blocks share a run of rows.  Each stages its half of every row (a
+// SPLIT (six to eight devices on rows of more than 320 groups): two blocks share a run of rows.  Each stages its half of every row (a
 // copy per device and row) and the BF16 rows, decodes its groups, adds up the selected features that lie among them (the
 // second block also those at or above L) and decodes the columns whose codes lie there.
 template <int B, int ND, bool SPLIT, bool FP32OUT, bool HAS_BIAS>
@@ -1601,17 +1601,40 @@ uint32_t dw_part_bytes(const tpq_ctx *c)
     return dw_split(c) ? DW_ROWS * dw_pitch((G + 1) / 2, c->bits) : dw_dev_bytes(L, c->bits);
 }
 
-// Ring depth; 0: the shape is the panel kernel's.  Five to eight devices: the 320 groups that a block has registers for, and rows
-// wide enough to give it warps (panel kernel and this one, us: 8 devices 1000 x 2304 11.5 and 7.3, 4000 x 2304 25.8 and 20.6,
-// 2000 x 2560 at 8 bits 20.1 and 13.2; 5 devices 15.2 and 12.2; 8 x 8000 x 1088 30.7 and 29.3, 5 devices 24.8 and 29.1; 8 x
-// 1000 x 576 4.9 and 5.9).  Wider rows, two blocks to a run: six devices or more and up to 8 rows an SM (8 devices 64 x 4608 4.5
-// and 3.0, 1000 x 4608 13.3 and 12.9, at 8 bits 15.4 and 13.4; 6 devices 200 x 3008 4.2 and 3.9; 4000 x 4608 40.9 and 41.8; 5
-// devices 1000 x 4416 11.0 and 11.8).
+// Whether this kernel is ahead of the panel kernel, six to eight devices and two blocks to a run of rows.  Both sides in ns, fitted
+// to 1200 launches of each (64 to 1184 rows of 2624 to 5120 features, every width; 4 % off on average, 28 % at worst).  Here a row
+// takes a copy per device and half, so its time hardly depends on the width.  The panel kernel takes steps: blocks of 16 rows,
+// one to an SM, two, or two with several chunks each; it is at its best where they fill one wave (8 x 740 x 2624, 3 bits, 7.1 us
+// against 9.1 here; 888 rows 11.3 and 10.1).  What this picks took 1.005 times as long as the faster of the two on average, 1.18 at
+// worst.
+bool dw_split_ahead(const tpq_ctx *c, int64_t T)
+{
+    struct { double one, one_dev, one_load, more, chunk, chunk_dev, load; } const fit[3] = {
+        {2690, 212, 65, 1680, 1640, 172, 147},   // 2 bits
+        {3470, 129, 62, 1590, 2050, 169, 171},   // 3 and 4 bits
+        {1850, 454, 75, 2310, 576, 473, 179}};   // more: two devices to a step instead of four
+    const auto &f = fit[c->bits == 2 ? 0 : c->bits <= 4 ? 1 : 2];
+    constexpr int RC = DS_THREADS / DS_CG * DS_R;  // rows of a chunk there
+    const int N = c->N, sm = c->sm_count, G = (c->E - c->k + 7) / 8, nd = dw_nd(N), warps = ((G + 1) / 2 + 31) / 32;
+    const int panels = (G + DS_CG - 1) / DS_CG;
+    const int64_t chunks = (T + RC - 1) / RC, room = 2 * sm / panels, deep = room < chunks ? room : chunks, runs = sm / 2;
+    const double load = (double)(panels * chunks) / sm, per_block = (double)((chunks + deep - 1) / deep);
+    const double panel = panels * deep <= sm ? f.one + (f.one_dev + f.one_load * load) * N
+                                             : f.more + per_block * (f.chunk + f.chunk_dev * N) + f.load * load * N;
+    return 1620.0 + 119.0 * nd + (double)((T + runs - 1) / runs) * (200.0 + nd * (16.4 + 5.9 * warps)) < panel;
+}
+
+// Ring depth; 0: the shape is the panel kernel's.  Up to four devices: this one.  Five to eight: from 160 groups on (below, 1024
+// features, 0.5 to 0.9 times the panel kernel's time up to 444 rows, 1.0 to 1.5 beyond).  Rows of 160 to 199 groups leave a
+// block five to seven warps: up to 16 rows an SM 0.6 to 1.05, beyond 0.95 to 1.2 at 2 to 4 bits, where the panel kernel's third
+// panel is nearly full, 0.9 to 1.05 at more and 0.65 to 0.95 at 8.  From 200 groups on 0.55 to 1.0 times.  Above 320, two blocks
+// to a run of rows: six devices or more, up to 8 rows an SM.
 int dw_stages(const tpq_ctx *c, int64_t T, int64_t out_stride)
 {
     const int L = c->E - c->k, G = (L + 7) / 8;
     if (c->N > 8 || c->E % 8 || out_stride % 8 || G > 640 || c->k > DW_MAX_K || (c->N > 4 && G < 160)) return 0;
-    if (dw_split(c) && (c->N < 6 || T > 8 * c->sm_count)) return 0;
+    if (c->N > 4 && G < 200 && T > 16 * c->sm_count && c->bits < (c->N > 5 ? 5 : 8)) return 0;
+    if (dw_split(c) && (c->N < 6 || T > 8 * c->sm_count || !dw_split_ahead(c, T))) return 0;
     int n = 4;
     while (n > 1 && dw_smem_bytes(dw_nd(c->N), dw_part_bytes(c), c->k, n) > (size_t)c->smem_optin) --n;
     return n > 1 ? n : 0;

@@ -338,3 +338,28 @@ def test_row_kernel_on_payloads_written_by_the_call_ahead(N, rows, short, E, k, 
         got.append(outs)
     assert all(torch.equal(a, b) for a, b in zip(*got))
     t.close()
+
+
+@pytest.mark.parametrize("N,T,E,k,bits,reducer", [
+    # five to eight devices: one group too few; 160 to 199 groups up to 16 rows an SM and above, by width; from 200 on
+    (8, 300, 1280, 15, 4, "dequant_stream<"), (7, 2368, 1408, 22, 3, "dequant_stream_rows<"), (7, 2369, 1408, 22, 3, "dequant_stream<"),
+    (5, 2369, 1408, 22, 7, "dequant_stream<"), (6, 2369, 1408, 22, 5, "dequant_stream_rows<"), (5, 2369, 1408, 22, 8, "dequant_stream_rows<"),
+    (5, 2369, 1624, 22, 2, "dequant_stream_rows<"),
+    # two blocks to a run of rows: where the panel kernel's blocks fill one wave and need two, the most rows, too few devices
+    (8, 740, 2624, 41, 3, "dequant_stream<"), (8, 888, 2624, 41, 3, "dequant_stream_rows<"), (8, 1184, 5120, 80, 8, "dequant_stream_rows<"),
+    (8, 1185, 5120, 80, 8, "dequant_stream<"), (5, 64, 4608, 72, 3, "dequant_stream<")])
+def test_which_reduction_serves_a_call(N, T, E, k, bits, reducer):
+    """The rule's lines for five to eight devices (148 SMs), each side the same sums as the shape-generic kernel."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the lines are stated for 148 SMs")
+    t, _, pls = _row_case(N, 1, 148 - T, E, k, bits, 0)
+    ptrs, got = [p.data_ptr() for p in pls], []
+    for path in (binding.PATH_GENERIC, binding.PATH_AUTO):
+        t.set_option(binding.TPQ_OPT_KERNEL_PATH, path)
+        out = torch.empty((T, E), dtype=torch.float32, device="cuda")
+        names = _kernels(lambda: t.dequant_reduce(ptrs, T, out.data_ptr(), binding.TPQ_OUT_FP32))
+        assert (reducer if path == binding.PATH_AUTO else "dequant_generic") in names
+        assert t.device_status() == 0
+        got.append(out)
+    assert torch.equal(*got)
+    t.close()
