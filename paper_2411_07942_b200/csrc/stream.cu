@@ -1849,13 +1849,13 @@ cudaError_t tpq_launch_dequant_stream(const tpq_ctx *c, const void *const *paylo
         const unsigned grid = (unsigned)((T + pp.rows_per_block - 1) / pp.rows_per_block * per_run);
         const int threads = 32 + DW_AUX + ((pp.half_groups ? pp.half_groups : G) + 31) / 32 * 32;
         size_t smem = dw_smem_bytes(dw_nd(c->N), pp.dev_bytes, k, pp.nstage);
-        // Blocks of several stages get an SM each: where two fit (narrow rows, or a device count that needs few registers) the next
-        // launch's blocks start two to an SM on the SMs that are free first, and the launch waits for those.  (1500 rows of 1024
-        // features, one to four devices, 3 to 8 bits, back to back: 0.83, 0.73, 0.78 and 0.81 times the time of the kernel that
-        // counted the devices at run time without this, 0.74, 0.65, 0.66 and 0.64 so; 3 x 3000 x 2304 0.98 and 0.73.  Blocks of
-        // one stage are better off two to an SM: 296 rows of 1536 1.03 and 1.10.)
+        // Where there are fewer blocks than SMs each gets one to itself: if two fit (narrow rows, or a device count that needs few
+        // registers) the next launch's blocks start two to an SM on the SMs that are free first, and the launch waits for those.
+        // (One to four devices of 512 to 3072 features, back to back, the time without this 1: 500 rows 0.96, 1500 rows of 1024
+        // features 0.83, 3 x 3000 x 2304 0.74.  With a block for every SM two to one are no loss, and their prologues overlap: 740
+        // rows 0.97 of the time with one, 1184 rows 0.98.)
         constexpr size_t ONE_PER_SM = 116 * 1024;
-        if (pp.rows_per_block > DW_ROWS && smem < ONE_PER_SM) smem = ONE_PER_SM;
+        if ((int)grid < c->sm_count && smem < ONE_PER_SM) smem = ONE_PER_SM;
         switch (c->bits) {
         case 2: e = launch_dequant_rows<2>(pp, fp32_out, grid, threads, smem, st); break;
         case 3: e = launch_dequant_rows<3>(pp, fp32_out, grid, threads, smem, st); break;
