@@ -46,7 +46,7 @@ cudaError_t dalloc(T **p, size_t n)
 
 void free_tables(tpq_tables &t)
 {
-    cudaFree(t.m); cudaFree(t.M); cudaFree(t.R); cudaFree(t.Rbar); cudaFree(t.key); cudaFree(t.s); cudaFree(t.inv_s);
+    cudaFree(t.m); cudaFree(t.M); cudaFree(t.R); cudaFree(t.Rbar); cudaFree(t.s); cudaFree(t.inv_s);
     cudaFree(t.s_k); cudaFree(t.s_slot); cudaFree(t.flag); cudaFree(t.hpre); cudaFree(t.pos); cudaFree(t.hp_idx);
     cudaFree(t.lp_idx); cudaFree(t.hole); cudaFree(t.filler); cudaFree(t.grp); cudaFree(t.status); cudaFree(t.push_done);
     memset(&t, 0, sizeof t);
@@ -191,7 +191,6 @@ tpq_status tpq_create(tpq_ctx **out, int n_shards, int n_features, int bits, flo
     if (e == cudaSuccess) e = dalloc(&t.M, NE);
     if (e == cudaSuccess) e = dalloc(&t.R, NE);
     if (e == cudaSuccess) e = dalloc(&t.Rbar, E);
-    if (e == cudaSuccess) e = dalloc(&t.key, E);
     if (e == cudaSuccess) e = dalloc(&t.s, NE);
     if (e == cudaSuccess) e = dalloc(&t.inv_s, NE);
     if (e == cudaSuccess) e = dalloc(&t.s_k, NE);
