@@ -10,8 +10,9 @@
 //                         which one row ends and the next begins; no barrier between warps; with a push mode
 //   quantize_stream_tile  any other rows: a block quantises 8 rows into bit strings in shared memory, then writes the
 //                         tile's bytes (8*L*B bits are a whole number of bytes) as words funnelled out of the strings
-//   dequant_stream_rows   up to four devices: the row kernel, code rows by bulk copies into a ring
-//   dequant_stream        more: a block's panel of code words comes in by 16-byte copies from the aligned place at or
+//   dequant_stream_rows   up to four devices, and five to eight where it is ahead: the row kernel, code rows by bulk copies into
+//                         a ring, one block or two to a run of rows
+//   dequant_stream        any others: a block's panel of code words comes in by 16-byte copies from the aligned place at or
 //                         below each row's first bit
 // Which calls they serve is decided in tpq_api.cu, by the rules at the end of this file.
 // Arithmetic as everywhere: u = fl(x * inv_s), clamp, round to nearest even; acc = fma(code, s, acc) over the
@@ -320,9 +321,9 @@ cudaError_t launch_quantize_tile(const QSParams &p, bool vec, int threads, dim3 
 //   and 16 of its first, or-ed together), for every row of the block and the row ahead of it.
 // A block may therefore start at any row.  Measured at 4 x 2048 x 5120, 51 selected, back to back: 23.1 us against 16.3 us
 // for its bytes at the copy rate (strings of whole tiles with a barrier of all consumers per 4 rows 43 us; one tile of 8 rows
-// per block, four blocks per SM, 29.5 us; the shape-generic kernel 114 us); 3 bits 25.0 us, 6 bits 28.0 us, 8 x 1000 x 4608 at
-// 8 bits 25.2 us.  Nearest limit: instruction issue.  A warp executes 102 instructions per 32 groups and row at 4 bits, 112 at 3,
-// 131 at 8, which take 67 to 71 % of the issue slots of the launch, with DRAM at a third.
+// per block, four blocks per SM, 29.5 us; the shape-generic kernel 114 us); 3 bits 24.5 us, 6 bits 26.9 us, 8 x 1000 x 4608 at
+// 8 bits 23.8 us.  Nearest limit: instruction issue.  A warp executes 103 instructions per 32 groups and row at 4 bits, 113 at 3,
+// 126 at 8, which take 71 to 74 % of the issue slots of the launch, with DRAM at a third.
 constexpr int QS_STAGE = 4;             // rows of a stage
 constexpr int QS_MAX_THREADS = 768;     // 80 registers a thread
 constexpr int QS_MAX_GPT = 2;           // groups of a consumer lane
@@ -769,9 +770,9 @@ cudaError_t launch_quantize_pipe(const QPipeParams &pp, bool push, int gpt, int 
 // the alignment: a segment starts at any bit, so the copies start at the 16-byte boundary at or below it and a
 // thread funnels its 8*B bits out of two (three) words; the shift is the same for all devices, so it is worked
 // out once per chunk and row.  Blocks are half the size, two to an SM, so that one's barrier hides behind the other's work.
-// 8 x 1000 x 4608 at 8 bits 15.4 us back to back (7.2 us for its bytes at the copy rate; one block of 512 threads per SM 22.1).
-// 61 instructions per warp of 32 groups and device take 52 % of the issue slots: 14 warps an SM (109 registers a thread) leave
-// one eligible a cycle between the chunk's barriers.
+// 5 x 1000 x 4608 at 8 bits 12.0 us back to back (5.0 us for its bytes at the copy rate), 8 devices 15.4 (one block of 512 threads
+// per SM 22.1).  With 8 devices 61 instructions per warp of 32 groups and device take 52 % of the issue slots: 14 warps an SM (109
+// registers a thread) leave one eligible a cycle between the chunk's barriers.
 // ----------------------------------------------------------------------------------------------
 constexpr int DS_THREADS = 256;  // two blocks share an SM, so that one's barrier hides behind the other's work
 constexpr int DS_CG = 64;        // groups of a panel
@@ -1160,21 +1161,24 @@ cudaError_t launch_dequant_stream(const DSParams &p, int fp32_out, cudaStream_t 
 }
 
 // ----------------------------------------------------------------------------------------------
-// Dequantise + reduce for up to four devices: the row kernel (dequant.cu) at bit granularity.
+// Dequantise + reduce for up to eight devices: the row kernel (dequant.cu) at bit granularity.  (When it is taken: dw_stages.)
 //
-// One persistent block per SM on a run of adjacent rows, DW_ROWS at a time (fewer in the first stage, which lands sooner).
+// One persistent block per SM on a run of adjacent rows, DW_ROWS at a time (fewer in the first stage, which lands sooner); for
+// rows of six to eight devices whose steps one block has no registers for, two blocks to a run (SPLIT below).
 // Warp 0 streams the devices' code rows and BF16 rows into a ring (two bulk copies per device and stage, between 16-byte
 // boundaries).  A main thread owns a group of 8 features with the steps of all devices in registers (0 at selected
 // features), funnels its bits out of two (three) words, stores the whole group and then overwrites the lanes of selected
 // features with the sums the auxiliary warps left in shared memory (same thread, same address: ordered).  An auxiliary
 // thread per rank h adds up the devices' BF16 values of selected feature h and decodes column L + h of the output where that
 // is a filler feature.  No warp waits for another's global stores.
-// What bounds it is the auxiliary warps' latency per stage (without selected features 9.6 us at 4 x 2048 x 5120, 3 bits), then
-// the decode.  Back to back, with the BF16 values loaded from memory a stage ahead, general loops in the auxiliary warps
-// and a device count read at run time, against this form: 4 x 2048 x 5120, 51 selected 14.9 and 12.0 us, 3 bits 14.5 and
-// 11.9, 6 bits 16.4 and 13.5; two devices 11.2 and 8.5; three 12.7 and 11.5 (6.6, 5.8, 8.2, 4.9 and 5.8 us for the bytes; the
-// Int4 row kernel 10.8).  Either half alone loses: the staged values behind general loops take 15.9 us, the compile-time
-// device count without them 15.2.
+// Four devices: 48 (4 bits) and 49 (3 bits) instructions per warp of 32 groups and device take 61 to 63 % of the issue slots and the
+// ALU pipe half of its cycles, with 1.7 to 1.8 eligible warps; the rest is the prologue and the drain.  Two blocks to a run, eight
+// devices at 8 bits: 41 instructions, 40 % of the slots, 0.7 eligible warps: 13 warps an SM (128 registers a thread) that wait
+// for loads.  Back to back, with the BF16 values loaded from memory a stage ahead, general loops in the auxiliary warps and a
+// device count read at run time, against this form: 4 x 2048 x 5120, 51 selected 15.0 and 12.0 us, 3 bits 14.6 and 11.7, 8 bits
+// 16.3 and 13.8; two devices 3 bits 11.1 and 8.3; three 12.8 and 10.3 (6.5, 5.8, 9.7, 4.5 and 5.1 us for the bytes; the Int4 row
+// kernel 10.8).  Either half alone loses: the staged values behind general loops take 15.9 us, the compile-time device count
+// without them 15.2.
 // ----------------------------------------------------------------------------------------------
 constexpr int DW_ROWS = 4, DW_AUX = 96, DW_MAX_K = 384;
 // most groups of a row, by the devices whose steps a main thread keeps in registers
