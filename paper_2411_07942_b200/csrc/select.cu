@@ -57,10 +57,10 @@ __global__ void __launch_bounds__(RG_THREADS) ranges_kernel(const float *m, cons
 // Rbar_a > Rbar_j, or Rbar_a == Rbar_j and a < j.  O(E^2) comparisons, a warp per feature: its lanes compare side by
 // side, four values per load (a few tens of KB, so the loads hit L1).  (One thread per feature, the values
 // through shared memory, left all but 18 SMs idle: 68 us at E = 4608.)
-// The keys are made once, by the kernel ahead, and lie in the array of the slots, which the tables' kernel writes when this one
-// has ended (one allocation less for a new context, whose nineteen take 400 to 850 us).  Those ahead of j's own four are
-// compared with one less: a comparison and an addition each.  (With the key made anew at every comparison, us per call:
-// 2 x 32768 380 and now 203, 2 x 131072 5250 and 2460; as comparisons of the values and their places 310 and 4100.)
+// The keys are made once, by the kernel ahead, and lie in the array of the prefix counts, which the kernels behind this one fill and
+// nobody else reads.  Those ahead of j's own four are compared with one less: a comparison and an addition each.  (With the key
+// made anew at every comparison, us per call: 2 x 32768 380 and now 203, 2 x 131072 5250 and 2460; as comparisons of the values
+// and their places 310 and 4100.)
 constexpr int TK_WARPS = 8;
 
 __global__ void __launch_bounds__(32 * TK_WARPS) topk_flags_kernel(const int32_t *key, int E, int k, uint8_t *flag)
@@ -257,13 +257,13 @@ cudaError_t tpq_launch_ranges(const tpq_tables &t, int N, int E, int bits, cudaS
 {
     ++*launches;
     return tpq_launch_pdl(ranges_kernel, dim3((E + RG_THREADS - 1) / RG_THREADS), dim3(RG_THREADS), 0, st, t.m, t.M, N, E,
-                          (float)((1 << bits) - 1), t.R, t.Rbar, t.pos, t.s, t.inv_s);
+                          (float)((1 << bits) - 1), t.R, t.Rbar, t.hpre, t.s, t.inv_s);
 }
 
 cudaError_t tpq_launch_topk_flags(const tpq_tables &t, int E, int k, cudaStream_t st, int64_t *launches)
 {
     ++*launches;
-    return tpq_launch_pdl(topk_flags_kernel, dim3((E + TK_WARPS - 1) / TK_WARPS), dim3(32 * TK_WARPS), 0, st, t.pos, E, k, t.flag);
+    return tpq_launch_pdl(topk_flags_kernel, dim3((E + TK_WARPS - 1) / TK_WARPS), dim3(32 * TK_WARPS), 0, st, t.hpre, E, k, t.flag);
 }
 
 cudaError_t tpq_launch_tables(const tpq_tables &t, int N, int E, int k, cudaStream_t st, int64_t *launches)

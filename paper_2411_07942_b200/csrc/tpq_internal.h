@@ -18,9 +18,9 @@ struct tpq_tables {
     float *s_k;          // [N][E] step with 0 at selected features (dequantiser's copy)
     float *s_slot;       // [N][E] step of the feature held by code slot c (slot order; 0 for c >= E-k)
     uint8_t *flag;       // [E]    1 = selected (kept in BF16)
-    int32_t *hpre;       // [E]    number of selected features before j
-    int32_t *pos;        // [E]    >= 0: code slot of feature j; < 0: -(h+1), h = rank among selected.  (While the tables are
-                         //        built: the aggregated range as an integer of the same order, select.cu.)
+    int32_t *hpre;       // [E]    number of selected features before j (until the tables are built: the aggregated range as an
+                         //        integer of the same order; used by select.cu only)
+    int32_t *pos;        // [E]    >= 0: code slot of feature j; < 0: -(h+1), h = rank among selected
     int32_t *hp_idx;     // [E]    first k entries: selected features, ascending
     int32_t *lp_idx;     // [E]    first L = E-k entries: feature held by code slot c (slot order below)
     int32_t *hole;       // [E]    first n_holes entries: selected features below L, ascending (slots to fill)
