@@ -309,3 +309,37 @@ def test_exchange_classes_with_one_rank():
             assert np.array_equal(out.view(torch.int16).cpu().numpy().view(np.uint16), want), (step, ex)
     assert push.step_no == 4
     t.close()
+
+
+def test_a_step_without_the_extension_module(monkeypatch):
+    """Every call of a step through ctypes alone gives the bytes and sums that the extension module's calls give."""
+    N, T, E, K = 2, 300, 1024, 128
+    t, _, ys = _ctx(N, T, E, 16, 4)
+    dev = [gu.dev_bf16(y) for y in ys]
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x, w = ((torch.randn(shape, generator=g, device="cuda")).to(torch.bfloat16) for shape in ((T, K), (E, K)))
+    slots = torch.empty_like(w)
+    t.permute_weight(w.data_ptr(), K, slots.data_ptr())
+    bias = torch.randn(E, generator=g, device="cuda")
+    P, got = t.payload_bytes(T), []
+    for calls in (binding._calls, binding._ctypes_only):
+        monkeypatch.setattr(binding, "_calls", calls)
+        pls = [torch.zeros(P, dtype=torch.uint8, device="cuda") for _ in range(2 * N + 1)]
+        outs = [torch.empty((T, E), dtype=torch.float32, device="cuda") for _ in range(3)]
+        words = torch.zeros(N, dtype=torch.int32, device="cuda")
+        ptrs = [p.data_ptr() for p in pls]
+        t.quantize_pack(0, dev[0].data_ptr(), T, ptrs[0], P)
+        t.quantize_pack_batch(0, [d.data_ptr() for d in dev], T, ptrs[:N], P)
+        for i in range(N):
+            t.quantize_pack_push(i, dev[i].data_ptr(), T, [ptrs[N + i]], [words.data_ptr() + 4 * i], P, 9)
+        t.linear_quantize_pack(0, x.data_ptr(), slots.data_ptr(), T, K, ptrs[2 * N], P)
+        t.dequant_reduce(ptrs[:N], T, outs[0].data_ptr(), binding.TPQ_OUT_FP32)
+        t.dequant_reduce(ptrs[:N], T, outs[1].data_ptr(), binding.TPQ_OUT_FP32, bias_ptr=bias.data_ptr())
+        t.dequant_reduce(ptrs[N:2 * N], T, outs[2].data_ptr(), binding.TPQ_OUT_FP32, arrived_ptr=words.data_ptr(), epoch=9)
+        t.calibrate_ranges(0, dev[0].data_ptr(), 1, T)
+        torch.cuda.synchronize()
+        assert t.device_status() == 0
+        got.append([*pls, *outs, words])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    assert torch.equal(got[0][0], got[0][N]) and torch.equal(got[0][2 * N + 1], got[0][2 * N + 3])
+    t.close()
