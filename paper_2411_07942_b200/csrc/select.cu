@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(RG_THREADS) ranges_kernel(const float *m, cons
 // side, four values per load (a few tens of KB, so the loads hit L1).  (One thread per feature, the values
 // through shared memory, left all but 18 SMs idle: 68 us at E = 4608.)
 // The keys are made once, by the kernel ahead, and lie in the array of the prefix counts, which the kernels behind this one fill and
-// nobody else reads.  Those ahead of j's own four are compared with one less: a comparison and an addition each.  (With the key
+// no step's kernel reads.  Those ahead of j's own four are compared with one less: a comparison and an addition each.  (With the key
 // made anew at every comparison, us per call: 2 x 32768 380 and now 203, 2 x 131072 5250 and 2460; as comparisons of the values
 // and their places 310 and 4100.)
 constexpr int TK_WARPS = 8;

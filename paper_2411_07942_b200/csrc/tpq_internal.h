@@ -19,7 +19,7 @@ struct tpq_tables {
     float *s_slot;       // [N][E] step of the feature held by code slot c (slot order; 0 for c >= E-k)
     uint8_t *flag;       // [E]    1 = selected (kept in BF16)
     int32_t *hpre;       // [E]    number of selected features before j (until the tables are built: the aggregated range as an
-                         //        integer of the same order; used by select.cu only)
+                         //        integer of the same order); read while a feature set is installed and by no step's kernel
     int32_t *pos;        // [E]    >= 0: code slot of feature j; < 0: -(h+1), h = rank among selected
     int32_t *hp_idx;     // [E]    first k entries: selected features, ascending
     int32_t *lp_idx;     // [E]    first L = E-k entries: feature held by code slot c (slot order below)
